@@ -91,7 +91,10 @@ int lbm3_set_fields(lbm3* h, const double* rho);
  * that the other tiles' share of the work leaves); the other tiles follow the wetting pass on an
  * internal higher-priority stream that is joined back before the call's work completes.  The
  * velocity of the last collision of the call is recorded for lbm3_fields / lbm3_diag.  A bulk
- * copy that does not complete within its wait limit is reported by the next lbm3_diag.  While more
+ * copy that does not complete within its wait limit is reported by the next lbm3_diag.  On grids
+ * with many pure tiles those around which one fluid is stored are advanced by a launch of their own
+ * that moves that fluid's populations only (the others' are zeros there), with the same results;
+ * its result does not depend on which launch takes a tile.  While more
  * than 8 steps remain, blocks of 8 steps are launched as one CUDA graph, captured on an internal
  * stream the first time it is needed (one graph per starting population buffer) and replayed on
  * the handle's stream: the same kernels in the same order, so the results do not depend on how
@@ -180,7 +183,8 @@ int lbm3_adjoint_release(lbm3* h);
 
 /* Size facts: out[0] = fluid nodes, out[1] = C_SB nodes, out[2] = algorithmic HBM bytes of the
  * fused step per timestep (216 B per fluid node with FP32 storage, 120 B with 16-bit offsets,
- * + 1 class byte per node), out[3] = fused-step launches per timestep, out[4] = wetting launches
+ * + 1 class byte per node; as if every node held all three fluids), out[3] = fused-step launches per
+ * timestep, out[4] = wetting launches
  * per timestep, out[5] = device bytes held by the handle, out[6] = algorithmic bytes of the
  * pure-tile launch, out[7] = nodes in pure tiles, out[8] = how the pure tiles move their
  * populations: 0 plain loads, 1 bulk tensor copies with two blocks per SM, 2 bulk tensor copies

@@ -68,9 +68,11 @@ struct lbm3 {
     long long pure_fluid = 0;
     // fluids present per tile (one byte per warp of the ring kernel's group, so no byte needs an
     // atomic or a clearing): pres[pp] describes the current state, the ring kernel writes the
-    // next one's for the pure tiles; every other tile keeps 0x07 (all fluids), and so does every
-    // tile after the state is replaced from outside.  pp turns with cur (and alone in the
-    // adjoint's slot-to-slot steps).
+    // next one's for the pure and wall tiles; every other tile keeps 0x07 (all fluids), and so does
+    // every tile after the state is replaced from outside.  While pp == cur, pres[b] describes
+    // buffer pop[b]: the planes of a fluid that a tile's word does not name hold zeros there, which
+    // launch_step_one relies on to leave them unwritten.  pp turns with cur (and alone in the
+    // adjoint's slot-to-slot steps, which therefore write every plane).
     uint64_t* pres[2] = {nullptr, nullptr};
     size_t pres_bytes = 0;
     int pp = 0;
@@ -80,6 +82,11 @@ struct lbm3 {
     // the wall tiles (the two sets are independent)
     cudaStream_t side2 = nullptr;
     cudaEvent_t ev_wet = nullptr, ev_join2 = nullptr;
+    // one: the pure tiles with one fluid around are launch_step_one's (kOneTiles); those with
+    // several run beside them on a third side stream
+    bool one = false;
+    cudaStream_t side3 = nullptr;
+    cudaEvent_t ev_join3 = nullptr;
     // CUDA graphs of kGraphSteps consecutive steps (an even count: a graph starts and ends on the
     // same population buffer), one per starting buffer, captured on the internal stream gcap
     // when lbm3_step first needs them and replayed on the caller's stream; dropped when a
@@ -199,9 +206,19 @@ void release(lbm3* h)
     if (h->ev_join) cudaEventDestroy(h->ev_join);
     if (h->ev_wet) cudaEventDestroy(h->ev_wet);
     if (h->ev_join2) cudaEventDestroy(h->ev_join2);
+    if (h->ev_join3) cudaEventDestroy(h->ev_join3);
+    if (h->side3) cudaStreamDestroy(h->side3);
     if (h->side2) cudaStreamDestroy(h->side2);
     if (h->side) cudaStreamDestroy(h->side);
 }
+
+// From this many pure tiles on, those with one fluid around are launch_step_one's, and the others
+// run beside them on a stream of their own.  Below it the step waits for the wetting pass and the
+// tiles after it, not for the pure tiles, and one more launch costs more than it hides: 2-3 % of
+// the step on 128 x 64 and on the 800 x 375 pillars (865 pure tiles), while the 2048 x 1024 ones
+// (6308) gain 12 %.  LBM3_ONE_TILES=<n> in the environment at lbm3_create sets another line (same
+// results).
+constexpr int kOneTiles = 4096;
 
 // Tensor maps of one [27][ny][nx] FP32 population buffer: as the two parts of the pull-source box
 // of a pure tile, (kTX + 8) x (kTY + 6) x kTmaPlanesA and x (27 - kTmaPlanesA) planes, and as its
@@ -304,18 +321,30 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
     if ((e = cudaEventRecord(h->ev_fork, h->stream)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) != cudaSuccess) return e;
     if (ev) record_timing(h, ev[0], h->stream);
-    if (h->ring)
-        launch_step_ring(h->P, h->tiles_pure, h->n_pure, h->ring_blocks, fo, u, io ? *h->io_box : h->tm_box[h->cur],
-                         pin, pout, h->stream);
-    else if (h->tma && h->precision == LBM3_FP32)
+    // pure tiles: those with several fluids around through the kernel of the storage and layout,
+    // those with one (launch_step_one) beside it; the two-blocks-per-SM kernel takes them all
+    if (h->n_pure > 0 && h->tma && h->precision == LBM3_FP32 && !h->ring) {
         launch_step_tma(h->P, h->tiles_pure, h->n_pure, h->tma_blocks, fo, u, h->tm_in_a[h->cur],
                         h->tm_in_b[h->cur], h->tm_out[1 - h->cur], h->stream);
-    else if (h->tma)
-        launch_step_tma16(h->precision, h->P, h->tiles_pure, h->n_pure, h->tma_blocks, fo, u, h->tm_in_a[h->cur],
-                          h->tm_in_b[h->cur], pin, pout, h->stream);
-    else
-        launch_step(h->precision, h->P, h->tiles_pure, h->n_pure, kTilesPure, fin, fo, h->type, h->Cw, u,
-                    pin, pout, h->stream);
+    } else if (h->n_pure > 0) {
+        const bool one = h->one;
+        cudaStream_t ms = one ? h->side3 : h->stream;
+        if (one && (e = cudaStreamWaitEvent(ms, h->ev_fork, 0)) != cudaSuccess) return e;
+        if (h->ring)
+            launch_step_ring(h->P, h->tiles_pure, h->n_pure, h->ring_blocks, fo, u,
+                             io ? *h->io_box : h->tm_box[h->cur], pin, pout, !one, ms);
+        else if (h->tma)
+            launch_step_tma16(h->precision, h->P, h->tiles_pure, h->n_pure, h->tma_blocks, fo, u, h->tm_in_a[h->cur],
+                              h->tm_in_b[h->cur], pin, pout, !one, ms);
+        else
+            launch_step(h->precision, h->P, h->tiles_pure, h->n_pure, kTilesPure, fin, fo, h->type, h->Cw, u,
+                        pin, pout, ms, !one);
+        if (one) {
+            launch_step_one(h->precision, h->P, h->tiles_pure, h->n_pure, fin, fo, u, pin, pout, io, h->stream);
+            if ((e = cudaEventRecord(h->ev_join3, ms)) != cudaSuccess) return e;
+            if ((e = cudaStreamWaitEvent(h->stream, h->ev_join3, 0)) != cudaSuccess) return e;
+        }
+    }
     if (ev) record_timing(h, ev[1], h->stream);
     if (ev) record_timing(h, ev[2], h->side);
     launch_wet(h->precision, h->P, h->nw, h->widx, h->wnrm, h->wang, fin, h->type, h->Cw, h->wcache, h->side,
@@ -686,12 +715,14 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
         e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
         if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, hi);
         if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, hi);
+        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side3, cudaStreamNonBlocking, hi);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->gcap, cudaStreamNonBlocking);
     }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_wet, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join2, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join3, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemcpy(h->type, cls.data(), N, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !widx.empty()) e = cudaMemcpy(h->widx, widx.data(), widx.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !wnrm.empty()) e = cudaMemcpy(h->wnrm, wnrm.data(), wnrm.size() * sizeof(double), cudaMemcpyHostToDevice);
@@ -744,6 +775,12 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
                 }
             }
         }
+    }
+    {
+        // the two-blocks-per-SM kernel takes every pure tile itself
+        const char* ov = std::getenv("LBM3_ONE_TILES");
+        const bool tma_only = h->tma && g->precision == LBM3_FP32 && !h->ring;
+        h->one = !tma_only && h->n_pure >= std::max(1, ov ? std::atoi(ov) : kOneTiles);
     }
     if (e != cudaSuccess) {
         const int code = e == cudaErrorMemoryAllocation ? LBM3_ERR_OOM : LBM3_ERR_CUDA;
@@ -1128,7 +1165,7 @@ int lbm3_adjoint_centroid(lbm3* h, int32_t nsteps, int32_t K, double* J_out, dou
                 } else {
                     r = slot_step(j, h->pop[1 - h->cur], true);  // the final state in the handle's buffer
                     h->cur = 1 - h->cur;
-                    if (h->pp != h->cur) pres_reset(h);
+                    pres_reset(h);  // the other word array describes a slot, not the other buffer
                 }
                 continue;
             }
@@ -1263,7 +1300,7 @@ int lbm3_info(const lbm3* h, int64_t out[9])
     // and 8 16-bit offsets (120 B); plus one class byte per node
     const long long per = h->precision == LBM3_FP32 ? 216 : 120;
     out[2] = h->n_fluid * per + h->P.N;
-    out[3] = (h->n_pure > 0) + (h->n_walltiles > 0) + (h->n_edgewall > 0) +
+    out[3] = (h->n_pure > 0) + h->one + (h->n_walltiles > 0) + (h->n_edgewall > 0) +
              (h->n_gen - h->n_walltiles - h->n_edgewall > 0);
     out[4] = h->nw > 0 ? 1 : 0;
     out[5] = (int64_t)h->bytes;

@@ -331,6 +331,10 @@ cudaError_t step_tma_prepare();
 cudaError_t step_tma16_prepare();
 void launch_step_tma(const Params& P, const int* tiles, int ntiles, int nblocks, const Pop& fout, float* u,
                      const CUtensorMap& tin_a, const CUtensorMap& tin_b, const CUtensorMap& tout, cudaStream_t s);
+// pure tiles around which pres_in holds one fluid, a warp each (any storage, any nx); the launches
+// below leave those out unless `all` is set; full_write: fout is not the buffer that pres_out described before this step
+void launch_step_one(int store, const Params& P, const int* tiles, int ntiles, const Pop& fin, const Pop& fout,
+                     float* u, const uint64_t* pres_in, uint64_t* pres_out, bool full_write, cudaStream_t s);
 // pure FP32 tiles through a ring of three bulk-copy buffers, one producer warp and two consumer
 // groups per block, one block per SM (nblocks blocks): tensor map of fin with the whole pull box
 // (kTX + 8, kTY + 6, 27) over the [27][ny][nx] buffer
@@ -338,14 +342,15 @@ size_t step_ring_smem_bytes();
 cudaError_t step_ring_prepare();
 // pres_in / pres_out: fluids present per tile in the step's input / output (see k_step_ring)
 void launch_step_ring(const Params& P, const int* tiles, int ntiles, int nblocks, const Pop& fout, float* u,
-                      const CUtensorMap& tin, const uint64_t* pres_in, uint64_t* pres_out, cudaStream_t s);
+                      const CUtensorMap& tin, const uint64_t* pres_in, uint64_t* pres_out, bool all,
+                      cudaStream_t s);
 // pure tiles of the 16-bit storage through bulk tensor copies (persistent, nblocks blocks): tensor
 // maps of the densities (box (kTX + 8, kTY + 6, 3) of [3][ny][nx] FP32) and of the offset planes
 // (box (kTX + 16, kTY + 6, 24) of [24][ny][nx] 16-bit words)
 size_t step_tma16_smem_bytes();
 void launch_step_tma16(int store, const Params& P, const int* tiles, int ntiles, int nblocks, const Pop& fout,
                        float* u, const CUtensorMap& trho, const CUtensorMap& toff, const uint64_t* pres_in,
-                       uint64_t* pres_out, cudaStream_t s);
+                       uint64_t* pres_out, bool all, cudaStream_t s);
 // tile lists of the fused step: pure tiles (no solid within 3 nodes, away from the domain
 // edge), wall tiles (solids near, halo inside the domain) and edge tiles (halo crossing the
 // domain edge: wrap, ghost columns, seam)
@@ -354,7 +359,7 @@ constexpr int kTilesPure = 0, kTilesWall = 1, kTilesEdge = 2;
 // and write them (see k_step), the other kinds ignore them
 void launch_step(int store, const Params& P, const int* tiles, int ntiles, int kind, const Pop& fin,
                  const Pop& fout, const uint8_t* type, const double* Cw, float* u, const uint64_t* pres_in,
-                 uint64_t* pres_out, cudaStream_t s);
+                 uint64_t* pres_out, cudaStream_t s, bool all = false);
 void launch_init(int store, const Params& P, const double* rho, const uint8_t* type, const Pop& f,
                  cudaStream_t s);
 void launch_fields(int store, const Params& P, const Pop& f, const uint8_t* type, float* rho_out,

@@ -510,6 +510,19 @@ __device__ __forceinline__ void stress_at(const Params& P, const uint8_t (*t)[HX
     pair_stress(P.sig12, c[1], c[2], gxk[1], gyk[1], gxk[2], gyk[2], rho2, Txx, Txy, Tyy);
 }
 
+// Fluids stored in the 3 x 3 tiles around a tile that lies inside the domain: the OR of its and its
+// neighbours' words (one byte per row of a tile, bit k: fluid k).
+__device__ __forceinline__ int fluids_around(const uint64_t* __restrict__ pres, int tile, int ntx)
+{
+    uint64_t nb = 0;
+#pragma unroll
+    for (int m = 0; m < 9; m++) nb |= pres[tile + (m / 3 - 1) * ntx + m % 3 - 1];
+    nb |= nb >> 32;
+    nb |= nb >> 16;
+    nb |= nb >> 8;
+    return (int)(nb & 7u);
+}
+
 // resident blocks per SM the wall-tile specialisation of the one-tile-per-block step kernel is
 // compiled for (registers capped at 65536 / (256 x this)); the others for four
 #ifndef LBM3_STEP_BLOCKS_PER_SM
@@ -536,7 +549,7 @@ __global__ void __launch_bounds__(TX* TY, (INNER && !PURE) ? kStepBlocksPerSm : 
                                                   const double* __restrict__ Cw,
                                                   float* __restrict__ uout,
                                                   const uint64_t* __restrict__ pres_in,
-                                                  uint64_t* __restrict__ pres_out)
+                                                  uint64_t* __restrict__ pres_out, const int all)
 {
     constexpr int NT = TX * TY;
     constexpr int HX = TX + 6, HY = TY + 6;  // geometry region (halo 3)
@@ -559,6 +572,8 @@ __global__ void __launch_bounds__(TX* TY, (INNER && !PURE) ? kStepBlocksPerSm : 
     if (!PURE && tid == 0) s_flags[0] = 0;  // published by the phase-0 barrier
     const int ntx = (P.nx + TX - 1) / TX;
     const int tile = tiles[blockIdx.x];
+    // the pure tiles with one fluid around are k_step_one's
+    if (PURE && !all && __popc((unsigned)fluids_around(pres_in, tile, ntx)) == 1) return;
     const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
     const int nx = P.nx;
     const int N = (int)P.N;
@@ -773,7 +788,7 @@ __global__ void __launch_bounds__(TX* TY, (INNER && !PURE) ? kStepBlocksPerSm : 
         r1 = ((q[9] + (q[10] + q[12])) + (q[11] + q[13])) + ((q[14] + q[16]) + (q[15] + q[17]));
         r2 = ((q[18] + (q[19] + q[21])) + (q[20] + q[22])) + ((q[23] + q[25]) + (q[24] + q[26]));
     }
-    if constexpr (INNER && !PURE) {
+    if constexpr (INNER || PURE) {
         // the fluids this warp's fluid nodes hold, for the tiles around this one in the next step
         const int own = own_fluid ? (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0) : 0;
         const int w = __reduce_or_sync(0xffffffffu, own);
@@ -1131,6 +1146,180 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
+// collide_mrt without a force, for nodes that hold one fluid: the terms of F are exact zeros there,
+// so leaving them out changes no bit of the result (but for the sign of a zero).  __fmul_rn where
+// the product is rounded there before the (zero) term is added, so that it is not fused here.
+__device__ __forceinline__ void collide_mrt_free(float f[kQ], float rho, float s1, float& ux, float& uy)
+{
+    const float d0 = f[0] - kW0;
+    const float d1 = f[1] - kW1, d2 = f[2] - kW1, d3 = f[3] - kW1, d4 = f[4] - kW1;
+    const float d5 = f[5] - kW5, d6 = f[6] - kW5, d7 = f[7] - kW5, d8 = f[8] - kW5;
+    const float b14 = (d1 + d3) + (d2 + d4);
+    const float b58 = (d5 + d7) + (d6 + d8);
+    const float drho = (d0 + b14) + b58 + (float)kDRho;
+    const float de = (-4.0f * d0 - b14 + 2.0f * b58) + (float)kDE;
+    const float deps = (4.0f * d0 - 2.0f * b14 + b58) + (float)kDEps;
+    const float jx = (f[1] - f[3]) + (f[5] - f[7]) + (f[8] - f[6]);
+    const float qx = -2.0f * (f[1] - f[3]) + (f[5] - f[7]) + (f[8] - f[6]);
+    const float jy = (f[2] - f[4]) + (f[5] - f[7]) + (f[6] - f[8]);
+    const float qy = -2.0f * (f[2] - f[4]) + (f[5] - f[7]) + (f[6] - f[8]);
+    const float pxx = (f[1] - f[2]) + (f[3] - f[4]);
+    const float pxy = (f[5] - f[6]) + (f[7] - f[8]);
+    const float irho = __fdividef(1.0f, rho);
+    ux = __fmul_rn(jx, irho);
+    uy = __fmul_rn(jy, irho);
+    const float u2 = ux * ux + uy * uy;
+    const float s4 = __fdividef(8.0f * (2.0f - s1), 8.0f - s1);
+    const float dE = __fmul_rn(-s1, de + 2.0f * drho - 3.0f * rho * u2);
+    const float dEps = __fmul_rn(-s1, deps - drho + 3.0f * rho * u2);
+    const float dqx = __fmul_rn(-s4, qx + rho * ux);
+    const float dqy = __fmul_rn(-s4, qy + rho * uy);
+    const float dpxx = __fmul_rn(-s1, pxx - rho * (ux * ux - uy * uy));
+    const float dpxy = __fmul_rn(-s1, pxy - rho * ux * uy);
+    const float c0 = (1.0f / 9.0f) * (dEps - dE);
+    const float ca = -(1.0f / 36.0f) * dE - (1.0f / 18.0f) * dEps;
+    const float cd = (1.0f / 18.0f) * dE + (1.0f / 36.0f) * dEps;
+    const float X1 = (1.0f / 6.0f) * -dqx, Y1 = (1.0f / 6.0f) * -dqy;
+    const float X2 = __fmul_rn(1.0f / 12.0f, dqx), Y2 = __fmul_rn(1.0f / 12.0f, dqy);
+    const float P4 = 0.25f * dpxx, Q4 = 0.25f * dpxy;
+    f[0] += c0;
+    f[1] += ca + X1 + P4;
+    f[2] += ca + Y1 - P4;
+    f[3] += ca - X1 + P4;
+    f[4] += ca - Y1 - P4;
+    f[5] += cd + X2 + Y2 + Q4;
+    f[6] += cd - X2 + Y2 - Q4;
+    f[7] += cd - X2 - Y2 + Q4;
+    f[8] += cd + X2 - Y2 - Q4;
+}
+
+// fraction r / rho of a fluid as collide_node forms it: the quotient corrected by its FMA residual
+__device__ __forceinline__ float fraction(float r, float rho)
+{
+    const float ir = __fdividef(1.0f, rho);
+    const float q = r * ir;
+    return fmaf(fmaf(-q, rho, r), ir, q);
+}
+
+// density of one fluid from its 9 post-streaming populations, in the order of phase_fields
+__device__ __forceinline__ float sum9(const float* q)
+{
+    return ((q[0] + (q[1] + q[3])) + (q[2] + q[4])) + ((q[5] + q[7]) + (q[6] + q[8]));
+}
+
+// write c f_a as the populations of fluid l of node i
+template <int STORE>
+__device__ __forceinline__ void store_fluid(const Params& P, const Pop& out, int l, int i, const float f[kQ], float c)
+{
+    const int N = (int)P.N;
+    if constexpr (STORE == kStoreF32) {
+        float* o = out.f + i + l * kQ * N;
+#pragma unroll
+        for (int a = 0; a < kQ; a++) o[P.off_plane[a]] = c * f[a];
+    } else {
+        float v[kQ];
+#pragma unroll
+        for (int a = 0; a < kQ; a++) v[a] = __fmul_rn(c, f[a]);  // rounded here, as store_node gets it
+        const float r = ((v[0] + (v[1] + v[3])) + (v[2] + v[4])) + ((v[5] + v[7]) + (v[6] + v[8]));
+        out.rho[l * N + i] = r;
+#pragma unroll
+        for (int a = 1; a < kQ; a++) out.off[(8 * l + a - 1) * N + i] = enc16<STORE>(v[a] - wq(a) * r);
+    }
+}
+
+// One node that holds fluid k alone, from the 9 post-streaming populations f of that fluid: its
+// velocity and, in f, its post-collision populations; the same bits as collide_node and the
+// recolouring give with the other two fluids' zeros.  false where they would not be: a density
+// whose fraction does not come out as 1 (a zero, an infinity or a NaN), which spreads to the
+// populations of the absent fluids too.
+__device__ __forceinline__ bool collide_single(const Params& P, int k, float f[kQ], float r, float& ux, float& uy)
+{
+    const float c = fraction(r, r);
+    const float D = r * (k == 0 ? P.inv_nu0 : (k == 1 ? P.inv_nu1 : P.inv_nu2));
+    const float s1 = __fdividef(D, 0.5f * D + 3.0f);
+    collide_mrt_free(f, r, s1, ux, uy);
+    return c == 1.0f;
+}
+
+// Pure tiles around which the step's input holds one fluid k (pres_in): k alone is in the tile
+// after the pull (a fluid absent from all of a node's sources stays absent, and the recolouring
+// keeps it at zero), so 9 populations per node are pulled, collided and written: 72 B per node
+// (40 B in the 16-bit storage) instead of 216 (120).  The other fluids' planes have to read as
+// zeros to whoever reads all 27 there, and do without being written: pres_out[tile] still
+// describes the output buffer as it was written two steps ago, and only a fluid that it names in a
+// row is cleared there, once.  So the planes of a fluid that a tile's word does not name are zeros
+// in that buffer.  (full_write: the output is not the buffer that pres_out described, so they are
+// cleared always.)  The other pure tiles are left to the kernels that move all 27 planes.
+//
+// One warp per tile, a row of 32 nodes at a time, two rows in flight: nothing is shared between
+// threads, each population is read once, and the loads of a warp are whole lines but for the
+// shift by one node in x.  It is bound by HBM, so what counts is warps in flight: no shared memory,
+// no barriers.  On the 4096 x 2048 pillars, 97 % of whose pure tiles are such, the pure tiles take
+// 173 us a step beside the other kernels instead of 338 (FP16: 190 instead of 410), and the step 240
+// instead of 353 (FP16: 310 instead of 425).  (Inside the ring kernel, with 9-plane boxes, the same
+// tiles took 1200 cycles of a consumer group and 1500 of its one producer each: 270 us.)
+constexpr int kOneThreads = 128;
+template <int TX, int TY, int STORE>
+__global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const int* __restrict__ tiles,
+                                                          const int ntiles, const Pop fin, const Pop fout,
+                                                          float* __restrict__ uout,
+                                                          const uint64_t* __restrict__ pres_in,
+                                                          uint64_t* __restrict__ pres_out, const int full_write)
+{
+    static_assert(TX == 32 && TY == 8, "one warp per tile, one byte of its word per row");
+    const int w = blockIdx.x * (kOneThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (w >= ntiles) return;
+    const int ntx = (P.nx + TX - 1) / TX;
+    const int tile = tiles[w];
+    const int around = fluids_around(pres_in, tile, ntx);
+    if (__popc((unsigned)around) != 1) return;
+    const uint64_t old = full_write ? 0x0707070707070707ull : pres_out[tile];
+    const int k = __ffs(around) - 1;
+    const int nx = P.nx, N = (int)P.N;
+    const int i0 = (tile / ntx) * TY * nx + (tile % ntx) * TX + lane;
+    uint64_t word = 0;
+#pragma unroll 2
+    for (int row = 0; row < TY; row++) {
+        const int i = i0 + row * nx;
+        float f[kQ];
+        if constexpr (STORE == kStoreF32) {
+            const float* b = fin.f + i + k * kQ * N;
+#pragma unroll
+            for (int a = 0; a < kQ; a++) f[a] = __ldg(b + P.off_pull[a]);
+        } else {
+            const float* rb = fin.rho + i + k * N;
+            const unsigned short* ob = fin.off + i + 8 * k * N;
+            float d[kQ];
+#pragma unroll
+            for (int a = 1; a < kQ; a++) d[a] = dec16<STORE>(__ldg(ob + (a - 1) * N));
+            f[0] = wq(0) * __ldg(rb) - sum_offsets(d);
+#pragma unroll
+            for (int a = 1; a < kQ; a++)
+                f[a] = wq(a) * __ldg(rb + P.off_pull16[a]) + dec16<STORE>(__ldg(ob + P.off_pull16o[a]));
+        }
+        const float r = sum9(f);
+        float ux, uy;
+        const bool plain = collide_single(P, k, f, r, ux, uy);
+        if (uout) {
+            uout[i] = ux;
+            uout[N + i] = uy;
+        }
+        const bool all = __all_sync(0xffffffffu, plain);
+        const int rowold = (int)(old >> (8 * row)) & 7;
+        // fluids to write: k, and those that this row of the buffer still holds, as zeros; all of
+        // them where a density has no fraction
+        const int write = all ? rowold | 1 << k : 7;
+#pragma unroll 1
+        for (int l = 0; l < kNF; l++) {
+            if (!(write & (1 << l))) continue;
+            const float c = plain ? (l == k ? 1.0f : 0.0f) : fraction(l == k ? r : 0.0f, r);
+            store_fluid<STORE>(P, fout, l, i, f, c);
+        }
+        word |= (uint64_t)(all ? 1 << k : 7) << (8 * row);
+    }
+    if (lane == 0) pres_out[tile] = word;
+}
+
 // Pure FP32 tiles through a ring of bulk tensor copies, warp-specialised: one producer warp and
 // two consumer groups of TX x TY threads per block, one block per SM (persistent).  Tile j of the
 // block (tiles[blockIdx.x + j gridDim.x]) lands in ring buffer j % 3 -- its 27-plane pull box,
@@ -1144,10 +1333,9 @@ __device__ __forceinline__ void mbar_arrive(uint32_t bar)
 // up on a buffer that is never released, and before exiting it waits (full limit) for every copy
 // it issued, so no copy lands in the shared memory of a later block.  The arithmetic is that of
 // k_step_tma and k_step<PURE>, so the results are identical.
-// Each warp also records the fluids its nodes hold (one byte of pres_out[tile] per warp); when
-// the 3 x 3 tiles around a tile held one fluid in the step's input (pres_in, read by the
-// producer), the tile is single-fluid after the pull, and its consumers skip the halo's phase
-// fields and the presence barrier, which only decide that (same results, fewer instructions).
+// The tiles with one fluid around are k_step_one's unless all is set; the producer passes over them, 32 at a time
+// (each lane looks one up).  Each warp records the fluids its nodes hold (one byte of
+// pres_out[tile] per warp), so that the tiles around know in the next step.
 constexpr int kRingBufs = 3;
 template <int TX, int TY>
 __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params P, const int* __restrict__ tiles,
@@ -1155,7 +1343,7 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
                                                                     float* __restrict__ uout,
                                                                     const __grid_constant__ CUtensorMap tm_in,
                                                                     const uint64_t* __restrict__ pres_in,
-                                                                    uint64_t* __restrict__ pres_out)
+                                                                    uint64_t* __restrict__ pres_out, const int all)
 {
     constexpr int NT = TX * TY;               // threads of a consumer group
     constexpr int NW = NT / 32;               // warps of a consumer group
@@ -1172,8 +1360,7 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
     __shared__ float s_txx[2][RY][RX], s_txy[2][RY][RX], s_tyy[2][RY][RX];
     __shared__ __align__(8) uint64_t s_full[2 * kRingBufs], s_empty[kRingBufs];
     __shared__ int s_flags[2][2];
-    __shared__ int s_single[2 * kRingBufs];  // by full-barrier slot: the tile's 3 x 3 tiles hold one fluid
-    __shared__ int s_tile[2 * kRingBufs];    // by full-barrier slot: the tile
+    __shared__ int s_tile[2 * kRingBufs];  // by full-barrier slot: the tile
     extern __shared__ unsigned char dsm[];
     float* ring = reinterpret_cast<float*>(dsm + ((128u - (smem_u32(dsm) & 127u)) & 127u));  // [3][27][BY][BX]
 
@@ -1191,51 +1378,40 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
 
     // ---------------- producer warp ----------------
     if (warp == 2 * NW) {
-        if (lane != 0) return;
-        // fluids stored in the 3 x 3 tiles around a tile (a pure tile is inner, so they exist)
-        auto around = [&](int t) {
-            uint64_t nb = 0;
-#pragma unroll
-            for (int dy = -1; dy <= 1; dy++)
-#pragma unroll
-                for (int dx = -1; dx <= 1; dx++) nb |= pres_in[t + dy * ntx + dx];
-            nb |= nb >> 32;
-            nb |= nb >> 16;
-            nb |= nb >> 8;
-            return (int)(nb & 7u);
-        };
-        // tile indices are loaded two tiles ahead and the fluids around a tile one tile ahead, so
-        // that no load waits on another within a tile and their latency passes while the
-        // producer waits for a free buffer
-        auto tile_at = [&](int jj) { return jj < njobs ? tiles[blockIdx.x + jj * gridDim.x] : 0; };
-        int tile_n = tile_at(0), tile_nn = tile_at(1);
-        int around_n = around(tile_n);
-        int issued = 0;
-        for (int j = 0; j < njobs; j++) {
+        // job j: the tile's box into buffer j % 3, which is free once the group that computed job
+        // j - 3 has pulled from it; no copy for tile -1, which ends the group's loop
+        auto send = [&](int tile, int j) {
             const int b = j % kRingBufs;
-            if (j >= kRingBufs) {
-                // buffer b is free once the group that computed tile j - 3 has pulled from it
-                bool ok = false;
+            if (j >= kRingBufs && tile >= 0) {
+                bool free = false;
                 const uint32_t par = (uint32_t)((j / kRingBufs - 1) & 1);
-                for (int it = 0; it < P.wait_polls && !ok; it++) ok = mbar_try_wait(smem_u32(&s_empty[b]), par);
-                if (!ok) {
-                    atomicOr(P.err, 1);
-                    break;
-                }
+                for (int it = 0; it < P.wait_polls && !free; it++) free = mbar_try_wait(smem_u32(&s_empty[b]), par);
+                if (!free) return false;
             }
-            const int tile = tile_n;
-            const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
             // written before the arrive, whose release the consumers' wait acquires
-            s_single[j % (2 * kRingBufs)] = __popc((unsigned)around_n) == 1;
             s_tile[j % (2 * kRingBufs)] = tile;
             const uint32_t full = smem_u32(&s_full[j % (2 * kRingBufs)]);
+            if (tile < 0) {
+                mbar_arrive(full);
+                return true;
+            }
             mbar_arrive_expect_tx(full, (uint32_t)NBOX * 4u);
-            tma_load_3d(smem_u32(ring + b * NBOXP), &tm_in, x0 - 4, y0 - 3, 0, full);
-            issued = j + 1;
-            tile_n = tile_nn;
-            tile_nn = tile_at(j + 2);
-            if (j + 1 < njobs) around_n = around(tile_n);
+            tma_load_3d(smem_u32(ring + b * NBOXP), &tm_in, (tile % ntx) * TX - 4, (tile / ntx) * TY - 3, 0, full);
+            return true;
+        };
+        int issued = 0;
+        bool ok = true;
+        for (int base = 0; base < njobs && ok; base += 32) {
+            const int mine = base + lane < njobs ? tiles[blockIdx.x + (base + lane) * gridDim.x] : -1;
+            const bool multi = mine >= 0 && (all || __popc((unsigned)fluids_around(pres_in, mine, ntx)) != 1);
+            for (unsigned todo = __ballot_sync(0xffffffffu, multi); todo && ok; todo &= todo - 1) {
+                const int tile = __shfl_sync(0xffffffffu, mine, __ffs(todo) - 1);
+                if (lane == 0) ok = send(tile, issued);
+                ok = __shfl_sync(0xffffffffu, ok, 0);
+                issued += ok;
+            }
         }
+        if (lane != 0) return;
         // every copy issued has landed before the block may exit
         for (int m = 0; m < 2 * kRingBufs; m++) {
             int last = -1;
@@ -1249,6 +1425,10 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
             for (int it = 0; it < kWaitLimit && !mbar_try_wait(smem_u32(&s_full[m]), par); it++) {
             }
         }
+        if (!ok) atomicOr(P.err, 1);
+        // no more tiles: one job without a copy for each group (after the waits above, which look
+        // at the last copy of each barrier)
+        for (int g = 0; g < 2 && ok; g++) ok = send(-1, issued + g);
         return;
     }
 
@@ -1286,7 +1466,7 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
         return (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0);
     };
 
-    for (int j = g, jj = 0; j < njobs; j += 2, jj++) {
+    for (int j = g, jj = 0;; j += 2, jj++) {
         const float* box = ring + (j % kRingBufs) * NBOXP;
         {
             bool ok = false;
@@ -1299,12 +1479,8 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
             }
         }
         const int tile = s_tile[j % (2 * kRingBufs)];
+        if (tile < 0) return;
         const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
-        // One fluid in the 3 x 3 tiles around: every node of the halo-2 region holds that fluid
-        // alone after the pull (a fluid absent from a node's sources stays absent), so the tile
-        // is not mixed, and its phase fields, which only the mixed path reads, are skipped.
-        const bool single = s_single[j % (2 * kRingBufs)];
-        if (single && tid == 0) flags[(jj + 1) & 1] = 0;  // all threads are past the last tile
         // ---- phase 1: pulls, densities and phase fields of the halo-2 region ----
         auto pull = [&](int cx, int cy, float q[27]) {
 #pragma unroll
@@ -1315,7 +1491,7 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
         };
         int present = 0;
         float q[27];
-        if (ring_node && !single) {
+        if (ring_node) {
             pull(rcx, rcy, q);
             const float a0 = ((q[0] + (q[1] + q[3])) + (q[2] + q[4])) + ((q[5] + q[7]) + (q[6] + q[8]));
             const float a1 = ((q[9] + (q[10] + q[12])) + (q[11] + q[13])) + ((q[14] + q[16]) + (q[15] + q[17]));
@@ -1338,25 +1514,22 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
             const int w = __reduce_or_sync(0xffffffffu, own);
             if (lane == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = (uint8_t)w;
         }
-        bool mixed = false;
-        if (!single) {
-            present |= store_phase(lx + 2, ly + 2, r0, r1, r2);
-            // fluids present in the group's phase-field region (one barrier; see fluids_present)
-            int cnt;
-            {
-                const int w = __reduce_or_sync(0xffffffffu, present);
-                if (lane == 0 && w) atomicOr(&flags[jj & 1], w);
-                group_sync(bar_id, NT);
-                const int v = flags[jj & 1];
-                if (tid == 0) flags[(jj + 1) & 1] = 0;
-                cnt = __popc(v & 7);
-            }
-            mixed = cnt != 1;
-
-            // ---- phase 2: stress tensor of Eq.(10) on the halo-1 region ----
-            if (mixed) stress_halo1<TX, TY>(P, ch, rh, s_txx[g], s_txy[g], s_tyy[g], tid);
+        present |= store_phase(lx + 2, ly + 2, r0, r1, r2);
+        // fluids present in the group's phase-field region (one barrier; see fluids_present)
+        int cnt;
+        {
+            const int w = __reduce_or_sync(0xffffffffu, present);
+            if (lane == 0 && w) atomicOr(&flags[jj & 1], w);
             group_sync(bar_id, NT);
+            const int v = flags[jj & 1];
+            if (tid == 0) flags[(jj + 1) & 1] = 0;
+            cnt = __popc(v & 7);
         }
+        const bool mixed = cnt != 1;
+
+        // ---- phase 2: stress tensor of Eq.(10) on the halo-1 region ----
+        if (mixed) stress_halo1<TX, TY>(P, ch, rh, s_txx[g], s_txy[g], s_tyy[g], tid);
+        group_sync(bar_id, NT);
 
         // ---- phase 3: force, collision, recolouring, 27 stores per node ----
         float Fx = 0.0f, Fy = 0.0f, gr[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
@@ -1614,30 +1787,30 @@ void launch_wet_init(int store, const Params& P, int nw, const int* widx, const 
 template <int STORE>
 static void launch_step_t(const Params& P, const int* tiles, int ntiles, int kind, const Pop& fin,
                           const Pop& fout, const uint8_t* type, const double* Cw, float* u,
-                          const uint64_t* pres_in, uint64_t* pres_out, cudaStream_t s)
+                          const uint64_t* pres_in, uint64_t* pres_out, bool all, cudaStream_t s)
 {
     if (kind == kTilesPure)
         k_step<kTX, kTY, true, true, STORE>
-            <<<ntiles, dim3(kTX, kTY), 0, s>>>(P, tiles, fin, fout, type, Cw, u, pres_in, pres_out);
+            <<<ntiles, dim3(kTX, kTY), 0, s>>>(P, tiles, fin, fout, type, Cw, u, pres_in, pres_out, all);
     else if (kind == kTilesWall)
         k_step<kTX, kTY, false, true, STORE>
-            <<<ntiles, dim3(kTX, kTY), 0, s>>>(P, tiles, fin, fout, type, Cw, u, pres_in, pres_out);
+            <<<ntiles, dim3(kTX, kTY), 0, s>>>(P, tiles, fin, fout, type, Cw, u, pres_in, pres_out, all);
     else
         k_step<kTX, kTY, false, false, STORE>
-            <<<ntiles, dim3(kTX, kTY), 0, s>>>(P, tiles, fin, fout, type, Cw, u, pres_in, pres_out);
+            <<<ntiles, dim3(kTX, kTY), 0, s>>>(P, tiles, fin, fout, type, Cw, u, pres_in, pres_out, all);
 }
 
 void launch_step(int store, const Params& P, const int* tiles, int ntiles, int kind, const Pop& fin,
                  const Pop& fout, const uint8_t* type, const double* Cw, float* u, const uint64_t* pres_in,
-                 uint64_t* pres_out, cudaStream_t s)
+                 uint64_t* pres_out, cudaStream_t s, bool all)
 {
     if (ntiles <= 0) return;
     if (store == kStoreF32)
-        launch_step_t<kStoreF32>(P, tiles, ntiles, kind, fin, fout, type, Cw, u, pres_in, pres_out, s);
+        launch_step_t<kStoreF32>(P, tiles, ntiles, kind, fin, fout, type, Cw, u, pres_in, pres_out, all, s);
     else if (store == kStoreF16)
-        launch_step_t<kStoreF16>(P, tiles, ntiles, kind, fin, fout, type, Cw, u, pres_in, pres_out, s);
+        launch_step_t<kStoreF16>(P, tiles, ntiles, kind, fin, fout, type, Cw, u, pres_in, pres_out, all, s);
     else
-        launch_step_t<kStoreBF16>(P, tiles, ntiles, kind, fin, fout, type, Cw, u, pres_in, pres_out, s);
+        launch_step_t<kStoreBF16>(P, tiles, ntiles, kind, fin, fout, type, Cw, u, pres_in, pres_out, all, s);
 }
 
 // Pure tiles of the 16-bit storage through the tensor memory accelerator, persistent, with the
@@ -1655,7 +1828,7 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
                                                             const __grid_constant__ CUtensorMap tm_rho,
                                                             const __grid_constant__ CUtensorMap tm_off,
                                                             const uint64_t* __restrict__ pres_in,
-                                                            uint64_t* __restrict__ pres_out)
+                                                            uint64_t* __restrict__ pres_out, const int all)
 {
     constexpr int NT = TX * TY;
     constexpr int CX = TX + 4, CY = TY + 4;
@@ -1671,7 +1844,8 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
     __shared__ float s_txx[RY][RX], s_txy[RY][RX], s_tyy[RY][RX];
     __shared__ __align__(8) uint64_t s_bar;
     __shared__ int s_flags[2];   // fluids present in the tile, by iteration parity
-    __shared__ int s_single[2];  // by iteration parity: the tile's 3 x 3 tiles hold one fluid
+    __shared__ int s_list[NT];   // tiles of the current batch
+    __shared__ int s_wn[NT / 32];
     extern __shared__ unsigned char dsm[];
     float* rbox = reinterpret_cast<float*>(dsm + ((128u - (smem_u32(dsm) & 127u)) & 127u));  // [3][BY][BX]
     const unsigned short* obox = reinterpret_cast<const unsigned short*>(rbox + NRP);          // [24][BY][OX]
@@ -1687,29 +1861,12 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
         tma_load_3d(smem_u32(rbox), &tm_rho, x0 - 4, y0 - 3, 0, bar);
         tma_load_3d(smem_u32(obox), &tm_off, x0 - 8, y0 - 3, 0, bar);
     };
-    // fluids stored in the 3 x 3 tiles around a tile (a pure tile is inner, so they exist): one
-    // fluid means the tile holds it alone after the pull (as in k_step_ring)
-    auto single_around = [&](int t) {
-        uint64_t nb = 0;
-#pragma unroll
-        for (int dy = -1; dy <= 1; dy++)
-#pragma unroll
-            for (int dx = -1; dx <= 1; dx++) nb |= pres_in[t + dy * ntx + dx];
-        nb |= nb >> 32;
-        nb |= nb >> 16;
-        nb |= nb >> 8;
-        return __popc((unsigned)(nb & 7u)) == 1 ? 1 : 0;
-    };
-    int tile = tiles[blockIdx.x];
-    int last = 0;
+    int last = -1;
     if (tid == 0) {
         mbar_init(bar, 1);
         fence_mbar_init();
-        issue(tile);
         s_flags[0] = s_flags[1] = 0;
-        s_single[0] = single_around(tile);
     }
-    __syncthreads();
 
     // pull of the node at (cx, cy) of the phase-field region from the boxes
     auto pull = [&](int cx, int cy, float q[27]) {
@@ -1745,109 +1902,116 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
     };
 
     int j = 0;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, j++) {
-        const bool more = t + (int)gridDim.x < ntiles;
-        const int next = more ? tiles[t + gridDim.x] : 0;
-        const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
-        bool ok = false;
-        for (int it = 0; it < P.wait_polls && !ok; it++) ok = mbar_try_wait(bar, j & 1);
-        if (__syncthreads_or(!ok)) {
-            // the copies did not complete in time: record it, give them a second bounded wait
-            // so that they do not land in a later block's shared memory, and stop
-            if (tid == 0) {
-                atomicOr(P.err, 1);
-                for (int it = 0; it < kWaitLimit && !mbar_try_wait(bar, last & 1); it++) {
+    const int mine = (ntiles - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    // the block's tiles in batches of one candidate per thread: those with one fluid around are
+    // k_step_one's, the others are listed
+    for (int base = 0; base < mine; base += NT) {
+        const int cand = base + tid < mine ? tiles[blockIdx.x + (base + tid) * gridDim.x] : -1;
+        const bool multi = cand >= 0 && (all || __popc((unsigned)fluids_around(pres_in, cand, ntx)) != 1);
+        const unsigned votes = __ballot_sync(0xffffffffu, multi);
+        if ((tid & 31) == 0) s_wn[tid >> 5] = __popc(votes);
+        __syncthreads();  // the counts, and every thread is past the last batch's list
+        int pos = __popc(votes & ((1u << (tid & 31)) - 1)), count = 0;
+        for (int w = 0; w < NT / 32; w++) {
+            if (w < (tid >> 5)) pos += s_wn[w];
+            count += s_wn[w];
+        }
+        if (multi) s_list[pos] = cand;
+        __syncthreads();
+        if (tid == 0 && count > 0) {
+            issue(s_list[0]);
+            last = j;
+        }
+        for (int m = 0; m < count; m++, j++) {
+            const bool more = m + 1 < count;
+            const int tile = s_list[m];
+            const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
+            bool ok = false;
+            for (int it = 0; it < P.wait_polls && !ok; it++) ok = mbar_try_wait(bar, j & 1);
+            if (__syncthreads_or(!ok)) {
+                // the copies did not complete in time: record it, give them a second bounded wait
+                // so that they do not land in a later block's shared memory, and stop
+                if (tid == 0) {
+                    atomicOr(P.err, 1);
+                    for (int it = 0; last >= 0 && it < kWaitLimit && !mbar_try_wait(bar, last & 1); it++) {
+                    }
+                }
+                return;
+            }
+
+            // ---- phase 1: pulls, densities and phase fields of the halo-2 region ----
+            int present = 0;
+            {
+                constexpr int NRING = CX * CY - TX * TY;
+                for (int r = tid; r < NRING; r += NT) {
+                    int cx, cy;
+                    if (r < 2 * CX) {
+                        cx = r % CX;
+                        cy = r / CX;
+                    } else if (r < 4 * CX) {
+                        cx = (r - 2 * CX) % CX;
+                        cy = CY - 2 + (r - 2 * CX) / CX;
+                    } else {
+                        const int rr0 = r - 4 * CX;  // 4 * TY side nodes
+                        const int side = rr0 / (2 * TY), rr = rr0 % (2 * TY);
+                        cy = 2 + rr / 2;
+                        cx = side == 0 ? (rr & 1) : CX - 2 + (rr & 1);
+                    }
+                    float q[27];
+                    pull(cx, cy, q);
+                    present |= store_phase(cx, cy, q);
                 }
             }
-            return;
-        }
-
-        const bool single = s_single[j & 1];
-        int single_next = 0;  // thread 0: for the next tile, written once this one is computed
-        // ---- phase 1: pulls, densities and phase fields of the halo-2 region ----
-        int present = 0;
-        if (!single) {
-            constexpr int NRING = CX * CY - TX * TY;
-            for (int r = tid; r < NRING; r += NT) {
-                int cx, cy;
-                if (r < 2 * CX) {
-                    cx = r % CX;
-                    cy = r / CX;
-                } else if (r < 4 * CX) {
-                    cx = (r - 2 * CX) % CX;
-                    cy = CY - 2 + (r - 2 * CX) / CX;
-                } else {
-                    const int rr0 = r - 4 * CX;  // 4 * TY side nodes
-                    const int side = rr0 / (2 * TY), rr = rr0 % (2 * TY);
-                    cy = 2 + rr / 2;
-                    cx = side == 0 ? (rr & 1) : CX - 2 + (rr & 1);
-                }
+            float f[kQ], r0, r1, r2;
+            {
                 float q[27];
-                pull(cx, cy, q);
-                present |= store_phase(cx, cy, q);
-            }
-        }
-        float f[kQ], r0, r1, r2;
-        {
-            float q[27];
-            pull(lx + 2, ly + 2, q);
-            if (!single) present |= store_phase(lx + 2, ly + 2, q);
+                pull(lx + 2, ly + 2, q);
+                present |= store_phase(lx + 2, ly + 2, q);
 #pragma unroll
-            for (int a = 0; a < kQ; a++) f[a] = (q[a] + q[9 + a]) + q[18 + a];
-            r0 = ((q[0] + (q[1] + q[3])) + (q[2] + q[4])) + ((q[5] + q[7]) + (q[6] + q[8]));
-            r1 = ((q[9] + (q[10] + q[12])) + (q[11] + q[13])) + ((q[14] + q[16]) + (q[15] + q[17]));
-            r2 = ((q[18] + (q[19] + q[21])) + (q[20] + q[22])) + ((q[23] + q[25]) + (q[24] + q[26]));
-        }
-        // the fluids this warp's nodes hold, for the tiles around this one in the next step
-        {
-            const int own = (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0);
-            const int w = __reduce_or_sync(0xffffffffu, own);
-            if ((tid & 31) == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = (uint8_t)w;
-        }
-        bool mixed = false;
-        if (single) {
-            __syncthreads();  // every pull is done before the boxes are refilled
-            if (tid == 0) s_flags[(j + 1) & 1] = 0;
-        } else {
-            mixed = fluids_present(present, s_flags, j, tid) != 1;
-        }
-        // the boxes are free: fetch the next tile's while this one computes
-        if (tid == 0 && more) {
-            issue(next);
-            last = j + 1;
-            single_next = single_around(next);
-        }
+                for (int a = 0; a < kQ; a++) f[a] = (q[a] + q[9 + a]) + q[18 + a];
+                r0 = ((q[0] + (q[1] + q[3])) + (q[2] + q[4])) + ((q[5] + q[7]) + (q[6] + q[8]));
+                r1 = ((q[9] + (q[10] + q[12])) + (q[11] + q[13])) + ((q[14] + q[16]) + (q[15] + q[17]));
+                r2 = ((q[18] + (q[19] + q[21])) + (q[20] + q[22])) + ((q[23] + q[25]) + (q[24] + q[26]));
+            }
+            // the fluids this warp's nodes hold, for the tiles around this one in the next step
+            {
+                const int own = (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0);
+                const int w = __reduce_or_sync(0xffffffffu, own);
+                if ((tid & 31) == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = (uint8_t)w;
+            }
+            const bool mixed = fluids_present(present, s_flags, j, tid) != 1;
+            // the boxes are free: fetch the next tile's while this one computes
+            if (tid == 0 && more) {
+                issue(s_list[m + 1]);
+                last = j + 1;
+            }
 
-        // ---- phase 2: stress tensor of Eq.(10) on the halo-1 region ----
-        if (!single) {
+            // ---- phase 2: stress tensor of Eq.(10) on the halo-1 region ----
             if (mixed) stress_halo1<TX, TY>(P, s_ch, s_rho, s_txx, s_txy, s_tyy, tid);
             __syncthreads();
-        }
 
-        // ---- phase 3: force, collision, recolouring, 16-bit stores ----
-        float Fx = 0.0f, Fy = 0.0f, g[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-        if (mixed) {
-            div_stress<RX>(s_txx, s_txy, s_tyy, lx + 1, ly + 1, Fx, Fy);
+            // ---- phase 3: force, collision, recolouring, 16-bit stores ----
+            float Fx = 0.0f, Fy = 0.0f, g[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+            if (mixed) {
+                div_stress<RX>(s_txx, s_txy, s_tyy, lx + 1, ly + 1, Fx, Fy);
 #pragma unroll
-            for (int k = 0; k < kNF; k++) grad9_f<CX>(s_ch[k], lx + 2, ly + 2, g[2 * k], g[2 * k + 1]);
+                for (int k = 0; k < kNF; k++) grad9_f<CX>(s_ch[k], lx + 2, ly + 2, g[2 * k], g[2 * k + 1]);
+            }
+            float ux, uy;
+            const Recolour rc = collide_node(P, f, r0, r1, r2, Fx, Fy, g, ux, uy);
+            const int i = (y0 + ly) * P.nx + x0 + lx;
+            if (uout) {
+                uout[i] = ux;
+                uout[P.N + i] = uy;
+            }
+            float v[27];
+#pragma unroll
+            for (int k = 0; k < kNF; k++)
+#pragma unroll
+                for (int a = 0; a < kQ; a++)
+                    v[9 * k + a] = rc.C[k] * f[a] + wq(a) * (rc.Vx[k] * (float)ex(a) + rc.Vy[k] * (float)ey(a));
+            store_node<STORE>(fout, P.N, i, v);
         }
-        float ux, uy;
-        const Recolour rc = collide_node(P, f, r0, r1, r2, Fx, Fy, g, ux, uy);
-        const int i = (y0 + ly) * P.nx + x0 + lx;
-        if (uout) {
-            uout[i] = ux;
-            uout[P.N + i] = uy;
-        }
-        tile = next;
-        float v[27];
-#pragma unroll
-        for (int k = 0; k < kNF; k++)
-#pragma unroll
-            for (int a = 0; a < kQ; a++)
-                v[9 * k + a] = rc.C[k] * f[a] + wq(a) * (rc.Vx[k] * (float)ex(a) + rc.Vy[k] * (float)ey(a));
-        store_node<STORE>(fout, P.N, i, v);
-        // read by every thread after the next tile's first barrier
-        if (tid == 0) s_single[(j + 1) & 1] = single_next;
     }
 }
 
@@ -1890,12 +2054,12 @@ cudaError_t step_ring_prepare()
 }
 
 void launch_step_ring(const Params& P, const int* tiles, int ntiles, int nblocks, const Pop& fout, float* u,
-                      const CUtensorMap& tin, const uint64_t* pres_in, uint64_t* pres_out, cudaStream_t s)
+                      const CUtensorMap& tin, const uint64_t* pres_in, uint64_t* pres_out, bool all, cudaStream_t s)
 {
     if (ntiles <= 0) return;
     const int nb = nblocks < ntiles ? nblocks : ntiles;
     k_step_ring<kTX, kTY><<<nb, 2 * kTX * kTY + 32, step_ring_smem_bytes(), s>>>(P, tiles, ntiles, fout.f, u, tin,
-                                                                                 pres_in, pres_out);
+                                                                                 pres_in, pres_out, all);
 }
 
 size_t step_tma16_smem_bytes()
@@ -1918,16 +2082,31 @@ cudaError_t step_tma16_prepare()
 
 void launch_step_tma16(int store, const Params& P, const int* tiles, int ntiles, int nblocks, const Pop& fout,
                        float* u, const CUtensorMap& trho, const CUtensorMap& toff, const uint64_t* pres_in,
-                       uint64_t* pres_out, cudaStream_t s)
+                       uint64_t* pres_out, bool all, cudaStream_t s)
 {
     if (ntiles <= 0) return;
     const int nb = nblocks < ntiles ? nblocks : ntiles;
     if (store == kStoreF16)
         k_step_tma16<kTX, kTY, kStoreF16><<<nb, dim3(kTX, kTY), step_tma16_smem_bytes(), s>>>(
-            P, tiles, ntiles, fout, u, trho, toff, pres_in, pres_out);
+            P, tiles, ntiles, fout, u, trho, toff, pres_in, pres_out, all);
     else
         k_step_tma16<kTX, kTY, kStoreBF16><<<nb, dim3(kTX, kTY), step_tma16_smem_bytes(), s>>>(
-            P, tiles, ntiles, fout, u, trho, toff, pres_in, pres_out);
+            P, tiles, ntiles, fout, u, trho, toff, pres_in, pres_out, all);
+}
+
+void launch_step_one(int store, const Params& P, const int* tiles, int ntiles, const Pop& fin, const Pop& fout,
+                     float* u, const uint64_t* pres_in, uint64_t* pres_out, bool full_write, cudaStream_t s)
+{
+    if (ntiles <= 0) return;
+    constexpr int per = kOneThreads / 32;
+    const unsigned nb = (unsigned)((ntiles + per - 1) / per);
+    const int fw = full_write ? 1 : 0;
+    if (store == kStoreF32)
+        k_step_one<kTX, kTY, kStoreF32><<<nb, kOneThreads, 0, s>>>(P, tiles, ntiles, fin, fout, u, pres_in, pres_out, fw);
+    else if (store == kStoreF16)
+        k_step_one<kTX, kTY, kStoreF16><<<nb, kOneThreads, 0, s>>>(P, tiles, ntiles, fin, fout, u, pres_in, pres_out, fw);
+    else
+        k_step_one<kTX, kTY, kStoreBF16><<<nb, kOneThreads, 0, s>>>(P, tiles, ntiles, fin, fout, u, pres_in, pres_out, fw);
 }
 
 void launch_init(int store, const Params& P, const double* rho, const uint8_t* type, const Pop& f,
