@@ -83,18 +83,18 @@ int lbm3_create(lbm3** out, const lbm3_grid* grid, const uint8_t* solid_mask,
  * step are the w-weighted means of each C_SB node's fluid neighbours.  rho: host [3][ny][nx]. */
 int lbm3_set_fields(lbm3* h, const double* rho);
 
-/* Advance nsteps >= 0 timesteps (Eq.1-22), asynchronously on the handle's stream.  Each step is
- * the wetting pass over the C_SB list (Eq.21-22) and the fused step kernel (Eq.1-16: densities,
- * gradients, interfacial force, MRT collision, recolouring, streaming with halfway bounce-back
- * and the x boundary).  Tiles with no solid node within 3 nodes run concurrently with the wetting
- * pass on the handle's stream (through bulk tensor copies when nx is a multiple of 4, on the SMs
- * that the other tiles' share of the work leaves); the other tiles follow the wetting pass on an
- * internal higher-priority stream that is joined back before the call's work completes.  The
- * velocity of the last collision of the call is recorded for lbm3_fields / lbm3_diag.  A bulk
- * copy that does not complete within its wait limit is reported by the next lbm3_diag.  On grids
+/* Advance nsteps >= 0 timesteps (Eq.1-22), asynchronously on the handle's stream.  A step is the
+ * fused Eq.1-16 (densities, gradients, interfacial force, MRT collision, recolouring, streaming with
+ * halfway bounce-back and the x boundary) on every tile, with the wetting of the C_SB nodes (Eq.21-22)
+ * in the tiles that see them.  Tiles with no solid node within 3 nodes and away from the domain edge
+ * (pure tiles) run on the handle's stream (through bulk tensor copies when nx is a multiple of 4, on
+ * the SMs that the other tiles' share of the work leaves); the other tiles run beside them on an
+ * internal higher-priority stream that is joined back before the call's work completes.  On grids
  * with many pure tiles those around which one fluid is stored are advanced by a launch of their own
- * that moves that fluid's populations only (the others' are zeros there), with the same results;
- * its result does not depend on which launch takes a tile.  While more
+ * that moves that fluid's populations only (the others' are zeros there).  The results do not depend
+ * on which launch takes a tile.  The velocity of the last collision of the call is recorded for
+ * lbm3_fields / lbm3_diag.  A bulk copy that does not complete within its wait limit is reported by
+ * the next lbm3_diag.  While more
  * than 8 steps remain, blocks of 8 steps are launched as one CUDA graph, captured on an internal
  * stream the first time it is needed (one graph per starting population buffer) and replayed on
  * the handle's stream: the same kernels in the same order, so the results do not depend on how
@@ -103,15 +103,14 @@ int lbm3_step(lbm3* h, int32_t nsteps);
 
 /* lbm3_step with per-launch timing: CUDA events are recorded around every launch on the stream
  * it runs on; after the last step the call synchronises and writes the summed times in ms:
- * ms_out[0] = wetting pass, ms_out[1] = fused step kernel on the pure tiles (no solid within
- * 3 nodes; main stream), ms_out[2] = fused step kernel on the other tiles (side stream, after the
- * wetting pass).  The pure-tile launch overlaps the other two. */
+ * ms_out[0] = wetting launch (none: about 0, the wetting is part of the tiles), ms_out[1] = pure tiles
+ * (no solid within 3 nodes; main stream), ms_out[2] = the other tiles (side stream).  The pure-tile
+ * launches overlap the other one. */
 int lbm3_step_timed(lbm3* h, int32_t nsteps, double ms_out[3]);
 
-/* lbm3_step_timed with the other tiles split by kind: ms_out[0] = wetting pass, ms_out[1] = pure
- * tiles, ms_out[2] = wall tiles (solids within 3 nodes, halo inside the domain), ms_out[3] = edge
- * tiles (halo crossing the domain edge; on a second internal stream, those with no solid within
- * 3 nodes from the start of the step, the others once the wetting pass is done), summed over the
+/* lbm3_step_timed with the device time of the run: ms_out[0] = wetting launch (none: about 0),
+ * ms_out[1] = pure tiles, ms_out[2] = the other tiles (solids within 3 nodes, or halo crossing the
+ * domain edge), ms_out[3] = edge tiles apart from those (none: about 0), summed over the
  * steps in ms, and ms_out[4] = the device time of the whole run, from the event before the first
  * step's first launch to one recorded after the last step (the host's read-back of the events
  * after the run is outside it).  Synchronises.  lbm3_step_timed's ms_out[2] is the sum of
@@ -143,7 +142,7 @@ int lbm3_wall_values(lbm3* h, double* c, int32_t cap);
 
 /* Checkpoint / resume.  The state of a simulation is its post-streaming populations
  * f_post [3][9][ny][nx] (fluid k, direction a; 0 at solid nodes) and the wall values
- * wall_c [3][ny][nx] that the next wetting pass reads in Eq.(21) (used at C_SB nodes only).
+ * wall_c [3][ny][nx] that the next step's wetting reads in Eq.(21) (used at C_SB nodes only).
  * lbm3_get_state copies both to host memory (synchronises); lbm3_set_state replaces the state
  * (the populations of directions entering from an open side are recomputed by Zou-He). */
 int lbm3_get_state(lbm3* h, double* f_post, double* wall_c);
@@ -185,7 +184,7 @@ int lbm3_adjoint_release(lbm3* h);
  * fused step per timestep (216 B per fluid node with FP32 storage, 120 B with 16-bit offsets,
  * + 1 class byte per node; as if every node held all three fluids), out[3] = fused-step launches per
  * timestep, out[4] = wetting launches
- * per timestep, out[5] = device bytes held by the handle, out[6] = algorithmic bytes of the
+ * per timestep (0: part of the fused step), out[5] = device bytes held by the handle, out[6] = algorithmic bytes of the
  * pure-tile launch, out[7] = nodes in pure tiles, out[8] = how the pure tiles move their
  * populations: 0 plain loads, 1 bulk tensor copies with two blocks per SM, 2 bulk tensor copies
  * through the warp-specialised ring (FP32 storage; LBM3_PURE_KERNEL=tma in the environment at

@@ -148,7 +148,7 @@ __global__ void a_dens(const Params P, const Adj A, const float* __restrict__ fs
         for (int j = 0; j < 27; j++) A.fpost[(long long)j * P.N + i] = q[j];
 }
 
-// A2: wetting with its decisions, 4 lanes per C_SB node (the same computation as k_wet)
+// A2: wetting with its decisions, 4 lanes per C_SB node (the same values as the step's)
 __global__ void a_wet(const Params P, const Adj A, int nw, const int* __restrict__ widx,
                       const double* __restrict__ wnrm, const float* __restrict__ wang,
                       const float* __restrict__ fs, const uint8_t* __restrict__ type,

@@ -1,6 +1,7 @@
 // lbm3_api.cu -- host side of the C ABI declared in include/lbm3.h: argument checks, node
 // classification (Section II.B), eighth-order solid normals (Eq.19-20), the compact wall list,
 // device buffers and the per-step launch sequence.
+#include <algorithm>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -23,7 +24,8 @@ struct lbm3 {
     // planes), the node classes, wall values, velocity, scratch
     Pop pop[2] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
     uint8_t* type = nullptr;
-    double* Cw = nullptr;          // [3][N] wall values (written at C_SB nodes only)
+    // [3][N] wall values (a step writes C_SB nodes only); cw[pp] are the current ones
+    double* cw[2] = {nullptr, nullptr};
     float* u = nullptr;
     float* scratch = nullptr;      // 3N floats for fields
     double* partials = nullptr;    // diagnostics block partials
@@ -43,28 +45,25 @@ struct lbm3 {
     int* widx = nullptr;
     double* wnrm = nullptr;
     float* wang = nullptr;
-    WetCache* wcache = nullptr;  // [4 nw] characteristic-line crossings of the wetting lanes
-    double* cw_keep = nullptr;   // set by the adjoint for one step: the wetting pass stores there
-                                 // the lagged wall values it reads
     // set by the adjoint for one step: the step reads io_in (through the tensor map io_box on the
     // ring path) and writes io_out instead of the two population buffers, whose turn is kept
     const Pop* io_in = nullptr;
     const Pop* io_out = nullptr;
+    double* io_cw_out = nullptr;  // and its wall values go there
     const CUtensorMap* io_box = nullptr;
     // the timing events of enqueue_step are recorded into a graph being captured (as nodes that
     // record them when the graph runs)
     bool ev_external = false;
     int nw = 0;
     long long n_fluid = 0;
-    // tiles of the fused step kernel: pure tiles (no solid within 3 nodes, away from the domain
-    // edge) run on the main stream and do not wait for the wetting pass; the other tiles run
-    // after the wetting pass on a higher-priority side stream
-    int* tiles_pure = nullptr;
-    int* tiles_gen = nullptr;
+    // tiles of the step kernels: gen, those near solids or the domain edge (launch_tile, on a
+    // higher-priority side stream), then the pure ones (no solid within 3 nodes, away from the edge;
+    // main stream)
+    TileSet gen{};
     int n_pure = 0, n_gen = 0;
-    int n_walltiles = 0;  // tiles_gen lists the inner wall tiles first, then the edge tiles
-    int n_edgewall = 0;   // of the edge tiles, those with a solid node within 3 nodes come first;
-                          // the others read no wall value and need not wait for the wetting pass
+    const int* tiles_pure = nullptr;
+    void* tile_mem[5] = {};  // the arrays of the set, and the pure tiles' list
+    int n_went = 0;          // entries of the wetting (gen.went), four lanes of its cache each
     long long pure_fluid = 0;
     // fluids present per tile (one byte per warp of the ring kernel's group, so no byte needs an
     // atomic or a clearing): pres[pp] describes the current state, the ring kernel writes the
@@ -78,10 +77,6 @@ struct lbm3 {
     int pp = 0;
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
-    // the edge tiles run on a second side stream once the wetting pass is done, concurrently with
-    // the wall tiles (the two sets are independent)
-    cudaStream_t side2 = nullptr;
-    cudaEvent_t ev_wet = nullptr, ev_join2 = nullptr;
     // one: the pure tiles with one fluid around are launch_step_one's (kOneTiles); those with
     // several run beside them on a third side stream
     bool one = false;
@@ -101,15 +96,14 @@ struct lbm3 {
     std::vector<int> wall_host;
     std::string err;
     // device memory of lbm3_adjoint_centroid, kept for later calls that need no more of it: the
-    // checkpoints (nck states), the segment's states (nsg), the final state, the work arrays,
-    // and two events that order the state copies; released by lbm3_adjoint_release or
+    // checkpoints (nck states), the segment's states (nsg), the final state and the work arrays;
+    // released by lbm3_adjoint_release or
     // lbm3_destroy
     struct AdjStore {
         float *ck_f = nullptr, *sg_f = nullptr, *fin_f = nullptr;
         double *ck_c = nullptr, *sg_c = nullptr, *fin_c = nullptr;
         int nck = 0, nsg = 0;
         AdjointWork* W = nullptr;
-        cudaEvent_t ev_in = nullptr, ev_saved = nullptr;
         std::vector<CUtensorMap> box;  // ring path: the tensor map of every segment slot
         // the sweep as a graph, for nsteps / K from state buffer g_cur
         cudaGraphExec_t gexec = nullptr;
@@ -184,8 +178,6 @@ void adj_release(lbm3* h)
         if (p) cudaFree(p);
     if (a.gexec) cudaGraphExecDestroy(a.gexec);
     adjoint_free(a.W);
-    if (a.ev_in) cudaEventDestroy(a.ev_in);
-    if (a.ev_saved) cudaEventDestroy(a.ev_saved);
     a = lbm3::AdjStore{};
 }
 
@@ -193,9 +185,9 @@ void release(lbm3* h)
 {
     adj_release(h);
     void* ptrs[] = {h->pop[0].f, h->pop[1].f, h->pop[0].rho, h->pop[1].rho, h->pop[0].off,
-                    h->pop[1].off, h->type, h->Cw, h->u, h->scratch, h->partials, h->dout,
-                    h->widx, h->wnrm, h->wang, h->tiles_pure, h->tiles_gen, h->err_flag, h->wcache,
-                    h->pres[0], h->pres[1]};
+                    h->pop[1].off, h->type, h->cw[0], h->cw[1], h->u, h->scratch, h->partials, h->dout,
+                    h->widx, h->wnrm, h->wang, h->err_flag, h->gen.cache, h->pres[0], h->pres[1],
+                    h->tile_mem[0], h->tile_mem[1], h->tile_mem[2], h->tile_mem[3], h->tile_mem[4]};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     h->pop[0] = h->pop[1] = Pop{nullptr, nullptr, nullptr};
@@ -204,17 +196,14 @@ void release(lbm3* h)
     if (h->gcap) cudaStreamDestroy(h->gcap);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
-    if (h->ev_wet) cudaEventDestroy(h->ev_wet);
-    if (h->ev_join2) cudaEventDestroy(h->ev_join2);
     if (h->ev_join3) cudaEventDestroy(h->ev_join3);
     if (h->side3) cudaStreamDestroy(h->side3);
-    if (h->side2) cudaStreamDestroy(h->side2);
     if (h->side) cudaStreamDestroy(h->side);
 }
 
 // From this many pure tiles on, those with one fluid around are launch_step_one's, and the others
-// run beside them on a stream of their own.  Below it the step waits for the wetting pass and the
-// tiles after it, not for the pure tiles, and one more launch costs more than it hides: 2-3 % of
+// run beside them on a stream of their own.  Below it the step waits for the tiles near solids, not
+// for the pure ones, and one more launch costs more than it hides: 2-3 % of
 // the step on 128 x 64 and on the 800 x 375 pillars (865 pure tiles), while the 2048 x 1024 ones
 // (6308) gain 12 %.  LBM3_ONE_TILES=<n> in the environment at lbm3_create sets another line (same
 // results).
@@ -295,11 +284,6 @@ bool make_tensor_maps16(const Params& P, const Pop& p, CUtensorMap* trho, CUtens
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// One timestep: fork the side streams off the main stream, run the pure tiles on the main stream
-// while the side stream runs the wetting pass and then the wall tiles, and the second side stream
-// the edge tiles (at once those without a solid node near them, after the wetting pass the
-// others), join.  With ev != NULL the launches are bracketed by the events ev[0..6] (main: 0-1
-// pure tiles; side: 2-3 wetting pass, 3-4 wall tiles; second side stream: 5-6 edge tiles).
 // a timing event of enqueue_step (a record node when captured into a graph)
 void record_timing(lbm3* h, cudaEvent_t ev, cudaStream_t s)
 {
@@ -309,17 +293,27 @@ void record_timing(lbm3* h, cudaEvent_t ev, cudaStream_t s)
         cudaEventRecord(ev, s);
 }
 
+// One timestep: fork the side streams off the main stream, run the pure tiles on the main stream
+// (those with several fluids around on a side stream of their own where launch_step_one takes the
+// others) and the other tiles, with the wetting of their solid boundary nodes, on the
+// higher-priority side stream; join.  With ev != NULL the launches are bracketed by the events ev[0..6]
+// (main: 0-1 pure tiles; side: 3-4 the other tiles; 2-3 and 5-6 enclose nothing).
 cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
 {
     cudaError_t e;
     const bool io = h->io_in != nullptr;
     const Pop& fin = io ? *h->io_in : h->pop[h->cur];
     const Pop& fo = io ? *h->io_out : h->pop[1 - h->cur];
+    double* cw_out = io ? h->io_cw_out : h->cw[1 - h->pp];
     float* u = last ? h->u : nullptr;
     const uint64_t* pin = h->pres[h->pp];
     uint64_t* pout = h->pres[1 - h->pp];
     if ((e = cudaEventRecord(h->ev_fork, h->stream)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) != cudaSuccess) return e;
+    if (ev) record_timing(h, ev[2], h->side);
+    if (ev) record_timing(h, ev[3], h->side);
+    launch_tile(h->precision, h->P, h->gen, fin, fo, cw_out, u, pin, pout, io, h->side);
+    if (ev) record_timing(h, ev[4], h->side);
     if (ev) record_timing(h, ev[0], h->stream);
     // pure tiles: those with several fluids around through the kernel of the storage and layout,
     // those with one (launch_step_one) beside it; the two-blocks-per-SM kernel takes them all
@@ -337,8 +331,7 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
             launch_step_tma16(h->precision, h->P, h->tiles_pure, h->n_pure, h->tma_blocks, fo, u, h->tm_in_a[h->cur],
                               h->tm_in_b[h->cur], pin, pout, !one, ms);
         else
-            launch_step(h->precision, h->P, h->tiles_pure, h->n_pure, kTilesPure, fin, fo, h->type, h->Cw, u,
-                        pin, pout, ms, !one);
+            launch_step_plain(h->precision, h->P, h->tiles_pure, h->n_pure, fin, fo, u, pin, pout, !one, ms);
         if (one) {
             launch_step_one(h->precision, h->P, h->tiles_pure, h->n_pure, fin, fo, u, pin, pout, io, h->stream);
             if ((e = cudaEventRecord(h->ev_join3, ms)) != cudaSuccess) return e;
@@ -346,38 +339,8 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
         }
     }
     if (ev) record_timing(h, ev[1], h->stream);
-    if (ev) record_timing(h, ev[2], h->side);
-    launch_wet(h->precision, h->P, h->nw, h->widx, h->wnrm, h->wang, fin, h->type, h->Cw, h->wcache, h->side,
-               h->cw_keep);
-    if (ev) record_timing(h, ev[3], h->side);
-    // edge tiles: those without a solid node near them start at once, the others after the
-    // wetting pass
-    const int n_edge = h->n_gen - h->n_walltiles, n_edge_free = n_edge - h->n_edgewall;
-    const int* tiles_edge = h->tiles_gen + h->n_walltiles;
-    const bool edges = n_edge > 0;
-    if (edges) {
-        if ((e = cudaStreamWaitEvent(h->side2, h->ev_fork, 0)) != cudaSuccess) return e;
-        if (ev) record_timing(h, ev[5], h->side2);
-        launch_step(h->precision, h->P, tiles_edge + h->n_edgewall, n_edge_free, kTilesEdge, fin, fo, h->type,
-                    h->Cw, u, pin, pout, h->side2);
-        if (h->n_edgewall > 0) {
-            if ((e = cudaEventRecord(h->ev_wet, h->side)) != cudaSuccess) return e;
-            if ((e = cudaStreamWaitEvent(h->side2, h->ev_wet, 0)) != cudaSuccess) return e;
-        }
-    }
-    launch_step(h->precision, h->P, h->tiles_gen, h->n_walltiles, kTilesWall, fin, fo, h->type, h->Cw, u, pin,
-                pout, h->side);
-    if (ev) record_timing(h, ev[4], h->side);
-    if (edges) {
-        launch_step(h->precision, h->P, tiles_edge, h->n_edgewall, kTilesEdge, fin, fo, h->type, h->Cw, u, pin,
-                    pout, h->side2);
-        if (ev) record_timing(h, ev[6], h->side2);
-        if ((e = cudaEventRecord(h->ev_join2, h->side2)) != cudaSuccess) return e;
-        if ((e = cudaStreamWaitEvent(h->stream, h->ev_join2, 0)) != cudaSuccess) return e;
-    } else if (ev) {
-        record_timing(h, ev[5], h->side);
-        record_timing(h, ev[6], h->side);
-    }
+    if (ev) record_timing(h, ev[5], h->side);
+    if (ev) record_timing(h, ev[6], h->side);
     if ((e = cudaEventRecord(h->ev_join, h->side)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(h->stream, h->ev_join, 0)) != cudaSuccess) return e;
     if (!io) h->cur = 1 - h->cur;
@@ -392,13 +355,15 @@ constexpr int kCopyWaitPolls = 1 << 22;
 
 // Error bits that the kernels set (bit 0: a bulk tensor copy outlived its wait), read after the
 // stream has been synchronised and cleared once read, so that each timeout is reported once.
-int take_kernel_error(lbm3* h, int* bits)
+int take_kernel_error(lbm3* h)
 {
-    *bits = 0;
-    cudaError_t e = cudaMemcpyAsync(bits, h->err_flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+    int bits = 0;
+    cudaError_t e = cudaMemcpyAsync(&bits, h->err_flag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e == cudaSuccess && *bits) e = cudaMemsetAsync(h->err_flag, 0, sizeof(int), h->stream);
-    return e == cudaSuccess ? LBM3_OK : fail(h, LBM3_ERR_CUDA, std::string("error bits: ") + cudaGetErrorString(e));
+    if (e == cudaSuccess && bits) e = cudaMemsetAsync(h->err_flag, 0, sizeof(int), h->stream);
+    if (e != cudaSuccess) return fail(h, LBM3_ERR_CUDA, std::string("error bits: ") + cudaGetErrorString(e));
+    if (bits & 1) return fail(h, LBM3_ERR_CUDA, "a bulk tensor copy of the step kernel did not complete in time");
+    return LBM3_OK;
 }
 
 // the state was replaced from outside: every tile may hold every fluid
@@ -570,7 +535,9 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
     }
 
     // ---- tiles of the fused step kernel (2-D prefix sums of the solid mask)
-    std::vector<int> tp, tg, te, tf;
+    std::vector<int> tp, tg, te;
+    std::vector<int> rec;
+    std::vector<int4> went;
     long long pure_fluid = 0;
     {
         std::vector<long long> ps((size_t)(nx + 1) * (ny + 1), 0);
@@ -599,34 +566,73 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
                 } else if (inner) {
                     tg.push_back(ty * ntx + tx);
                 } else {
-                    // an edge tile: any solid node within 3 nodes, across a periodic side too?
-                    bool near_solid = false;
-                    for (int y = y0 - 3; y < y0 + kTY + 3 && !near_solid; y++) {
-                        int yy = y;
-                        if (yy < 0 || yy >= ny) {
-                            if (!g->periodic_y) continue;
-                            yy = (yy % ny + ny) % ny;
-                        }
-                        for (int x = x0 - 3; x < x0 + kTX + 3; x++) {
-                            int xx = x;
-                            if (xx < 0 || xx >= nx) {
-                                if (g->bc_x != kPeriodic && g->bc_x != kModPer) continue;
-                                xx = (xx % nx + nx) % nx;
-                            }
-                            if (solid[(size_t)yy * nx + xx]) {
-                                near_solid = true;
-                                break;
-                            }
-                        }
-                    }
-                    (near_solid ? te : tf).push_back(ty * ntx + tx);
+                    te.push_back(ty * ntx + tx);
                 }
             }
+        // ---- the C_SB nodes that each of those wets, and the tiles whose stored fluids can reach it
+        tg.insert(tg.end(), te.begin(), te.end());
+        std::vector<int> wof(N, -1);
+        for (size_t w = 0; w < widx.size(); w++) wof[widx[w]] = (int)w;
+        std::vector<int> owner(widx.size(), -1);
+        for (const int tile : tg) {
+            const int x0 = (tile % ntx) * kTX, y0 = (tile / ntx) * kTY;
+            std::vector<int> near;
+            const int first = (int)went.size();
+            bool open = false;
+            for (int Y = y0 - 3; Y < y0 + kTY + 3; Y++) {
+                int y = Y;
+                if (y < 0 || y >= ny) {
+                    if (!g->periodic_y) continue;
+                    y = ((y % ny) + ny) % ny;
+                }
+                for (int X = x0 - 3; X < x0 + kTX + 3; X++) {
+                    int x = X, par = 0;
+                    if (g->bc_x == kZouHe) {
+                        // a column that Zou-He completes may hold what nobody stored near it
+                        if (X <= 0 || X >= nx - 1) open = true;
+                        if (X < 0 || X >= nx) continue;
+                    } else if (x < 0 || x >= nx) {
+                        if (g->bc_x == kWalls) continue;
+                        const int q = floordiv_i(x, nx);
+                        x -= q * nx;
+                        par = g->bc_x == kModPer ? q & 1 : 0;
+                    }
+                    const size_t i = (size_t)y * nx + x;
+                    if (!solid[i]) {
+                        const int code = 2 * ((y / kTY) * ntx + x / kTX) + par;
+                        if (std::find(near.begin(), near.end(), code) == near.end()) near.push_back(code);
+                    } else if (cls[i] == kSB && X >= x0 - 2 && X < x0 + kTX + 2 && Y >= y0 - 2 && Y < y0 + kTY + 2) {
+                        const bool mine = X >= x0 && X < x0 + kTX && X < nx && Y >= y0 && Y < y0 + kTY && Y < ny;
+                        if (mine || owner[wof[i]] < 0) {
+                            if (owner[wof[i]] >= 0) went[owner[wof[i]]].z &= ~kWetOwner;
+                            owner[wof[i]] = (int)went.size();
+                        }
+                        went.push_back(make_int4((int)i, wof[i],
+                                                 (X - x0 + 2) | (Y - y0 + 2) << 8 | (par ? kWetPar : 0) |
+                                                     (owner[wof[i]] == (int)went.size() ? kWetOwner : 0),
+                                                 0));
+                    }
+                }
+            }
+            if (open || (int)near.size() > kTileRecInts - kTileRecHead) near.assign(1, -1);
+            near.resize(kTileRecInts - kTileRecHead, -2);
+            rec.insert(rec.end(), {tile, first, (int)went.size() - first});
+            rec.insert(rec.end(), near.begin(), near.end());
+        }
     }
-    const int n_wall_tiles = (int)tg.size();
-    const int n_edge_wall = (int)te.size();
-    tg.insert(tg.end(), te.begin(), te.end());
-    tg.insert(tg.end(), tf.begin(), tf.end());
+    // flags of the fluid nodes: the directions that bounce back there, and the domain's edges
+    std::vector<uint16_t> nflag(N, 0);
+    for (int y = 0; y < ny; y++)
+        for (int x = 0; x < nx; x++) {
+            const size_t i = (size_t)y * nx + x;
+            if (solid[i]) continue;
+            int f = (x == 0 ? kNodeX0 : 0) | (x == nx - 1 ? kNodeXN : 0) | (y == 0 ? kNodeY0 : 0) |
+                    (y == ny - 1 ? kNodeYN : 0);
+            if (cls[i] == kFB)
+                for (int a = 1; a < kQ; a++) f |= S(x - ex(a), y - ey(a)) << a;
+            nflag[i] = (uint16_t)f;
+        }
+    const int n_gen = (int)tg.size();
 
     // ---- parameters
     lbm3* h = new lbm3();
@@ -662,9 +668,8 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
     h->nw = (int)widx.size();
     h->n_fluid = n_fluid;
     h->n_pure = (int)tp.size();
-    h->n_gen = (int)tg.size();
-    h->n_walltiles = n_wall_tiles;
-    h->n_edgewall = n_edge_wall;
+    h->n_gen = n_gen;
+    h->n_went = (int)went.size();
     h->pure_fluid = pure_fluid;
     h->wall_host = widx;
 
@@ -684,7 +689,8 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
         }
     }
     if (e == cudaSuccess) e = dmalloc((void**)&h->type, N);
-    if (e == cudaSuccess) e = dmalloc((void**)&h->Cw, 3 * N * sizeof(double));
+    for (int b = 0; b < 2; b++)
+        if (e == cudaSuccess) e = dmalloc((void**)&h->cw[b], 3 * N * sizeof(double));
     if (e == cudaSuccess) e = dmalloc((void**)&h->u, 2 * N * sizeof(float));
     if (e == cudaSuccess) e = dmalloc((void**)&h->scratch, 3 * N * sizeof(float));
     if (e == cudaSuccess) e = dmalloc((void**)&h->partials, (size_t)diag_blocks(P) * 8 * sizeof(double));
@@ -696,38 +702,41 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
     if (e == cudaSuccess) e = dmalloc((void**)&h->widx, widx.size() * sizeof(int));
     if (e == cudaSuccess) e = dmalloc((void**)&h->wnrm, wnrm.size() * sizeof(double));
     if (e == cudaSuccess) e = dmalloc((void**)&h->wang, wang.size() * sizeof(float));
-    if (e == cudaSuccess) e = dmalloc((void**)&h->wcache, 4 * widx.size() * sizeof(WetCache));
-    if (e == cudaSuccess) {
-        reset_wet_cache(h->wcache, (int)widx.size(), nullptr);
-        e = cudaGetLastError();
+    WetLane* cache = nullptr;
+    if (e == cudaSuccess) e = dmalloc((void**)&cache, 4 * (size_t)h->n_went * sizeof(WetLane));
+    h->gen.cache = cache;
+    {
+        std::vector<double2> en;
+        for (const int4& w : went) en.push_back(make_double2(wnrm[2 * w.y], wnrm[2 * w.y + 1]));
+        const void* from[5] = {rec.data(), went.data(), nflag.data(), tp.data(), en.data()};
+        const size_t size[5] = {rec.size() * sizeof(int), went.size() * sizeof(int4), nflag.size() * sizeof(uint16_t),
+                                tp.size() * sizeof(int), en.size() * sizeof(double2)};
+        for (int j = 0; j < 5; j++) {
+            if (e == cudaSuccess) e = dmalloc(&h->tile_mem[j], size[j]);
+            if (e == cudaSuccess && size[j]) e = cudaMemcpy(h->tile_mem[j], from[j], size[j], cudaMemcpyHostToDevice);
+        }
     }
     h->pres_bytes = (size_t)((nx + kTX - 1) / kTX) * ((ny + kTY - 1) / kTY) * sizeof(uint64_t);
     for (int b = 0; b < 2; b++) {
         if (e == cudaSuccess) e = dmalloc((void**)&h->pres[b], h->pres_bytes);
         if (e == cudaSuccess) e = cudaMemset(h->pres[b], 0x07, h->pres_bytes);
     }
-    if (e == cudaSuccess) e = dmalloc((void**)&h->tiles_pure, tp.size() * sizeof(int));
-    if (e == cudaSuccess) e = dmalloc((void**)&h->tiles_gen, tg.size() * sizeof(int));
-    if (e == cudaSuccess && !tp.empty()) e = cudaMemcpy(h->tiles_pure, tp.data(), tp.size() * sizeof(int), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess && !tg.empty()) e = cudaMemcpy(h->tiles_gen, tg.data(), tg.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
         int lo = 0, hi = 0;
         e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
         if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, hi);
-        if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, hi);
         if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&h->side3, cudaStreamNonBlocking, hi);
         if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&h->gcap, cudaStreamNonBlocking);
     }
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_wet, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join2, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join3, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMemcpy(h->type, cls.data(), N, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !widx.empty()) e = cudaMemcpy(h->widx, widx.data(), widx.size() * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !wnrm.empty()) e = cudaMemcpy(h->wnrm, wnrm.data(), wnrm.size() * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess && !wang.empty()) e = cudaMemcpy(h->wang, wang.data(), wang.size() * sizeof(float), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(h->Cw, 0, 3 * N * sizeof(double));
+    for (int b = 0; b < 2; b++)
+        if (e == cudaSuccess) e = cudaMemset(h->cw[b], 0, 3 * N * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(h->u, 0, 2 * N * sizeof(float));
     // pure tiles through bulk tensor copies where the layout allows them (row pitch a multiple of
     // 16 bytes: nx % 4 == 0 for FP32 populations, nx % 8 == 0 for 16-bit offset planes);
@@ -750,7 +759,7 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
                 ep = f32 ? step_tma_prepare() : step_tma16_prepare();
                 if (ep != cudaSuccess) cudaGetLastError();
             }
-            // SMs left free for the wetting pass and the wall / edge tiles, which run on the side
+            // SMs left free for the wall / edge tiles, which run on the side
             // stream while the persistent pure-tile kernel holds its SMs: their share of the step's
             // work, in units of a pure tile's SM time as measured on the 4096 x 2048 pillars (a
             // wall or edge tile 1.8, the wetting pass 0.038 per C_SB node: 30 of 152 SMs there).
@@ -776,6 +785,9 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
             }
         }
     }
+    h->gen = TileSet{n_gen, (const int*)h->tile_mem[0], (const int4*)h->tile_mem[1], (const double2*)h->tile_mem[4], h->wang, h->gen.cache,
+                     h->type, (const uint16_t*)h->tile_mem[2]};
+    h->tiles_pure = (const int*)h->tile_mem[3];
     {
         // the two-blocks-per-SM kernel takes every pure tile itself
         const char* ov = std::getenv("LBM3_ONE_TILES");
@@ -810,7 +822,8 @@ int lbm3_set_fields(lbm3* h, const double* rho)
     CUDA_TRY(h, pres_reset(h));
     CUDA_TRY(h, cudaMemsetAsync(h->err_flag, 0, sizeof(int), h->stream));
     launch_init(h->precision, h->P, drho, h->type, h->pop[0], h->stream);
-    launch_wet_init(h->precision, h->P, h->nw, h->widx, h->pop[0], h->type, h->Cw, h->stream);
+    launch_wet_init(h->precision, h->P, h->nw, h->widx, h->pop[0], h->type, h->cw[h->pp], h->stream);
+    launch_wet_look(h->P, h->gen, h->n_went, h->cw[h->pp], h->stream);
     CUDA_TRY(h, cudaMemsetAsync(h->u, 0, 2 * N * sizeof(float), h->stream));
     CUDA_TRY(h, cudaFreeAsync(drho, h->stream));
     CUDA_TRY(h, cudaGetLastError());
@@ -928,9 +941,7 @@ int lbm3_fields(lbm3* h, double* rho_out, double* u_out)
     for (size_t i = 0; i < 3 * N; i++) rho_out[i] = tmp[i];
     if (u_out)
         for (size_t i = 0; i < 2 * N; i++) u_out[i] = tu[i];
-    int bits = 0;
-    if (int rc = take_kernel_error(h, &bits)) return rc;
-    if (bits & 1) return fail(h, LBM3_ERR_CUDA, "a bulk tensor copy of the step kernel did not complete in time");
+    if (int rc = take_kernel_error(h)) return rc;
     return LBM3_OK;
 }
 
@@ -941,9 +952,7 @@ int lbm3_diag(lbm3* h, double out[8])
     launch_diag(h->precision, h->P, h->pop[h->cur], h->type, h->u, h->partials, h->dout, h->stream);
     CUDA_TRY(h, cudaGetLastError());
     CUDA_TRY(h, cudaMemcpyAsync(out, h->dout, 8 * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
-    int bits = 0;
-    if (int rc = take_kernel_error(h, &bits)) return rc;
-    if (bits & 1) return fail(h, LBM3_ERR_CUDA, "a bulk tensor copy of the step kernel did not complete in time");
+    if (int rc = take_kernel_error(h)) return rc;
     if (out[7] > 0.0 || !(out[6] > 0.0)) return fail(h, LBM3_ERR_DIVERGED, "non-finite or non-positive density");
     return LBM3_OK;
 }
@@ -964,7 +973,7 @@ int lbm3_wall_values(lbm3* h, double* c, int32_t cap)
     if (!h->ready) return fail(h, LBM3_ERR_STATE, "lbm3_set_fields has not been called");
     const size_t N = (size_t)h->P.N;
     std::vector<double> cw(3 * N);
-    CUDA_TRY(h, cudaMemcpyAsync(cw.data(), h->Cw, 3 * N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    CUDA_TRY(h, cudaMemcpyAsync(cw.data(), h->cw[h->pp], 3 * N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     const int n = std::min<int>(cap, h->nw);
     for (int j = 0; j < n; j++) {
@@ -989,7 +998,7 @@ int lbm3_get_state(lbm3* h, double* f_post, double* wall_c)
     std::vector<double> cw;
     if (wall_c) {
         cw.resize(3 * N);
-        CUDA_TRY(h, cudaMemcpyAsync(cw.data(), h->Cw, 3 * N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+        CUDA_TRY(h, cudaMemcpyAsync(cw.data(), h->cw[h->pp], 3 * N * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
     }
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     for (size_t i = 0; i < 27 * N; i++) f_post[i] = tmp[i];
@@ -1008,7 +1017,10 @@ int lbm3_set_state(lbm3* h, const double* f_post, const double* wall_c)
     CUDA_TRY(h, pres_reset(h));
     CUDA_TRY(h, cudaMemsetAsync(h->err_flag, 0, sizeof(int), h->stream));
     launch_set_state(h->precision, h->P, dpost, h->type, h->pop[0], h->stream);
-    CUDA_TRY(h, cudaMemcpyAsync(h->Cw, wall_c, 3 * N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+    // both arrays: a step writes the C_SB nodes' values only
+    for (int b = 0; b < 2; b++)
+        CUDA_TRY(h, cudaMemcpyAsync(h->cw[b], wall_c, 3 * N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+    launch_wet_look(h->P, h->gen, h->n_went, h->cw[h->pp], h->stream);
     CUDA_TRY(h, cudaMemsetAsync(h->u, 0, 2 * N * sizeof(float), h->stream));
     CUDA_TRY(h, cudaFreeAsync(dpost, h->stream));
     CUDA_TRY(h, cudaGetLastError());
@@ -1028,8 +1040,8 @@ int lbm3_set_wall_angles(lbm3* h, const double* angles)
     }
     if (!a.empty())
         CUDA_TRY(h, cudaMemcpyAsync(h->wang, a.data(), a.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream));
-    // the wetting pass keeps each lane's angle with the wall values it came from: forget them
-    reset_wet_cache(h->wcache, h->nw, h->stream);
+    // the lines that the next step reads were looked for with the old angles
+    if (h->ready) launch_wet_look(h->P, h->gen, h->n_went, h->cw[h->pp], h->stream);
     CUDA_TRY(h, cudaGetLastError());
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     return LBM3_OK;
@@ -1069,12 +1081,10 @@ int lbm3_adjoint_centroid(lbm3* h, int32_t nsteps, int32_t K, double* J_out, dou
         if (e == cudaSuccess) e = cudaMalloc((void**)&st.sg_c, cb * seglen);
         if (e == cudaSuccess) e = cudaMalloc((void**)&st.fin_f, fb);
         if (e == cudaSuccess) e = cudaMalloc((void**)&st.fin_c, cb);
-        // the wetting pass stores only the C_SB nodes' wall values into a state's slot; the rest
+        // a step stores only the C_SB nodes' wall values into a state's slot; the rest
         // stays 0, as in the handle's own array
-        if (e == cudaSuccess) e = cudaMemset(st.ck_c, 0, cb * nck);
+            if (e == cudaSuccess) e = cudaMemset(st.ck_c, 0, cb * nck);
         if (e == cudaSuccess) e = cudaMemset(st.sg_c, 0, cb * seglen);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&st.ev_in, cudaEventDisableTiming);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&st.ev_saved, cudaEventDisableTiming);
         if (e == cudaSuccess) e = adjoint_alloc(h->P, h->nw, &st.W);
         if (e == cudaSuccess && h->ring) {
             st.box.resize(seglen);
@@ -1096,53 +1106,46 @@ int lbm3_adjoint_centroid(lbm3* h, int32_t nsteps, int32_t K, double* J_out, dou
         if (e != cudaSuccess) adj_release(h);
     };
     cudaStream_t s = h->stream;
-    // A state is saved while the next step runs, which only reads its populations: they are
-    // copied on the adjoint's side stream, which the step after next waits for, as it overwrites
-    // them; that step's wetting pass stores the wall values it starts from (saved_step).  A save
-    // that no step follows (the final state) copies the wall values itself.
-    cudaStream_t cs = adjoint_side_stream(W);
-    bool copying = false;
-    auto save_wait = [&]() {
-        if (copying) cudaStreamWaitEvent(s, st.ev_saved, 0);
-        copying = false;
-    };
-    auto save = [&](float* df, double* dc, bool stepped) {
-        save_wait();
-        cudaEventRecord(st.ev_in, s);
-        cudaStreamWaitEvent(cs, st.ev_in, 0);
-        cudaMemcpyAsync(df, h->pop[h->cur].f, fb, cudaMemcpyDeviceToDevice, cs);
-        cudaEventRecord(st.ev_saved, cs);
-        copying = true;
-        if (!stepped || h->nw == 0) cudaMemcpyAsync(dc, h->Cw, cb, cudaMemcpyDeviceToDevice, s);
-    };
-    // one step whose lagged wall values go to dc (or nowhere)
-    auto saved_step = [&](double* dc, bool last) {
-        h->cw_keep = h->nw > 0 ? dc : nullptr;
-        const cudaError_t r = enqueue_step(h, last, nullptr);
-        h->cw_keep = nullptr;
-        return r;
-    };
-    // Where the step kernels can read any buffer (the ring path, through the slot's tensor map, or
-    // the plain kernels), a segment's steps go from slot to slot of the store and its states need
-    // no copy: one step from slot j to `out`, its lagged wall values to slot j's
+    // Where the step kernels can read any buffer (the ring path, through the slot's tensor map, the
+    // plain kernels), a segment's steps go from slot to slot of the store.
     const bool direct = h->ring || !h->tma;
+    // the current state into a slot of a store
+    auto save = [&](float* df, double* dc) {
+        cudaMemcpyAsync(df, h->pop[h->cur].f, fb, cudaMemcpyDeviceToDevice, s);
+        cudaMemcpyAsync(dc, h->cw[h->pp], cb, cudaMemcpyDeviceToDevice, s);
+    };
     auto slot = [&](int j) { return Pop{sg_f + (size_t)j * 27 * N, nullptr, nullptr}; };
-    auto slot_step = [&](int j, const Pop& out, bool last) {
+    // one step from slot j to `out`, its wall values to cw_out
+    auto slot_step = [&](int j, const Pop& out, double* cw_out, bool last) {
         const Pop in = slot(j);
         h->io_in = &in;
         h->io_out = &out;
+        h->io_cw_out = cw_out;
         h->io_box = h->ring ? &st.box[j] : nullptr;
-        const cudaError_t r = saved_step(sg_c + (size_t)j * 3 * N, last);
+        const cudaError_t r = enqueue_step(h, last, nullptr);
         h->io_in = h->io_out = nullptr;
+        h->io_cw_out = nullptr;
         h->io_box = nullptr;
         return r;
     };
+    // n steps from slot 0 on, slot to slot
+    auto slot_steps = [&](int n) {
+        cudaError_t r = cudaSuccess;
+        for (int j = 0; j < n && r == cudaSuccess; j++) r = slot_step(j, slot(j + 1), sg_c + (size_t)(j + 1) * 3 * N, false);
+        return r;
+    };
+    // n steps of the handle's own buffers
+    auto own_steps = [&](int n) {
+        cudaError_t r = cudaSuccess;
+        for (int j = 0; j < n && r == cudaSuccess; j++) r = enqueue_step(h, false, nullptr);
+        return r;
+    };
     auto restore = [&](const float* df, const double* dc) {
-        save_wait();
         h->cur = 0;
         pres_reset(h);
         cudaMemcpyAsync(h->pop[0].f, df, fb, cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(h->Cw, dc, cb, cudaMemcpyDeviceToDevice, s);
+        cudaMemcpyAsync(h->cw[0], dc, cb, cudaMemcpyDeviceToDevice, s);
+        launch_wet_look(h->P, h->gen, h->n_went, h->cw[0], s);
     };
     // The whole sweep, enqueued without a host round trip (the seed reads J from the device
     // diagnostics): the forward pass with checkpoints, whose last segment's states go straight to
@@ -1151,60 +1154,47 @@ int lbm3_adjoint_centroid(lbm3* h, int32_t nsteps, int32_t K, double* J_out, dou
     // back into the handle.  capturing: recorded into a graph (no host waits allowed).
     auto enqueue_all = [&](bool capturing) -> cudaError_t {
         cudaError_t r = cudaSuccess;
-        const int t_last = (nseg - 1) * K;
-        for (int t = 0; t < nsteps && r == cudaSuccess; t++) {
-            double* dc = nullptr;
-            if (t >= t_last && direct) {
-                if (t == t_last) {
-                    save_wait();
-                    cudaMemcpyAsync(sg_f, h->pop[h->cur].f, fb, cudaMemcpyDeviceToDevice, s);
-                }
-                const int j = t - t_last;
-                if (t + 1 < nsteps) {
-                    r = slot_step(j, slot(j + 1), false);
-                } else {
-                    r = slot_step(j, h->pop[1 - h->cur], true);  // the final state in the handle's buffer
-                    h->cur = 1 - h->cur;
-                    pres_reset(h);  // the other word array describes a slot, not the other buffer
-                }
-                continue;
-            }
-            if (t >= t_last) {
-                dc = sg_c + (size_t)(t - t_last) * 3 * N;
-                save(sg_f + (size_t)(t - t_last) * 27 * N, dc, true);
-            } else if (t % K == 0) {
-                dc = ck_c + (size_t)(t / K) * 3 * N;
-                save(ck_f + (size_t)(t / K) * 27 * N, dc, true);
-            } else {
-                save_wait();  // the copy of the previous state is done before this step overwrites it
-            }
-            r = saved_step(dc, t == nsteps - 1);
+        const int t_last = (nseg - 1) * K, n_last = nsteps - t_last;
+        for (int seg = 0; seg < nseg - 1 && r == cudaSuccess; seg++) {
+            save(ck_f + (size_t)seg * 27 * N, ck_c + (size_t)seg * 3 * N);
+            r = own_steps(K);
         }
-        save_wait();
+        if (r != cudaSuccess) return r;
+        if (direct) {
+            save(sg_f, sg_c);
+            r = slot_steps(n_last - 1);
+            // the final state in the handle's other buffer
+            const int c = 1 - h->cur;
+            if (r == cudaSuccess) r = slot_step(n_last - 1, h->pop[c], h->cw[c], true);
+            h->cur = c;
+            pres_reset(h);  // the words describe the slots, not the handle's buffers
+        } else {
+            for (int j = 0; j < n_last && r == cudaSuccess; j++) {
+                save(sg_f + (size_t)j * 27 * N, sg_c + (size_t)j * 3 * N);
+                r = enqueue_step(h, j == n_last - 1, nullptr);
+            }
+        }
         if (r != cudaSuccess) return r;
         launch_diag(h->precision, h->P, h->pop[h->cur], h->type, h->u, h->partials, h->dout, s);
-        save(fin_f, fin_c, false);
-        save_wait();
+        save(fin_f, fin_c);
         cudaMemsetAsync(adjoint_dang(W), 0, sizeof(double) * 3 * (size_t)std::max(h->nw, 1), s);
         cudaMemsetAsync(adjoint_du(W), 0, sizeof(double), s);
         adjoint_seed(h->P, W, h->pop[h->cur].f, h->type, h->dout, s);
         for (int seg = nseg - 1; seg >= 0 && r == cudaSuccess; seg--) {
             const int t0 = seg * K, t1 = std::min(nsteps, t0 + K);
             if (seg < nseg - 1 && direct) {
-                // the checkpoint into slot 0 and the wall values into the handle, then slot to slot
+                // the checkpoint into slot 0, then slot to slot
                 pres_reset(h);
                 cudaMemcpyAsync(sg_f, ck_f + (size_t)seg * 27 * N, fb, cudaMemcpyDeviceToDevice, s);
-                cudaMemcpyAsync(h->Cw, ck_c + (size_t)seg * 3 * N, cb, cudaMemcpyDeviceToDevice, s);
-                for (int t = t0; t < t1 - 1 && r == cudaSuccess; t++) r = slot_step(t - t0, slot(t - t0 + 1), false);
-                cudaMemcpyAsync(sg_c + (size_t)(t1 - 1 - t0) * 3 * N, h->Cw, cb, cudaMemcpyDeviceToDevice, s);
+                cudaMemcpyAsync(sg_c, ck_c + (size_t)seg * 3 * N, cb, cudaMemcpyDeviceToDevice, s);
+                launch_wet_look(h->P, h->gen, h->n_went, sg_c, s);
+                r = slot_steps(t1 - t0 - 1);
             } else if (seg < nseg - 1) {
                 restore(ck_f + (size_t)seg * 27 * N, ck_c + (size_t)seg * 3 * N);
-                for (int t = t0; t < t1; t++) {
-                    double* dc = sg_c + (size_t)(t - t0) * 3 * N;
-                    save(sg_f + (size_t)(t - t0) * 27 * N, dc, t < t1 - 1);
-                    if (t < t1 - 1 && (r = saved_step(dc, false)) != cudaSuccess) break;
+                for (int t = t0; t < t1 && r == cudaSuccess; t++) {
+                    save(sg_f + (size_t)(t - t0) * 27 * N, sg_c + (size_t)(t - t0) * 3 * N);
+                    if (t < t1 - 1) r = enqueue_step(h, false, nullptr);
                 }
-                save_wait();
             }
             // the intermediates of step t - 1 are prepared on the adjoint's side stream while the
             // reverse of step t runs
@@ -1262,7 +1252,6 @@ int lbm3_adjoint_centroid(lbm3* h, int32_t nsteps, int32_t K, double* J_out, dou
         }
         h->cur = cur0;  // the capture ran nothing
         h->pp = cur0;
-        copying = false;
     }
     if (st.gexec) {
         e = cudaGraphLaunch(st.gexec, s);
@@ -1280,9 +1269,7 @@ int lbm3_adjoint_centroid(lbm3* h, int32_t nsteps, int32_t K, double* J_out, dou
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     cleanup();
     if (e != cudaSuccess) return fail(h, LBM3_ERR_CUDA, std::string("adjoint: ") + cudaGetErrorString(e));
-    int bits = 0;
-    if (int rc = take_kernel_error(h, &bits)) return rc;
-    if (bits & 1) return fail(h, LBM3_ERR_CUDA, "a bulk tensor copy of the step kernel did not complete in time");
+    if (int rc = take_kernel_error(h)) return rc;
     *J_out = d[3] / d[0];
     for (int w = 0; w < h->nw; w++)
         for (int j = 0; j < 3; j++) dJ_dangles[3 * w + j] = dang[(size_t)j * h->nw + w];
@@ -1300,11 +1287,10 @@ int lbm3_info(const lbm3* h, int64_t out[9])
     // and 8 16-bit offsets (120 B); plus one class byte per node
     const long long per = h->precision == LBM3_FP32 ? 216 : 120;
     out[2] = h->n_fluid * per + h->P.N;
-    out[3] = (h->n_pure > 0) + h->one + (h->n_walltiles > 0) + (h->n_edgewall > 0) +
-             (h->n_gen - h->n_walltiles - h->n_edgewall > 0);
-    out[4] = h->nw > 0 ? 1 : 0;
+    out[3] = (h->n_pure > 0) + h->one + (h->n_gen > 0);
+    out[4] = 0;  // the wetting is part of the tiles' launch
     out[5] = (int64_t)h->bytes;
-    // the pure-tile launch reads and writes 27 FP32 populations per node and no class bytes
+    // as if every node of the pure tiles held all three fluids
     out[6] = h->pure_fluid * per;
     out[7] = h->pure_fluid;
     out[8] = h->ring ? 2 : (h->tma ? 1 : 0);

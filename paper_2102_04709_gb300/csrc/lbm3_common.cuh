@@ -198,7 +198,8 @@ __device__ __forceinline__ void zou_he(const Params& P, float p[27], bool inlet)
     }
 }
 
-// Post-streaming populations of fluid k for the pull from a stored buffer.
+// Post-streaming populations of fluid k for the pull from a stored buffer.  (Plain loads: the kernel
+// that marches many steps in one launch writes what it read through the same pointers before.)
 template <int STORE>
 struct Store;
 
@@ -211,7 +212,7 @@ struct Store<kStoreF32> {
     // population a of (storage) fluid k stored at node idx
     __device__ __forceinline__ float get(int k, int a, int idx) const
     {
-        return __ldg(f + (long long)(k * kQ + a) * N + idx);
+        return f[(long long)(k * kQ + a) * N + idx];
     }
 };
 
@@ -224,11 +225,11 @@ struct Store16 {
     // offset of population a >= 1 of fluid k at node idx
     __device__ __forceinline__ float offset(int k, int a, int idx) const
     {
-        return dec16<STORE>(__ldg(off + (long long)(8 * k + a - 1) * N + idx));
+        return dec16<STORE>(off[(long long)(8 * k + a - 1) * N + idx]);
     }
     __device__ __forceinline__ float get(int k, int a, int idx) const
     {
-        const float r = __ldg(rho + (long long)k * N + idx);
+        const float r = rho[(long long)k * N + idx];
         if (a > 0) return wq(a) * r + offset(k, a, idx);
         float d[kQ];
 #pragma unroll
@@ -295,30 +296,49 @@ __device__ void pull_global(const Params& P, const S& st, const uint8_t* __restr
     if (outlet) zou_he(P, p, false);
 }
 
-// Where the characteristic line of one lane of the wetting pass (C_SB node, wetted fluid, side)
-// met the fluid for the local contact angle th of Eq.(21) it was marched with: the line depends
-// on th and the fixed geometry only, so while a node's th repeats bit for bit (every node away
-// from a moving contact line) the march is skipped and its crossing reused.  th itself is kept
-// with the two wall values (wm, wl) of Eq.(21) it came from, so that while those repeat it is
-// not recomputed either (the wall angles are fixed between resets of the cache).  th, wm, wl =
-// NaN: none yet.
-struct WetCache {
+// Where the characteristic line of one lane (C_SB node, wetted fluid, side) meets the fluid in the
+// next step: for the local contact angle th of Eq.(21), which comes from the wall values wm, wl (kept
+// in the lanes of side 0).  The line depends on th and the fixed geometry only, so it is marched anew
+// only where th changed, and th computed anew only where wm or wl did.  ia, fa and ib, fb: storage
+// index and flags of the one or two nodes that bracket the crossing (-1: none), fr its fraction from
+// a to b.
+struct alignas(16) WetLane {
     double th, fr, wm, wl;
-    int kind, ax, ay, bx, by, pad;
+    int ia, fa, ib, fb;
+};
+// flags of a fluid node: bits 0-8, direction a bounces back there; its column and row are the first
+// or last ones; (in a lane) it lies an odd number of seams away from the C_SB node, or in the tile's
+// phase-field region
+constexpr int kNodePar = 1 << 9;
+constexpr int kNodeNear = 1 << 14;
+constexpr int kNodeX0 = 1 << 10, kNodeXN = 1 << 11, kNodeY0 = 1 << 12, kNodeYN = 1 << 13;
+
+// A list of tiles with what a step needs to know of each: a record of 32 words -- the tile, its first
+// entry and their number in went (the C_SB nodes of its phase-field region, four lanes of the cache
+// each), and, from word kTileRecHead on, the tiles whose stored fluids can reach it: 2 x tile, + 1
+// across the modified periodic seam, -1 for any fluid (an open column in reach), -2 for none.
+// Entry: node, its place in the wall list, and its position in the region (cx | cy << 8) with the
+// flags below.
+constexpr int kWetOwner = 1 << 16;  // this tile writes the node's wall values
+constexpr int kWetPar = 1 << 17;    // seen across the modified periodic seam
+constexpr int kTileRecInts = 32, kTileRecHead = 3;
+struct TileSet {
+    int ntiles;
+    const int* rec;
+    const int4* went;
+    const double2* wnrm;  // by entry: the outward normal
+    const float* wang;    // by place in the wall list: the three angles
+    WetLane* cache;
+    const uint8_t* type;
+    const uint16_t* nflag;  // flags of every fluid node (0 at solid ones)
 };
 
 // ---- kernel launchers (lbm3_step.cu); `store` is kStoreF32 / kStoreF16 / kStoreBF16 ----
-// Cw_prev (or nullptr): where the wetting pass also stores the lagged wall values it reads
-void launch_wet(int store, const Params& P, int nw, const int* widx, const double* wnrm,
-                const float* wang, const Pop& f, const uint8_t* type, double* Cw, WetCache* cache,
-                cudaStream_t s, double* Cw_prev = nullptr);
-void reset_wet_cache(WetCache* cache, int nw, cudaStream_t s);
 void launch_wet_init(int store, const Params& P, int nw, const int* widx, const Pop& f,
                      const uint8_t* type, double* Cw, cudaStream_t s);
-// tile of the fused step kernel (interior nodes per CTA)
+// tile of the step kernels (nodes per CTA); pure tile: free of solid nodes within 3 nodes of it and
+// away from the domain edges; tiles: list of tile indices ty * ceil(nx / kTX) + tx
 constexpr int kTX = 32, kTY = 8;
-// tiles: list of tile indices ty * ceil(nx / kTX) + tx; pure = every listed tile is free of solid
-// nodes within 3 nodes of it and away from the domain edges
 // pure FP32 tiles through bulk tensor copies (persistent, nblocks blocks): the dynamic shared
 // memory they need, the one-time attribute set-up, and the launch with tensor maps of fin
 // (boxes (kTX + 8, kTY + 6, kTmaPlanesA) and (kTX + 8, kTY + 6, 27 - kTmaPlanesA)) and fout
@@ -351,15 +371,15 @@ size_t step_tma16_smem_bytes();
 void launch_step_tma16(int store, const Params& P, const int* tiles, int ntiles, int nblocks, const Pop& fout,
                        float* u, const CUtensorMap& trho, const CUtensorMap& toff, const uint64_t* pres_in,
                        uint64_t* pres_out, bool all, cudaStream_t s);
-// tile lists of the fused step: pure tiles (no solid within 3 nodes, away from the domain
-// edge), wall tiles (solids near, halo inside the domain) and edge tiles (halo crossing the
-// domain edge: wrap, ghost columns, seam)
-constexpr int kTilesPure = 0, kTilesWall = 1, kTilesEdge = 2;
-// pres_in / pres_out: fluids present per tile in the step's input / output; the wall tiles read
-// and write them (see k_step), the other kinds ignore them
-void launch_step(int store, const Params& P, const int* tiles, int ntiles, int kind, const Pop& fin,
-                 const Pop& fout, const uint8_t* type, const double* Cw, float* u, const uint64_t* pres_in,
-                 uint64_t* pres_out, cudaStream_t s, bool all = false);
+// pure tiles by plain loads, any storage and nx
+void launch_step_plain(int store, const Params& P, const int* tiles, int ntiles, const Pop& fin, const Pop& fout,
+                       float* u, const uint64_t* pres_in, uint64_t* pres_out, bool all, cudaStream_t s);
+// tiles of any kind, one per block; cw_out: the wall values of this step (those of the last one are in
+// the cache's lines)
+void launch_tile(int store, const Params& P, const TileSet& T, const Pop& fin, const Pop& fout, double* cw_out, float* u,
+                 const uint64_t* pres_in, uint64_t* pres_out, bool full_write, cudaStream_t s);
+// the cache's lines from the wall values Cw, after those or the wall angles were replaced
+void launch_wet_look(const Params& P, const TileSet& T, int entries, const double* Cw, cudaStream_t s);
 void launch_init(int store, const Params& P, const double* rho, const uint8_t* type, const Pop& f,
                  cudaStream_t s);
 void launch_fields(int store, const Params& P, const Pop& f, const uint8_t* type, float* rho_out,

@@ -67,8 +67,8 @@ __device__ __forceinline__ bool node_is_fluid(const Params& P, const uint8_t* __
 // are summed with error-free transformations and divided in float-float arithmetic (div_df), so
 // the value is the fraction of the stored FP32 populations to about 44 bits (a node holding one
 // fluid gives exactly 0 or 1) without a double-precision division, which is slow on this GPU.
-// (kept out of line: the wetting pass calls it up to ten times per lane, and inlining each call
-// made that kernel wait on its instruction cache)
+// (kept out of line: its callers call it up to ten times per lane, and inlining each call made them
+// wait on the instruction cache)
 template <class S>
 __device__ __noinline__ double node_C(const Params& P, const S& st, const uint8_t* __restrict__ type, int X,
                          int Y, int k)

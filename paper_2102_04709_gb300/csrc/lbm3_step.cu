@@ -2,12 +2,14 @@
 // lattice Boltzmann model with the characteristic-line wetting condition
 // (arXiv:2102.04709, Section II).
 //
-//   k_wet      Eq.(21)-(22) and the characteristic lines of Section II.B, one thread per
-//              solid boundary node (C_SB), FP64 ray geometry
-//   k_step     fused Eq.(1)-(16): pull-streaming with halfway bounce-back (and the x boundary),
-//              densities and phase fields, isotropic gradients (Eq.12), the surface-stress
-//              tensor and its divergence (Eq.10), MRT collision with forcing (Eq.1-9, 11),
-//              recolouring (Eq.13-15); one CTA per TX x TY tile, halo staged in shared memory
+//   tiles (TX x TY nodes, halo staged in shared memory): fused Eq.(1)-(16): pull-streaming with
+//              halfway bounce-back (and the x boundary), densities and phase fields, isotropic
+//              gradients (Eq.12), the surface-stress tensor and its divergence (Eq.10), MRT
+//              collision with forcing (Eq.1-9, 11), recolouring (Eq.13-15)
+//     k_tile     tiles near solids or the domain edge, one per CTA, with the wetting of their
+//                solid boundary nodes (Eq.21-22, characteristic lines, FP64 ray geometry)
+//     k_step_one, k_step_ring, k_step_tma, k_step_tma16, k_step_plain    pure tiles: no solid
+//                within 3 nodes, away from the domain edge
 //   k_init     rest-equilibrium initial state written as the pre-image of a pull
 //   k_fields   post-streaming densities
 //   k_diag     FP64 block partials of mass, centroid, max|u|, min rho, non-finite count
@@ -20,96 +22,6 @@
 namespace lbm3k {
 
 namespace {
-
-// Four lanes per C_SB node: lane = 2 * k + side, for the wetted fluids k = 0, 1 and the two
-// characteristic lines (rotated by +phi and -phi from n_s).  Each lane marches its line over the
-// class bytes, then gathers C at the one or two nodes it found; Eq.(22) combines the two lines
-// of a fluid with a shuffle, and lane 0 writes the wall values (and, when Cw_prev is given, the
-// lagged ones it started from, which the adjoint keeps for every step).
-template <class S>
-__global__ void __launch_bounds__(128) k_wet(const Params P, const int nw, const int* __restrict__ widx,
-                                             const double* __restrict__ wnrm,
-                                             const float* __restrict__ wang, const S st,
-                                             const uint8_t* __restrict__ type, double* __restrict__ Cw,
-                                             WetCache* __restrict__ cache, double* __restrict__ Cw_prev)
-{
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    const int w = g >> 2;
-    const int k = (g >> 1) & 1, side = g & 1;
-    const bool valid = w < nw;
-    int i = 0, px = 0, py = 0;
-    double th = 90.0;
-    Crossing cr{0, 0, 0, 0, 0, 0.0};
-    if (valid) {
-        i = widx[w];
-        px = i % P.nx;
-        py = i / P.nx;
-        // Eq.(21) with the wall values of the previous step
-        const double Cr = Cw[i], Cg = Cw[P.N + i], Cb = Cw[2 * P.N + i];
-        if (Cw_prev && (g & 3) == 0) {
-            Cw_prev[i] = Cr;
-            Cw_prev[P.N + i] = Cg;
-            Cw_prev[2 * P.N + i] = Cb;
-        }
-        const double wm = Cb, wl = k == 0 ? Cg : Cr;  // the weights of Eq.(21) for fluid k
-        const WetCache c = cache[g];
-        if (c.wm == wm && c.wl == wl) {
-            // the same wall values as last time: the same angle, line and crossing
-            th = c.th;
-            cr = Crossing{c.kind, c.ax, c.ay, c.bx, c.by, c.fr};
-        } else {
-            const double t_rg = wang[3 * w], t_br = wang[3 * w + 1], t_gb = wang[3 * w + 2];
-            th = k == 0 ? local_angle(wm, 180.0 - t_br, wl, t_rg) : local_angle(wm, t_gb, wl, 180.0 - t_rg);
-            if (c.th == th) {
-                // the same angle as when this lane last marched: the same line, the same crossing
-                cr = Crossing{c.kind, c.ax, c.ay, c.bx, c.by, c.fr};
-            } else {
-                const double nx_ = wnrm[2 * w], ny_ = wnrm[2 * w + 1];
-                const double dev = fabs(90.0 - th);
-                const double phi = dev < kPhiSnap ? 0.0 : dev * (M_PI / 180.0);
-                double sn, cs;
-                sincos(phi, &sn, &cs);
-                if (side) sn = -sn;
-                // the line makes the angle phi with n_s (tangent (-n_y, n_x))
-                cr = characteristic_line<S>(P, type, px, py, cs * nx_ - sn * ny_, cs * ny_ + sn * nx_);
-            }
-            cache[g] = WetCache{th, cr.fr, wm, wl, cr.kind, cr.ax, cr.ay, cr.bx, cr.by, 0};
-        }
-    }
-    double ca = 0.0, cb = 0.0;
-    if (valid && cr.kind >= 1) ca = node_C(P, st, type, cr.ax, cr.ay, k);
-    if (valid && cr.kind == 2) cb = node_C(P, st, type, cr.bx, cr.by, k);
-    if (valid && cr.kind == 0) ca = neighbour_mean(P, st, type, px, py, k);
-    const double cd = cr.kind == 2 ? ca + cr.fr * (cb - ca) : ca;
-    // Eq.(22): max of the two lines for theta_k <= 90 deg, min otherwise
-    const double other = __shfl_xor_sync(0xffffffffu, cd, 1);
-    const double cp = th <= 90.0 ? fmax(cd, other) : fmin(cd, other);
-    const double cg = __shfl_xor_sync(0xffffffffu, cp, 2);
-    if (valid && (g & 3) == 0) {
-        // fractions stay in [0, 1] (a no-op unless 16-bit storage rounded a density below 0)
-        double c0 = fmin(fmax(cp, 0.0), 1.0), c1 = fmin(fmax(cg, 0.0), 1.0);
-        const double s = c0 + c1;
-        if (s > 1.0) {
-            c0 /= s;
-            c1 /= s;
-        }
-        Cw[i] = c0;
-        Cw[P.N + i] = c1;
-        Cw[2 * P.N + i] = fmax(0.0, 1.0 - c0 - c1);
-    }
-}
-
-// initial wall values: w-weighted mean of the fluid neighbours, for each fluid
-template <class S>
-__global__ void k_wet_init(const Params P, const int nw, const int* __restrict__ widx, const S st,
-                           const uint8_t* __restrict__ type, double* __restrict__ Cw)
-{
-    const int w = blockIdx.x * blockDim.x + threadIdx.x;
-    if (w >= nw) return;
-    const int i = widx[w];
-    const int px = i % P.nx, py = i / P.nx;
-    for (int k = 0; k < kNF; k++) Cw[k * P.N + i] = neighbour_mean(P, st, type, px, py, k);
-}
 
 // ------------------------------------------------------------------------------------------
 // fused step
@@ -287,11 +199,6 @@ constexpr int kWaitLimit = 1 << 22;
 // lagged wetting feedback amplifies the rounding of single-precision phase fields.  Away from
 // such nodes the phase fields near walls are those of one fluid and a float suffices.
 constexpr double kMixEps = 1e-6;
-__device__ __forceinline__ bool mixed_wall(const double* __restrict__ Cw, long long N, long long i)
-{
-    const double m = fmax(fmax(Cw[i], Cw[N + i]), Cw[2 * N + i]);
-    return m < 1.0 - kMixEps;
-}
 
 // Eq.(12) derivative of a float field held in shared memory
 template <int W>
@@ -427,42 +334,36 @@ __device__ __forceinline__ int phase_fields(bool df, const float q[27], float (*
     return (r[0] != 0.0f ? 1 : 0) | (r[1] != 0.0f ? 2 : 0) | (r[2] != 0.0f ? 4 : 0);
 }
 
-// Wall values of a C_SB node at (cx, cy) of the phase-field region (FP64 from the wetting pass,
-// split into hi + lo; labels relabelled across a modified periodic seam when par); rho := 1 at
-// solid nodes.  Returns the fluids with a nonzero wall value.
-template <int CX, int CY>
-__device__ __forceinline__ int wall_fields(const double* __restrict__ Cw, long long N, int in, bool par,
-                                           float (*ch)[CY][CX], float (*cl)[CY][CX], float (*rh)[CX], int cx,
-                                           int cy)
+// Geometry word of a position of a tile's halo-3 region: the storage index of the node it shows
+// (its own, wrapped, or the boundary-column node beyond an open side), the node's class, and
+// whether the position lies beyond an open side or an odd number of seams away.
+constexpr int kGeoIdx = (1 << 27) - 1;  // 27 nx ny < 2^31
+constexpr int kGeoSolid = 1 << 28;      // bit 1 of the class
+constexpr int kGeoGhost = 1 << 29;
+constexpr int kGeoPar = 1 << 30;
+__device__ __forceinline__ int geo_class(int g) { return (g >> 27) & 3; }
+__device__ __forceinline__ int geo_word(const Params& P, const uint8_t* __restrict__ type, int X, int Y)
 {
-    int present = 0;
-#pragma unroll
-    for (int k = 0; k < kNF; k++) {
-        const double c = Cw[(long long)relabel(k, par) * N + in];
-        const float h = (float)c;
-        ch[k][cy][cx] = h;
-        cl[k][cy][cx] = (float)(c - (double)h);
-        if (c != 0.0) present |= 1 << k;
-    }
-    rh[cy][cx] = 1.0f;
-    return present;
+    const Loc L = locate(P, X, Y);
+    if (L.kind == 1) return kSI << 27;
+    return L.idx | (int)(__ldg(type + L.idx) & 3) << 27 | (L.kind == 2 ? kGeoGhost : 0) | (L.par ? kGeoPar : 0);
 }
 
 // Eq.(12) gradients (gxk, gyk) and the Eq.(10) stress of position (rx, ry) of the stress region
-// of a tile with solids: class bytes t of the geometry region (halo 3), phase fields of the
+// of a tile with solids: geometry words t of the halo-3 region, phase fields of the
 // phase-field region (halo 2).  At a C_SB centre a neighbour without a value of its own takes
 // the extrapolation 2 C(P) - C(P - e_a) (its rounding error carried in the lo word), or C(P)
 // when P - e_a has none either; lo words exist only in float-float (df) tiles.
 template <int HX, int CX, int CY>
-__device__ __forceinline__ void stress_at(const Params& P, const uint8_t (*t)[HX], const float (*ch)[CY][CX],
+__device__ __forceinline__ void stress_at(const Params& P, const int (*t)[HX], const float (*ch)[CY][CX],
                                           const float (*cl)[CY][CX], const float (*rh)[CX], bool df, int rx,
                                           int ry, float gxk[kNF], float gyk[kNF], float& Txx, float& Txy,
                                           float& Tyy)
 {
     const int cx = rx + 1, cy = ry + 1, hx = rx + 2, hy = ry + 2;
     Txx = Txy = Tyy = 0.f;
-    const uint8_t tc = t[hy][hx];
-    if ((tc & 3) == kSI) {
+    const int tc = geo_class(t[hy][hx]);
+    if (tc == kSI) {
 #pragma unroll
         for (int k = 0; k < kNF; k++) gxk[k] = gyk[k] = 0.0f;
         return;
@@ -471,26 +372,27 @@ __device__ __forceinline__ void stress_at(const Params& P, const uint8_t (*t)[HX
     float c[kNF];
 #pragma unroll
     for (int k = 0; k < kNF; k++) c[k] = ch[k][cy][cx];
-    if ((tc & 3) == kSB) {
+    if (tc == kSB) {
+        // where neighbour a takes its value from: itself, or through the centre from the opposite
+        // neighbour (bit a of ext), or the centre (bit a of ctr)
+        int ext = 0, ctr = 0;
 #pragma unroll
+        for (int a = 1; a < kQ; a++)
+            if (geo_class(t[hy + ey(a)][hx + ex(a)]) == kSI)
+                (geo_class(t[hy - ey(a)][hx - ex(a)]) == kSI ? ctr : ext) |= 1 << a;
+#pragma unroll 1
         for (int k = 0; k < kNF; k++) {
             float v[kQ], vl[kQ];
             const float h0 = ch[k][cy][cx], l0 = df ? cl[k][cy][cx] : 0.0f;
 #pragma unroll
             for (int a = 1; a < kQ; a++) {
-                if ((t[hy + ey(a)][hx + ex(a)] & 3) != kSI) {
-                    v[a] = ch[k][cy + ey(a)][cx + ex(a)];
-                    vl[a] = df ? cl[k][cy + ey(a)][cx + ex(a)] : 0.0f;
-                } else if ((t[hy - ey(a)][hx - ex(a)] & 3) == kSI) {
-                    v[a] = h0;
-                    vl[a] = l0;
-                } else {
-                    const float oh = ch[k][cy - ey(a)][cx - ex(a)];
-                    const float ol = df ? cl[k][cy - ey(a)][cx - ex(a)] : 0.0f;
-                    float e;
-                    two_sum(2.0f * h0, -oh, v[a], e);
-                    vl[a] = (2.0f * l0 - ol) + e;
-                }
+                const bool x = ext >> a & 1, c = ctr >> a & 1;
+                const int yy = c ? cy : (x ? cy - ey(a) : cy + ey(a)), xx = c ? cx : (x ? cx - ex(a) : cx + ex(a));
+                const float oh = ch[k][yy][xx], ol = df ? cl[k][yy][xx] : 0.0f;
+                float e;
+                two_sum(2.0f * h0, -oh, v[a], e);
+                vl[a] = x ? (2.0f * l0 - ol) + e : ol;
+                v[a] = x ? v[a] : oh;
             }
             gxk[k] = (1.0f / 3.0f) * (v[1] - v[3]) + (1.0f / 12.0f) * ((v[5] - v[7]) + (v[8] - v[6])) +
                      ((1.0f / 3.0f) * (vl[1] - vl[3]) + (1.0f / 12.0f) * ((vl[5] - vl[7]) + (vl[8] - vl[6])));
@@ -522,359 +424,6 @@ __device__ __forceinline__ int fluids_around(const uint64_t* __restrict__ pres, 
     nb |= nb >> 8;
     return (int)(nb & 7u);
 }
-
-// resident blocks per SM the wall-tile specialisation of the one-tile-per-block step kernel is
-// compiled for (registers capped at 65536 / (256 x this)); the others for four
-#ifndef LBM3_STEP_BLOCKS_PER_SM
-#define LBM3_STEP_BLOCKS_PER_SM 5
-#endif
-constexpr int kStepBlocksPerSm = LBM3_STEP_BLOCKS_PER_SM;
-
-// One CTA per TX x TY tile of interior nodes.
-//   phase 0: class bytes (and, for tiles touching the domain edge, storage indices and seam
-//            parities) of the halo-3 region into shared memory
-//   phase 1: pull-streaming of every fluid node of the halo-2 region, densities rho_k and the
-//            phase fields C_k; the tile's own nodes keep their 9 post-streaming totals and 3
-//            densities in registers
-//   phase 2: the Eq.(10) stress tensor on the halo-1 region
-//   phase 3: force, velocity, MRT collision with forcing, recolouring, 27 stores per node
-// Tiles whose halo-3 region stays inside the domain take arithmetic source indices and skip the
-// bounce-back tests at C_FI nodes; only tiles whose halo-2 region holds a C_SB node with mixed
-// wall values (a contact line at or near it) carry the float-float phase fields, decided anew
-// every step from the wall values of this step's wetting pass.
-template <int TX, int TY, bool PURE, bool INNER, int STORE>
-__global__ void __launch_bounds__(TX* TY, (INNER && !PURE) ? kStepBlocksPerSm : 4) k_step(const Params P, const int* __restrict__ tiles,
-                                                  const Pop fin, const Pop fout,
-                                                  const uint8_t* __restrict__ type,
-                                                  const double* __restrict__ Cw,
-                                                  float* __restrict__ uout,
-                                                  const uint64_t* __restrict__ pres_in,
-                                                  uint64_t* __restrict__ pres_out, const int all)
-{
-    constexpr int NT = TX * TY;
-    constexpr int HX = TX + 6, HY = TY + 6;  // geometry region (halo 3)
-    constexpr int CX = TX + 4, CY = TY + 4;  // phase-field region (halo 2)
-    constexpr int RX = TX + 2, RY = TY + 2;  // stress region (halo 1)
-    __shared__ int s_idx[HY][HX];            // storage index (tiles at the domain edge only)
-    __shared__ uint8_t s_t[HY][HX];          // class bits 0-1; bit 3: ghost beyond an open side
-    __shared__ uint8_t s_par[HX];
-    __shared__ float s_ch[kNF][CY][CX], s_cl[kNF][CY][CX];  // C_k = hi (+ lo in wall tiles)
-    __shared__ float s_rho[CY][CX];
-    __shared__ float s_txx[RY][RX], s_txy[RY][RX], s_tyy[RY][RX];
-    __shared__ float s_g[2 * kNF][TY][TX];   // colour gradients of the tile's own nodes
-    __shared__ int s_flags[2];                // fluids present (wall and edge tiles)
-    // wall tiles: fluids stored in the 3 x 3 tiles around (one word each), and the fluids with a
-    // nonzero wall value at the C_SB nodes of the phase-field region (one word per warp)
-    __shared__ uint64_t s_nb[9];
-    __shared__ int s_wp[TX * TY / 32];
-
-    const int tid = threadIdx.x + TX * threadIdx.y;
-    if (!PURE && tid == 0) s_flags[0] = 0;  // published by the phase-0 barrier
-    const int ntx = (P.nx + TX - 1) / TX;
-    const int tile = tiles[blockIdx.x];
-    // the pure tiles with one fluid around are k_step_one's
-    if (PURE && !all && __popc((unsigned)fluids_around(pres_in, tile, ntx)) == 1) return;
-    const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
-    const int nx = P.nx;
-    const int N = (int)P.N;
-    // halo-3 region inside the domain: no wrap, no ghost, no seam (INNER: every listed tile).
-    // A PURE tile is also free of solid nodes in that region (every node it touches is in C_FI).
-    const bool inner = PURE || INNER || (x0 >= 3 && y0 >= 3 && x0 + TX + 3 <= P.nx && y0 + TY + 3 <= P.ny);
-
-    // ---- phase 0: geometry of the halo-3 region ----
-    int wall = 0, wp = 0;
-    if (PURE) {
-    } else if (inner) {
-        if constexpr (INNER) {
-            if (tid < 9) s_nb[tid] = pres_in[tile + (tid / 3 - 1) * ntx + (tid % 3 - 1)];
-        }
-        for (int j = tid; j < HX * HY; j += NT) {
-            const int hx = j % HX, hy = j / HX;
-            const uint8_t t = __ldg(type + (y0 + hy - 3) * nx + (x0 + hx - 3));
-            s_t[hy][hx] = t;
-            if ((t & 3) == kSB && hx >= 1 && hx <= CX && hy >= 1 && hy <= CY) {
-                const long long in = (long long)(y0 + hy - 3) * nx + (x0 + hx - 3);
-                const double c0 = Cw[in], c1 = Cw[P.N + in], c2 = Cw[2 * P.N + in];
-                if (fmax(fmax(c0, c1), c2) < 1.0 - kMixEps) wall = 1;  // mixed_wall
-                wp |= (c0 != 0.0 ? 1 : 0) | (c1 != 0.0 ? 2 : 0) | (c2 != 0.0 ? 4 : 0);
-            }
-        }
-        if constexpr (INNER) {
-            const int w = __reduce_or_sync(0xffffffffu, wp);
-            if ((tid & 31) == 0) s_wp[tid >> 5] = w;
-        }
-    } else {
-        for (int j = tid; j < HX * HY; j += NT) {
-            const int hx = j % HX, hy = j / HX;
-            const int X = x0 + hx - 3, Y = y0 + hy - 3;
-            const Loc L = locate(P, X, Y);
-            uint8_t t = kSI;
-            if (L.kind != 1) {
-                t = __ldg(type + L.idx);
-                if (L.kind == 2) t |= 8;
-            }
-            s_t[hy][hx] = t;
-            s_idx[hy][hx] = L.idx;
-            if (hy == 0) s_par[hx] = parity_x(P, X);
-            if ((t & 3) == kSB && hx >= 1 && hx <= CX && hy >= 1 && hy <= CY && mixed_wall(Cw, P.N, L.idx))
-                wall = 1;
-        }
-    }
-    const bool df = PURE ? false : __syncthreads_or(wall);
-    // A wall tile whose 3 x 3 tiles stored one fluid, and whose C_SB nodes in the phase-field
-    // region have wall values of that fluid only, holds that fluid alone in the region after
-    // the pull: it is not mixed, and its halo's phase fields, which only the mixed path reads,
-    // are skipped (same results).  The plain float path only (no float-float words).
-    bool single = false;
-    if constexpr (INNER && !PURE) {
-        if (!df) {
-            uint64_t nb = 0;
-#pragma unroll
-            for (int t = 0; t < 9; t++) nb |= s_nb[t];
-            nb |= nb >> 32;
-            nb |= nb >> 16;
-            nb |= nb >> 8;
-            int bits = (int)(nb & 7u);
-#pragma unroll
-            for (int w = 0; w < TX * TY / 32; w++) bits |= s_wp[w];
-            single = __popc(bits) == 1;
-        }
-    }
-
-    // ---- phase 1: post-streaming populations, densities and phase fields ----
-    // pull of the fluid node at (hx, hy) of the geometry region into q[27]
-    auto pull = [&](int hx, int hy, float q[27]) {
-        const uint8_t t = PURE ? (uint8_t)kFI : s_t[hy][hx];
-        if (inner) {
-            const int i = (y0 + hy - 3) * nx + (x0 + hx - 3);
-            const bool fi = PURE || (t & 3) == kFI;
-            if constexpr (STORE == kStoreF32) {
-                const float* b = fin.f + i;
-                if (fi) {
-#pragma unroll
-                    for (int a = 0; a < kQ; a++)
-#pragma unroll
-                        for (int k = 0; k < kNF; k++) q[9 * k + a] = __ldg(b + P.off_pull[k * kQ + a]);
-                } else {
-#pragma unroll
-                    for (int a = 0; a < kQ; a++) {
-                        const bool bb = s_t[hy - ey(a)][hx - ex(a)] & 2;
-#pragma unroll
-                        for (int k = 0; k < kNF; k++)
-                            q[9 * k + a] = __ldg(b + (bb ? P.off_plane[k * kQ + opp(a)] : P.off_pull[k * kQ + a]));
-                    }
-                }
-            } else {
-                // own node: rho_k and the 8 offsets (the rest population and any bounce-back)
-                const float* rb = fin.rho + i;
-                const unsigned short* ob = fin.off + i;
-#pragma unroll
-                for (int k = 0; k < kNF; k++) {
-                    const float rk = __ldg(rb + k * N);
-                    float d[kQ];
-#pragma unroll
-                    for (int a = 1; a < kQ; a++) d[a] = dec16<STORE>(__ldg(ob + (8 * k + a - 1) * N));
-                    q[9 * k] = wq(0) * rk - sum_offsets(d);
-#pragma unroll
-                    for (int a = 1; a < kQ; a++) {
-                        const bool bb = !fi && (s_t[hy - ey(a)][hx - ex(a)] & 2);
-                        if (bb) {
-                            q[9 * k + a] = wq(opp(a)) * rk + d[opp(a)];
-                        } else {
-                            const int o = P.off_pull16[k * kQ + a];
-                            q[9 * k + a] = wq(a) * __ldg(fin.rho + i + o) +
-                                           dec16<STORE>(__ldg(ob + P.off_pull16o[k * kQ + a]));
-                        }
-                    }
-                }
-            }
-            return;
-        }
-        if (t & 8) {
-            // ghost beyond an open side: copy of the boundary-column node (zero gradient)
-            const Store<STORE> st(fin, P.N);
-            pull_global(P, st, type, x0 + hx - 3, y0 + hy - 3, q);
-            return;
-        }
-        const Store<STORE> st(fin, P.N);
-        const bool pn = s_par[hx];
-        const int in = s_idx[hy][hx];
-        bool inl = false, outl = false;
-#pragma unroll
-        for (int a = 0; a < kQ; a++) {
-            const int sx = hx - ex(a), sy = hy - ey(a);
-            const uint8_t ts = s_t[sy][sx];
-            if (ts & 8) {
-                if (x0 + hx - 3 == 0) inl = true; else outl = true;
-#pragma unroll
-                for (int k = 0; k < kNF; k++) q[9 * k + a] = 0.0f;
-            } else if (ts & 2) {
-#pragma unroll
-                for (int k = 0; k < kNF; k++) q[9 * k + a] = st.get(relabel(k, pn), opp(a), in);
-            } else {
-                const bool ps = s_par[sx];
-                const int is = s_idx[sy][sx];
-#pragma unroll
-                for (int k = 0; k < kNF; k++) q[9 * k + a] = st.get(relabel(k, ps), a, is);
-            }
-        }
-        if (inl) zou_he(P, q, true);
-        if (outl) zou_he(P, q, false);
-    };
-    // densities / phase fields of the position (cx, cy) of the phase-field region from q, and which
-    // fluids occur in the region (bit k: some rho_k != 0, or a wall value C_k != 0 at a C_SB node)
-    int present = 0;
-    auto store_phase = [&](int cx, int cy, const float q[27]) {
-        present |= phase_fields<CX, CY>(df, q, s_ch, s_cl, s_rho, cx, cy);
-    };
-    auto fill = [&](int cx, int cy, float q[27]) -> bool {
-        const int hx = cx + 1, hy = cy + 1;
-        const uint8_t t = PURE ? (uint8_t)kFI : s_t[hy][hx];
-        if (!(t & 2)) {
-            pull(hx, hy, q);
-            store_phase(cx, cy, q);
-            return true;
-        }
-        if ((t & 3) == kSB) {
-            // wall value from the wetting pass (FP64, split into hi + lo); rho := 1 at solid nodes
-            const int in = inner ? (y0 + hy - 3) * nx + (x0 + hx - 3) : s_idx[hy][hx];
-            const bool pr = inner ? false : s_par[hx];
-            present |= wall_fields<CX, CY>(Cw, P.N, in, pr, s_ch, s_cl, s_rho, cx, cy);
-        } else {
-#pragma unroll
-            for (int k = 0; k < kNF; k++) s_ch[k][cy][cx] = s_cl[k][cy][cx] = 0.0f;
-            s_rho[cy][cx] = 0.0f;
-        }
-        return false;
-    };
-
-    if (!single) {
-        // ring of the halo-2 region: rows 0, 1, CY-2, CY-1 and columns 0, 1, CX-2, CX-1
-        constexpr int NRING = CX * CY - TX * TY;
-        for (int j = tid; j < NRING; j += NT) {
-            int cx, cy;
-            if (j < 2 * CX) {
-                cx = j % CX;
-                cy = j / CX;
-            } else if (j < 4 * CX) {
-                cx = (j - 2 * CX) % CX;
-                cy = CY - 2 + (j - 2 * CX) / CX;
-            } else {
-                const int r = j - 4 * CX;  // 4 * TY side nodes
-                const int side = r / (2 * TY), rr = r % (2 * TY);
-                cy = 2 + rr / 2;
-                cx = side == 0 ? (rr & 1) : CX - 2 + (rr & 1);
-            }
-            float q[27];
-            fill(cx, cy, q);
-        }
-    }
-    const int lx = threadIdx.x, ly = threadIdx.y;
-    const int gx = x0 + lx, gy = y0 + ly;
-    // own node: keep the 9 post-streaming totals and the 3 densities
-    float f[kQ], r0, r1, r2;
-    bool own_fluid;
-    {
-        float q[27];
-        if (single) {
-            own_fluid = !(s_t[ly + 3][lx + 3] & 2);
-            if (own_fluid) pull(lx + 3, ly + 3, q);
-        } else {
-            own_fluid = fill(lx + 2, ly + 2, q);
-        }
-#pragma unroll
-        for (int a = 0; a < kQ; a++) f[a] = (q[a] + q[9 + a]) + q[18 + a];
-        r0 = ((q[0] + (q[1] + q[3])) + (q[2] + q[4])) + ((q[5] + q[7]) + (q[6] + q[8]));
-        r1 = ((q[9] + (q[10] + q[12])) + (q[11] + q[13])) + ((q[14] + q[16]) + (q[15] + q[17]));
-        r2 = ((q[18] + (q[19] + q[21])) + (q[20] + q[22])) + ((q[23] + q[25]) + (q[24] + q[26]));
-    }
-    if constexpr (INNER || PURE) {
-        // the fluids this warp's fluid nodes hold, for the tiles around this one in the next step
-        const int own = own_fluid ? (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0) : 0;
-        const int w = __reduce_or_sync(0xffffffffu, own);
-        if ((tid & 31) == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = (uint8_t)w;
-    }
-    // fluids present in the phase-field region: one barrier for tiles that had one already (the
-    // word was cleared before the phase-0 barrier), three for the pure tiles of the plain path
-    const bool mixed =
-        single ? false : (PURE ? single_fluid_or(present) : fluids_present(present, s_flags, 0, tid)) != 1;
-
-    // ---- phase 2: stress tensor of Eq.(10) on the halo-1 region ----
-    for (int j = mixed ? tid : RX * RY; j < RX * RY; j += NT) {
-        const int rx = j % RX, ry = j / RX;
-        float Txx = 0.f, Txy = 0.f, Tyy = 0.f;
-        float gxk[kNF], gyk[kNF];
-        if (PURE) {
-            const float rho = s_rho[ry + 1][rx + 1];
-            float c[kNF];
-#pragma unroll
-            for (int k = 0; k < kNF; k++) {
-                c[k] = s_ch[k][ry + 1][rx + 1];
-                grad9_f<CX>(s_ch[k], rx + 1, ry + 1, gxk[k], gyk[k]);
-            }
-            const float rho2 = rho * rho;
-            pair_stress(P.sig01, c[0], c[1], gxk[0], gyk[0], gxk[1], gyk[1], rho2, Txx, Txy, Tyy);
-            pair_stress(P.sig02, c[0], c[2], gxk[0], gyk[0], gxk[2], gyk[2], rho2, Txx, Txy, Tyy);
-            pair_stress(P.sig12, c[1], c[2], gxk[1], gyk[1], gxk[2], gyk[2], rho2, Txx, Txy, Tyy);
-        } else {
-            stress_at<HX, CX, CY>(P, s_t, s_ch, s_cl, s_rho, df, rx, ry, gxk, gyk, Txx, Txy, Tyy);
-        }
-        if (rx >= 1 && rx <= TX && ry >= 1 && ry <= TY) {
-#pragma unroll
-            for (int k = 0; k < kNF; k++) {
-                s_g[2 * k][ry - 1][rx - 1] = gxk[k];
-                s_g[2 * k + 1][ry - 1][rx - 1] = gyk[k];
-            }
-        }
-        s_txx[ry][rx] = Txx;
-        s_txy[ry][rx] = Txy;
-        s_tyy[ry][rx] = Tyy;
-    }
-    if (!single) __syncthreads();
-
-    if (!own_fluid || gx >= P.nx || gy >= P.ny) return;
-
-    // ---- interfacial force F_s = div T (Eq.10 with Eq.12) ----
-    float Fx = 0.0f, Fy = 0.0f, g[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    if (mixed) {
-        div_stress<RX>(s_txx, s_txy, s_tyy, lx + 1, ly + 1, Fx, Fy);
-        // own colour gradients from phase 2
-#pragma unroll
-        for (int k = 0; k < 6; k++) g[k] = s_g[k][ly][lx];
-    }
-    // ---- velocity, MRT collision with forcing, recolouring coefficients ----
-    float ux, uy;
-    const Recolour rc = collide_node(P, f, r0, r1, r2, Fx, Fy, g, ux, uy);
-    const int i = gy * nx + gx;
-    if (uout) {
-        uout[i] = ux;
-        uout[N + i] = uy;
-    }
-    const float* Cs = rc.C;
-    const float* Vx = rc.Vx;
-    const float* Vy = rc.Vy;
-    if constexpr (STORE == kStoreF32) {
-        float* o = fout.f + i;
-#pragma unroll
-        for (int k = 0; k < kNF; k++) {
-#pragma unroll
-            for (int a = 0; a < kQ; a++) {
-                const float v = Cs[k] * f[a] + wq(a) * (Vx[k] * (float)ex(a) + Vy[k] * (float)ey(a));
-                o[P.off_plane[k * kQ + a]] = v;
-            }
-        }
-    } else {
-        float v[27];
-#pragma unroll
-        for (int k = 0; k < kNF; k++)
-#pragma unroll
-            for (int a = 0; a < kQ; a++)
-                v[9 * k + a] = Cs[k] * f[a] + wq(a) * (Vx[k] * (float)ex(a) + Vy[k] * (float)ey(a));
-        store_node<STORE>(fout, P.N, i, v);
-    }
-}
-
-
 
 // Eq.(10) stress on the halo-1 region of a pure tile from the phase fields of its halo-2 region
 // (float path: no solid, no float-float words)
@@ -914,7 +463,7 @@ __device__ __forceinline__ void stress_halo1(const Params& P, const float (*s_ch
 // The 27 output planes are written directly (STAGE = false: 72 KB of shared memory per block)
 // or staged in shared memory and written by one bulk tensor store per tile (STAGE = true,
 // 100 KB).  kTmaBlocksPerSm = 2 blocks per SM: three (the most that fit) measured slower.
-// Same arithmetic as k_step<PURE>, so the two give identical results.
+// Same arithmetic as k_step_plain, so the two give identical results.
 template <int TX, int TY, bool STAGE>
 __global__ void __launch_bounds__(TX* TY, kTmaBlocksPerSm) k_step_tma(const Params P, const int* __restrict__ tiles,
                                                         const int ntiles, float* __restrict__ fout,
@@ -1241,6 +790,796 @@ __device__ __forceinline__ bool collide_single(const Params& P, int k, float f[k
     return c == 1.0f;
 }
 
+// write the 27 recoloured post-collision populations of node i
+template <int STORE>
+__device__ __forceinline__ void store_recoloured(const Params& P, const Pop& out, int i, const float f[kQ],
+                                                 const Recolour& rc)
+{
+    if constexpr (STORE == kStoreF32) {
+        float* o = out.f + i;
+#pragma unroll
+        for (int k = 0; k < kNF; k++)
+#pragma unroll
+            for (int a = 0; a < kQ; a++)
+                o[P.off_plane[k * kQ + a]] =
+                    rc.C[k] * f[a] + wq(a) * (rc.Vx[k] * (float)ex(a) + rc.Vy[k] * (float)ey(a));
+    } else {
+        float v[27];
+#pragma unroll
+        for (int k = 0; k < kNF; k++)
+#pragma unroll
+            for (int a = 0; a < kQ; a++)
+                v[9 * k + a] = rc.C[k] * f[a] + wq(a) * (rc.Vx[k] * (float)ex(a) + rc.Vy[k] * (float)ey(a));
+        store_node<STORE>(out, P.N, i, v);
+    }
+}
+
+// position j of the ring that the halo-2 region of a tile has around the tile's own nodes
+template <int TX, int TY>
+__device__ __forceinline__ void ring_position(int j, int& cx, int& cy)
+{
+    constexpr int CX = TX + 4, CY = TY + 4;
+    if (j < 2 * CX) {
+        cx = j % CX;
+        cy = j / CX;
+    } else if (j < 4 * CX) {
+        cx = (j - 2 * CX) % CX;
+        cy = CY - 2 + (j - 2 * CX) / CX;
+    } else {
+        const int r = j - 4 * CX;  // 4 * TY side nodes
+        const int side = r / (2 * TY), rr = r % (2 * TY);
+        cy = 2 + rr / 2;
+        cx = side == 0 ? (rr & 1) : CX - 2 + (rr & 1);
+    }
+}
+
+// Pure tiles by plain loads (nx not a multiple of what the bulk copies need): one CTA per TX x TY
+// tile.  Pull-streaming of every node of the halo-2 region (densities and phase fields C_k; the
+// tile's own nodes keep their 9 post-streaming totals and 3 densities in registers), the Eq.(10)
+// stress on the halo-1 region, then force, velocity, MRT collision with forcing, recolouring and 27
+// stores per node.  all: take the tiles with one fluid around too, which are k_step_one's otherwise.
+template <int TX, int TY, int STORE>
+__global__ void __launch_bounds__(TX* TY, 4) k_step_plain(const Params P, const int* __restrict__ tiles, const Pop fin,
+                                                        const Pop fout, float* __restrict__ uout,
+                                                        const uint64_t* __restrict__ pres_in,
+                                                        uint64_t* __restrict__ pres_out, const int all)
+{
+    constexpr int NT = TX * TY;
+    constexpr int CX = TX + 4, CY = TY + 4;  // phase-field region (halo 2)
+    constexpr int RX = TX + 2, RY = TY + 2;  // stress region (halo 1)
+    __shared__ float s_ch[kNF][CY][CX];
+    __shared__ float s_rho[CY][CX];
+    __shared__ float s_txx[RY][RX], s_txy[RY][RX], s_tyy[RY][RX];
+
+    const int lx = threadIdx.x, ly = threadIdx.y, tid = lx + TX * ly;
+    const int ntx = (P.nx + TX - 1) / TX;
+    const int tile = tiles[blockIdx.x];
+    if (!all && __popc((unsigned)fluids_around(pres_in, tile, ntx)) == 1) return;
+    const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
+    const int nx = P.nx;
+    const int N = (int)P.N;
+    // pull of the node at (cx, cy) of the phase-field region
+    auto pull = [&](int cx, int cy, float q[27]) {
+        const int i = (y0 + cy - 2) * nx + (x0 + cx - 2);
+        if constexpr (STORE == kStoreF32) {
+            const float* b = fin.f + i;
+#pragma unroll
+            for (int a = 0; a < kQ; a++)
+#pragma unroll
+                for (int k = 0; k < kNF; k++) q[9 * k + a] = __ldg(b + P.off_pull[k * kQ + a]);
+        } else {
+            const unsigned short* ob = fin.off + i;
+#pragma unroll
+            for (int k = 0; k < kNF; k++) {
+                float d[kQ];
+#pragma unroll
+                for (int a = 1; a < kQ; a++) d[a] = dec16<STORE>(__ldg(ob + (8 * k + a - 1) * N));
+                q[9 * k] = wq(0) * __ldg(fin.rho + i + k * N) - sum_offsets(d);
+#pragma unroll
+                for (int a = 1; a < kQ; a++)
+                    q[9 * k + a] = wq(a) * __ldg(fin.rho + i + P.off_pull16[k * kQ + a]) +
+                                   dec16<STORE>(__ldg(ob + P.off_pull16o[k * kQ + a]));
+            }
+        }
+    };
+    // the lo words of float-float fields do not exist here
+    float(*none)[CY][CX] = nullptr;
+    int present = 0;
+    constexpr int NRING = CX * CY - TX * TY;
+    static_assert(NRING <= NT, "the ring of the halo-2 region must not exceed one node per thread");
+    if (tid < NRING) {
+        int cx, cy;
+        ring_position<TX, TY>(tid, cx, cy);
+        float q[27];
+        pull(cx, cy, q);
+        present |= phase_fields<CX, CY>(false, q, s_ch, none, s_rho, cx, cy);
+    }
+    float f[kQ], r0, r1, r2;
+    {
+        float q[27];
+        pull(lx + 2, ly + 2, q);
+        present |= phase_fields<CX, CY>(false, q, s_ch, none, s_rho, lx + 2, ly + 2);
+#pragma unroll
+        for (int a = 0; a < kQ; a++) f[a] = (q[a] + q[9 + a]) + q[18 + a];
+        r0 = sum9(q);
+        r1 = sum9(q + 9);
+        r2 = sum9(q + 18);
+    }
+    // the fluids this warp's nodes hold, for the tiles around this one in the next step
+    {
+        const int own = (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0);
+        const int w = __reduce_or_sync(0xffffffffu, own);
+        if (lx == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[ly] = (uint8_t)w;
+    }
+    const bool mixed = single_fluid_or(present) != 1;
+
+    if (mixed) stress_halo1<TX, TY>(P, s_ch, s_rho, s_txx, s_txy, s_tyy, tid);
+    __syncthreads();
+
+    float Fx = 0.0f, Fy = 0.0f, g[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    if (mixed) {
+        div_stress<RX>(s_txx, s_txy, s_tyy, lx + 1, ly + 1, Fx, Fy);
+#pragma unroll
+        for (int k = 0; k < kNF; k++) grad9_f<CX>(s_ch[k], lx + 2, ly + 2, g[2 * k], g[2 * k + 1]);
+    }
+    float ux, uy;
+    const Recolour rc = collide_node(P, f, r0, r1, r2, Fx, Fy, g, ux, uy);
+    const int i = (y0 + ly) * nx + x0 + lx;
+    if (uout) {
+        uout[i] = ux;
+        uout[N + i] = uy;
+    }
+    store_recoloured<STORE>(P, fout, i, f, rc);
+}
+
+// ------------------------------------------------------------------------------------------
+// tiles of any kind: solids, domain edges, the seam, open sides
+// ------------------------------------------------------------------------------------------
+// population dir of fluid k stored at node src
+template <int STORE>
+__device__ __forceinline__ void load_fluid(const Params& P, const Pop& fin, int src, int dir, int k, float& q)
+{
+    const int N = (int)P.N;
+    if constexpr (STORE == kStoreF32) {
+        q = fin.f[src + (k * kQ + dir) * N];
+    } else {
+        const float rk = fin.rho[src + k * N];
+        const unsigned short* ob = fin.off + src + (8 * k - 1) * N;
+        if (dir > 0) {
+            q = (dir < 5 ? wq(1) : wq(5)) * rk + dec16<STORE>(ob[dir * N]);
+        } else {
+            float d[kQ];
+#pragma unroll
+            for (int a = 1; a < kQ; a++) d[a] = dec16<STORE>(ob[a * N]);
+            q = wq(0) * rk - sum_offsets(d);
+        }
+    }
+}
+
+// population dir of the three fluids stored at node src: q[0], q[9], q[18] (rest: dir is 0)
+template <int STORE>
+__device__ __forceinline__ void load_direction(const Params& P, const Pop& fin, int src, int dir, float* q)
+{
+    const int N = (int)P.N;
+    if constexpr (STORE == kStoreF32) {
+        const float* f = fin.f + src + dir * N;
+#pragma unroll
+        for (int k = 0; k < kNF; k++) q[9 * k] = f[k * kQ * N];
+    } else {
+#pragma unroll
+        for (int k = 0; k < kNF; k++) load_fluid<STORE>(P, fin, src, dir, k, q[9 * k]);
+    }
+}
+
+// storage index and flags of the fluid node at unwrapped (X, Y)
+__device__ __forceinline__ void wet_node(const Params& P, const uint16_t* __restrict__ nflag, int X, int Y, int& idx, int& fl)
+{
+    const Loc L = locate(P, X, Y);
+    idx = L.idx;
+    fl = (int)__ldg(nflag + L.idx) | (L.par ? kNodePar : 0);
+}
+
+// C_k at such a node, in the frame of the C_SB node: node_C without a search for the sources, all
+// of whose loads are issued at once (one dependent load of a class byte per direction made the
+// separate wetting pass take 20 us on the smallest grids)
+template <int STORE>
+__device__ __forceinline__ double wet_fraction(const Params& P, const Pop& fin, int idx, int fl, int k)
+{
+    const int nx = P.nx;
+    const int xm = fl & kNodeX0 ? nx - 1 : -1, xp = fl & kNodeXN ? 1 - nx : 1;
+    const int ym = fl & kNodeY0 ? (P.ny - 1) * nx : -nx, yp = fl & kNodeYN ? (1 - P.ny) * nx : nx;
+    const bool seam = P.bc_x == kModPer, open = P.bc_x == kZouHe;
+    float q[27];
+#pragma unroll
+    for (int a = 0; a < kQ; a++) {
+        const bool bb = a > 0 && (fl >> a & 1);
+        const bool over = (ex(a) == 1 && (fl & kNodeX0)) || (ex(a) == -1 && (fl & kNodeXN));
+        const int d = (ex(a) == 1 ? xm : (ex(a) == -1 ? xp : 0)) + (ey(a) == 1 ? ym : (ey(a) == -1 ? yp : 0));
+        // beyond an open side nothing is stored: the node itself is read and its value dropped
+        const int src = bb || (open && over) ? idx : idx + d;
+        load_direction<STORE>(P, fin, src, bb ? opp(a) : a, q + a);
+        if (seam && (((fl & kNodePar) != 0) != (over && !bb))) {
+            const float t = q[a];
+            q[a] = q[18 + a];
+            q[18 + a] = t;
+        }
+        if (open && over) q[a] = q[9 + a] = q[18 + a] = 0.0f;
+    }
+    if (open && (fl & (kNodeX0 | kNodeXN))) zou_he(P, q, (fl & kNodeX0) != 0);
+    float rh[kNF], rl[kNF];
+#pragma unroll
+    for (int j = 0; j < kNF; j++) sum9_df(q + 9 * j, rh[j], rl[j]);
+    float th, tl, sh, sl, dh;
+    two_sum(rh[0], rh[1], th, tl);
+    two_sum(th, rh[2], sh, sl);
+    const float dl = (tl + sl) + ((rl[0] + rl[1]) + rl[2]);
+    two_sum(sh, dl, dh, sl);
+    const float nh = k == 0 ? rh[0] : rh[1];
+    const float nl = k == 0 ? rl[0] : rl[1];
+    float qh, ql;
+    div_df(nh, nl, dh, sl, qh, ql);
+    return (double)qh + (double)ql;
+}
+
+// the w-weighted neighbour mean, where a line meets no fluid (out of line: rarely called)
+template <int STORE>
+__device__ __noinline__ double wet_mean(const Params& P, const Pop& fin, const uint8_t* __restrict__ type, int px, int py,
+                                        int k)
+{
+    const Store<STORE> st(fin, P.N);
+    return neighbour_mean(P, st, type, px, py, k);
+}
+
+// whether the node at unwrapped (X, Y) is fluid, from the geometry words of a tile where they reach:
+// it is at (hx, hy) there
+template <int HX, int HY>
+__device__ __forceinline__ bool fluid_near(const Params& P, const uint8_t* __restrict__ type, const int (*geo)[HX], int hx,
+                                           int hy, int X, int Y)
+{
+    if ((unsigned)hx < (unsigned)HX && (unsigned)hy < (unsigned)HY) return !(geo[hy][hx] & (kGeoSolid | kGeoGhost));
+    return node_is_fluid<Store<kStoreF32>>(P, type, X, Y);
+}
+
+// Where the line from (px, py) along (dx, dy) first crosses a grid line between two fluid nodes,
+// found in single precision: true with the crossed line (vertical x = X or horizontal y = Y) and the
+// node below or left of the crossing (ax, ay).  Every decision up to there -- which line comes
+// first, between which nodes -- has to be clear by a margin of kRayMargin, some twenty times the
+// rounding of the positions (up to 16 long, directions rounded to 6e-8) and a hundred times
+// kRayEps; otherwise false, and the double-precision march decides.  (hx, hy): the place of (px, py)
+// in the tile's geometry words.
+constexpr float kRayMargin = 1e-4f;
+template <int HX, int HY>
+__device__ __forceinline__ bool float_crossing(const Params& P, const uint8_t* __restrict__ type, const int (*geo)[HX], int hx,
+                                               int hy, int px, int py, float dx, float dy, bool& vertical, int& ax,
+                                               int& ay)
+{
+    const float adx = fabsf(dx), ady = fabsf(dy);
+    if (!(fminf(adx, ady) >= kRayMargin)) return false;
+    const int sx = dx > 0.0f ? 1 : -1, sy = dy > 0.0f ? 1 : -1;
+    const float ix = __fdividef(1.0f, adx), iy = __fdividef(1.0f, ady);
+    int m = 1, n = 1;  // the next vertical and horizontal grid line, counted from the node
+#pragma unroll 1
+    for (int it = 0; it < 64; it++) {
+        const float tX = m * ix, tY = n * iy;
+        const float t = fminf(tX, tY);
+        if (t > (float)kRayTmax - 0.01f || fabsf(tX - tY) < kRayMargin) return false;
+        vertical = tX < tY;
+        // position along the crossed line, relative to the node
+        const float r = vertical ? t * dy : t * dx;
+        const float rf = floorf(r), fr = r - rf;
+        if (fr < kRayMargin || fr > 1.0f - kRayMargin) return false;
+        const int fl = (int)rf, rx = vertical ? m * sx : fl, ry = vertical ? fl : n * sy;
+        if (fluid_near<HX, HY>(P, type, geo, hx + rx, hy + ry, px + rx, py + ry) &&
+            fluid_near<HX, HY>(P, type, geo, hx + rx + !vertical, hy + ry + vertical, px + rx + !vertical,
+                               py + ry + vertical)) {
+            ax = px + rx;
+            ay = py + ry;
+            return true;
+        }
+        if (vertical) m++; else n++;
+    }
+    return false;
+}
+
+// The line of one side of the C_SB node of entry en (normal n) for the local angle th, into its lane.
+// The search is done in single precision where that is safe, the crossing itself with the
+// expressions of characteristic_line.  geo: the tile's geometry words (or null).
+template <int TX, int TY>
+__device__ __forceinline__ void wet_line(const Params& P, const TileSet& T, const int (*geo)[TX + 6], const int4 en,
+                                         const double2 n, double th, int side, WetLane& c)
+{
+    constexpr int HX = TX + 6, HY = TY + 6;
+    const int node = en.x, px = node % P.nx, py = node / P.nx;
+    const int hx = (en.z & 255) + 1, hy = (en.z >> 8 & 255) + 1;  // where the geometry words have the node
+    const double dev = fabs(90.0 - th);
+    const double phi = dev < kPhiSnap ? 0.0 : dev * (M_PI / 180.0);
+    double sn, cs;
+    sincos(phi, &sn, &cs);
+    if (side) sn = -sn;
+    // the line makes the angle phi with n_s (tangent (-n_y, n_x))
+    const double dx = fma(cs, n.x, -__dmul_rn(sn, n.y)), dy = fma(cs, n.y, __dmul_rn(sn, n.x));
+    Crossing cr{0, 0, 0, 0, 0, 0.0};
+    bool vertical;
+    if (float_crossing<HX, HY>(P, T.type, geo, geo ? hx : 1 << 30, hy, px, py, (float)dx, (float)dy, vertical, cr.ax,
+                               cr.ay)) {
+        cr.kind = 2;
+        cr.bx = cr.ax + !vertical;
+        cr.by = cr.ay + vertical;
+        // without fused multiply-add, as characteristic_line
+        const double t = (double)(vertical ? cr.ax - px : cr.ay - py) / (vertical ? dx : dy);
+        const double s = __dadd_rn((double)(vertical ? py : px), __dmul_rn(t, vertical ? dy : dx));
+        cr.fr = s - (double)(vertical ? cr.ay : cr.ax);
+    } else {
+        cr = characteristic_line<Store<kStoreF32>>(P, T.type, px, py, dx, dy);
+    }
+    c.fr = cr.fr;
+    c.ia = c.ib = -1;
+    c.fa = c.fb = 0;
+    auto bracket = [&](int X, int Y, int& idx, int& fl) {
+        wet_node(P, T.nflag, X, Y, idx, fl);
+        const int gx = hx + X - px, gy = hy + Y - py;
+        if (gx >= 1 && gx <= HX - 2 && gy >= 1 && gy <= HY - 2) fl |= kNodeNear;
+    };
+    if (cr.kind >= 1) bracket(cr.ax, cr.ay, c.ia, c.fa);
+    if (cr.kind == 2) bracket(cr.bx, cr.by, c.ib, c.fb);
+}
+
+// Threads of a block: one for every node of a tile's halo-2 region (432 of 512), so that each phase
+// of a tile is one pass: with 256, which pulled the tile's nodes and the ring around it in turn, a
+// tile took 13000 cycles instead of the sum of its memory latencies.
+constexpr int kTileThreads = 512;
+constexpr int kNoTile = -2;
+constexpr int kWetNodes = kTileThreads / 8;  // C_SB nodes wetted at a time
+
+template <int TX, int TY>
+struct TileShared {
+    static constexpr int HX = TX + 6, HY = TY + 6;  // geometry region (halo 3)
+    static constexpr int CX = TX + 4, CY = TY + 4;  // phase-field region (halo 2)
+    static constexpr int RX = TX + 2, RY = TY + 2;  // stress region (halo 1)
+    int geo[HY][HX];
+    float ch[kNF][CY][CX], cl[kNF][CY][CX];  // C_k = hi + lo
+    float rho[CY][CX];
+    float txx[RY][RX], txy[RY][RX], tyy[RY][RX];
+    int4 went[kWetNodes];         // the C_SB nodes of a pass,
+    double2 nrm[kWetNodes];       // their normals,
+    double raw[kWetNodes][2];     // Eq.(22)'s values of the wetted fluids there, before the limits,
+    double wv[kNF][kWetNodes];    // and the three wall values
+    double th[2 * kWetNodes];     // angles whose lines have to be looked for,
+    short list[2 * kWetNodes];    // and of which node x 2 + fluid
+    int wall, flags, todo;        // what the C_SB nodes hold, the fluids present, the list's length
+};
+
+// the same finite number, compared as words (a comparison of doubles is one of their slow instructions)
+__device__ __forceinline__ bool same_number(double a, double b)
+{
+    const long long x = __double_as_longlong(a);
+    return x == __double_as_longlong(b) && (x & 0x7ff0000000000000LL) != 0x7ff0000000000000LL;
+}
+
+// The lines of the next step for the m C_SB nodes of a pass (entries e0 ..), whose wall values of
+// this step are in S.wv: Eq.(21), and where its angle changed, the march.  By nt threads (t: this
+// one's number), whole warps; nothing of this step waits for it, so two warps that have no node of
+// the region do it while the others go on.  The nodes whose angle changed are packed first: an SM
+// issues a double-precision warp instruction in some twenty to thirty cycles, and with all lanes
+// marching before the wetting, a wall tile took 14 us for it.
+template <int TX, int TY>
+__device__ __forceinline__ void wet_look(const Params& P, const TileSet& T, int e0, int m, int t, int nt, int bar,
+                                         TileShared<TX, TY>& S, int* count)
+{
+    if (t == 0) *count = 0;
+    group_sync(bar, nt);
+#pragma unroll 1
+    for (int j0 = 0; j0 < 2 * m; j0 += nt) {
+        const int j = j0 + t, n = j >> 1, k = j & 1;
+        bool turned = false;
+        double th = 0.0;
+        if (j < 2 * m) {
+            const int w = S.went[n].y;
+            WetLane* const c = T.cache + (4 * (long long)(e0 + n) + 2 * k);
+            const double wm = S.wv[2][n], wl = S.wv[1 - k][n];  // the weights of Eq.(21) for fluid k
+            const double om = c[0].wm, ol = c[0].wl, oth = c[0].th;
+            const float t_rg = T.wang[3 * w], t_x = T.wang[3 * w + (k == 0 ? 1 : 2)];
+            if (!(same_number(om, wm) && same_number(ol, wl))) {
+                th = k == 0 ? local_angle(wm, 180.0 - t_x, wl, t_rg) : local_angle(wm, t_x, wl, 180.0 - t_rg);
+                c[0].wm = wm;
+                c[0].wl = wl;
+                // the same angle as when these lanes last marched: the same lines, the same crossings
+                turned = !same_number(oth, th);
+            }
+        }
+        const unsigned votes = __ballot_sync(0xffffffffu, turned);
+        int at = 0;
+        if ((t & 31) == 0 && votes) at = atomicAdd(count, __popc(votes));
+        at = __shfl_sync(0xffffffffu, at, 0) + __popc(votes & ((1u << (t & 31)) - 1));
+        if (turned) {
+            S.list[at] = (short)j;
+            S.th[at] = th;
+        }
+    }
+    group_sync(bar, nt);
+#pragma unroll 1
+    for (int i = t; i < 2 * *count; i += nt) {
+        const int j = S.list[i >> 1], n = j >> 1, k = j & 1, side = i & 1;
+        WetLane* const c = T.cache + (4 * (long long)(e0 + n) + 2 * k + side);
+        WetLane d;
+        d.th = S.th[i >> 1];
+        wet_line<TX, TY>(P, T, S.geo, S.went[n], S.nrm[n], d.th, side, d);
+        c->th = d.th;
+        c->fr = d.fr;
+        *reinterpret_cast<int4*>(&c->ia) = make_int4(d.ia, d.fa, d.ib, d.fb);
+    }
+}
+
+// Wetting of the C_SB nodes of a tile's phase-field region (entries e0 .. e0 + cnt of the set's
+// list): C at the nodes that bracket the crossings of the two characteristic lines of the two wetted
+// fluids, which the last step looked for (wet_look), and Eq.(22).  Eight lanes per node -- lane =
+// 4 k + 2 side + end -- pull one of the up to two nodes of a line each.  The values go to the region's
+// phase fields (rho := 1 there), to S.wv and, for the nodes that the tile owns, to cw_out.  A node
+// near several tiles is wetted by each of them, with the same result: 1.6 times the work of a pass
+// over the nodes, but no launch that the tiles have to wait for.  one: the fluids around; where that
+// is one, the nodes of the region hold it alone (C_k exactly 1 or 0) and need no pull.  Returns the
+// fluids with a nonzero wall value (bit k), and in bit 3 whether some node's values are mixed.
+template <int TX, int TY, int STORE>
+__device__ __forceinline__ int wet_entries(const Params& P, const TileSet& T, int e0, int cnt, int one,
+                                           const Pop& fin, double* cw_out, TileShared<TX, TY>& S)
+{
+    const long long N = P.N;
+    const int tid = threadIdx.x;
+    int bits = 0;
+#pragma unroll 1
+    for (int b0 = 0; b0 < cnt; b0 += kWetNodes) {
+        const int m = min(cnt - b0, kWetNodes);  // nodes of this pass
+        if (b0 > 0) {
+            // the pass before: its lines of the next step, then this one's nodes in its place
+            __syncthreads();
+            wet_look<TX, TY>(P, T, e0 + b0 - kWetNodes, kWetNodes, tid, kTileThreads, 0, S, &S.flags);
+            __syncthreads();
+            if (tid < m) {
+                S.went[tid] = T.went[e0 + b0 + tid];
+                S.nrm[tid] = T.wnrm[e0 + b0 + tid];
+            }
+            if (tid == 0) S.flags = 0;
+            __syncthreads();
+        }
+        if ((tid & ~31) < 8 * m) {
+            const bool valid = tid < 8 * m;
+            const int end = tid & 1, side = tid >> 1 & 1, k = tid >> 2 & 1;
+            const int e = valid ? tid >> 3 : 0;
+            const WetLane c = T.cache[4 * (long long)(e0 + b0 + e) + 2 * k + side];
+            double v = 0.0;
+            if (valid) {
+                const int4 en = S.went[e];
+                const int idx = end ? c.ib : c.ia, fl = end ? c.fb : c.fa, node = en.x;
+                if (idx >= 0 && (fl & kNodeNear) && __popc((unsigned)one) == 1)
+                    v = one >> relabel(k, en.z & kWetPar) & 1 ? 1.0 : 0.0;  // in the tile's frame
+                else if (idx >= 0)
+                    v = wet_fraction<STORE>(P, fin, idx, fl, k);
+                else if (end == 0)
+                    v = wet_mean<STORE>(P, fin, T.type, node % P.nx, node / P.nx, k);
+            }
+            const double o = __shfl_xor_sync(0xffffffffu, v, 1);
+            const double ca = end ? o : v, cb = end ? v : o;
+            double cd = ca;
+            if (c.ib >= 0 && !same_number(ca, cb)) cd = ca + c.fr * (cb - ca);
+            // Eq.(22): max of the two lines for theta_k <= 90 deg, min otherwise
+            const double other = __shfl_xor_sync(0xffffffffu, cd, 2);
+            double cp = cd;
+            if (!same_number(cd, other))
+                cp = c.th <= 90.0 ? fmax(cd, other) : fmin(cd, other);
+            if (valid && (tid & 3) == 0) S.raw[e][k] = cp;
+        }
+        __syncthreads();
+        if (tid < m) {
+            double c0 = S.raw[tid][0], c1 = S.raw[tid][1], c2;
+            const bool z0 = same_number(c0, 0.0), z1 = same_number(c1, 0.0);
+            // one fluid at the node: no double-precision instructions
+            const bool pure = (z0 && z1) || (z0 && same_number(c1, 1.0)) || (z1 && same_number(c0, 1.0));
+            if (pure) {
+                c2 = z0 && z1 ? 1.0 : 0.0;
+            } else {
+                // fractions stay in [0, 1] (a no-op unless 16-bit storage rounded a density below 0)
+                c0 = fmin(fmax(c0, 0.0), 1.0);
+                c1 = fmin(fmax(c1, 0.0), 1.0);
+                const double s = c0 + c1;
+                if (s > 1.0) {
+                    c0 /= s;
+                    c1 /= s;
+                }
+                c2 = fmax(0.0, 1.0 - c0 - c1);
+            }
+            S.wv[0][tid] = c0;
+            S.wv[1][tid] = c1;
+            S.wv[2][tid] = c2;
+            const int4 en = S.went[tid];
+            if (en.z & kWetOwner) {
+                cw_out[en.x] = c0;
+                cw_out[N + en.x] = c1;
+                cw_out[2 * N + en.x] = c2;
+            }
+            // FP64 split into hi + lo, relabelled across a modified periodic seam
+            const int cx = en.z & 255, cy = en.z >> 8 & 255;
+            const bool par = en.z & kWetPar;
+            const double cc[kNF] = {par ? c2 : c0, c1, par ? c0 : c2};
+#pragma unroll
+            for (int j = 0; j < kNF; j++) {
+                float h, l = 0.0f;
+                if (pure) {
+                    h = same_number(cc[j], 0.0) ? 0.0f : 1.0f;
+                } else {
+                    h = (float)cc[j];
+                    l = (float)(cc[j] - (double)h);
+                }
+                S.ch[j][cy][cx] = h;
+                S.cl[j][cy][cx] = l;
+                if (!same_number(cc[j], 0.0)) bits |= 1 << j;
+            }
+            S.rho[cy][cx] = 1.0f;
+            if (!pure && fmax(fmax(c0, c1), c2) < 1.0 - kMixEps) bits |= 8;
+        }
+    }
+    return bits;
+}
+
+// the lines of the current wall values Cw, for every entry of the set (after the state or the wall
+// angles were replaced): what wet_look does at the end of a step
+__global__ void k_wet_look(const Params P, const TileSet T, const int n, const double* __restrict__ Cw)
+{
+    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= 4 * n) return;
+    const int4 en = T.went[j >> 2];
+    const int side = j & 1, k = j >> 1 & 1;
+    const double wm = Cw[2 * P.N + en.x], wl = Cw[(1 - k) * P.N + en.x];
+    const float t_rg = T.wang[3 * en.y], t_x = T.wang[3 * en.y + (k == 0 ? 1 : 2)];
+    WetLane d;
+    d.wm = wm;
+    d.wl = wl;
+    d.th = k == 0 ? local_angle(wm, 180.0 - t_x, wl, t_rg) : local_angle(wm, t_x, wl, 180.0 - t_rg);
+    wet_line<kTX, kTY>(P, T, nullptr, en, T.wnrm[j >> 2], d.th, side, d);
+    T.cache[j] = d;
+}
+
+// initial wall values: w-weighted mean of the fluid neighbours, for each fluid
+template <class S>
+__global__ void k_wet_init(const Params P, const int nw, const int* __restrict__ widx, const S st,
+                           const uint8_t* __restrict__ type, double* __restrict__ Cw)
+{
+    const int w = blockIdx.x * blockDim.x + threadIdx.x;
+    if (w >= nw) return;
+    const int i = widx[w];
+    const int px = i % P.nx, py = i / P.nx;
+    for (int k = 0; k < kNF; k++) {
+        Cw[k * P.N + i] = neighbour_mean(P, st, type, px, py, k);
+    }
+}
+
+// One step of tile T.rec[blockIdx.x] (any kind): thread t < TX TY has the tile's node t, the next ones a
+// node of the ring that the halo-2 region has around it.
+//   geometry words of the halo-3 region into shared memory
+//   wetting of the C_SB nodes of the phase-field region
+//   one fluid around (the words of the tiles that the halo-3 region touches, and the wall values):
+//     9 populations per own node as in k_step_one
+//   else the pulls, phase fields, stress, force, collision and recolouring of all three fluids;
+//     where a C_SB node of the region has mixed wall values (a contact line at or near it) the
+//     phase fields are float-float, decided anew every step
+// What bounds it: on small grids the chain of memory latencies (about 700 cycles each) and instruction
+// cache misses (6 of its stalls per issued instruction on 128 x 64) in a wall tile, 18000 cycles of
+// which the wetting is 8500; so what is known early is loaded early: the tile's record in one load,
+// all that hangs on it in the next.  It takes the place of a wetting pass and two launches behind it:
+// a step of 128 x 64 takes 17.5 us instead of 27.6, of 320 x 180 17.2 instead of 27.9, of the 800 x 375
+// pillars 28.6 instead of 35.5, and of the 4096 x 2048 ones 223 instead of 240.
+// (Measured and left out: many steps in one cooperative launch whose blocks wait for one another, 14 to
+// 80 us where this took 12 to 44; the region's populations copied to shared memory during the wetting,
+// no gain; 256 threads a tile, each with two nodes of the region in turn, 1.5 times slower.)
+template <int TX, int TY, int STORE>
+__global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const TileSet T, const Pop fin, const Pop fout,
+                                                          double* cw_out, float* uout, const uint64_t* pres_in,
+                                                          uint64_t* pres_out, const int full_write)
+{
+    using TS = TileShared<TX, TY>;
+    constexpr int NT = kTileThreads, CX = TS::CX, CY = TS::CY, RX = TS::RX, RY = TS::RY, HX = TS::HX, HY = TS::HY;
+    constexpr int NOWN = TX * TY, NC = CX * CY, NR = RX * RY;
+    static_assert(TX == 32 && TY == 8 && NC <= NT, "one warp per row, one node of the region per thread");
+    // the warps that have a node of the region; the others look for the lines of the next step
+    constexpr int NB = (NC + 31) / 32 * 32;
+    static_assert(NT - NB >= 32, "a warp for the lines");
+    __shared__ TS S;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int N = (int)P.N;
+    const int word32 = T.rec[blockIdx.x * kTileRecInts + lane];  // one word of the record per lane
+    const int tile = __shfl_sync(0xffffffffu, word32, 0), e0 = __shfl_sync(0xffffffffu, word32, 1),
+              cnt = __shfl_sync(0xffffffffu, word32, 2);
+    const int nbr = lane >= kTileRecHead ? word32 : kNoTile;
+    const int ntx = (P.nx + TX - 1) / TX;
+    const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
+    for (int j = tid; j < HX * HY; j += NT) {
+        const int hx = j % HX, hy = j / HX;
+        S.geo[hy][hx] = geo_word(P, T.type, x0 + hx - 3, y0 + hy - 3);
+    }
+    if (tid < min(cnt, kWetNodes)) {
+        S.went[tid] = T.went[e0 + tid];
+        S.nrm[tid] = T.wnrm[e0 + tid];
+    }
+    if (tid == 0) S.wall = S.flags = 0;
+    // fluids stored in the tiles that the halo-3 region touches (every warp for itself)
+    int around = nbr == -1 ? 7 : 0;  // an open column: any fluid
+    if (nbr >= 0) {
+        uint64_t b = pres_in[nbr >> 1];
+        b |= b >> 32;
+        b |= b >> 16;
+        b |= b >> 8;
+        const int v = (int)(b & 7u);
+        around = nbr & 1 ? (v & 2) | (v & 1) << 2 | v >> 2 : v;  // across the seam
+    }
+    const bool inside = tid < NOWN;  // a node of the tile itself, row tid / 32 (one warp)
+    uint8_t* const word = reinterpret_cast<uint8_t*>(pres_out + tile) + (tid >> 5);
+    const int old = !inside || full_write ? 7 : *word;  // what this row of the output buffer still holds
+    around = __reduce_or_sync(0xffffffffu, around);
+    __syncthreads();
+
+    // this thread's position in the phase-field region
+    int cx = 0, cy = 0;
+    if (inside) {
+        cx = lane + 2;
+        cy = (tid >> 5) + 2;
+    } else if (tid < NC) {
+        ring_position<TX, TY>(tid - NOWN, cx, cy);
+    }
+    int hx = cx + 1, hy = cy + 1;
+    int own = tid < NC ? S.geo[hy][hx] : kGeoSolid;
+    const bool own_fluid = inside && !(own & kGeoSolid) && x0 + cx - 2 < P.nx && y0 + cy - 2 < P.ny;
+    int px = hx;
+    if (own & kGeoGhost) {
+        // beyond an open side: the boundary-column node (zero gradient)
+        const int X = x0 + hx - 3;
+        px += X < 0 ? -X : P.nx - 1 - X;
+    }
+    bool df = false;
+    int wp = 0;
+    if (cnt > 0) {
+        const int b = __reduce_or_sync(
+            0xffffffffu, wet_entries<TX, TY, STORE>(P, T, e0, cnt, around, fin, cw_out, S));
+        if (lane == 0 && b) atomicOr(&S.wall, b);
+        __syncthreads();
+        df = S.wall & 8;
+        wp = S.wall & 7;
+    }
+    if (tid >= NB) {
+        if (cnt > 0) {
+            const int last = (cnt - 1) / kWetNodes * kWetNodes;
+            wet_look<TX, TY>(P, T, e0 + last, cnt - last, tid - NB, NT - NB, 2, S, &S.todo);
+        }
+        return;
+    }
+    if (!df && __popc((unsigned)(around | wp)) == 1) {
+        // ---- one fluid: as in k_step_one ----
+        if (!inside) return;
+        const int k = __ffs(around | wp) - 1, i = own & kGeoIdx;
+        bool plain = true;
+        float f[kQ], r = 1.0f, ux = 0.0f, uy = 0.0f;
+        if (own_fluid) {
+#pragma unroll
+            for (int a = 0; a < kQ; a++) {
+                const int g = S.geo[hy - ey(a)][hx - ex(a)];
+                const bool bb = g & kGeoSolid;
+                const int s = bb ? own : g;
+                load_fluid<STORE>(P, fin, s & kGeoIdx, bb ? opp(a) : a, (s & kGeoPar) && k != 1 ? 2 - k : k, f[a]);
+            }
+            r = sum9(f);
+            plain = collide_single(P, k, f, r, ux, uy);
+        }
+        const bool all = __all_sync(0xffffffffu, plain);
+        if (own_fluid) {
+            if (uout) {
+                uout[i] = ux;
+                uout[N + i] = uy;
+            }
+            const int write = all ? old | 1 << k : 7;
+#pragma unroll 1
+            for (int l = 0; l < kNF; l++) {
+                if (!(write & (1 << l))) continue;
+                const float c = plain ? (l == k ? 1.0f : 0.0f) : fraction(l == k ? r : 0.0f, r);
+                store_fluid<STORE>(P, fout, l, i, f, c);
+            }
+        }
+        const unsigned some = __ballot_sync(0xffffffffu, own_fluid);
+        if (lane == 0) *word = (uint8_t)(some ? (all ? 1 << k : 7) : 0);
+        return;
+    }
+
+    // ---- pulls, densities and phase fields of the halo-2 region ----
+    int present = wp;
+    float f[kQ], r0 = 0.0f, r1 = 0.0f, r2 = 0.0f;
+    if (!(own & kGeoSolid)) {
+        own = S.geo[hy][px];
+        hx = px;
+        float q[27];
+        bool open = false;
+#pragma unroll
+        for (int a = 0; a < kQ; a++) {
+            const int g = S.geo[hy - ey(a)][hx - ex(a)];
+            const bool bb = g & kGeoSolid;
+            const int s = bb ? own : g;
+            load_direction<STORE>(P, fin, s & kGeoIdx, bb ? opp(a) : a, q + a);
+        }
+#pragma unroll
+        for (int a = 1; a < kQ; a++) {
+            const int g = S.geo[hy - ey(a)][hx - ex(a)];
+            if ((g & kGeoSolid ? own : g) & kGeoPar) {
+                const float t = q[a];
+                q[a] = q[18 + a];
+                q[18 + a] = t;
+            }
+            if (g & kGeoGhost) {
+                open = true;
+                q[a] = q[9 + a] = q[18 + a] = 0.0f;
+            }
+        }
+        if (own & kGeoPar) {
+            const float t = q[0];
+            q[0] = q[18];
+            q[18] = t;
+        }
+        if (open) zou_he(P, q, x0 + hx - 3 == 0);
+        present |= phase_fields<CX, CY>(df, q, S.ch, S.cl, S.rho, cx, cy);
+#pragma unroll
+        for (int a = 0; a < kQ; a++) f[a] = (q[a] + q[9 + a]) + q[18 + a];
+        r0 = sum9(q);
+        r1 = sum9(q + 9);
+        r2 = sum9(q + 18);
+    } else if (geo_class(own) == kSI && tid < NC) {
+#pragma unroll
+        for (int k = 0; k < kNF; k++) S.ch[k][cy][cx] = S.cl[k][cy][cx] = 0.0f;
+        S.rho[cy][cx] = 0.0f;
+    }
+    {
+        // the fluids this row's fluid nodes hold, for the tiles around in the next step
+        const int b = own_fluid ? (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0) : 0;
+        const int w = __reduce_or_sync(0xffffffffu, b);
+        if (inside && lane == 0) *word = (uint8_t)w;
+        const int pw = __reduce_or_sync(0xffffffffu, present);
+        if (lane == 0 && pw) atomicOr(&S.flags, pw);
+    }
+    group_sync(1, NB);
+    const bool mixed = __popc((unsigned)(S.flags & 7)) != 1;
+
+    // ---- stress tensor of Eq.(10) on the halo-1 region; gradients of the own nodes ----
+    float Fx = 0.0f, Fy = 0.0f, gr[6] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    if (mixed) {
+        if (tid < NR) {
+            int rx = cx - 1, ry = cy - 1;
+            if (!inside) {
+                // the ring of the halo-1 region: two rows, then two columns
+                const int j = tid - NOWN;
+                ry = j < 2 * RX ? (j < RX ? 0 : RY - 1) : 1 + (j - 2 * RX) / 2;
+                rx = j < 2 * RX ? j % RX : ((j - 2 * RX) & 1 ? RX - 1 : 0);
+            }
+            float Txx, Txy, Tyy, gxk[kNF], gyk[kNF];
+            stress_at<HX, CX, CY>(P, S.geo, S.ch, S.cl, S.rho, df, rx, ry, gxk, gyk, Txx, Txy, Tyy);
+            S.txx[ry][rx] = Txx;
+            S.txy[ry][rx] = Txy;
+            S.tyy[ry][rx] = Tyy;
+#pragma unroll
+            for (int k = 0; k < kNF; k++) {
+                gr[2 * k] = gxk[k];
+                gr[2 * k + 1] = gyk[k];
+            }
+        }
+        group_sync(1, NB);
+        if (own_fluid) div_stress<RX>(S.txx, S.txy, S.tyy, cx - 1, cy - 1, Fx, Fy);
+    }
+    // ---- velocity, MRT collision with forcing, recolouring, stores ----
+    if (own_fluid) {
+        const int i = own & kGeoIdx;
+        float ux, uy;
+        const Recolour rc = collide_node(P, f, r0, r1, r2, Fx, Fy, gr, ux, uy);
+        if (uout) {
+            uout[i] = ux;
+            uout[N + i] = uy;
+        }
+        store_recoloured<STORE>(P, fout, i, f, rc);
+    }
+}
+
 // Pure tiles around which the step's input holds one fluid k (pres_in): k alone is in the tile
 // after the pull (a fluid absent from all of a node's sources stays absent, and the recolouring
 // keeps it at zero), so 9 populations per node are pulled, collided and written: 72 B per node
@@ -1332,7 +1671,7 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
 // bounded: a consumer that gives up sets the error bit and its group returns; the producer gives
 // up on a buffer that is never released, and before exiting it waits (full limit) for every copy
 // it issued, so no copy lands in the shared memory of a later block.  The arithmetic is that of
-// k_step_tma and k_step<PURE>, so the results are identical.
+// k_step_tma and k_step_plain, so the results are identical.
 // The tiles with one fluid around are k_step_one's unless all is set; the producer passes over them, 32 at a time
 // (each lane looks one up).  Each warp records the fluids its nodes hold (one byte of
 // pres_out[tile] per warp), so that the tiles around know in the next step.
@@ -1746,35 +2085,6 @@ void with_store(int store, const Pop& p, long long N, Fn fn)
         fn(Store<kStoreBF16>(p, N));
 }
 
-void launch_wet(int store, const Params& P, int nw, const int* widx, const double* wnrm,
-                const float* wang, const Pop& f, const uint8_t* type, double* Cw, WetCache* cache,
-                cudaStream_t s, double* Cw_prev)
-{
-    if (nw <= 0) return;
-    const long long threads = 4LL * nw;
-    with_store(store, f, P.N, [&](auto st) {
-        k_wet<<<(unsigned)((threads + 127) / 128), 128, 0, s>>>(P, nw, widx, wnrm, wang, st, type, Cw, cache, Cw_prev);
-    });
-}
-
-__global__ void k_wet_cache_reset(WetCache* cache, int n)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        const double nan = __longlong_as_double(0x7ff8000000000000LL);  // never equal
-        cache[i].th = nan;
-        cache[i].wm = nan;
-        cache[i].wl = nan;
-    }
-}
-
-void reset_wet_cache(WetCache* cache, int nw, cudaStream_t s)
-{
-    if (nw <= 0) return;
-    const int n = 4 * nw;
-    k_wet_cache_reset<<<(n + 255) / 256, 256, 0, s>>>(cache, n);
-}
-
 void launch_wet_init(int store, const Params& P, int nw, const int* widx, const Pop& f,
                      const uint8_t* type, double* Cw, cudaStream_t s)
 {
@@ -1784,33 +2094,35 @@ void launch_wet_init(int store, const Params& P, int nw, const int* widx, const 
     });
 }
 
-template <int STORE>
-static void launch_step_t(const Params& P, const int* tiles, int ntiles, int kind, const Pop& fin,
-                          const Pop& fout, const uint8_t* type, const double* Cw, float* u,
-                          const uint64_t* pres_in, uint64_t* pres_out, bool all, cudaStream_t s)
-{
-    if (kind == kTilesPure)
-        k_step<kTX, kTY, true, true, STORE>
-            <<<ntiles, dim3(kTX, kTY), 0, s>>>(P, tiles, fin, fout, type, Cw, u, pres_in, pres_out, all);
-    else if (kind == kTilesWall)
-        k_step<kTX, kTY, false, true, STORE>
-            <<<ntiles, dim3(kTX, kTY), 0, s>>>(P, tiles, fin, fout, type, Cw, u, pres_in, pres_out, all);
-    else
-        k_step<kTX, kTY, false, false, STORE>
-            <<<ntiles, dim3(kTX, kTY), 0, s>>>(P, tiles, fin, fout, type, Cw, u, pres_in, pres_out, all);
-}
-
-void launch_step(int store, const Params& P, const int* tiles, int ntiles, int kind, const Pop& fin,
-                 const Pop& fout, const uint8_t* type, const double* Cw, float* u, const uint64_t* pres_in,
-                 uint64_t* pres_out, cudaStream_t s, bool all)
+void launch_step_plain(int store, const Params& P, const int* tiles, int ntiles, const Pop& fin, const Pop& fout,
+                       float* u, const uint64_t* pres_in, uint64_t* pres_out, bool all, cudaStream_t s)
 {
     if (ntiles <= 0) return;
+    const dim3 b(kTX, kTY);
     if (store == kStoreF32)
-        launch_step_t<kStoreF32>(P, tiles, ntiles, kind, fin, fout, type, Cw, u, pres_in, pres_out, all, s);
+        k_step_plain<kTX, kTY, kStoreF32><<<ntiles, b, 0, s>>>(P, tiles, fin, fout, u, pres_in, pres_out, all);
     else if (store == kStoreF16)
-        launch_step_t<kStoreF16>(P, tiles, ntiles, kind, fin, fout, type, Cw, u, pres_in, pres_out, all, s);
+        k_step_plain<kTX, kTY, kStoreF16><<<ntiles, b, 0, s>>>(P, tiles, fin, fout, u, pres_in, pres_out, all);
     else
-        launch_step_t<kStoreBF16>(P, tiles, ntiles, kind, fin, fout, type, Cw, u, pres_in, pres_out, all, s);
+        k_step_plain<kTX, kTY, kStoreBF16><<<ntiles, b, 0, s>>>(P, tiles, fin, fout, u, pres_in, pres_out, all);
+}
+
+void launch_tile(int store, const Params& P, const TileSet& T, const Pop& fin, const Pop& fout, double* cw_out, float* u,
+                 const uint64_t* pres_in, uint64_t* pres_out, bool full_write, cudaStream_t s)
+{
+    if (T.ntiles <= 0) return;
+    const int nt = kTileThreads, fw = full_write ? 1 : 0;
+    if (store == kStoreF32)
+        k_tile<kTX, kTY, kStoreF32><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw);
+    else if (store == kStoreF16)
+        k_tile<kTX, kTY, kStoreF16><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw);
+    else
+        k_tile<kTX, kTY, kStoreBF16><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw);
+}
+
+void launch_wet_look(const Params& P, const TileSet& T, int entries, const double* Cw, cudaStream_t s)
+{
+    if (entries > 0) k_wet_look<<<(4 * entries + 127) / 128, 128, 0, s>>>(P, T, entries, Cw);
 }
 
 // Pure tiles of the 16-bit storage through the tensor memory accelerator, persistent, with the

@@ -182,14 +182,14 @@ class Lbm3:
 
     def step_timed(self, n):
         """Advance n steps; return CUDA-event times in ms summed over the steps:
-        (wetting pass, fused kernel on pure tiles, fused kernel on the other tiles)."""
+        (wetting launch -- none, about 0 --, pure tiles, the other tiles)."""
         out = np.zeros(3)
         _check(self._h, load().lbm3_step_timed(self._h, int(n), _dp(out)))
         return float(out[0]), float(out[1]), float(out[2])
 
     def step_timed_detail(self, n):
-        """Advance n steps; return CUDA-event times in ms summed over the steps: (wetting pass,
-        pure tiles, wall tiles, edge tiles, the whole run on the device)."""
+        """Advance n steps; return CUDA-event times in ms summed over the steps: (0,
+        pure tiles, the other tiles, 0, the whole run on the device)."""
         out = np.zeros(5)
         _check(self._h, load().lbm3_step_timed_detail(self._h, int(n), _dp(out)))
         return tuple(float(v) for v in out)
