@@ -312,7 +312,10 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
     if ((e = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) != cudaSuccess) return e;
     if (ev) record_timing(h, ev[2], h->side);
     if (ev) record_timing(h, ev[3], h->side);
-    launch_tile(h->precision, h->P, h->gen, fin, fo, cw_out, u, pin, pout, io, h->side);
+    // steps between the adjoint's slots write every plane and wall value: the tiles all of theirs
+    const bool light = h->one && !io;
+    if (light) launch_step_one(h->precision, h->P, h->gen, nullptr, 0, fin, fo, u, pin, pout, false, h->side);
+    launch_tile(h->precision, h->P, h->gen, fin, fo, cw_out, u, pin, pout, io, light, h->side);
     if (ev) record_timing(h, ev[4], h->side);
     if (ev) record_timing(h, ev[0], h->stream);
     // pure tiles: those with several fluids around through the kernel of the storage and layout,
@@ -333,7 +336,9 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
         else
             launch_step_plain(h->precision, h->P, h->tiles_pure, h->n_pure, fin, fo, u, pin, pout, !one, ms);
         if (one) {
-            launch_step_one(h->precision, h->P, h->tiles_pure, h->n_pure, fin, fo, u, pin, pout, io, h->stream);
+            TileSet none = h->gen;
+            none.ntiles = 0;
+            launch_step_one(h->precision, h->P, none, h->tiles_pure, h->n_pure, fin, fo, u, pin, pout, io, h->stream);
             if ((e = cudaEventRecord(h->ev_join3, ms)) != cudaSuccess) return e;
             if ((e = cudaStreamWaitEvent(h->stream, h->ev_join3, 0)) != cudaSuccess) return e;
         }
@@ -579,13 +584,14 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
             std::vector<int> near;
             const int first = (int)went.size();
             bool open = false;
-            for (int Y = y0 - 3; Y < y0 + kTY + 3; Y++) {
+            constexpr int H = kNearHalo + 1;
+            for (int Y = y0 - H; Y < y0 + kTY + H; Y++) {
                 int y = Y;
                 if (y < 0 || y >= ny) {
                     if (!g->periodic_y) continue;
                     y = ((y % ny) + ny) % ny;
                 }
-                for (int X = x0 - 3; X < x0 + kTX + 3; X++) {
+                for (int X = x0 - H; X < x0 + kTX + H; X++) {
                     int x = X, par = 0;
                     if (g->bc_x == kZouHe) {
                         // a column that Zou-He completes may hold what nobody stored near it
@@ -620,12 +626,15 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
             rec.insert(rec.end(), near.begin(), near.end());
         }
     }
-    // flags of the fluid nodes: the directions that bounce back there, and the domain's edges
+    // flags of the nodes: the directions that bounce back there, and the domain's edges
     std::vector<uint16_t> nflag(N, 0);
     for (int y = 0; y < ny; y++)
         for (int x = 0; x < nx; x++) {
             const size_t i = (size_t)y * nx + x;
-            if (solid[i]) continue;
+            if (solid[i]) {
+                nflag[i] = (uint16_t)kNodeSolid;
+                continue;
+            }
             int f = (x == 0 ? kNodeX0 : 0) | (x == nx - 1 ? kNodeXN : 0) | (y == 0 ? kNodeY0 : 0) |
                     (y == ny - 1 ? kNodeYN : 0);
             if (cls[i] == kFB)
@@ -1040,7 +1049,9 @@ int lbm3_set_wall_angles(lbm3* h, const double* angles)
     }
     if (!a.empty())
         CUDA_TRY(h, cudaMemcpyAsync(h->wang, a.data(), a.size() * sizeof(float), cudaMemcpyHostToDevice, h->stream));
-    // the lines that the next step reads were looked for with the old angles
+    // the lines that the next step reads were looked for with the old angles (and the words say that
+    // they have settled)
+    CUDA_TRY(h, pres_reset(h));
     if (h->ready) launch_wet_look(h->P, h->gen, h->n_went, h->cw[h->pp], h->stream);
     CUDA_TRY(h, cudaGetLastError());
     CUDA_TRY(h, cudaStreamSynchronize(h->stream));

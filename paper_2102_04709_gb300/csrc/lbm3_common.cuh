@@ -307,10 +307,13 @@ struct alignas(16) WetLane {
     int ia, fa, ib, fb;
 };
 // flags of a fluid node: bits 0-8, direction a bounces back there; its column and row are the first
-// or last ones; (in a lane) it lies an odd number of seams away from the C_SB node, or in the tile's
-// phase-field region
+// or last ones; (in a lane) it lies an odd number of seams away from the C_SB node, or within
+// kNearHalo of the tile.  Solid nodes: kNodeSolid.
 constexpr int kNodePar = 1 << 9;
-constexpr int kNodeNear = 1 << 14;
+constexpr int kNodeNear = 1 << 14, kNodeSolid = 1 << 15;
+// a tile's record names the tiles within kNearHalo + 1 of it: the words of those say what a node within
+// kNearHalo holds after the pull
+constexpr int kNearHalo = 5;
 constexpr int kNodeX0 = 1 << 10, kNodeXN = 1 << 11, kNodeY0 = 1 << 12, kNodeYN = 1 << 13;
 
 // A list of tiles with what a step needs to know of each: a record of 32 words -- the tile, its first
@@ -330,7 +333,7 @@ struct TileSet {
     const float* wang;    // by place in the wall list: the three angles
     WetLane* cache;
     const uint8_t* type;
-    const uint16_t* nflag;  // flags of every fluid node (0 at solid ones)
+    const uint16_t* nflag;  // flags of every node
 };
 
 // ---- kernel launchers (lbm3_step.cu); `store` is kStoreF32 / kStoreF16 / kStoreBF16 ----
@@ -351,10 +354,13 @@ cudaError_t step_tma_prepare();
 cudaError_t step_tma16_prepare();
 void launch_step_tma(const Params& P, const int* tiles, int ntiles, int nblocks, const Pop& fout, float* u,
                      const CUtensorMap& tin_a, const CUtensorMap& tin_b, const CUtensorMap& tout, cudaStream_t s);
-// pure tiles around which pres_in holds one fluid, a warp each (any storage, any nx); the launches
-// below leave those out unless `all` is set; full_write: fout is not the buffer that pres_out described before this step
-void launch_step_one(int store, const Params& P, const int* tiles, int ntiles, const Pop& fin, const Pop& fout,
-                     float* u, const uint64_t* pres_in, uint64_t* pres_out, bool full_write, cudaStream_t s);
+// tiles around which pres_in holds one fluid, a warp each (any storage, any nx): the pure ones of the
+// list, and those of T in which nothing of the wetting changes (none of T if T.ntiles is 0); launch_tile
+// with `one`, and the launches below unless `all` is set, leave them out.  full_write: fout is not the
+// buffer that pres_out described before this step
+void launch_step_one(int store, const Params& P, const TileSet& T, const int* tiles, int ntiles, const Pop& fin,
+                     const Pop& fout, float* u, const uint64_t* pres_in, uint64_t* pres_out, bool full_write,
+                     cudaStream_t s);
 // pure FP32 tiles through a ring of three bulk-copy buffers, one producer warp and two consumer
 // groups per block, one block per SM (nblocks blocks): tensor map of fin with the whole pull box
 // (kTX + 8, kTY + 6, 27) over the [27][ny][nx] buffer
@@ -377,7 +383,7 @@ void launch_step_plain(int store, const Params& P, const int* tiles, int ntiles,
 // tiles of any kind, one per block; cw_out: the wall values of this step (those of the last one are in
 // the cache's lines)
 void launch_tile(int store, const Params& P, const TileSet& T, const Pop& fin, const Pop& fout, double* cw_out, float* u,
-                 const uint64_t* pres_in, uint64_t* pres_out, bool full_write, cudaStream_t s);
+                 const uint64_t* pres_in, uint64_t* pres_out, bool full_write, bool one, cudaStream_t s);
 // the cache's lines from the wall values Cw, after those or the wall angles were replaced
 void launch_wet_look(const Params& P, const TileSet& T, int entries, const double* Cw, cudaStream_t s);
 void launch_init(int store, const Params& P, const double* rho, const uint8_t* type, const Pop& f,

@@ -1118,7 +1118,8 @@ __device__ __forceinline__ void wet_line(const Params& P, const TileSet& T, cons
     auto bracket = [&](int X, int Y, int& idx, int& fl) {
         wet_node(P, T.nflag, X, Y, idx, fl);
         const int gx = hx + X - px, gy = hy + Y - py;
-        if (gx >= 1 && gx <= HX - 2 && gy >= 1 && gy <= HY - 2) fl |= kNodeNear;
+        if (gx >= 3 - kNearHalo && gx <= HX - 4 + kNearHalo && gy >= 3 - kNearHalo && gy <= HY - 4 + kNearHalo)
+            fl |= kNodeNear;
     };
     if (cr.kind >= 1) bracket(cr.ax, cr.ay, c.ia, c.fa);
     if (cr.kind == 2) bracket(cr.bx, cr.by, c.ib, c.fb);
@@ -1217,8 +1218,9 @@ __device__ __forceinline__ void wet_look(const Params& P, const TileSet& T, int 
 // phase fields (rho := 1 there), to S.wv and, for the nodes that the tile owns, to cw_out.  A node
 // near several tiles is wetted by each of them, with the same result: 1.6 times the work of a pass
 // over the nodes, but no launch that the tiles have to wait for.  one: the fluids around; where that
-// is one, the nodes of the region hold it alone (C_k exactly 1 or 0) and need no pull.  Returns the
-// fluids with a nonzero wall value (bit k), and in bit 3 whether some node's values are mixed.
+// is one, the nodes near the region hold it alone (C_k exactly 1 or 0) and need no pull.  Returns the
+// fluids with a nonzero wall value (bit k), in bit 3 whether some node's values are mixed, and in bit 4
+// whether a line ends in a node that is not near.
 template <int TX, int TY, int STORE>
 __device__ __forceinline__ int wet_entries(const Params& P, const TileSet& T, int e0, int cnt, int one,
                                            const Pop& fin, double* cw_out, TileShared<TX, TY>& S)
@@ -1250,6 +1252,7 @@ __device__ __forceinline__ int wet_entries(const Params& P, const TileSet& T, in
             if (valid) {
                 const int4 en = S.went[e];
                 const int idx = end ? c.ib : c.ia, fl = end ? c.fb : c.fa, node = en.x;
+                if (idx >= 0 ? !(fl & kNodeNear) : end == 0) bits |= 16;
                 if (idx >= 0 && (fl & kNodeNear) && __popc((unsigned)one) == 1)
                     v = one >> relabel(k, en.z & kWetPar) & 1 ? 1.0 : 0.0;  // in the tile's frame
                 else if (idx >= 0)
@@ -1352,6 +1355,35 @@ __global__ void k_wet_init(const Params P, const int nw, const int* __restrict__
     }
 }
 
+// Fluids stored in the tiles of a record (this lane's entry of the list: nbr), for the whole warp.
+__device__ __forceinline__ int fluids_reaching(const uint64_t* __restrict__ pres, int nbr)
+{
+    int around = nbr == -1 ? 7 : 0;  // an open column: any fluid
+    if (nbr >= 0) {
+        uint64_t b = pres[nbr >> 1];
+        b |= b >> 32;
+        b |= b >> 16;
+        b |= b >> 8;
+        const int v = (int)(b & 7u);
+        around = nbr & 1 ? (v & 2) | (v & 1) << 2 | v >> 2 : v;  // across the seam
+    }
+    return __reduce_or_sync(0xffffffffu, around);
+}
+
+// The upper bits of a tile's word (byte 0: bits 4-5 a number of steps, at most 2, 6-7 a fluid k): for
+// how many steps the wall values of every C_SB node that the tile sees have been those of k alone,
+// with lines that end in nodes near it.  After two both arrays of wall values hold them, and while the
+// tiles around keep holding k alone nothing of the wetting changes.
+__device__ __forceinline__ int settled_steps(uint64_t word, int around)
+{
+    return __popc((unsigned)around) == 1 && (int)(word >> 6 & 3) == __ffs(around) - 1 ? (int)(word >> 4 & 3) : 0;
+}
+// a tile that needs no wetting and holds one fluid after the pull: k_step_one's
+__device__ __forceinline__ bool settled_single(int around, int cnt, uint64_t word)
+{
+    return __popc((unsigned)around) == 1 && (cnt == 0 || settled_steps(word, around) == 2);
+}
+
 // One step of tile T.rec[blockIdx.x] (any kind): thread t < TX TY has the tile's node t, the next ones a
 // node of the ring that the halo-2 region has around it.
 //   geometry words of the halo-3 region into shared memory
@@ -1373,7 +1405,7 @@ __global__ void k_wet_init(const Params P, const int nw, const int* __restrict__
 template <int TX, int TY, int STORE>
 __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const TileSet T, const Pop fin, const Pop fout,
                                                           double* cw_out, float* uout, const uint64_t* pres_in,
-                                                          uint64_t* pres_out, const int full_write)
+                                                          uint64_t* pres_out, const int full_write, const int one)
 {
     using TS = TileShared<TX, TY>;
     constexpr int NT = kTileThreads, CX = TS::CX, CY = TS::CY, RX = TS::RX, RY = TS::RY, HX = TS::HX, HY = TS::HY;
@@ -1391,6 +1423,15 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
     const int nbr = lane >= kTileRecHead ? word32 : kNoTile;
     const int ntx = (P.nx + TX - 1) / TX;
     const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
+    // fluids stored in the tiles that reach the region (every warp for itself), and whether the
+    // tile's wall values have settled
+    int around;
+    uint64_t mine;
+    if (one) {
+        around = fluids_reaching(pres_in, nbr);
+        mine = pres_in[tile];
+        if (settled_single(around, cnt, mine)) return;  // k_step_one's
+    }
     for (int j = tid; j < HX * HY; j += NT) {
         const int hx = j % HX, hy = j / HX;
         S.geo[hy][hx] = geo_word(P, T.type, x0 + hx - 3, y0 + hy - 3);
@@ -1400,20 +1441,13 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
         S.nrm[tid] = T.wnrm[e0 + tid];
     }
     if (tid == 0) S.wall = S.flags = 0;
-    // fluids stored in the tiles that the halo-3 region touches (every warp for itself)
-    int around = nbr == -1 ? 7 : 0;  // an open column: any fluid
-    if (nbr >= 0) {
-        uint64_t b = pres_in[nbr >> 1];
-        b |= b >> 32;
-        b |= b >> 16;
-        b |= b >> 8;
-        const int v = (int)(b & 7u);
-        around = nbr & 1 ? (v & 2) | (v & 1) << 2 | v >> 2 : v;  // across the seam
+    if (!one) {
+        around = fluids_reaching(pres_in, nbr);
+        mine = pres_in[tile];
     }
     const bool inside = tid < NOWN;  // a node of the tile itself, row tid / 32 (one warp)
     uint8_t* const word = reinterpret_cast<uint8_t*>(pres_out + tile) + (tid >> 5);
-    const int old = !inside || full_write ? 7 : *word;  // what this row of the output buffer still holds
-    around = __reduce_or_sync(0xffffffffu, around);
+    const int old = !inside || full_write ? 7 : *word & 7;  // what this row of the output buffer still holds
     __syncthreads();
 
     // this thread's position in the phase-field region
@@ -1443,6 +1477,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
         df = S.wall & 8;
         wp = S.wall & 7;
     }
+    // steps in a row in which one fluid was around and every wall value and line was that fluid's
+    const int quiet = cnt > 0 && S.wall == around ? min(settled_steps(mine, around) + 1, 2) : 0;
     if (tid >= NB) {
         if (cnt > 0) {
             const int last = (cnt - 1) / kWetNodes * kWetNodes;
@@ -1482,7 +1518,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
             }
         }
         const unsigned some = __ballot_sync(0xffffffffu, own_fluid);
-        if (lane == 0) *word = (uint8_t)(some ? (all ? 1 << k : 7) : 0);
+        if (lane == 0) *word = (uint8_t)((some ? (all ? 1 << k : 7) : 0) | (tid == 0 ? quiet << 4 | k << 6 : 0));
         return;
     }
 
@@ -1590,6 +1626,10 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
 // in that buffer.  (full_write: the output is not the buffer that pres_out described, so they are
 // cleared always.)  The other pure tiles are left to the kernels that move all 27 planes.
 //
+// The tiles near solids or the domain edge in which nothing of the wetting changes (settled_single) are
+// done the same way, with the flags of each node (directions that bounce back, wraps) in place of fixed
+// offsets.
+//
 // One warp per tile, a row of 32 nodes at a time, two rows in flight: nothing is shared between
 // threads, each population is read once, and the loads of a warp are whole lines but for the
 // shift by one node in x.  It is bound by HBM, so what counts is warps in flight: no shared memory,
@@ -1598,8 +1638,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
 // instead of 353 (FP16: 310 instead of 425).  (Inside the ring kernel, with 9-plane boxes, the same
 // tiles took 1200 cycles of a consumer group and 1500 of its one producer each: 270 us.)
 constexpr int kOneThreads = 128;
-template <int TX, int TY, int STORE>
-__global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const int* __restrict__ tiles,
+template <int TX, int TY, int STORE, bool PURE>
+__global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const TileSet T, const int* __restrict__ tiles,
                                                           const int ntiles, const Pop fin, const Pop fout,
                                                           float* __restrict__ uout,
                                                           const uint64_t* __restrict__ pres_in,
@@ -1607,54 +1647,95 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
 {
     static_assert(TX == 32 && TY == 8, "one warp per tile, one byte of its word per row");
     const int w = blockIdx.x * (kOneThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (w >= ntiles) return;
+    if (w >= (PURE ? ntiles : T.ntiles)) return;
     const int ntx = (P.nx + TX - 1) / TX;
-    const int tile = tiles[w];
-    const int around = fluids_around(pres_in, tile, ntx);
-    if (__popc((unsigned)around) != 1) return;
+    int tile, around;
+    uint64_t word = 0;
+    if constexpr (PURE) {
+        tile = tiles[w];
+        around = fluids_around(pres_in, tile, ntx);
+        if (__popc((unsigned)around) != 1) return;
+    } else {
+        const int r = T.rec[w * kTileRecInts + lane];
+        tile = __shfl_sync(0xffffffffu, r, 0);
+        const int cnt = __shfl_sync(0xffffffffu, r, 2);
+        const uint64_t mine = pres_in[tile];
+        around = fluids_reaching(pres_in, lane >= kTileRecHead ? r : -2);
+        if (!settled_single(around, cnt, mine)) return;
+        word = mine & 0xf0;  // settled it stays
+    }
     const uint64_t old = full_write ? 0x0707070707070707ull : pres_out[tile];
     const int k = __ffs(around) - 1;
     const int nx = P.nx, N = (int)P.N;
-    const int i0 = (tile / ntx) * TY * nx + (tile % ntx) * TX + lane;
-    uint64_t word = 0;
+    const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
+    const int rows = PURE ? TY : min(TY, P.ny - y0);
+    const bool column = PURE || x0 + lane < nx;
 #pragma unroll 2
-    for (int row = 0; row < TY; row++) {
-        const int i = i0 + row * nx;
+    for (int row = 0; row < rows; row++) {
+        const int i = (y0 + row) * nx + x0 + lane;
         float f[kQ];
-        if constexpr (STORE == kStoreF32) {
-            const float* b = fin.f + i + k * kQ * N;
+        bool fluid = true;
+        if constexpr (PURE) {
+            if constexpr (STORE == kStoreF32) {
+                const float* b = fin.f + i + k * kQ * N;
 #pragma unroll
-            for (int a = 0; a < kQ; a++) f[a] = __ldg(b + P.off_pull[a]);
+                for (int a = 0; a < kQ; a++) f[a] = __ldg(b + P.off_pull[a]);
+            } else {
+                const float* rb = fin.rho + i + k * N;
+                const unsigned short* ob = fin.off + i + 8 * k * N;
+                float d[kQ];
+#pragma unroll
+                for (int a = 1; a < kQ; a++) d[a] = dec16<STORE>(__ldg(ob + (a - 1) * N));
+                f[0] = wq(0) * __ldg(rb) - sum_offsets(d);
+#pragma unroll
+                for (int a = 1; a < kQ; a++)
+                    f[a] = wq(a) * __ldg(rb + P.off_pull16[a]) + dec16<STORE>(__ldg(ob + P.off_pull16o[a]));
+            }
         } else {
-            const float* rb = fin.rho + i + k * N;
-            const unsigned short* ob = fin.off + i + 8 * k * N;
-            float d[kQ];
+            const int fl = column ? (int)__ldg(T.nflag + i) : kNodeSolid;
+            fluid = !(fl & kNodeSolid);
+            if (fluid) {
+                const int xm = fl & kNodeX0 ? nx - 1 : -1, xp = fl & kNodeXN ? 1 - nx : 1;
+                const int ym = fl & kNodeY0 ? (P.ny - 1) * nx : -nx, yp = fl & kNodeYN ? (1 - P.ny) * nx : nx;
 #pragma unroll
-            for (int a = 1; a < kQ; a++) d[a] = dec16<STORE>(__ldg(ob + (a - 1) * N));
-            f[0] = wq(0) * __ldg(rb) - sum_offsets(d);
-#pragma unroll
-            for (int a = 1; a < kQ; a++)
-                f[a] = wq(a) * __ldg(rb + P.off_pull16[a]) + dec16<STORE>(__ldg(ob + P.off_pull16o[a]));
+                for (int a = 0; a < kQ; a++) {
+                    const bool bb = a > 0 && (fl >> a & 1);
+                    const bool over = (ex(a) == 1 && (fl & kNodeX0)) || (ex(a) == -1 && (fl & kNodeXN));
+                    const int d = (ex(a) == 1 ? xm : (ex(a) == -1 ? xp : 0)) + (ey(a) == 1 ? ym : (ey(a) == -1 ? yp : 0));
+                    const bool swap = P.bc_x == kModPer && over && !bb && k != 1;
+                    load_fluid<STORE>(P, fin, bb ? i : i + d, bb ? opp(a) : a, swap ? 2 - k : k, f[a]);
+                }
+            }
         }
-        const float r = sum9(f);
-        float ux, uy;
-        const bool plain = collide_single(P, k, f, r, ux, uy);
-        if (uout) {
-            uout[i] = ux;
-            uout[N + i] = uy;
+        float r = 1.0f, ux = 0.0f, uy = 0.0f;
+        bool plain = true;
+        if (fluid) {
+            r = sum9(f);
+            plain = collide_single(P, k, f, r, ux, uy);
+            if (uout) {
+                uout[i] = ux;
+                uout[N + i] = uy;
+            }
         }
         const bool all = __all_sync(0xffffffffu, plain);
         const int rowold = (int)(old >> (8 * row)) & 7;
         // fluids to write: k, and those that this row of the buffer still holds, as zeros; all of
         // them where a density has no fraction
         const int write = all ? rowold | 1 << k : 7;
+        if (fluid) {
+            if (write == 1 << k) {
+                store_fluid<STORE>(P, fout, k, i, f, 1.0f);
+            } else {
 #pragma unroll 1
-        for (int l = 0; l < kNF; l++) {
-            if (!(write & (1 << l))) continue;
-            const float c = plain ? (l == k ? 1.0f : 0.0f) : fraction(l == k ? r : 0.0f, r);
-            store_fluid<STORE>(P, fout, l, i, f, c);
+                for (int l = 0; l < kNF; l++) {
+                    if (!(write & (1 << l))) continue;
+                    const float c = plain ? (l == k ? 1.0f : 0.0f) : fraction(l == k ? r : 0.0f, r);
+                    store_fluid<STORE>(P, fout, l, i, f, c);
+                }
+            }
         }
-        word |= (uint64_t)(all ? 1 << k : 7) << (8 * row);
+        const bool some = PURE || __ballot_sync(0xffffffffu, fluid);
+        word |= (uint64_t)(some ? (all ? 1 << k : 7) : 0) << (8 * row);
     }
     if (lane == 0) pres_out[tile] = word;
 }
@@ -2108,16 +2189,16 @@ void launch_step_plain(int store, const Params& P, const int* tiles, int ntiles,
 }
 
 void launch_tile(int store, const Params& P, const TileSet& T, const Pop& fin, const Pop& fout, double* cw_out, float* u,
-                 const uint64_t* pres_in, uint64_t* pres_out, bool full_write, cudaStream_t s)
+                 const uint64_t* pres_in, uint64_t* pres_out, bool full_write, bool one, cudaStream_t s)
 {
     if (T.ntiles <= 0) return;
     const int nt = kTileThreads, fw = full_write ? 1 : 0;
     if (store == kStoreF32)
-        k_tile<kTX, kTY, kStoreF32><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw);
+        k_tile<kTX, kTY, kStoreF32><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw, one);
     else if (store == kStoreF16)
-        k_tile<kTX, kTY, kStoreF16><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw);
+        k_tile<kTX, kTY, kStoreF16><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw, one);
     else
-        k_tile<kTX, kTY, kStoreBF16><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw);
+        k_tile<kTX, kTY, kStoreBF16><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw, one);
 }
 
 void launch_wet_look(const Params& P, const TileSet& T, int entries, const double* Cw, cudaStream_t s)
@@ -2406,19 +2487,23 @@ void launch_step_tma16(int store, const Params& P, const int* tiles, int ntiles,
             P, tiles, ntiles, fout, u, trho, toff, pres_in, pres_out, all);
 }
 
-void launch_step_one(int store, const Params& P, const int* tiles, int ntiles, const Pop& fin, const Pop& fout,
-                     float* u, const uint64_t* pres_in, uint64_t* pres_out, bool full_write, cudaStream_t s)
+void launch_step_one(int store, const Params& P, const TileSet& T, const int* tiles, int ntiles, const Pop& fin,
+                     const Pop& fout, float* u, const uint64_t* pres_in, uint64_t* pres_out, bool full_write,
+                     cudaStream_t s)
 {
-    if (ntiles <= 0) return;
     constexpr int per = kOneThreads / 32;
-    const unsigned nb = (unsigned)((ntiles + per - 1) / per);
     const int fw = full_write ? 1 : 0;
+    const unsigned nb = (unsigned)((ntiles + per - 1) / per), ng = (unsigned)((T.ntiles + per - 1) / per);
+    auto go = [&](auto pure, auto general) {
+        if (nb > 0) pure<<<nb, kOneThreads, 0, s>>>(P, T, tiles, ntiles, fin, fout, u, pres_in, pres_out, fw);
+        if (ng > 0) general<<<ng, kOneThreads, 0, s>>>(P, T, tiles, ntiles, fin, fout, u, pres_in, pres_out, fw);
+    };
     if (store == kStoreF32)
-        k_step_one<kTX, kTY, kStoreF32><<<nb, kOneThreads, 0, s>>>(P, tiles, ntiles, fin, fout, u, pres_in, pres_out, fw);
+        go(k_step_one<kTX, kTY, kStoreF32, true>, k_step_one<kTX, kTY, kStoreF32, false>);
     else if (store == kStoreF16)
-        k_step_one<kTX, kTY, kStoreF16><<<nb, kOneThreads, 0, s>>>(P, tiles, ntiles, fin, fout, u, pres_in, pres_out, fw);
+        go(k_step_one<kTX, kTY, kStoreF16, true>, k_step_one<kTX, kTY, kStoreF16, false>);
     else
-        k_step_one<kTX, kTY, kStoreBF16><<<nb, kOneThreads, 0, s>>>(P, tiles, ntiles, fin, fout, u, pres_in, pres_out, fw);
+        go(k_step_one<kTX, kTY, kStoreBF16, true>, k_step_one<kTX, kTY, kStoreBF16, false>);
 }
 
 void launch_init(int store, const Params& P, const double* rho, const uint8_t* type, const Pop& f,
