@@ -201,13 +201,14 @@ void release(lbm3* h)
     if (h->side) cudaStreamDestroy(h->side);
 }
 
-// From this many pure tiles on, those with one fluid around are launch_step_one's, and the others
-// run beside them on a stream of their own.  Below it the step waits for the tiles near solids, not
-// for the pure ones, and one more launch costs more than it hides: 2-3 % of
-// the step on 128 x 64 and on the 800 x 375 pillars (865 pure tiles), while the 2048 x 1024 ones
-// (6308) gain 12 %.  LBM3_ONE_TILES=<n> in the environment at lbm3_create sets another line (same
-// results).
-constexpr int kOneTiles = 4096;
+// From this many pure tiles on, the tiles with one fluid around are launch_step_one's, and the pure
+// ones with several run beside them on a stream of their own.  On smaller grids the fluids soon reach
+// every tile, the step waits for the tiles near solids, and two more launches cost more than they hide:
+// after 1500 steps the 512 x 512 cylinder (805 pure tiles) takes 25.5 us a step with them and 22.9
+// without, the 800 x 375 pillars (865) 28.6 and 28.9, the 1030 x 517 ones (1571) 36 and 42, a
+// 1024 x 1024 cylinder (3700) 60 and 67.  LBM3_ONE_TILES=<n> in the environment at lbm3_create sets
+// another line (same results).
+constexpr int kOneTiles = 1200;
 
 // Tensor maps of one [27][ny][nx] FP32 population buffer: as the two parts of the pull-source box
 // of a pure tile, (kTX + 8) x (kTY + 6) x kTmaPlanesA and x (27 - kTmaPlanesA) planes, and as its
@@ -314,8 +315,10 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
     if (ev) record_timing(h, ev[3], h->side);
     // steps between the adjoint's slots write every plane and wall value: the tiles all of theirs
     const bool light = h->one && !io;
-    if (light) launch_step_one(h->precision, h->P, h->gen, nullptr, 0, fin, fo, u, pin, pout, false, h->side);
     launch_tile(h->precision, h->P, h->gen, fin, fo, cw_out, u, pin, pout, io, light, h->side);
+    // (behind the tiles that take long: in front of them, or of the pure tiles on either stream, it delays
+    // what the step waits for, 5-10 % on the 2048 x 1024 pillars)
+    if (light) launch_step_one(h->precision, h->P, h->gen, nullptr, 0, fin, fo, u, pin, pout, false, h->side);
     if (ev) record_timing(h, ev[4], h->side);
     if (ev) record_timing(h, ev[0], h->stream);
     // pure tiles: those with several fluids around through the kernel of the storage and layout,

@@ -1630,14 +1630,17 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
 // done the same way, with the flags of each node (directions that bounce back, wraps) in place of fixed
 // offsets.
 //
-// One warp per tile, a row of 32 nodes at a time, two rows in flight: nothing is shared between
-// threads, each population is read once, and the loads of a warp are whole lines but for the
-// shift by one node in x.  It is bound by HBM, so what counts is warps in flight: no shared memory,
-// no barriers.  On the 4096 x 2048 pillars, 97 % of whose pure tiles are such, the pure tiles take
-// 173 us a step beside the other kernels instead of 338 (FP16: 190 instead of 410), and the step 240
-// instead of 353 (FP16: 310 instead of 425).  (Inside the ring kernel, with 9-plane boxes, the same
+// A warp takes kOneRows rows of 32 nodes, two in flight: nothing is shared between threads, each
+// population is read once, and the loads of a warp are whole lines but for the shift by one node in x.
+// It is bound by issue (250 instructions a row, 318 with lane-wise plane addresses) and HBM, so what
+// counts is warps in flight: no shared memory, no barriers.  On the 4096 x 2048 pillars, 97 % of whose
+// pure tiles are such, the pure tiles took 338 us a step (FP16: 410) in the kernels that move all 27
+// planes; the whole step, all kernels, takes 174 us with this one (FP16: 176).  (Inside the ring kernel, with 9-plane boxes, the same
 // tiles took 1200 cycles of a consumer group and 1500 of its one producer each: 270 us.)
 constexpr int kOneThreads = 128;
+// rows of a pure tile per warp (a tile near solids: 1, there are few of them and each row waits for its
+// flags first); 8, 4 and 2 rows: 180, 175 and 182 us a step of the 4096 x 2048 pillars
+constexpr int kOneRows = 4;
 template <int TX, int TY, int STORE, bool PURE>
 __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const TileSet T, const int* __restrict__ tiles,
                                                           const int ntiles, const Pop fin, const Pop fout,
@@ -1645,15 +1648,27 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
                                                           const uint64_t* __restrict__ pres_in,
                                                           uint64_t* __restrict__ pres_out, const int full_write)
 {
-    static_assert(TX == 32 && TY == 8, "one warp per tile, one byte of its word per row");
-    const int w = blockIdx.x * (kOneThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    static_assert(TX == 32 && TY == 8, "a row per warp instruction, one byte of the tile's word per row");
+    constexpr int RW = PURE ? kOneRows : 1;  // rows of a warp
+    const int u = blockIdx.x * (kOneThreads / 32) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    const int w = u / (TY / RW), row0 = u % (TY / RW) * RW;
     if (w >= (PURE ? ntiles : T.ntiles)) return;
     const int ntx = (P.nx + TX - 1) / TX;
     int tile, around;
     uint64_t word = 0;
     if constexpr (PURE) {
-        tile = tiles[w];
-        around = fluids_around(pres_in, tile, ntx);
+        // one lane per tile around; what a warp reduction returns is uniform to the compiler, which
+        // then addresses the planes by uniform registers
+        tile = __reduce_or_sync(0xffffffffu, tiles[w]);
+        int v = 0;
+        if (lane < 9) {
+            uint64_t b = pres_in[tile + (lane / 3 - 1) * ntx + lane % 3 - 1];
+            b |= b >> 32;
+            b |= b >> 16;
+            b |= b >> 8;
+            v = (int)(b & 7u);
+        }
+        around = __reduce_or_sync(0xffffffffu, v);
         if (__popc((unsigned)around) != 1) return;
     } else {
         const int r = T.rec[w * kTileRecInts + lane];
@@ -1664,22 +1679,35 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
         if (!settled_single(around, cnt, mine)) return;
         word = mine & 0xf0;  // settled it stays
     }
+    if (!PURE && row0 >= P.ny - (tile / ntx) * TY) {
+        if (lane == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[row0] = 0;
+        return;
+    }
     const uint64_t old = full_write ? 0x0707070707070707ull : pres_out[tile];
     const int k = __ffs(around) - 1;
     const int nx = P.nx, N = (int)P.N;
     const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
-    const int rows = PURE ? TY : min(TY, P.ny - y0);
+    const int rows = PURE ? row0 + RW : min(row0 + RW, P.ny - y0);
     const bool column = PURE || x0 + lane < nx;
+    // the fluid's planes at the tile's corner (FP32 storage)
+    const int corner = y0 * nx + x0;
+    const float* src[kQ];
+    float* dst[kQ];
+#pragma unroll
+    for (int a = 0; a < kQ; a++) {
+        src[a] = fin.f + (corner + k * kQ * N + P.off_pull[a]);
+        dst[a] = fout.f + (corner + k * kQ * N + P.off_plane[a]);
+    }
 #pragma unroll 2
-    for (int row = 0; row < rows; row++) {
+    for (int row = row0; row < rows; row++) {
         const int i = (y0 + row) * nx + x0 + lane;
         float f[kQ];
         bool fluid = true;
         if constexpr (PURE) {
             if constexpr (STORE == kStoreF32) {
-                const float* b = fin.f + i + k * kQ * N;
+                const unsigned o = (unsigned)(row * nx + lane);
 #pragma unroll
-                for (int a = 0; a < kQ; a++) f[a] = __ldg(b + P.off_pull[a]);
+                for (int a = 0; a < kQ; a++) f[a] = __ldg(src[a] + o);
             } else {
                 const float* rb = fin.rho + i + k * N;
                 const unsigned short* ob = fin.off + i + 8 * k * N;
@@ -1724,7 +1752,13 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
         const int write = all ? rowold | 1 << k : 7;
         if (fluid) {
             if (write == 1 << k) {
-                store_fluid<STORE>(P, fout, k, i, f, 1.0f);
+                if constexpr (STORE == kStoreF32) {
+                    const unsigned o = (unsigned)(row * nx + lane);
+#pragma unroll
+                    for (int a = 0; a < kQ; a++) dst[a][o] = f[a];
+                } else {
+                    store_fluid<STORE>(P, fout, k, i, f, 1.0f);
+                }
             } else {
 #pragma unroll 1
                 for (int l = 0; l < kNF; l++) {
@@ -1735,9 +1769,13 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
             }
         }
         const bool some = PURE || __ballot_sync(0xffffffffu, fluid);
-        word |= (uint64_t)(some ? (all ? 1 << k : 7) : 0) << (8 * row);
+        const int byte = some ? (all ? 1 << k : 7) : 0;
+        if constexpr (RW == TY)
+            word |= (uint64_t)byte << (8 * row);
+        else if (lane == 0)
+            reinterpret_cast<uint8_t*>(pres_out + tile)[row] = (uint8_t)(byte | (row == 0 ? (int)word : 0));
     }
-    if (lane == 0) pres_out[tile] = word;
+    if (RW == TY && lane == 0) pres_out[tile] = word;
 }
 
 // Pure FP32 tiles through a ring of bulk tensor copies, warp-specialised: one producer warp and
@@ -2493,7 +2531,8 @@ void launch_step_one(int store, const Params& P, const TileSet& T, const int* ti
 {
     constexpr int per = kOneThreads / 32;
     const int fw = full_write ? 1 : 0;
-    const unsigned nb = (unsigned)((ntiles + per - 1) / per), ng = (unsigned)((T.ntiles + per - 1) / per);
+    const unsigned nb = (unsigned)(((long long)ntiles * (kTY / kOneRows) + per - 1) / per);
+    const unsigned ng = (unsigned)(((long long)T.ntiles * kTY + per - 1) / per);
     auto go = [&](auto pure, auto general) {
         if (nb > 0) pure<<<nb, kOneThreads, 0, s>>>(P, T, tiles, ntiles, fin, fout, u, pres_in, pres_out, fw);
         if (ng > 0) general<<<ng, kOneThreads, 0, s>>>(P, T, tiles, ntiles, fin, fout, u, pres_in, pres_out, fw);
