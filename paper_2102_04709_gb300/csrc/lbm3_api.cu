@@ -467,17 +467,24 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
 
     // ---- node classes: a node is a boundary node when any D2Q9 neighbour is of the other kind
     std::vector<uint8_t> cls(N);
+    // flags of the nodes: the directions that bounce back there, and the domain's edges
+    std::vector<uint16_t> nflag(N);
     long long n_fluid = 0;
     for (int y = 0; y < ny; y++)
         for (int x = 0; x < nx; x++) {
             const int me = S(x, y);
             bool touch = false;
+            int flag = (x == 0 ? kNodeX0 : 0) | (x == nx - 1 ? kNodeXN : 0) | (y == 0 ? kNodeY0 : 0) |
+                       (y == ny - 1 ? kNodeYN : 0);
             for (int a = 1; a < kQ; a++) {
                 if (!me && S.outside_solid(x + ex(a), y + ey(a)))
                     return fail(nullptr, LBM3_ERR_INVALID,
                                 "a fluid node touches a wall side: make the boundary rows/columns solid");
-                if (S(x + ex(a), y + ey(a)) != me) touch = true;
+                const int other = S(x + ex(a), y + ey(a));
+                if (other != me) touch = true;
+                flag |= other << opp(a);  // what comes along opp(a) would come from there
             }
+            nflag[(size_t)y * nx + x] = (uint16_t)(me ? kNodeSolid : flag);
             cls[(size_t)y * nx + x] = me ? (touch ? kSB : kSI) : (touch ? kFB : kFI);
             n_fluid += !me;
         }
@@ -582,45 +589,70 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
         std::vector<int> wof(N, -1);
         for (size_t w = 0; w < widx.size(); w++) wof[widx[w]] = (int)w;
         std::vector<int> owner(widx.size(), -1);
+        // tiles with a fluid node (the others are never written)
+        std::vector<uint8_t> live((size_t)ntx * nty, 0);
+        for (const int t : tp) live[t] = 1;
+        for (const int t : tg) live[t] = 1;
         for (const int tile : tg) {
             const int x0 = (tile % ntx) * kTX, y0 = (tile / ntx) * kTY;
-            std::vector<int> near;
             const int first = (int)went.size();
-            bool open = false;
+            // columns and rows as the boundaries continue them: -1 where there is nothing
             constexpr int H = kNearHalo + 1;
-            for (int Y = y0 - H; Y < y0 + kTY + H; Y++) {
-                int y = Y;
-                if (y < 0 || y >= ny) {
-                    if (!g->periodic_y) continue;
-                    y = ((y % ny) + ny) % ny;
-                }
-                for (int X = x0 - H; X < x0 + kTX + H; X++) {
-                    int x = X, par = 0;
-                    if (g->bc_x == kZouHe) {
-                        // a column that Zou-He completes may hold what nobody stored near it
-                        if (X <= 0 || X >= nx - 1) open = true;
-                        if (X < 0 || X >= nx) continue;
-                    } else if (x < 0 || x >= nx) {
-                        if (g->bc_x == kWalls) continue;
+            int col[kTX + 2 * H], par[kTX + 2 * H], row[kTY + 2 * H];
+            bool open = false;
+            for (int j = 0; j < kTX + 2 * H; j++) {
+                int x = x0 + j - H;
+                par[j] = 0;
+                // a column that Zou-He completes may hold what nobody stored near it
+                if (g->bc_x == kZouHe && (x <= 0 || x >= nx - 1)) open = true;
+                if (x < 0 || x >= nx) {
+                    if (g->bc_x == kZouHe || g->bc_x == kWalls) {
+                        x = -1;
+                    } else {
                         const int q = floordiv_i(x, nx);
                         x -= q * nx;
-                        par = g->bc_x == kModPer ? q & 1 : 0;
+                        par[j] = g->bc_x == kModPer ? q & 1 : 0;
                     }
+                }
+                col[j] = x;
+            }
+            for (int j = 0; j < kTY + 2 * H; j++) {
+                const int y = y0 + j - H;
+                row[j] = y >= 0 && y < ny ? y : (g->periodic_y ? ((y % ny) + ny) % ny : -1);
+            }
+            std::vector<int> near, across;
+            for (int j = 0; j < kTX + 2 * H; j++)
+                if (col[j] >= 0) {
+                    const int c = 2 * (col[j] / kTX) + par[j];
+                    if (std::find(across.begin(), across.end(), c) == across.end()) across.push_back(c);
+                }
+            int seen = -1;
+            for (int j = 0; j < kTY + 2 * H; j++) {
+                if (row[j] < 0 || row[j] / kTY == seen) continue;
+                seen = row[j] / kTY;
+                for (const int c : across) {
+                    const int t = seen * ntx + c / 2, code = 2 * t + (c & 1);
+                    if (live[t] && std::find(near.begin(), near.end(), code) == near.end()) near.push_back(code);
+                }
+            }
+            for (int cy = 0; cy < kTY + 4; cy++) {
+                const int y = row[cy + H - 2];
+                if (y < 0) continue;
+                for (int cx = 0; cx < kTX + 4; cx++) {
+                    const int x = col[cx + H - 2];
+                    if (x < 0) continue;
                     const size_t i = (size_t)y * nx + x;
-                    if (!solid[i]) {
-                        const int code = 2 * ((y / kTY) * ntx + x / kTX) + par;
-                        if (std::find(near.begin(), near.end(), code) == near.end()) near.push_back(code);
-                    } else if (cls[i] == kSB && X >= x0 - 2 && X < x0 + kTX + 2 && Y >= y0 - 2 && Y < y0 + kTY + 2) {
-                        const bool mine = X >= x0 && X < x0 + kTX && X < nx && Y >= y0 && Y < y0 + kTY && Y < ny;
-                        if (mine || owner[wof[i]] < 0) {
-                            if (owner[wof[i]] >= 0) went[owner[wof[i]]].z &= ~kWetOwner;
-                            owner[wof[i]] = (int)went.size();
-                        }
-                        went.push_back(make_int4((int)i, wof[i],
-                                                 (X - x0 + 2) | (Y - y0 + 2) << 8 | (par ? kWetPar : 0) |
-                                                     (owner[wof[i]] == (int)went.size() ? kWetOwner : 0),
-                                                 0));
+                    if (cls[i] != kSB) continue;
+                    // the tile that has the node writes its wall values, else the first that sees it
+                    const int w = wof[i], X = x0 + cx - 2, Y = y0 + cy - 2;
+                    const bool mine = cx >= 2 && cx < kTX + 2 && cy >= 2 && cy < kTY + 2 && X < nx && Y < ny;
+                    int own = 0;
+                    if (mine || owner[w] < 0) {
+                        if (owner[w] >= 0) went[owner[w]].z &= ~kWetOwner;
+                        owner[w] = (int)went.size();
+                        own = kWetOwner;
                     }
+                    went.push_back(make_int4((int)i, w, cx | cy << 8 | (par[cx + H - 2] ? kWetPar : 0) | own, 0));
                 }
             }
             if (open || (int)near.size() > kTileRecInts - kTileRecHead) near.assign(1, -1);
@@ -629,21 +661,6 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
             rec.insert(rec.end(), near.begin(), near.end());
         }
     }
-    // flags of the nodes: the directions that bounce back there, and the domain's edges
-    std::vector<uint16_t> nflag(N, 0);
-    for (int y = 0; y < ny; y++)
-        for (int x = 0; x < nx; x++) {
-            const size_t i = (size_t)y * nx + x;
-            if (solid[i]) {
-                nflag[i] = (uint16_t)kNodeSolid;
-                continue;
-            }
-            int f = (x == 0 ? kNodeX0 : 0) | (x == nx - 1 ? kNodeXN : 0) | (y == 0 ? kNodeY0 : 0) |
-                    (y == ny - 1 ? kNodeYN : 0);
-            if (cls[i] == kFB)
-                for (int a = 1; a < kQ; a++) f |= S(x - ex(a), y - ey(a)) << a;
-            nflag[i] = (uint16_t)f;
-        }
     const int n_gen = (int)tg.size();
 
     // ---- parameters

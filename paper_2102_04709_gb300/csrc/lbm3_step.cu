@@ -1181,7 +1181,8 @@ __device__ __forceinline__ void wet_look(const Params& P, const TileSet& T, int 
             const double om = c[0].wm, ol = c[0].wl, oth = c[0].th;
             const float t_rg = T.wang[3 * w], t_x = T.wang[3 * w + (k == 0 ? 1 : 2)];
             if (!(same_number(om, wm) && same_number(ol, wl))) {
-                th = k == 0 ? local_angle(wm, 180.0 - t_x, wl, t_rg) : local_angle(wm, t_x, wl, 180.0 - t_rg);
+                const double a = 180.0 - (k == 0 ? t_x : t_rg);  // an angle seen from the other side
+                th = local_angle(wm, k == 0 ? a : (double)t_x, wl, k == 0 ? (double)t_rg : a);
                 c[0].wm = wm;
                 c[0].wl = wl;
                 // the same angle as when these lanes last marched: the same lines, the same crossings
