@@ -77,6 +77,9 @@ struct lbm3 {
     int pp = 0;
     cudaStream_t side = nullptr;
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    // chain: a small grid, every tile in one launch per step (kChainTiles); the records of the pure
+    // tiles then follow those of gen
+    bool chain = false;
     // one: the pure tiles with one fluid around are launch_step_one's (kOneTiles); those with
     // several run beside them on a third side stream
     bool one = false;
@@ -204,11 +207,21 @@ void release(lbm3* h)
 // From this many pure tiles on, the tiles with one fluid around are launch_step_one's, and the pure
 // ones with several run beside them on a stream of their own.  On smaller grids the fluids soon reach
 // every tile, the step waits for the tiles near solids, and two more launches cost more than they hide:
-// after 1500 steps the 512 x 512 cylinder (805 pure tiles) takes 25.5 us a step with them and 22.9
+// after 1500 steps the 512 x 512 cylinder (805 pure tiles) took 25.5 us a step with them and 22.9
 // without, the 800 x 375 pillars (865) 28.6 and 28.9, the 1030 x 517 ones (1571) 36 and 42, a
 // 1024 x 1024 cylinder (3700) 60 and 67.  LBM3_ONE_TILES=<n> in the environment at lbm3_create sets
 // another line (same results).
 constexpr int kOneTiles = 1200;
+
+// Tiles up to which a step is one launch of all of them (k_tile, two blocks per SM: four rounds of
+// blocks), one launch behind the other with no fork to the side streams and no join, and the start of a
+// step (its record, the geometry words) under the end of the one before (programmatic dependent launch).
+// Beyond, k_tile's time for a pure tile counts: us a step with the launches beside one another and with
+// one, after 300 and 1500 steps: 128 x 64 16.3 16.5 / 15.4 15.5, 450 x 31 18.1 18.2 / 16.7 17.0,
+// 2048 x 128 (1024 tiles) 17.3 19.2 / 16.8 17.3, the 512 x 512 cylinder (1024) 21.7 23.2 / 21.7 23.6, the
+// 800 x 375 pillars (1175) 23.4 29.3 / 21.5 25.0, the 1030 x 517 ones (2145) 27.4 36.1 / 36.8 44.9.
+// LBM3_CHAIN_TILES=<n> in the environment at lbm3_create sets another line (same results).
+constexpr int kChainTiles = 1200;
 
 // Tensor maps of one [27][ny][nx] FP32 population buffer: as the two parts of the pull-source box
 // of a pure tile, (kTX + 8) x (kTY + 6) x kTmaPlanesA and x (27 - kTmaPlanesA) planes, and as its
@@ -294,6 +307,14 @@ void record_timing(lbm3* h, cudaEvent_t ev, cudaStream_t s)
         cudaEventRecord(ev, s);
 }
 
+// polls of an mbarrier before a step kernel gives up on a tile's bulk copies (a completed copy
+// takes a few microseconds; this is seconds of polling)
+constexpr int kCopyWaitPolls = 1 << 22;
+
+// whether a step is one launch of every tile.  A lowered copy-wait limit is for the bulk copies of the
+// other launches.
+bool chained(const lbm3* h) { return h->chain && h->P.wait_polls == kCopyWaitPolls; }
+
 // One timestep: fork the side streams off the main stream, run the pure tiles on the main stream
 // (those with several fluids around on a side stream of their own where launch_step_one takes the
 // others) and the other tiles, with the wetting of their solid boundary nodes, on the
@@ -309,13 +330,25 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
     float* u = last ? h->u : nullptr;
     const uint64_t* pin = h->pres[h->pp];
     uint64_t* pout = h->pres[1 - h->pp];
+    if (chained(h)) {
+        // a small grid: every tile in one launch, one step behind the other on the main stream
+        for (int j = 0; ev && j < 4; j++) record_timing(h, ev[j], h->stream);
+        TileSet all = h->gen;
+        all.ntiles = h->n_gen + h->n_pure;
+        e = launch_tile(h->precision, h->P, all, fin, fo, cw_out, u, pin, pout, io, false, !ev, h->stream);
+        for (int j = 4; ev && j < 7; j++) record_timing(h, ev[j], h->stream);
+        if (!io) h->cur = 1 - h->cur;
+        h->pp = 1 - h->pp;
+        return e;
+    }
     if ((e = cudaEventRecord(h->ev_fork, h->stream)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) != cudaSuccess) return e;
     if (ev) record_timing(h, ev[2], h->side);
     if (ev) record_timing(h, ev[3], h->side);
     // steps between the adjoint's slots write every plane and wall value: the tiles all of theirs
     const bool light = h->one && !io;
-    launch_tile(h->precision, h->P, h->gen, fin, fo, cw_out, u, pin, pout, io, light, h->side);
+    e = launch_tile(h->precision, h->P, h->gen, fin, fo, cw_out, u, pin, pout, io, light, false, h->side);
+    if (e != cudaSuccess) return e;
     // (behind the tiles that take long: in front of them, or of the pure tiles on either stream, it delays
     // what the step waits for, 5-10 % on the 2048 x 1024 pillars)
     if (light) launch_step_one(h->precision, h->P, h->gen, nullptr, 0, fin, fo, u, pin, pout, false, h->side);
@@ -357,10 +390,6 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
 }
 
 constexpr int kGraphSteps = 8;
-// polls of an mbarrier before a step kernel gives up on a tile's bulk copies (a completed copy
-// takes a few microseconds; this is seconds of polling)
-constexpr int kCopyWaitPolls = 1 << 22;
-
 // Error bits that the kernels set (bit 0: a bulk tensor copy outlived its wait), read after the
 // stream has been synchronised and cleared once read, so that each timeout is reported once.
 int take_kernel_error(lbm3* h)
@@ -662,6 +691,17 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
         }
     }
     const int n_gen = (int)tg.size();
+    const char* chain_env = std::getenv("LBM3_CHAIN_TILES");
+    const bool chain = n_gen + (int)tp.size() <= (chain_env ? std::atoi(chain_env) : kChainTiles);
+    if (chain) {
+        // a pure tile's record: no C_SB node, the 3 x 3 tiles around (it is inner, so they exist)
+        const int ntx = (nx + kTX - 1) / kTX;
+        for (const int t : tp) {
+            rec.insert(rec.end(), {t, 0, 0});
+            for (int m = 0; m < kTileRecInts - kTileRecHead; m++)
+                rec.push_back(m < 9 ? 2 * (t + (m / 3 - 1) * ntx + m % 3 - 1) : -2);
+        }
+    }
 
     // ---- parameters
     lbm3* h = new lbm3();
@@ -698,6 +738,7 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
     h->n_fluid = n_fluid;
     h->n_pure = (int)tp.size();
     h->n_gen = n_gen;
+    h->chain = chain;
     h->n_went = (int)went.size();
     h->pure_fluid = pure_fluid;
     h->wall_host = widx;
@@ -1318,7 +1359,7 @@ int lbm3_info(const lbm3* h, int64_t out[9])
     // and 8 16-bit offsets (120 B); plus one class byte per node
     const long long per = h->precision == LBM3_FP32 ? 216 : 120;
     out[2] = h->n_fluid * per + h->P.N;
-    out[3] = (h->n_pure > 0) + h->one + (h->n_gen > 0);
+    out[3] = chained(h) ? 1 : (h->n_pure > 0) + 2 * h->one + (h->n_gen > 0);
     out[4] = 0;  // the wetting is part of the tiles' launch
     out[5] = (int64_t)h->bytes;
     // as if every node of the pure tiles held all three fluids

@@ -198,8 +198,9 @@ __device__ __forceinline__ void zou_he(const Params& P, float p[27], bool inlet)
     }
 }
 
-// Post-streaming populations of fluid k for the pull from a stored buffer.  (Plain loads: the kernel
-// that marches many steps in one launch writes what it read through the same pointers before.)
+// Post-streaming populations of fluid k for the pull from a stored buffer.  (Plain loads, not those for
+// data that nobody writes during a kernel: with programmatic dependent launch the step before still
+// writes the buffer while the first blocks of the next start.)
 template <int STORE>
 struct Store;
 
@@ -381,9 +382,11 @@ void launch_step_tma16(int store, const Params& P, const int* tiles, int ntiles,
 void launch_step_plain(int store, const Params& P, const int* tiles, int ntiles, const Pop& fin, const Pop& fout,
                        float* u, const uint64_t* pres_in, uint64_t* pres_out, bool all, cudaStream_t s);
 // tiles of any kind, one per block; cw_out: the wall values of this step (those of the last one are in
-// the cache's lines)
-void launch_tile(int store, const Params& P, const TileSet& T, const Pop& fin, const Pop& fout, double* cw_out, float* u,
-                 const uint64_t* pres_in, uint64_t* pres_out, bool full_write, bool one, cudaStream_t s);
+// the cache's lines); chain: the launch before on the stream is another such one, whose end this one's
+// blocks wait for themselves (programmatic dependent launch)
+cudaError_t launch_tile(int store, const Params& P, const TileSet& T, const Pop& fin, const Pop& fout, double* cw_out,
+                        float* u, const uint64_t* pres_in, uint64_t* pres_out, bool full_write, bool one, bool chain,
+                        cudaStream_t s);
 // the cache's lines from the wall values Cw, after those or the wall angles were replaced
 void launch_wet_look(const Params& P, const TileSet& T, int entries, const double* Cw, cudaStream_t s);
 void launch_init(int store, const Params& P, const double* rho, const uint8_t* type, const Pop& f,

@@ -1356,6 +1356,12 @@ __global__ void k_wet_init(const Params P, const int nw, const int* __restrict__
     }
 }
 
+// Programmatic dependent launch (nothing happens in a launch without it): let the next kernel of the
+// stream start its blocks where there is room; wait until the kernels before have ended and their
+// writes can be read.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Fluids stored in the tiles of a record (this lane's entry of the list: nbr), for the whole warp.
 __device__ __forceinline__ int fluids_reaching(const uint64_t* __restrict__ pres, int nbr)
 {
@@ -1428,7 +1434,9 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
     // tile's wall values have settled
     int around;
     uint64_t mine;
+    launch_dependents();
     if (one) {
+        wait_prerequisites();
         around = fluids_reaching(pres_in, nbr);
         mine = pres_in[tile];
         if (settled_single(around, cnt, mine)) return;  // k_step_one's
@@ -1443,6 +1451,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
     }
     if (tid == 0) S.wall = S.flags = 0;
     if (!one) {
+        wait_prerequisites();  // up to here nothing that a step writes was read
         around = fluids_reaching(pres_in, nbr);
         mine = pres_in[tile];
     }
@@ -2227,17 +2236,27 @@ void launch_step_plain(int store, const Params& P, const int* tiles, int ntiles,
         k_step_plain<kTX, kTY, kStoreBF16><<<ntiles, b, 0, s>>>(P, tiles, fin, fout, u, pres_in, pres_out, all);
 }
 
-void launch_tile(int store, const Params& P, const TileSet& T, const Pop& fin, const Pop& fout, double* cw_out, float* u,
-                 const uint64_t* pres_in, uint64_t* pres_out, bool full_write, bool one, cudaStream_t s)
+cudaError_t launch_tile(int store, const Params& P, const TileSet& T, const Pop& fin, const Pop& fout, double* cw_out,
+                        float* u, const uint64_t* pres_in, uint64_t* pres_out, bool full_write, bool one, bool chain,
+                        cudaStream_t s)
 {
-    if (T.ntiles <= 0) return;
-    const int nt = kTileThreads, fw = full_write ? 1 : 0;
-    if (store == kStoreF32)
-        k_tile<kTX, kTY, kStoreF32><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw, one);
-    else if (store == kStoreF16)
-        k_tile<kTX, kTY, kStoreF16><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw, one);
-    else
-        k_tile<kTX, kTY, kStoreBF16><<<T.ntiles, nt, 0, s>>>(P, T, fin, fout, cw_out, u, pres_in, pres_out, fw, one);
+    if (T.ntiles <= 0) return cudaSuccess;
+    const int fw = full_write ? 1 : 0, on = one ? 1 : 0;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(T.ntiles);
+    cfg.blockDim = dim3(kTileThreads);
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = chain ? 1 : 0;
+    auto go = [&](auto kernel) {
+        return cudaLaunchKernelEx(&cfg, kernel, P, T, fin, fout, cw_out, u, pres_in, pres_out, fw, on);
+    };
+    if (store == kStoreF32) return go(k_tile<kTX, kTY, kStoreF32>);
+    if (store == kStoreF16) return go(k_tile<kTX, kTY, kStoreF16>);
+    return go(k_tile<kTX, kTY, kStoreBF16>);
 }
 
 void launch_wet_look(const Params& P, const TileSet& T, int entries, const double* Cw, cudaStream_t s)

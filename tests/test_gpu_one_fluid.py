@@ -1,6 +1,6 @@
-"""Pure tiles with one fluid around (their own launch, which moves nine populations per node) against
-the launches that move all 27: the same bits, whichever takes a tile.  LBM3_ONE_TILES moves the
-line between the two at lbm3_create."""
+"""The launches that a tile can be done by: those for one fluid, which move nine populations per node,
+those that move all 27 by bulk copies or plain loads, and the one launch of all tiles: the same bits,
+whichever takes it.  LBM3_ONE_TILES, LBM3_DISABLE_TMA and LBM3_CHAIN_TILES choose at lbm3_create."""
 import numpy as np
 import pytest
 
@@ -20,39 +20,41 @@ def gpu():
     return lbm3
 
 
-def pair(gpu, monkeypatch, w, precision):
+def variants(gpu, monkeypatch, w, precision):
     sims = []
-    for line in ("1", "1000000000"):
-        monkeypatch.setenv("LBM3_ONE_TILES", line)
+    for one, chain, plain in (("1", "0", "0"), ("1000000000", "0", "0"), ("1000000000", "0", "1"), ("1", "1000000000", "0")):
+        monkeypatch.setenv("LBM3_ONE_TILES", one)
+        monkeypatch.setenv("LBM3_CHAIN_TILES", chain)
+        monkeypatch.setenv("LBM3_DISABLE_TMA", plain)
         sims.append(gpu.Lbm3.from_workload(w, precision=precision))
-    assert sims[0].info()["step_kernels"] == sims[1].info()["step_kernels"] + 1
+    assert [s.info()["step_kernels"] for s in sims] == [4, 2, 2, 1]
     return sims
 
 
-def same(a, b):
-    for x, y in zip(a.get_state() + a.fields(), b.get_state() + b.fields()):
-        assert np.array_equal(x, y, equal_nan=True)
-    assert np.array_equal(a.diag(check=False), b.diag(check=False), equal_nan=True)
+def same(a, *others):
+    x = a.get_state() + a.fields() + (a.diag(check=False),)
+    for b in others:
+        for p, q in zip(x, b.get_state() + b.fields() + (b.diag(check=False),)):
+            assert np.array_equal(p, q, equal_nan=True)
 
 
 # nx a multiple of 8 (bulk copies), of 4 (FP32 only) and odd (plain loads); a droplet that moves and
 # spreads over tiles that held one fluid before
 @pytest.mark.parametrize("precision", [0, 1, 2], ids=["fp32", "fp16", "bf16"])
 @pytest.mark.parametrize("nx,ny", [(320, 120), (324, 119), (319, 123)])
-def test_one_fluid_tiles_match_the_general_kernels(gpu, monkeypatch, precision, nx, ny):
+def test_every_launch_gives_the_same_bits(gpu, monkeypatch, precision, nx, ny):
     w = W.pillars(nx=nx, ny=ny, count=3, r_lo=6.0, r_hi=9.0, x_lo=150.0, x_hi=260.0, gap=8.0, seed=5,
                   drop=(60.0, 60.0), r_core=8.0, r_shell=14.0, u_in=0.05)
-    a, b = pair(gpu, monkeypatch, w, precision)
+    sims = variants(gpu, monkeypatch, w, precision)
     for n in (1, 2, 13, 60):  # odd and even counts: either buffer, single launches and graphs
-        a.step(n)
-        b.step(n)
-        same(a, b)
-    f, c = a.get_state()
-    a.set_state(f, c)
-    b.set_state(f, c)
-    a.step(11)
-    b.step(11)
-    same(a, b)
+        for s in sims:
+            s.step(n)
+        same(*sims)
+    f, c = sims[0].get_state()
+    for s in sims:
+        s.set_state(f, c)
+        s.step(11)
+    same(*sims)
 
 
 # a density without a fraction (0, infinite, NaN) in a region of one fluid spreads to the absent
@@ -61,16 +63,15 @@ def test_one_fluid_tiles_match_the_general_kernels(gpu, monkeypatch, precision, 
 @pytest.mark.parametrize("value", [0.0, np.inf, np.nan])
 def test_one_fluid_tiles_without_a_fraction(gpu, monkeypatch, precision, value):
     w = W.janus_cylinder(nx=256, ny=128, Rs=10.0, Rj=9.0)
-    a, b = pair(gpu, monkeypatch, w, precision)
-    a.step(20)
-    b.step(20)
-    f, c = a.get_state()
+    sims = variants(gpu, monkeypatch, w, precision)
+    for s in sims:
+        s.step(20)
+    f, c = sims[0].get_state()
     f[:, :, 30, 60] = 0.0
     f[1, :, 30, 60] = value
-    for s in (a, b):
-        s.set_state(f, c)
-        s.step(1)
-    same(a, b)
-    a.step(6)
-    b.step(6)
-    same(a, b)
+    for n in (1, 6):
+        for s in sims:
+            if n == 1:
+                s.set_state(f, c)
+            s.step(n)
+        same(*sims)
