@@ -501,6 +501,23 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
     long long n_fluid = 0;
     for (int y = 0; y < ny; y++)
         for (int x = 0; x < nx; x++) {
+            if (x > 0 && x < nx - 1 && y > 0 && y < ny - 1) {
+                // inside the domain: nine plain reads (with the boundaries' rules for each of them this
+                // loop was most of a set-up)
+                const uint8_t* m = solid + (size_t)y * nx + x;
+                const int me = m[0] != 0;
+                int flag = 0, others = 0;
+                for (int a = 1; a < kQ; a++) {
+                    const int other = m[ey(a) * nx + ex(a)] != 0;
+                    others += other;
+                    flag |= other << opp(a);  // what comes along opp(a) would come from there
+                }
+                const bool touch = others != (me ? kQ - 1 : 0);
+                nflag[(size_t)y * nx + x] = (uint16_t)(me ? kNodeSolid : flag);
+                cls[(size_t)y * nx + x] = me ? (touch ? kSB : kSI) : (touch ? kFB : kFI);
+                n_fluid += !me;
+                continue;
+            }
             const int me = S(x, y);
             bool touch = false;
             int flag = (x == 0 ? kNodeX0 : 0) | (x == nx - 1 ? kNodeXN : 0) | (y == 0 ? kNodeY0 : 0) |
@@ -511,7 +528,7 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
                                 "a fluid node touches a wall side: make the boundary rows/columns solid");
                 const int other = S(x + ex(a), y + ey(a));
                 if (other != me) touch = true;
-                flag |= other << opp(a);  // what comes along opp(a) would come from there
+                flag |= other << opp(a);
             }
             nflag[(size_t)y * nx + x] = (uint16_t)(me ? kNodeSolid : flag);
             cls[(size_t)y * nx + x] = me ? (touch ? kSB : kSI) : (touch ? kFB : kFI);
