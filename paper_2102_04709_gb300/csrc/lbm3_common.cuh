@@ -391,8 +391,8 @@ cudaError_t launch_tile(int store, const Params& P, const TileSet& T, const Pop&
 void launch_wet_look(const Params& P, const TileSet& T, int entries, const double* Cw, cudaStream_t s);
 void launch_init(int store, const Params& P, const double* rho, const uint8_t* type, const Pop& f,
                  cudaStream_t s);
-void launch_fields(int store, const Params& P, const Pop& f, const uint8_t* type, float* rho_out,
-                   cudaStream_t s);
+void launch_fields(int store, const Params& P, const Pop& f, const uint8_t* type, double* rho_out, cudaStream_t s);
+void launch_widen(long long n, const float* in, double* out, cudaStream_t s);
 void launch_get_state(int store, const Params& P, const Pop& f, const uint8_t* type, float* post,
                       cudaStream_t s);
 void launch_set_state(int store, const Params& P, const double* post, const uint8_t* type,

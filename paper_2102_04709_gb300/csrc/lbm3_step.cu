@@ -2057,9 +2057,9 @@ __global__ void k_init(const Params P, const double* __restrict__ rho,
     store_node<STORE>(f, P.N, i, v);
 }
 
+// post-streaming densities in double precision, as the caller gets them
 template <class S>
-__global__ void k_fields(const Params P, const S st, const uint8_t* __restrict__ type,
-                         float* __restrict__ rho_out)
+__global__ void k_fields(const Params P, const S st, const uint8_t* __restrict__ type, double* __restrict__ rho_out)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= P.N) return;
@@ -2073,7 +2073,14 @@ __global__ void k_fields(const Params P, const S st, const uint8_t* __restrict__
             for (int a = 0; a < kQ; a++) r[k] += p[9 * k + a];
     }
 #pragma unroll
-    for (int k = 0; k < kNF; k++) rho_out[(long long)k * P.N + i] = r[k];
+    for (int k = 0; k < kNF; k++) rho_out[(long long)k * P.N + i] = (double)r[k];
+}
+
+// n numbers in double precision
+__global__ void k_widen(const long long n, const float* __restrict__ in, double* __restrict__ out)
+{
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) out[i] = (double)in[i];
 }
 
 // post-streaming populations of every fluid node (0 at solid nodes)
@@ -2577,12 +2584,16 @@ void launch_init(int store, const Params& P, const double* rho, const uint8_t* t
         k_init<kStoreBF16><<<nb, 256, 0, s>>>(P, rho, type, f);
 }
 
-void launch_fields(int store, const Params& P, const Pop& f, const uint8_t* type, float* rho_out,
-                   cudaStream_t s)
+void launch_fields(int store, const Params& P, const Pop& f, const uint8_t* type, double* rho_out, cudaStream_t s)
 {
     with_store(store, f, P.N, [&](auto st) {
         k_fields<<<(unsigned)((P.N + 255) / 256), 256, 0, s>>>(P, st, type, rho_out);
     });
+}
+
+void launch_widen(long long n, const float* in, double* out, cudaStream_t s)
+{
+    k_widen<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(n, in, out);
 }
 
 void launch_get_state(int store, const Params& P, const Pop& f, const uint8_t* type, float* post,
