@@ -835,6 +835,8 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
     for (int b = 0; b < 2; b++)
         if (e == cudaSuccess) e = cudaMemset(h->cw[b], 0, 3 * N * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(h->u, 0, 2 * N * sizeof(float));
+    const char* one_env = std::getenv("LBM3_ONE_TILES");
+    const bool many = h->n_pure >= std::max(1, one_env ? std::atoi(one_env) : kOneTiles);
     // pure tiles through bulk tensor copies where the layout allows them (row pitch a multiple of
     // 16 bytes: nx % 4 == 0 for FP32 populations, nx % 8 == 0 for 16-bit offset planes);
     // LBM3_DISABLE_TMA=1 in the environment keeps the plain kernel
@@ -856,13 +858,15 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
                 ep = f32 ? step_tma_prepare() : step_tma16_prepare();
                 if (ep != cudaSuccess) cudaGetLastError();
             }
-            // SMs left free for the wall / edge tiles, which run on the side
-            // stream while the persistent pure-tile kernel holds its SMs: their share of the step's
-            // work, in units of a pure tile's SM time as measured on the 4096 x 2048 pillars (a
-            // wall or edge tile 1.8, the wetting pass 0.038 per C_SB node: 30 of 152 SMs there).
-            // LBM3_SPARE_SMS=<n> in the environment at lbm3_create sets the count instead.
+            // SMs left free for the other kernels of a step while the persistent pure-tile kernel holds
+            // its own.  Where k_step_one takes most of the pure tiles, half of them: us a step after 200
+            // and 4500 steps with 30, 60, 76 and 105 left, FP32 4096 x 2048 164 185 / 158 178 / 156 173 /
+            // 149 185, BF16 2048 x 1024 with 30 to 76 61 to 62, 83 to 87.  Where it takes them all, the
+            // other tiles' share of the step's work, in units of a pure tile's SM time (such a tile 1.8,
+            // 0.038 per C_SB node).  LBM3_SPARE_SMS=<n> in the environment at lbm3_create sets the count
+            // instead.
             const double wg = 1.8 * h->n_gen + 0.038 * h->nw;
-            int spare = std::min(sms / 2, (int)std::lround(sms * wg / (wg + h->n_pure)));
+            int spare = many ? sms / 2 : std::min(sms / 2, (int)std::lround(sms * wg / (wg + h->n_pure)));
             if (const char* ov = std::getenv("LBM3_SPARE_SMS"))
                 spare = std::max(0, std::min(sms - 1, std::atoi(ov)));
             h->tma_blocks = (f32 ? kTmaBlocksPerSm : kTma16BlocksPerSm) * (sms - spare);
@@ -887,9 +891,8 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
     h->tiles_pure = (const int*)h->tile_mem[3];
     {
         // the two-blocks-per-SM kernel takes every pure tile itself
-        const char* ov = std::getenv("LBM3_ONE_TILES");
         const bool tma_only = h->tma && g->precision == LBM3_FP32 && !h->ring;
-        h->one = !tma_only && h->n_pure >= std::max(1, ov ? std::atoi(ov) : kOneTiles);
+        h->one = !tma_only && many;
     }
     if (e != cudaSuccess) {
         const int code = e == cudaErrorMemoryAllocation ? LBM3_ERR_OOM : LBM3_ERR_CUDA;

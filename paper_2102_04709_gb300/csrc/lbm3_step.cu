@@ -412,18 +412,99 @@ __device__ __forceinline__ void stress_at(const Params& P, const int (*t)[HX], c
     pair_stress(P.sig12, c[1], c[2], gxk[1], gyk[1], gxk[2], gyk[2], rho2, Txx, Txy, Tyy);
 }
 
-// Fluids stored in the 3 x 3 tiles around a tile that lies inside the domain: the OR of its and its
-// neighbours' words (one byte per row of a tile, bit k: fluid k).
+// ---- what the words of the tiles say (one byte per row of 32 nodes) ----
+// Bits 0-2: the fluids that the row's nodes hold; 0 only where it has no fluid node.  Bits 3-4: 0, or
+// d + 1 where the row is calm in fluid d: every node's total populations are at least kCalmMin, its
+// density at most kCalmRho, and the share C of the two other fluids at most kCalmShare, in what is
+// stored.  (Bits 5-6 of byte 0: settled_steps.)
+//
+// Where everything that can reach a node within two links is calm in the same d, the other fluids stay
+// traces there: a pulled share is the mean of its sources' with the total populations as weights
+// (between 0 and kCalmShare; in the FP16 storage, where the traces' offsets round to 0 and the sources
+// keep w_a rho_k, at most 10 times that: 1.4 / (9 / 64)), so it is at most 2e-13 at every fluid node of
+// the phase-field region, and the wall values of the C_SB nodes there are compared with that.  A gradient
+// component of such a share is at most three times as large (the extrapolation beyond a C_SB node
+// doubles one value and subtracts another), those of C_d are rounding (1e-6) and come times a share in
+// G_kl, and |G_kl|^2 < 8e-25 for every pair: below kG2Eps, so the stress of Eq.(10) and the normals of
+// Eq.(13) are exact zeros.  What the recolouring splits is then C_k f alone, from the node's own
+// populations: no halo, no phase fields, no barriers.  Traces spread by a node a step and soon are
+// in most tiles (of the 512 x 512 cylinder in 95 % after 1000 steps, of which 5 % hold shares above
+// 1e-12): us a step after 1000 steps without and with this, 512 x 512 23.6 / 19.7, the 800 x 375
+// pillars 22.8 / 21.2 and after 6000 28.1 / 24.2; bf16 2048 x 1024 after 4500 105 / 87.
+constexpr float kCalmMin = 1.0f / 64.0f, kCalmRho = 1.4f, kCalmWall = 2e-13f;
+__host__ __device__ constexpr float calm_share(int store) { return store == kStoreF16 ? 1.9e-14f : 1.9e-13f; }
+
+// a node's part of the above: bits 3-5 the fluids with more than a trace, bit 6 not calm at all; f: the
+// total populations that are stored
+template <int STORE>
+__device__ __forceinline__ int calm_bits(const float f[kQ], float rho, float c0, float c1, float c2)
+{
+    const float m = fminf(fminf(fminf(fminf(f[0], f[1]), fminf(f[2], f[3])), fminf(fminf(f[4], f[5]), fminf(f[6], f[7]))), f[8]);
+    constexpr float T = calm_share(STORE);
+    return (fabsf(c0) > T ? 8 : 0) | (fabsf(c1) > T ? 16 : 0) | (fabsf(c2) > T ? 32 : 0) |
+           (m >= kCalmMin && rho <= kCalmRho ? 0 : 64);
+}
+__device__ __forceinline__ int present_bits(float r0, float r1, float r2)
+{
+    return (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0);
+}
+// the row's byte from the OR of its nodes' bits (a row without any density has NaNs in all planes)
+__device__ __forceinline__ uint8_t row_byte(int v)
+{
+    const int d = v >> 3 & 7;
+    if (v & 64) return (uint8_t)(v & 7 ? v & 7 : 7);
+    return (uint8_t)((v & 7) | (__popc(d) == 1 ? __ffs(d) << 3 : 0));
+}
+
+// the fluids that a tile holds
+__device__ __forceinline__ int word_fluids(uint64_t b)
+{
+    b |= b >> 32;
+    b |= b >> 16;
+    b |= b >> 8;
+    return (int)(b & 7u);
+}
+// d + 1 of the tile's first row with a fluid node (0: not calm)
+__device__ __forceinline__ int word_calm(uint64_t b)
+{
+    const uint64_t rows = (b | b >> 1 | b >> 2) & 0x0101010101010101ull;
+    return rows ? (int)(b >> (__ffsll((long long)rows) + 2) & 3u) : 0;
+}
+// whether every row with a fluid node is calm in fluid d1 - 1
+__device__ __forceinline__ bool word_calm_in(uint64_t b, int d1)
+{
+    const uint64_t rows = (b | b >> 1 | b >> 2) & 0x0101010101010101ull;
+    return d1 > 0 && !((b ^ 0x0808080808080808ull * (uint64_t)d1) & (rows << 3 | rows << 4));
+}
+
+// How a tile that lies inside the domain can be done, from the words of the 3 x 3 tiles around it:
+// the fluids stored there (bits 0-2), and bit 3 where all is calm in one fluid.
 __device__ __forceinline__ int fluids_around(const uint64_t* __restrict__ pres, int tile, int ntx)
 {
+    const int d1 = word_calm(pres[tile]);
     uint64_t nb = 0;
+    bool calm = true;
 #pragma unroll
-    for (int m = 0; m < 9; m++) nb |= pres[tile + (m / 3 - 1) * ntx + m % 3 - 1];
-    nb |= nb >> 32;
-    nb |= nb >> 16;
-    nb |= nb >> 8;
-    return (int)(nb & 7u);
+    for (int m = 0; m < 9; m++) {
+        const uint64_t b = pres[tile + (m / 3 - 1) * ntx + m % 3 - 1];
+        nb |= b;
+        calm = calm && word_calm_in(b, d1);
+    }
+    return word_fluids(nb) | (calm ? 8 : 0);
 }
+// the same, by a whole warp with one word per lane
+__device__ __forceinline__ int fluids_around_warp(const uint64_t* __restrict__ pres, int tile, int ntx, int lane)
+{
+    uint64_t b = 0;
+    if (lane < 9) b = pres[tile + (lane / 3 - 1) * ntx + lane % 3 - 1];
+    const int d1 = __shfl_sync(0xffffffffu, word_calm(b), 4);
+    const bool calm = __all_sync(0xffffffffu, lane >= 9 || word_calm_in(b, d1));
+    return __reduce_or_sync(0xffffffffu, word_fluids(b)) | (calm ? 8 : 0);
+}
+// one fluid: k_step_one's tiles
+__device__ __forceinline__ bool one_fluid(int around) { return __popc((unsigned)around & 7u) == 1; }
+// In the list of tiles of the kernels that move all 27 planes: the tile is calm, no gradients needed.
+constexpr int kCalmTile = 1 << 30;
 
 // Eq.(10) stress on the halo-1 region of a pure tile from the phase fields of its halo-2 region
 // (float path: no solid, no float-float words)
@@ -790,6 +871,39 @@ __device__ __forceinline__ bool collide_single(const Params& P, int k, float f[k
     return c == 1.0f;
 }
 
+// One node at which |G_kl| vanishes for every pair (see calm_bits), from its 9 post-streaming totals f
+// and densities: collide_node without force and normals, and the recolouring, to the planes of the
+// fluids in write.  Returns its bits for row_byte.
+template <int STORE>
+__device__ __forceinline__ int collide_calm(const Params& P, const Pop& fout, float* uout, int i, float f[kQ], float r0,
+                                            float r1, float r2, int write)
+{
+    const float rho = (r0 + r1) + r2;
+    const float c[kNF] = {fraction(r0, rho), fraction(r1, rho), fraction(r2, rho)};
+    const float D = (r0 * P.inv_nu0 + r1 * P.inv_nu1) + r2 * P.inv_nu2;
+    const float s1 = __fdividef(D, 0.5f * D + 3.0f);
+    float ux, uy;
+    collide_mrt_free(f, rho, s1, ux, uy);
+    if (uout) {
+        uout[i] = ux;
+        uout[P.N + i] = uy;
+    }
+#pragma unroll
+    for (int l = 0; l < kNF; l++)
+        if (write >> l & 1) store_fluid<STORE>(P, fout, l, i, f, c[l]);
+    return present_bits(r0, r1, r2) | calm_bits<STORE>(f, rho, c[0], c[1], c[2]);
+}
+
+// the bits of a recoloured node for row_byte (one that the recolouring shifts is not calm: its traces are
+// not C_k f)
+template <int STORE>
+__device__ __forceinline__ int recoloured_bits(const float f[kQ], float r0, float r1, float r2, const Recolour& rc)
+{
+    const bool shifts = rc.Vx[0] != 0.0f || rc.Vy[0] != 0.0f || rc.Vx[1] != 0.0f || rc.Vy[1] != 0.0f ||
+                        rc.Vx[2] != 0.0f || rc.Vy[2] != 0.0f;
+    return present_bits(r0, r1, r2) | calm_bits<STORE>(f, (r0 + r1) + r2, rc.C[0], rc.C[1], rc.C[2]) | (shifts ? 64 : 0);
+}
+
 // write the 27 recoloured post-collision populations of node i
 template <int STORE>
 __device__ __forceinline__ void store_recoloured(const Params& P, const Pop& out, int i, const float f[kQ],
@@ -854,7 +968,8 @@ __global__ void __launch_bounds__(TX* TY, 4) k_step_plain(const Params P, const 
     const int lx = threadIdx.x, ly = threadIdx.y, tid = lx + TX * ly;
     const int ntx = (P.nx + TX - 1) / TX;
     const int tile = tiles[blockIdx.x];
-    if (!all && __popc((unsigned)fluids_around(pres_in, tile, ntx)) == 1) return;
+    const int around = fluids_around_warp(pres_in, tile, ntx, tid & 31);
+    if (!all && one_fluid(around)) return;
     const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
     const int nx = P.nx;
     const int N = (int)P.N;
@@ -882,6 +997,17 @@ __global__ void __launch_bounds__(TX* TY, 4) k_step_plain(const Params P, const 
             }
         }
     };
+    if (around & 8) {
+        // all but one fluid as traces: the node's own populations are enough
+        float q[27], f[kQ];
+        pull(lx + 2, ly + 2, q);
+#pragma unroll
+        for (int a = 0; a < kQ; a++) f[a] = (q[a] + q[9 + a]) + q[18 + a];
+        const int v = collide_calm<STORE>(P, fout, uout, (y0 + ly) * nx + x0 + lx, f, sum9(q), sum9(q + 9), sum9(q + 18), 7);
+        const int w = __reduce_or_sync(0xffffffffu, v);
+        if (lx == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[ly] = row_byte(w);
+        return;
+    }
     // the lo words of float-float fields do not exist here
     float(*none)[CY][CX] = nullptr;
     int present = 0;
@@ -905,12 +1031,6 @@ __global__ void __launch_bounds__(TX* TY, 4) k_step_plain(const Params P, const 
         r1 = sum9(q + 9);
         r2 = sum9(q + 18);
     }
-    // the fluids this warp's nodes hold, for the tiles around this one in the next step
-    {
-        const int own = (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0);
-        const int w = __reduce_or_sync(0xffffffffu, own);
-        if (lx == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[ly] = (uint8_t)w;
-    }
     const bool mixed = single_fluid_or(present) != 1;
 
     if (mixed) stress_halo1<TX, TY>(P, s_ch, s_rho, s_txx, s_txy, s_tyy, tid);
@@ -930,6 +1050,9 @@ __global__ void __launch_bounds__(TX* TY, 4) k_step_plain(const Params P, const 
         uout[N + i] = uy;
     }
     store_recoloured<STORE>(P, fout, i, f, rc);
+    // what this warp's nodes hold, for the tiles around this one in the next step
+    const int w = __reduce_or_sync(0xffffffffu, recoloured_bits<STORE>(f, r0, r1, r2, rc));
+    if (lx == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[ly] = row_byte(w);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1220,11 +1343,12 @@ __device__ __forceinline__ void wet_look(const Params& P, const TileSet& T, int 
 // near several tiles is wetted by each of them, with the same result: 1.6 times the work of a pass
 // over the nodes, but no launch that the tiles have to wait for.  one: the fluids around; where that
 // is one, the nodes near the region hold it alone (C_k exactly 1 or 0) and need no pull.  Returns the
-// fluids with a nonzero wall value (bit k), in bit 3 whether some node's values are mixed, and in bit 4
-// whether a line ends in a node that is not near.
+// fluids with a nonzero wall value (bit k), in bit 3 whether some node's values are mixed, in bit 4
+// whether a line ends in a node that is not near, and in bit 5 whether some value of a fluid other than
+// calm - 1 is more than a trace.
 template <int TX, int TY, int STORE>
 __device__ __forceinline__ int wet_entries(const Params& P, const TileSet& T, int e0, int cnt, int one,
-                                           const Pop& fin, double* cw_out, TileShared<TX, TY>& S)
+                                           int calm, const Pop& fin, double* cw_out, TileShared<TX, TY>& S)
 {
     const long long N = P.N;
     const int tid = threadIdx.x;
@@ -1316,6 +1440,7 @@ __device__ __forceinline__ int wet_entries(const Params& P, const TileSet& T, in
                 S.ch[j][cy][cx] = h;
                 S.cl[j][cy][cx] = l;
                 if (!same_number(cc[j], 0.0)) bits |= 1 << j;
+                if (j + 1 != calm && !(h <= kCalmWall)) bits |= 32;
             }
             S.rho[cy][cx] = 1.0f;
             if (!pure && fmax(fmax(c0, c1), c2) < 1.0 - kMixEps) bits |= 8;
@@ -1362,33 +1487,35 @@ __global__ void k_wet_init(const Params P, const int nw, const int* __restrict__
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_prerequisites() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// Fluids stored in the tiles of a record (this lane's entry of the list: nbr), for the whole warp.
-__device__ __forceinline__ int fluids_reaching(const uint64_t* __restrict__ pres, int nbr)
+// fluids_around for the tiles of a record (this lane's entry of the list: nbr; own: the tile's word)
+__device__ __forceinline__ int fluids_reaching(const uint64_t* __restrict__ pres, int nbr, uint64_t own)
 {
     int around = nbr == -1 ? 7 : 0;  // an open column: any fluid
+    bool calm = nbr < -1;
     if (nbr >= 0) {
-        uint64_t b = pres[nbr >> 1];
-        b |= b >> 32;
-        b |= b >> 16;
-        b |= b >> 8;
-        const int v = (int)(b & 7u);
-        around = nbr & 1 ? (v & 2) | (v & 1) << 2 | v >> 2 : v;  // across the seam
+        const uint64_t b = pres[nbr >> 1];
+        const int v = word_fluids(b), d1 = word_calm(own);
+        const bool seam = nbr & 1;  // across it fluids 0 and 2 swap
+        around = seam ? (v & 2) | (v & 1) << 2 | v >> 2 : v;
+        calm = word_calm_in(b, seam && d1 > 0 ? 4 - d1 : d1);
     }
-    return __reduce_or_sync(0xffffffffu, around);
+    around = __reduce_or_sync(0xffffffffu, around);
+    return around | (__all_sync(0xffffffffu, calm) ? 8 : 0);
 }
 
-// The upper bits of a tile's word (byte 0: bits 4-5 a number of steps, at most 2, 6-7 a fluid k): for
-// how many steps the wall values of every C_SB node that the tile sees have been those of k alone,
-// with lines that end in nodes near it.  After two both arrays of wall values hold them, and while the
-// tiles around keep holding k alone nothing of the wetting changes.
+// Bits 5-6 of a tile's word (at most 2): for how many steps the wall values of every C_SB node that the
+// tile sees have been those of the one fluid around it alone, with lines that end in nodes near it.
+// After two both arrays of wall values hold them, and while the tiles around keep holding that fluid
+// alone nothing of the wetting changes.  (The tile itself is among those, and has a fluid node, so it
+// is the same fluid.)
 __device__ __forceinline__ int settled_steps(uint64_t word, int around)
 {
-    return __popc((unsigned)around) == 1 && (int)(word >> 6 & 3) == __ffs(around) - 1 ? (int)(word >> 4 & 3) : 0;
+    return __popc((unsigned)around & 7u) == 1 ? (int)(word >> 5 & 3) : 0;
 }
 // a tile that needs no wetting and holds one fluid after the pull: k_step_one's
 __device__ __forceinline__ bool settled_single(int around, int cnt, uint64_t word)
 {
-    return __popc((unsigned)around) == 1 && (cnt == 0 || settled_steps(word, around) == 2);
+    return __popc((unsigned)around & 7u) == 1 && (cnt == 0 || settled_steps(word, around) == 2);
 }
 
 // One step of tile T.rec[blockIdx.x] (any kind): thread t < TX TY has the tile's node t, the next ones a
@@ -1437,8 +1564,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
     launch_dependents();
     if (one) {
         wait_prerequisites();
-        around = fluids_reaching(pres_in, nbr);
         mine = pres_in[tile];
+        around = fluids_reaching(pres_in, nbr, mine);
         if (settled_single(around, cnt, mine)) return;  // k_step_one's
     }
     for (int j = tid; j < HX * HY; j += NT) {
@@ -1452,9 +1579,11 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
     if (tid == 0) S.wall = S.flags = 0;
     if (!one) {
         wait_prerequisites();  // up to here nothing that a step writes was read
-        around = fluids_reaching(pres_in, nbr);
         mine = pres_in[tile];
+        around = fluids_reaching(pres_in, nbr, mine);
     }
+    bool calm = around & 8;
+    around &= 7;
     const bool inside = tid < NOWN;  // a node of the tile itself, row tid / 32 (one warp)
     uint8_t* const word = reinterpret_cast<uint8_t*>(pres_out + tile) + (tid >> 5);
     const int old = !inside || full_write ? 7 : *word & 7;  // what this row of the output buffer still holds
@@ -1481,11 +1610,12 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
     int wp = 0;
     if (cnt > 0) {
         const int b = __reduce_or_sync(
-            0xffffffffu, wet_entries<TX, TY, STORE>(P, T, e0, cnt, around, fin, cw_out, S));
+            0xffffffffu, wet_entries<TX, TY, STORE>(P, T, e0, cnt, around, word_calm(mine), fin, cw_out, S));
         if (lane == 0 && b) atomicOr(&S.wall, b);
         __syncthreads();
         df = S.wall & 8;
         wp = S.wall & 7;
+        calm = calm && !(S.wall & 40);
     }
     // steps in a row in which one fluid was around and every wall value and line was that fluid's
     const int quiet = cnt > 0 && S.wall == around ? min(settled_steps(mine, around) + 1, 2) : 0;
@@ -1528,7 +1658,38 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
             }
         }
         const unsigned some = __ballot_sync(0xffffffffu, own_fluid);
-        if (lane == 0) *word = (uint8_t)((some ? (all ? 1 << k : 7) : 0) | (tid == 0 ? quiet << 4 | k << 6 : 0));
+        const bool still = __all_sync(0xffffffffu, !own_fluid || (calm_bits<STORE>(f, r, 0.0f, 0.0f, 0.0f) == 0));
+        if (lane == 0)
+            *word = (uint8_t)((some ? (all ? 1 << k | (still ? (k + 1) << 3 : 0) : 7) : 0) | (tid == 0 ? quiet << 5 : 0));
+        return;
+    }
+    if (calm) {
+        // ---- several fluids, all but one as traces: no gradients (calm_bits) ----
+        if (!inside) return;
+        int bits = 0;
+        if (own_fluid) {
+            float f[kQ], r[kNF] = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+            for (int a = 0; a < kQ; a++) f[a] = 0.0f;
+#pragma unroll
+            for (int k = 0; k < kNF; k++) {
+                if (!(around >> k & 1)) continue;
+                float q[kQ];
+#pragma unroll
+                for (int a = 0; a < kQ; a++) {
+                    const int g = S.geo[hy - ey(a)][hx - ex(a)];
+                    const bool bb = g & kGeoSolid;
+                    const int s = bb ? own : g;
+                    load_fluid<STORE>(P, fin, s & kGeoIdx, bb ? opp(a) : a, (s & kGeoPar) && k != 1 ? 2 - k : k, q[a]);
+                }
+                r[k] = sum9(q);
+#pragma unroll
+                for (int a = 0; a < kQ; a++) f[a] = f[a] + q[a];
+            }
+            bits = collide_calm<STORE>(P, fout, uout, own & kGeoIdx, f, r[0], r[1], r[2], old | around);
+        }
+        const int v = __reduce_or_sync(0xffffffffu, bits);
+        if (lane == 0) *word = row_byte(v);
         return;
     }
 
@@ -1578,10 +1739,6 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
         S.rho[cy][cx] = 0.0f;
     }
     {
-        // the fluids this row's fluid nodes hold, for the tiles around in the next step
-        const int b = own_fluid ? (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0) : 0;
-        const int w = __reduce_or_sync(0xffffffffu, b);
-        if (inside && lane == 0) *word = (uint8_t)w;
         const int pw = __reduce_or_sync(0xffffffffu, present);
         if (lane == 0 && pw) atomicOr(&S.flags, pw);
     }
@@ -1614,6 +1771,8 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
         if (own_fluid) div_stress<RX>(S.txx, S.txy, S.tyy, cx - 1, cy - 1, Fx, Fy);
     }
     // ---- velocity, MRT collision with forcing, recolouring, stores ----
+    if (!inside) return;
+    int bits = 0;
     if (own_fluid) {
         const int i = own & kGeoIdx;
         float ux, uy;
@@ -1623,7 +1782,11 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
             uout[N + i] = uy;
         }
         store_recoloured<STORE>(P, fout, i, f, rc);
+        bits = recoloured_bits<STORE>(f, r0, r1, r2, rc);
     }
+    // what this row's fluid nodes hold, for the tiles around in the next step
+    const int v = __reduce_or_sync(0xffffffffu, bits);
+    if (lane == 0) *word = row_byte(v);
 }
 
 // Pure tiles around which the step's input holds one fluid k (pres_in): k alone is in the tile
@@ -1671,13 +1834,7 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
         // then addresses the planes by uniform registers
         tile = __reduce_or_sync(0xffffffffu, tiles[w]);
         int v = 0;
-        if (lane < 9) {
-            uint64_t b = pres_in[tile + (lane / 3 - 1) * ntx + lane % 3 - 1];
-            b |= b >> 32;
-            b |= b >> 16;
-            b |= b >> 8;
-            v = (int)(b & 7u);
-        }
+        if (lane < 9) v = word_fluids(pres_in[tile + (lane / 3 - 1) * ntx + lane % 3 - 1]);
         around = __reduce_or_sync(0xffffffffu, v);
         if (__popc((unsigned)around) != 1) return;
     } else {
@@ -1685,9 +1842,9 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
         tile = __shfl_sync(0xffffffffu, r, 0);
         const int cnt = __shfl_sync(0xffffffffu, r, 2);
         const uint64_t mine = pres_in[tile];
-        around = fluids_reaching(pres_in, lane >= kTileRecHead ? r : -2);
+        around = fluids_reaching(pres_in, lane >= kTileRecHead ? r : kNoTile, mine) & 7;
         if (!settled_single(around, cnt, mine)) return;
-        word = mine & 0xf0;  // settled it stays
+        word = mine & 0x60;  // settled it stays
     }
     if (!PURE && row0 >= P.ny - (tile / ntx) * TY) {
         if (lane == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[row0] = 0;
@@ -1746,16 +1903,18 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
             }
         }
         float r = 1.0f, ux = 0.0f, uy = 0.0f;
-        bool plain = true;
+        bool plain = true, still = true;
         if (fluid) {
             r = sum9(f);
             plain = collide_single(P, k, f, r, ux, uy);
+            still = calm_bits<STORE>(f, r, 0.0f, 0.0f, 0.0f) == 0;
             if (uout) {
                 uout[i] = ux;
                 uout[N + i] = uy;
             }
         }
         const bool all = __all_sync(0xffffffffu, plain);
+        still = __all_sync(0xffffffffu, still);
         const int rowold = (int)(old >> (8 * row)) & 7;
         // fluids to write: k, and those that this row of the buffer still holds, as zeros; all of
         // them where a density has no fraction
@@ -1779,7 +1938,7 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
             }
         }
         const bool some = PURE || __ballot_sync(0xffffffffu, fluid);
-        const int byte = some ? (all ? 1 << k : 7) : 0;
+        const int byte = some ? (all ? 1 << k | (still ? (k + 1) << 3 : 0) : 7) : 0;
         if constexpr (RW == TY)
             word |= (uint64_t)byte << (8 * row);
         else if (lane == 0)
@@ -1864,16 +2023,18 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
                 return true;
             }
             mbar_arrive_expect_tx(full, (uint32_t)NBOX * 4u);
-            tma_load_3d(smem_u32(ring + b * NBOXP), &tm_in, (tile % ntx) * TX - 4, (tile / ntx) * TY - 3, 0, full);
+            const int t = tile & (kCalmTile - 1);
+            tma_load_3d(smem_u32(ring + b * NBOXP), &tm_in, (t % ntx) * TX - 4, (t / ntx) * TY - 3, 0, full);
             return true;
         };
         int issued = 0;
         bool ok = true;
         for (int base = 0; base < njobs && ok; base += 32) {
             const int mine = base + lane < njobs ? tiles[blockIdx.x + (base + lane) * gridDim.x] : -1;
-            const bool multi = mine >= 0 && (all || __popc((unsigned)fluids_around(pres_in, mine, ntx)) != 1);
+            const int around = mine >= 0 ? fluids_around(pres_in, mine, ntx) : 0;
+            const bool multi = mine >= 0 && (all || !one_fluid(around));
             for (unsigned todo = __ballot_sync(0xffffffffu, multi); todo && ok; todo &= todo - 1) {
-                const int tile = __shfl_sync(0xffffffffu, mine, __ffs(todo) - 1);
+                const int tile = __shfl_sync(0xffffffffu, around & 8 ? mine | kCalmTile : mine, __ffs(todo) - 1);
                 if (lane == 0) ok = send(tile, issued);
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 issued += ok;
@@ -1934,7 +2095,8 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
         return (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0);
     };
 
-    for (int j = g, jj = 0;; j += 2, jj++) {
+    int jj = 0;  // tiles so far that used the flags
+    for (int j = g;; j += 2) {
         const float* box = ring + (j % kRingBufs) * NBOXP;
         {
             bool ok = false;
@@ -1946,8 +2108,10 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
                 return;
             }
         }
-        const int tile = s_tile[j % (2 * kRingBufs)];
-        if (tile < 0) return;
+        const int job = s_tile[j % (2 * kRingBufs)];
+        if (job < 0) return;
+        const bool calm = job & kCalmTile;
+        const int tile = job & (kCalmTile - 1);
         const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
         // ---- phase 1: pulls, densities and phase fields of the halo-2 region ----
         auto pull = [&](int cx, int cy, float q[27]) {
@@ -1959,7 +2123,7 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
         };
         int present = 0;
         float q[27];
-        if (ring_node) {
+        if (ring_node && !calm) {
             pull(rcx, rcy, q);
             const float a0 = ((q[0] + (q[1] + q[3])) + (q[2] + q[4])) + ((q[5] + q[7]) + (q[6] + q[8]));
             const float a1 = ((q[9] + (q[10] + q[12])) + (q[11] + q[13])) + ((q[14] + q[16]) + (q[15] + q[17]));
@@ -1976,11 +2140,14 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
         r0 = ((q[0] + (q[1] + q[3])) + (q[2] + q[4])) + ((q[5] + q[7]) + (q[6] + q[8]));
         r1 = ((q[9] + (q[10] + q[12])) + (q[11] + q[13])) + ((q[14] + q[16]) + (q[15] + q[17]));
         r2 = ((q[18] + (q[19] + q[21])) + (q[20] + q[22])) + ((q[23] + q[25]) + (q[24] + q[26]));
-        // the fluids this warp's nodes hold, for the tiles around this one in the next step
-        {
-            const int own = (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0);
-            const int w = __reduce_or_sync(0xffffffffu, own);
-            if (lane == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = (uint8_t)w;
+        if (calm) {
+            // all but one fluid as traces: no gradients.  (No barrier until the next tile's, which may write
+            // the phase fields: nobody reads them here.)
+            const int v = collide_calm<kStoreF32>(P, Pop{fout, nullptr, nullptr}, uout, (y0 + ly) * P.nx + x0 + lx, f, r0,
+                                                  r1, r2, 7);
+            const int w = __reduce_or_sync(0xffffffffu, v);
+            if (lane == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = row_byte(w);
+            continue;
         }
         present |= store_phase(lx + 2, ly + 2, r0, r1, r2);
         // fluids present in the group's phase-field region (one barrier; see fluids_present)
@@ -1992,6 +2159,7 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
             const int v = flags[jj & 1];
             if (tid == 0) flags[(jj + 1) & 1] = 0;
             cnt = __popc(v & 7);
+            jj++;
         }
         const bool mixed = cnt != 1;
 
@@ -2020,6 +2188,9 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
             for (int a = 0; a < kQ; a++)
                 o[P.off_plane[k * kQ + a]] =
                     rc.C[k] * f[a] + wq(a) * (rc.Vx[k] * (float)ex(a) + rc.Vy[k] * (float)ey(a));
+        // what this warp's nodes hold, for the tiles around this one in the next step
+        const int w = __reduce_or_sync(0xffffffffu, recoloured_bits<kStoreF32>(f, r0, r1, r2, rc));
+        if (lane == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = row_byte(w);
         // the next tile's phase fields overwrite ch / rh only after its own barriers; the stress
         // arrays after its phase-1 barrier, by which time every thread here has read them
     }
@@ -2365,7 +2536,8 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
     // k_step_one's, the others are listed
     for (int base = 0; base < mine; base += NT) {
         const int cand = base + tid < mine ? tiles[blockIdx.x + (base + tid) * gridDim.x] : -1;
-        const bool multi = cand >= 0 && (all || __popc((unsigned)fluids_around(pres_in, cand, ntx)) != 1);
+        const int around = cand >= 0 ? fluids_around(pres_in, cand, ntx) : 0;
+        const bool multi = cand >= 0 && (all || !one_fluid(around));
         const unsigned votes = __ballot_sync(0xffffffffu, multi);
         if ((tid & 31) == 0) s_wn[tid >> 5] = __popc(votes);
         __syncthreads();  // the counts, and every thread is past the last batch's list
@@ -2374,15 +2546,16 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
             if (w < (tid >> 5)) pos += s_wn[w];
             count += s_wn[w];
         }
-        if (multi) s_list[pos] = cand;
+        if (multi) s_list[pos] = around & 8 ? cand | kCalmTile : cand;
         __syncthreads();
         if (tid == 0 && count > 0) {
-            issue(s_list[0]);
+            issue(s_list[0] & (kCalmTile - 1));
             last = j;
         }
         for (int m = 0; m < count; m++, j++) {
             const bool more = m + 1 < count;
-            const int tile = s_list[m];
+            const bool calm = s_list[m] & kCalmTile;
+            const int tile = s_list[m] & (kCalmTile - 1);
             const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
             bool ok = false;
             for (int it = 0; it < P.wait_polls && !ok; it++) ok = mbar_try_wait(bar, j & 1);
@@ -2401,7 +2574,7 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
             int present = 0;
             {
                 constexpr int NRING = CX * CY - TX * TY;
-                for (int r = tid; r < NRING; r += NT) {
+                for (int r = tid; r < NRING && !calm; r += NT) {
                     int cx, cy;
                     if (r < 2 * CX) {
                         cx = r % CX;
@@ -2424,24 +2597,26 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
             {
                 float q[27];
                 pull(lx + 2, ly + 2, q);
-                present |= store_phase(lx + 2, ly + 2, q);
+                if (!calm) present |= store_phase(lx + 2, ly + 2, q);
 #pragma unroll
                 for (int a = 0; a < kQ; a++) f[a] = (q[a] + q[9 + a]) + q[18 + a];
                 r0 = ((q[0] + (q[1] + q[3])) + (q[2] + q[4])) + ((q[5] + q[7]) + (q[6] + q[8]));
                 r1 = ((q[9] + (q[10] + q[12])) + (q[11] + q[13])) + ((q[14] + q[16]) + (q[15] + q[17]));
                 r2 = ((q[18] + (q[19] + q[21])) + (q[20] + q[22])) + ((q[23] + q[25]) + (q[24] + q[26]));
             }
-            // the fluids this warp's nodes hold, for the tiles around this one in the next step
-            {
-                const int own = (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0);
-                const int w = __reduce_or_sync(0xffffffffu, own);
-                if ((tid & 31) == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = (uint8_t)w;
-            }
             const bool mixed = fluids_present(present, s_flags, j, tid) != 1;
             // the boxes are free: fetch the next tile's while this one computes
             if (tid == 0 && more) {
-                issue(s_list[m + 1]);
+                issue(s_list[m + 1] & (kCalmTile - 1));
                 last = j + 1;
+            }
+
+            const int i = (y0 + ly) * P.nx + x0 + lx;
+            if (calm) {
+                // all but one fluid as traces: no gradients
+                const int w = __reduce_or_sync(0xffffffffu, collide_calm<STORE>(P, fout, uout, i, f, r0, r1, r2, 7));
+                if ((tid & 31) == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = row_byte(w);
+                continue;
             }
 
             // ---- phase 2: stress tensor of Eq.(10) on the halo-1 region ----
@@ -2457,7 +2632,6 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
             }
             float ux, uy;
             const Recolour rc = collide_node(P, f, r0, r1, r2, Fx, Fy, g, ux, uy);
-            const int i = (y0 + ly) * P.nx + x0 + lx;
             if (uout) {
                 uout[i] = ux;
                 uout[P.N + i] = uy;
@@ -2469,6 +2643,9 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
                 for (int a = 0; a < kQ; a++)
                     v[9 * k + a] = rc.C[k] * f[a] + wq(a) * (rc.Vx[k] * (float)ex(a) + rc.Vy[k] * (float)ey(a));
             store_node<STORE>(fout, P.N, i, v);
+            // what this warp's nodes hold, for the tiles around this one in the next step
+            const int w = __reduce_or_sync(0xffffffffu, recoloured_bits<STORE>(f, r0, r1, r2, rc));
+            if ((tid & 31) == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = row_byte(w);
         }
     }
 }

@@ -75,3 +75,25 @@ def test_one_fluid_tiles_without_a_fraction(gpu, monkeypatch, precision, value):
                 s.set_state(f, c)
             s.step(n)
         same(*sims)
+
+
+# tiles with only traces of all fluids but one take no gradients: the same bits as with them, which every
+# tile takes in the step after a set_state; pillars among the traces, in every launch that has both ways
+@pytest.mark.parametrize("nx,ny,chain", [(320, 120, "1000000000"), (320, 120, "0"), (319, 123, "0")],
+                         ids=["one-launch", "ring", "plain"])
+def test_traces_match_the_general_way(gpu, monkeypatch, nx, ny, chain):
+    w = W.pillars(nx=nx, ny=ny, count=6, r_lo=5.0, r_hi=8.0, x_lo=110.0, x_hi=280.0, gap=8.0, seed=5,
+                  drop=(60.0, 60.0), r_core=8.0, r_shell=14.0, u_in=0.02)
+    monkeypatch.setenv("LBM3_ONE_TILES", "1")
+    monkeypatch.setenv("LBM3_CHAIN_TILES", chain)
+    a = gpu.Lbm3.from_workload(w)
+    b = gpu.Lbm3.from_workload(w)
+    a.step(150)
+    r = np.abs(a.fields()[0])
+    assert np.count_nonzero((r > 0) & (r < 1e-13)) > nx * ny // 4  # there are traces, and over many tiles
+    b.set_state(*a.get_state())
+    for _ in range(40):
+        b.set_state(*b.get_state())
+        a.step(1)
+        b.step(1)
+    same(a, b)
