@@ -32,6 +32,7 @@ struct AdjLine {
 
 struct Adj {
     int nxp;  // nx + 2
+    const uint16_t* nflag;  // [N] flags of the nodes (kNodeX0 ...)
     // forward intermediates
     float* fpost;  // [27][N]
     float* C;      // [3][NP]
@@ -63,6 +64,17 @@ struct Adj {
 };
 
 __device__ __forceinline__ int pad(const Adj& A, int x, int y) { return y * A.nxp + x + 1; }
+
+// a fluid node inside the domain with fluid nodes all around: its neighbours are where the plain
+// offsets say, and no class has to be looked up (a load and a dependent one per direction).  With that,
+// and the lanes of a_wet doubled, a step of the 512 x 256 sweep takes 70.7 us instead of 81.4, of the
+// 250 x 125 one 58.5 instead of 67.1.  (Measured and left out: A1 and A2 in one launch and B3b in
+// B4's, 73.1; A2 on a stream of its own with the wall values from the stored states, 75.5; all in one
+// stream, 88, with programmatic dependent launch 98.)
+__device__ __forceinline__ bool plain_node(int fl)
+{
+    return !(fl & (0x1fe | kNodeX0 | kNodeXN | kNodeY0 | kNodeYN | kNodeSolid));
+}
 
 // The lattice position (X, Y), unwrapped, brought into the domain in place, as locate() does but
 // without dividing its index back into coordinates: 0 inside, 1 solid beyond a wall side (X, Y
@@ -133,8 +145,7 @@ __global__ void a_dens(const Params P, const Adj A, const float* __restrict__ fs
         return;
     }
     float q[27];
-    const Store<kStoreF32> st(fs, P.N);
-    pull_global(P, st, type, x, y, q);
+    pull_node<kStoreF32>(P, Pop{const_cast<float*>(fs), nullptr, nullptr}, i, (int)A.nflag[i], q);
     float r[kNF];
     for (int k = 0; k < kNF; k++) {
         float s = 0.f;
@@ -148,20 +159,26 @@ __global__ void a_dens(const Params P, const Adj A, const float* __restrict__ fs
         for (int j = 0; j < 27; j++) A.fpost[(long long)j * P.N + i] = q[j];
 }
 
-// A2: wetting with its decisions, 4 lanes per C_SB node (the same values as the step's)
+// A2: wetting with its decisions (the same values as the step's), 8 lanes per C_SB node -- lane =
+// 4 k + 2 side + end -- of which two pull the two nodes that bracket a crossing.  What bounds it is the
+// chain of the line, a pull's loads and the combination; with four lanes that pulled both nodes in turn,
+// class by class, it took 23.6 us at 512 x 256 (now 14.5), half of the intermediates' time.
 __global__ void a_wet(const Params P, const Adj A, int nw, const int* __restrict__ widx,
                       const double* __restrict__ wnrm, const float* __restrict__ wang,
                       const float* __restrict__ fs, const uint8_t* __restrict__ type,
                       const double* __restrict__ cw_lag)
 {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    const int w = g >> 2, lane = g & 3;
+    const int g8 = blockIdx.x * blockDim.x + threadIdx.x;
+    const int w = g8 >> 3, lane = g8 >> 1 & 3, end = g8 & 1, g = g8 >> 1;
     const int k = lane >> 1, side = lane & 1;
     const bool valid = w < nw;
     const Store<kStoreF32> st(fs, P.N);
     int i = 0, px = 0, py = 0;
     double th = 90.0, dfr = 0.0;
     Crossing cr{0, 0, 0, 0, 0, 0.0};
+    AdjLine c{};
+    if (valid) c = A.wline[g];
+    __syncwarp();  // read by both ends before one of them writes it
     if (valid) {
         i = widx[w];
         px = i % P.nx;
@@ -169,7 +186,6 @@ __global__ void a_wet(const Params P, const Adj A, int nw, const int* __restrict
         const double Cr = cw_lag[i], Cg = cw_lag[P.N + i], Cb = cw_lag[2 * P.N + i];
         const double t_rg = wang[3 * w], t_br = wang[3 * w + 1], t_gb = wang[3 * w + 2];
         th = k == 0 ? local_angle(Cb, 180.0 - t_br, Cg, t_rg) : local_angle(Cb, t_gb, Cr, 180.0 - t_rg);
-        const AdjLine c = A.wline[g];
         if (c.th == th) {
             cr = Crossing{c.kind, c.ax, c.ay, c.bx, c.by, c.fr};
             dfr = c.dfr;
@@ -192,21 +208,27 @@ __global__ void a_wet(const Params P, const Adj A, int nw, const int* __restrict
                     ds = (double)(cr.ay - py) * (ddx * dy - dx * ddy) / (dy * dy);
                 dfr = ds * (90.0 - th > 0 ? -1.0 : 1.0) * (M_PI / 180.0);
             }
-            A.wline[g] = AdjLine{th, cr.fr, dfr, cr.kind, cr.ax, cr.ay, cr.bx, cr.by, 0};
+            // (both ends found the same line)
+            if (end == 0) A.wline[g] = AdjLine{th, cr.fr, dfr, cr.kind, cr.ax, cr.ay, cr.bx, cr.by, 0};
         }
     }
-    double ca = 0.0, cb = 0.0;
-    if (valid && cr.kind >= 1) ca = node_C(P, st, type, cr.ax, cr.ay, k);
-    if (valid && cr.kind == 2) cb = node_C(P, st, type, cr.bx, cr.by, k);
-    if (valid && cr.kind == 0) ca = neighbour_mean(P, st, type, px, py, k);
+    double v = 0.0;
+    if (valid && cr.kind == 0 && end == 0) v = neighbour_mean(P, st, type, px, py, k);
+    if (valid && (end ? cr.kind == 2 : cr.kind >= 1)) {
+        int idx, fl;
+        wet_node(P, A.nflag, end ? cr.bx : cr.ax, end ? cr.by : cr.ay, idx, fl);
+        v = wet_fraction<kStoreF32>(P, Pop{const_cast<float*>(fs), nullptr, nullptr}, idx, fl, k);
+    }
+    const double o = __shfl_xor_sync(0xffffffffu, v, 1);
+    const double ca = end ? o : v, cb = end ? v : o;
     const double cd = cr.kind == 2 ? ca + cr.fr * (cb - ca) : ca;
-    const double other = __shfl_xor_sync(0xffffffffu, cd, 1);
+    const double other = __shfl_xor_sync(0xffffffffu, cd, 2);
     const bool takes_max = th <= 90.0;
     const double cp = takes_max ? fmax(cd, other) : fmin(cd, other);
     // the chosen side (ties: side 0)
     const int sel = (takes_max ? (cd > other || (cd == other && side == 0)) : (cd < other || (cd == other && side == 0))) ? side : 1 - side;
-    const double cg = __shfl_xor_sync(0xffffffffu, cp, 2);
-    if (valid) {
+    const double cg = __shfl_xor_sync(0xffffffffu, cp, 4);
+    if (valid && end == 0) {
         const int j = lane * nw + w;
         A.wkind[j] = cr.kind;
         int kk;
@@ -300,10 +322,17 @@ __global__ void a_grad_stress(const Params P, const Adj A, const uint8_t* __rest
     const int p = pad(A, gx, y);
     float c[kNF], gxk[kNF], gyk[kNF], m[kQ];
     int src[kQ], src2[kQ];
-    stencil_geom(P, A, type, gx, y, cls, src, src2, m);
+    const bool plain = gx >= 0 && gx < P.nx && plain_node((int)A.nflag[y * P.nx + gx]);
+    if (!plain) stencil_geom(P, A, type, gx, y, cls, src, src2, m);
     for (int k = 0; k < kNF; k++) {
         float v[kQ];
-        stencil_C(P, A, k, src, src2, m, v);
+        if (plain) {
+            const float* Ck = A.C + k * NP + p;
+#pragma unroll
+            for (int a = 0; a < kQ; a++) v[a] = Ck[ey(a) * A.nxp + ex(a)];
+        } else {
+            stencil_C(P, A, k, src, src2, m, v);
+        }
         c[k] = v[0];
         gxk[k] = (1.0f / 3.0f) * (v[1] - v[3]) + (1.0f / 12.0f) * ((v[5] - v[7]) + (v[8] - v[6]));
         gyk[k] = (1.0f / 3.0f) * (v[2] - v[4]) + (1.0f / 12.0f) * ((v[5] - v[7]) + (v[6] - v[8]));
@@ -330,8 +359,11 @@ __global__ void a_force(const Params P, const Adj A, const uint8_t* __restrict__
     if (type[i] & 2) return;
     const int NP = P.ny * A.nxp;
     float Fx = 0.f, Fy = 0.f;
+    const bool plain = plain_node((int)A.nflag[i]);
+    const int p = pad(A, x, y);
+#pragma unroll
     for (int a = 1; a < kQ; a++) {
-        const int q = tpos(P, A, x + ex(a), y + ey(a));
+        const int q = plain ? p + ey(a) * A.nxp + ex(a) : tpos(P, A, x + ex(a), y + ey(a));
         const float c = 3.0f * wq(a);
         Fx += c * (A.T[q] * ex(a) + A.T[NP + q] * ey(a));
         Fy += c * (A.T[NP + q] * ex(a) + A.T[2 * NP + q] * ey(a));
@@ -546,7 +578,17 @@ __device__ __forceinline__ void div_adjoint(const Params& P, const Adj& A, const
                                             int y, int p, float lT[3])
 {
     float lxx = 0.f, lxy = 0.f, lyy = 0.f;
-    for (int a = 1; a < kQ; a++) {
+    const bool plain = gx >= 0 && gx < P.nx && plain_node((int)A.nflag[y * P.nx + gx]);
+#pragma unroll
+    for (int a = 1; a < kQ && plain; a++) {
+        const int qi = (y - ey(a)) * P.nx + gx - ex(a);
+        const float c = 3.0f * wq(a);
+        const float lFx = A.l_F[qi], lFy = A.l_F[P.N + qi];
+        lxx += c * ex(a) * lFx;
+        lxy += c * (ey(a) * lFx + ex(a) * lFy);
+        lyy += c * ey(a) * lFy;
+    }
+    for (int a = 1; a < kQ && !plain; a++) {
         // the fluid node q = p - e_a looked up T at p in direction a
         int qx = gx - ex(a), qy = y - ey(a);
         if (wrap_xy(P, qx, qy) != 0) continue;
@@ -618,6 +660,14 @@ __global__ void b_stress_grad(const Params P, const Adj A, const uint8_t* __rest
         lg[k][0] = A.l_g[(2 * k) * NP + p];
         lg[k][1] = A.l_g[(2 * k + 1) * NP + p];
     }
+    // no interface here (no pair's gradient) and none of the recolouring: nothing to add
+    auto pair_acts = [&](int k, int l) {
+        const float Gx = c[l] * g[k][0] - c[k] * g[l][0], Gy = c[l] * g[k][1] - c[k] * g[l][1];
+        return Gx * Gx + Gy * Gy > 1e-24f;
+    };
+    bool any = pair_acts(0, 1) || pair_acts(0, 2) || pair_acts(1, 2);
+    for (int k = 0; k < kNF; k++) any = any || lg[k][0] != 0.f || lg[k][1] != 0.f;
+    if (!any) return;
     float lT[3];
     div_adjoint(P, A, type, gx, y, p, lT);
     float lrho = 0.f;
@@ -884,16 +934,16 @@ __global__ void b_pull(const Params P, const Adj A, const uint8_t* __restrict__ 
         const double lU = zouhe_adjoint(P, A, x == 0, i, lk);
         if (lU != 0.0) atomicAdd(A.d_u, lU);
     }
+    const int fl = (int)A.nflag[i];
+    const int xm = fl & kNodeX0 ? P.nx - 1 : -1, xp = fl & kNodeXN ? 1 - P.nx : 1;
+    const int ym = fl & kNodeY0 ? (P.ny - 1) * P.nx : -P.nx, yp = fl & kNodeYN ? (1 - P.ny) * P.nx : P.nx;
 #pragma unroll
     for (int a = 0; a < kQ; a++) {
-        int X = x - ex(a), Y = y - ey(a);
-        const int sk = wrap_xy(P, X, Y);
-        int dst = i, dir = opp(a);
-        if (sk == 2) continue;  // entered through an open side: a Zou-He unknown, no stored source
-        if (sk == 0 && !(type[Y * P.nx + X] & 2)) {
-            dst = Y * P.nx + X;
-            dir = a;
-        }
+        const bool bb = a > 0 && (fl >> a & 1);
+        const bool over = (ex(a) == 1 && (fl & kNodeX0)) || (ex(a) == -1 && (fl & kNodeXN));
+        if (zh && over) continue;  // entered through an open side: a Zou-He unknown, no stored source
+        const int dst = bb ? i : i + (ex(a) == 1 ? xm : (ex(a) == -1 ? xp : 0)) + (ey(a) == 1 ? ym : (ey(a) == -1 ? yp : 0));
+        const int dir = bb ? opp(a) : a;
         for (int k = 0; k < kNF; k++) A.l_fs[(long long)(9 * k + dir) * P.N + dst] = lk[9 * k + a];
     }
     if (zcol)
@@ -947,7 +997,7 @@ static cudaError_t amalloc(void** p, size_t b, size_t& tot)
     return cudaMalloc(p, b ? b : 16);
 }
 
-cudaError_t adjoint_alloc(const Params& P, int nw, AdjointWork** out)
+cudaError_t adjoint_alloc(const Params& P, int nw, const uint16_t* nflag, AdjointWork** out)
 {
     AdjointWork* W = new AdjointWork();
     *out = W;
@@ -961,6 +1011,7 @@ cudaError_t adjoint_alloc(const Params& P, int nw, AdjointWork** out)
     };
     Adj& S = W->A[0];
     S.nxp = P.nx + 2;
+    S.nflag = nflag;
     // shared by both views
     M((void**)&S.wline, 4 * nwz * sizeof(AdjLine));
     if (e == cudaSuccess) e = cudaMemset(S.wline, 0xff, 4 * nwz * sizeof(AdjLine));  // th = NaN: march
@@ -1071,7 +1122,7 @@ cudaError_t adjoint_prepare(const Params& P, AdjointWork* W, int t, bool wait_re
     const dim3 gp((P.nx + 2 + 127) / 128, P.ny);
     a_dens<<<gp, 128, 0, s>>>(P, A, fs, type);
     if (nw > 0)
-        a_wet<<<(unsigned)((4LL * nw + 127) / 128), 128, 0, s>>>(P, A, nw, widx, wnrm, wang, fs, type, cw_lag);
+        a_wet<<<(unsigned)((8LL * nw + 127) / 128), 128, 0, s>>>(P, A, nw, widx, wnrm, wang, fs, type, cw_lag);
     a_grad_stress<<<gp, 128, 0, s>>>(P, A, type, P.sig01, P.sig02, P.sig12);
     a_force<<<dim3((P.nx + 127) / 128, P.ny), 128, 0, s>>>(P, A, type);
     return cudaEventRecord(W->ev_a[c], s);

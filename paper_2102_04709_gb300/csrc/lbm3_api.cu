@@ -1183,7 +1183,7 @@ int lbm3_adjoint_centroid(lbm3* h, int32_t nsteps, int32_t K, double* J_out, dou
         // stays 0, as in the handle's own array
             if (e == cudaSuccess) e = cudaMemset(st.ck_c, 0, cb * nck);
         if (e == cudaSuccess) e = cudaMemset(st.sg_c, 0, cb * seglen);
-        if (e == cudaSuccess) e = adjoint_alloc(h->P, h->nw, &st.W);
+        if (e == cudaSuccess) e = adjoint_alloc(h->P, h->nw, h->gen.nflag, &st.W);
         if (e == cudaSuccess && h->ring) {
             st.box.resize(seglen);
             for (int j = 0; j < seglen && e == cudaSuccess; j++)

@@ -400,7 +400,7 @@ void launch_set_state(int store, const Params& P, const double* post, const uint
 int diag_blocks(const Params& P);
 // adjoint (lbm3_adjoint.cu)
 struct AdjointWork;
-cudaError_t adjoint_alloc(const Params& P, int nw, AdjointWork** out);
+cudaError_t adjoint_alloc(const Params& P, int nw, const uint16_t* nflag, AdjointWork** out);
 void adjoint_free(AdjointWork* W);
 size_t adjoint_bytes(const AdjointWork* W);
 double* adjoint_dang(AdjointWork* W);

@@ -1058,92 +1058,6 @@ __global__ void __launch_bounds__(TX* TY, 4) k_step_plain(const Params P, const 
 // ------------------------------------------------------------------------------------------
 // tiles of any kind: solids, domain edges, the seam, open sides
 // ------------------------------------------------------------------------------------------
-// population dir of fluid k stored at node src
-template <int STORE>
-__device__ __forceinline__ void load_fluid(const Params& P, const Pop& fin, int src, int dir, int k, float& q)
-{
-    const int N = (int)P.N;
-    if constexpr (STORE == kStoreF32) {
-        q = fin.f[src + (k * kQ + dir) * N];
-    } else {
-        const float rk = fin.rho[src + k * N];
-        const unsigned short* ob = fin.off + src + (8 * k - 1) * N;
-        if (dir > 0) {
-            q = (dir < 5 ? wq(1) : wq(5)) * rk + dec16<STORE>(ob[dir * N]);
-        } else {
-            float d[kQ];
-#pragma unroll
-            for (int a = 1; a < kQ; a++) d[a] = dec16<STORE>(ob[a * N]);
-            q = wq(0) * rk - sum_offsets(d);
-        }
-    }
-}
-
-// population dir of the three fluids stored at node src: q[0], q[9], q[18] (rest: dir is 0)
-template <int STORE>
-__device__ __forceinline__ void load_direction(const Params& P, const Pop& fin, int src, int dir, float* q)
-{
-    const int N = (int)P.N;
-    if constexpr (STORE == kStoreF32) {
-        const float* f = fin.f + src + dir * N;
-#pragma unroll
-        for (int k = 0; k < kNF; k++) q[9 * k] = f[k * kQ * N];
-    } else {
-#pragma unroll
-        for (int k = 0; k < kNF; k++) load_fluid<STORE>(P, fin, src, dir, k, q[9 * k]);
-    }
-}
-
-// storage index and flags of the fluid node at unwrapped (X, Y)
-__device__ __forceinline__ void wet_node(const Params& P, const uint16_t* __restrict__ nflag, int X, int Y, int& idx, int& fl)
-{
-    const Loc L = locate(P, X, Y);
-    idx = L.idx;
-    fl = (int)__ldg(nflag + L.idx) | (L.par ? kNodePar : 0);
-}
-
-// C_k at such a node, in the frame of the C_SB node: node_C without a search for the sources, all
-// of whose loads are issued at once (one dependent load of a class byte per direction made the
-// separate wetting pass take 20 us on the smallest grids)
-template <int STORE>
-__device__ __forceinline__ double wet_fraction(const Params& P, const Pop& fin, int idx, int fl, int k)
-{
-    const int nx = P.nx;
-    const int xm = fl & kNodeX0 ? nx - 1 : -1, xp = fl & kNodeXN ? 1 - nx : 1;
-    const int ym = fl & kNodeY0 ? (P.ny - 1) * nx : -nx, yp = fl & kNodeYN ? (1 - P.ny) * nx : nx;
-    const bool seam = P.bc_x == kModPer, open = P.bc_x == kZouHe;
-    float q[27];
-#pragma unroll
-    for (int a = 0; a < kQ; a++) {
-        const bool bb = a > 0 && (fl >> a & 1);
-        const bool over = (ex(a) == 1 && (fl & kNodeX0)) || (ex(a) == -1 && (fl & kNodeXN));
-        const int d = (ex(a) == 1 ? xm : (ex(a) == -1 ? xp : 0)) + (ey(a) == 1 ? ym : (ey(a) == -1 ? yp : 0));
-        // beyond an open side nothing is stored: the node itself is read and its value dropped
-        const int src = bb || (open && over) ? idx : idx + d;
-        load_direction<STORE>(P, fin, src, bb ? opp(a) : a, q + a);
-        if (seam && (((fl & kNodePar) != 0) != (over && !bb))) {
-            const float t = q[a];
-            q[a] = q[18 + a];
-            q[18 + a] = t;
-        }
-        if (open && over) q[a] = q[9 + a] = q[18 + a] = 0.0f;
-    }
-    if (open && (fl & (kNodeX0 | kNodeXN))) zou_he(P, q, (fl & kNodeX0) != 0);
-    float rh[kNF], rl[kNF];
-#pragma unroll
-    for (int j = 0; j < kNF; j++) sum9_df(q + 9 * j, rh[j], rl[j]);
-    float th, tl, sh, sl, dh;
-    two_sum(rh[0], rh[1], th, tl);
-    two_sum(th, rh[2], sh, sl);
-    const float dl = (tl + sl) + ((rl[0] + rl[1]) + rl[2]);
-    two_sum(sh, dl, dh, sl);
-    const float nh = k == 0 ? rh[0] : rh[1];
-    const float nl = k == 0 ? rl[0] : rl[1];
-    float qh, ql;
-    div_df(nh, nl, dh, sl, qh, ql);
-    return (double)qh + (double)ql;
-}
-
 // the w-weighted neighbour mean, where a line meets no fluid (out of line: rarely called)
 template <int STORE>
 __device__ __noinline__ double wet_mean(const Params& P, const Pop& fin, const uint8_t* __restrict__ type, int px, int py,
