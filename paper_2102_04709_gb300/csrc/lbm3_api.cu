@@ -859,14 +859,15 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
                 if (ep != cudaSuccess) cudaGetLastError();
             }
             // SMs left free for the other kernels of a step while the persistent pure-tile kernel holds
-            // its own.  Where k_step_one takes most of the pure tiles, half of them: us a step after 200
-            // and 4500 steps with 30, 60, 76 and 105 left, FP32 4096 x 2048 164 185 / 158 178 / 156 173 /
-            // 149 185, BF16 2048 x 1024 with 30 to 76 61 to 62, 83 to 87.  Where it takes them all, the
+            // its own.  Where k_step_one takes most of the pure tiles, half of them beside the FP32 kernel
+            // and 2/5 beside the 16-bit one: us a step after 200 and 4500 steps with 30, 60, 76 and 105
+            // left, FP32 4096 x 2048 164 185 / 158 178 / 156 173 / 149 185, FP16 163 184 / 163 182 /
+            // 161 194 / -, BF16 2048 x 1024 61 83 / 61 83 / 61 88 / -.  Where it takes them all, the
             // other tiles' share of the step's work, in units of a pure tile's SM time (such a tile 1.8,
             // 0.038 per C_SB node).  LBM3_SPARE_SMS=<n> in the environment at lbm3_create sets the count
             // instead.
             const double wg = 1.8 * h->n_gen + 0.038 * h->nw;
-            int spare = many ? sms / 2 : std::min(sms / 2, (int)std::lround(sms * wg / (wg + h->n_pure)));
+            int spare = many ? (f32 ? sms / 2 : sms * 2 / 5) : std::min(sms / 2, (int)std::lround(sms * wg / (wg + h->n_pure)));
             if (const char* ov = std::getenv("LBM3_SPARE_SMS"))
                 spare = std::max(0, std::min(sms - 1, std::atoi(ov)));
             h->tma_blocks = (f32 ? kTmaBlocksPerSm : kTma16BlocksPerSm) * (sms - spare);
