@@ -105,7 +105,8 @@ int lbm3_step(lbm3* h, int32_t nsteps);
  * it runs on; after the last step the call synchronises and writes the summed times in ms:
  * ms_out[0] = wetting launch (none: about 0, the wetting is part of the tiles), ms_out[1] = pure tiles
  * (no solid within 3 nodes; main stream), ms_out[2] = the other tiles (side stream).  The pure-tile
- * launches overlap the other one. */
+ * launches overlap the other one.  On small grids, where one launch takes every tile, ms_out[2] is
+ * its time and ms_out[1] about 0. */
 int lbm3_step_timed(lbm3* h, int32_t nsteps, double ms_out[3]);
 
 /* lbm3_step_timed with the device time of the run: ms_out[0] = wetting launch (none: about 0),

@@ -1438,6 +1438,7 @@ __device__ __forceinline__ bool settled_single(int around, int cnt, uint64_t wor
 //   wetting of the C_SB nodes of the phase-field region
 //   one fluid around (the words of the tiles that the halo-3 region touches, and the wall values):
 //     9 populations per own node as in k_step_one
+//   all but one fluid as traces (calm_bits): the own nodes' populations, no gradients
 //   else the pulls, phase fields, stress, force, collision and recolouring of all three fluids;
 //     where a C_SB node of the region has mixed wall values (a contact line at or near it) the
 //     phase fields are float-float, decided anew every step
@@ -1445,8 +1446,9 @@ __device__ __forceinline__ bool settled_single(int around, int cnt, uint64_t wor
 // cache misses (6 of its stalls per issued instruction on 128 x 64) in a wall tile, 18000 cycles of
 // which the wetting is 8500; so what is known early is loaded early: the tile's record in one load,
 // all that hangs on it in the next.  It takes the place of a wetting pass and two launches behind it:
-// a step of 128 x 64 takes 17.5 us instead of 27.6, of 320 x 180 17.2 instead of 27.9, of the 800 x 375
-// pillars 28.6 instead of 35.5, and of the 4096 x 2048 ones 223 instead of 240.
+// a step of 128 x 64 took 17.5 us instead of 27.6, of 320 x 180 17.2 instead of 27.9, of the 800 x 375
+// pillars 28.6 instead of 35.5, and of the 4096 x 2048 ones 223 instead of 240 (with what came after --
+// one launch per step, calm tiles -- now 15.4, 16.4, 21 and 156).
 // (Measured and left out: many steps in one cooperative launch whose blocks wait for one another, 14 to
 // 80 us where this took 12 to 44; the region's populations copied to shared memory during the wetting,
 // no gain; 256 threads a tile, each with two nodes of the region in turn, 1.5 times slower.)
@@ -1719,11 +1721,12 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
 //
 // A warp takes kOneRows rows of 32 nodes, two in flight: nothing is shared between threads, each
 // population is read once, and the loads of a warp are whole lines but for the shift by one node in x.
-// It is bound by issue (250 instructions a row, 318 with lane-wise plane addresses) and HBM, so what
-// counts is warps in flight: no shared memory, no barriers.  On the 4096 x 2048 pillars, 97 % of whose
+// It is bound by issue (261 instructions a row, 11 of them for the row's calm bits, 68 more with lane-wise
+// plane addresses) and HBM, so what counts is warps in flight: no shared memory, no barriers.  On the 4096 x 2048 pillars, 97 % of whose
 // pure tiles are such, the pure tiles took 338 us a step (FP16: 410) in the kernels that move all 27
-// planes; the whole step, all kernels, takes 174 us with this one (FP16: 176).  (Inside the ring kernel, with 9-plane boxes, the same
-// tiles took 1200 cycles of a consumer group and 1500 of its one producer each: 270 us.)
+// planes; the whole step, all kernels, takes 156 us with this one (FP16: 163).  (Inside the ring kernel,
+// with 9-plane boxes, the same tiles took 1200 cycles of a consumer group and 1500 of its one producer
+// each: 270 us.)
 constexpr int kOneThreads = 128;
 // rows of a pure tile per warp (a tile near solids: 1, there are few of them and each row waits for its
 // flags first); 8, 4 and 2 rows: 180, 175 and 182 us a step of the 4096 x 2048 pillars
