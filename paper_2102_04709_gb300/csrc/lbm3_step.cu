@@ -1721,8 +1721,10 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
 //
 // A warp takes kOneRows rows of 32 nodes, two in flight: nothing is shared between threads, each
 // population is read once, and the loads of a warp are whole lines but for the shift by one node in x.
-// It is bound by issue (261 instructions a row, 11 of them for the row's calm bits, 68 more with lane-wise
-// plane addresses) and HBM, so what counts is warps in flight: no shared memory, no barriers.  On the 4096 x 2048 pillars, 97 % of whose
+// It is bound by HBM: alone on the 4096 x 2048 pillars 82 us for 547 MB, the rate of a copy, at 261
+// instructions a row (11 of them for the row's calm bits; 68 more with lane-wise plane addresses) and 64 %
+// issue, so what counts is warps in flight: no shared memory, no barriers.  (Two rows per thread in packed
+// single-precision instructions, with 62 registers instead of 40: 158 us a step instead of 156.)  On the 4096 x 2048 pillars, 97 % of whose
 // pure tiles are such, the pure tiles took 338 us a step (FP16: 410) in the kernels that move all 27
 // planes; the whole step, all kernels, takes 156 us with this one (FP16: 163).  (Inside the ring kernel,
 // with 9-plane boxes, the same tiles took 1200 cycles of a consumer group and 1500 of its one producer
