@@ -1,6 +1,7 @@
 """The launches that a tile can be done by: those for one fluid, which move nine populations per node,
 those that move all 27 by bulk copies or plain loads, and the one launch of all tiles: the same bits,
-whichever takes it.  LBM3_ONE_TILES, LBM3_DISABLE_TMA and LBM3_CHAIN_TILES choose at lbm3_create."""
+whichever takes it.  LBM3_ONE_TILES, LBM3_DISABLE_TMA, LBM3_CHAIN_TILES and LBM3_PURE_KERNEL
+choose at lbm3_create."""
 import numpy as np
 import pytest
 
@@ -21,13 +22,18 @@ def gpu():
 
 
 def variants(gpu, monkeypatch, w, precision):
-    sims = []
-    for one, chain, plain in (("1", "0", "0"), ("1000000000", "0", "0"), ("1000000000", "0", "1"), ("1", "1000000000", "0")):
+    sims, kernels = [], [4, 2, 2, 1]
+    ways = [("1", "0", "0", ""), ("1000000000", "0", "0", ""), ("1000000000", "0", "1", ""), ("1", "1000000000", "0", "")]
+    if precision == 0 and w.nx % 4 == 0:
+        ways.append(("1", "0", "0", "tma"))  # the two-blocks-per-SM kernel takes every pure tile
+        kernels.append(2)
+    for one, chain, plain, pure in ways:
         monkeypatch.setenv("LBM3_ONE_TILES", one)
         monkeypatch.setenv("LBM3_CHAIN_TILES", chain)
         monkeypatch.setenv("LBM3_DISABLE_TMA", plain)
+        monkeypatch.setenv("LBM3_PURE_KERNEL", pure)
         sims.append(gpu.Lbm3.from_workload(w, precision=precision))
-    assert [s.info()["step_kernels"] for s in sims] == [4, 2, 2, 1]
+    assert [s.info()["step_kernels"] for s in sims] == kernels
     return sims
 
 
