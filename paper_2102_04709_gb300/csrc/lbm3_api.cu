@@ -65,13 +65,14 @@ struct lbm3 {
     void* tile_mem[5] = {};  // the arrays of the set, and the pure tiles' list
     int n_went = 0;          // entries of the wetting (gen.went), four lanes of its cache each
     long long pure_fluid = 0;
-    // fluids present per tile (one byte per warp of the ring kernel's group, so no byte needs an
-    // atomic or a clearing): pres[pp] describes the current state, the ring kernel writes the
-    // next one's for the pure and wall tiles; every other tile keeps 0x07 (all fluids), and so does
-    // every tile after the state is replaced from outside.  While pp == cur, pres[b] describes
-    // buffer pop[b]: the planes of a fluid that a tile's word does not name hold zeros there, which
-    // launch_step_one relies on to leave them unwritten.  pp turns with cur (and alone in the
-    // adjoint's slot-to-slot steps, which therefore write every plane).
+    // a word per tile, what its rows hold (one byte per row, written by one warp, so no byte needs an
+    // atomic or a clearing): pres[pp] describes the current state, and every launch of a step writes the
+    // next one's for the tiles that it advances (launch_step_tma, which does not look what they hold, as
+    // 0x07: all fluids), so that a run may go from one set of launches to another between any two steps.
+    // All words say 0x07 after the state is replaced from outside, those of tiles without a fluid node
+    // for ever.  While pp == cur, pres[b] describes buffer pop[b]: the planes of a fluid that a tile's
+    // word does not name hold zeros there, which launch_step_one relies on to leave them unwritten.  pp
+    // turns with cur (and alone in the adjoint's slot-to-slot steps, which therefore write every plane).
     uint64_t* pres[2] = {nullptr, nullptr};
     size_t pres_bytes = 0;
     int pp = 0;
@@ -358,7 +359,7 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
     // those with one (launch_step_one) beside it; the two-blocks-per-SM kernel takes them all
     if (h->n_pure > 0 && h->tma && h->precision == LBM3_FP32 && !h->ring) {
         launch_step_tma(h->P, h->tiles_pure, h->n_pure, h->tma_blocks, fo, u, h->tm_in_a[h->cur],
-                        h->tm_in_b[h->cur], h->tm_out[1 - h->cur], h->stream);
+                        h->tm_in_b[h->cur], h->tm_out[1 - h->cur], pout, h->stream);
     } else if (h->n_pure > 0) {
         const bool one = h->one;
         cudaStream_t ms = one ? h->side3 : h->stream;

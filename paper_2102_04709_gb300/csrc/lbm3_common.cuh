@@ -354,7 +354,8 @@ size_t step_tma_smem_bytes();
 cudaError_t step_tma_prepare();
 cudaError_t step_tma16_prepare();
 void launch_step_tma(const Params& P, const int* tiles, int ntiles, int nblocks, const Pop& fout, float* u,
-                     const CUtensorMap& tin_a, const CUtensorMap& tin_b, const CUtensorMap& tout, cudaStream_t s);
+                     const CUtensorMap& tin_a, const CUtensorMap& tin_b, const CUtensorMap& tout, uint64_t* pres_out,
+                     cudaStream_t s);
 // tiles around which pres_in holds one fluid, a warp each (any storage, any nx): the pure ones of the
 // list, and those of T in which nothing of the wetting changes (none of T if T.ntiles is 0); launch_tile
 // with `one`, and the launches below unless `all` is set, leave them out.  full_write: fout is not the

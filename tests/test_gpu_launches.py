@@ -1,0 +1,58 @@
+"""The launches that a step is made of on larger grids -- the persistent kernels of the pure tiles, the
+one-fluid launches, the tiles near solids beside them -- on grids small enough for the oracle, which by
+themselves would be done by one launch of every tile (LBM3_CHAIN_TILES=0 splits them); and what the
+tiles' words and cached lines say after a change from outside."""
+import pytest
+
+from paper_2102_04709_gb300 import workloads as W
+from tests.test_gpu_one_fluid import same
+
+pytestmark = pytest.mark.gpu
+
+NEVER, ALWAYS = "1000000000", "1"
+
+
+@pytest.fixture(scope="module")
+def gpu():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2102_04709_gb300 import build, lbm3
+    build.build()
+    lbm3.load()
+    return lbm3
+
+
+def choose(monkeypatch, one=NEVER, chain="0", plain="0", pure=""):
+    monkeypatch.setenv("LBM3_ONE_TILES", one)
+    monkeypatch.setenv("LBM3_CHAIN_TILES", chain)
+    monkeypatch.setenv("LBM3_DISABLE_TMA", plain)
+    monkeypatch.setenv("LBM3_PURE_KERNEL", pure)
+
+
+def pillars(nx=320, ny=120, u_in=0.05):
+    return W.pillars(nx=nx, ny=ny, count=6, r_lo=5.0, r_hi=8.0, x_lo=110.0, x_hi=280.0, gap=8.0, seed=5,
+                     drop=(60.0, 60.0), r_core=8.0, r_shell=14.0, u_in=u_in)
+
+
+# ---- the tiles' words when the launches change ----
+# A copy-wait limit other than the default takes a small grid from one launch of every tile to the split
+# ones, and back: whatever launch takes over, the words must describe the state that the others left.
+# (2^20 polls: no wait runs out.)
+@pytest.mark.parametrize("precision,pure", [(0, "tma"), (0, ""), (1, "")], ids=["fp32-tma", "fp32-ring", "fp16"])
+def test_a_change_of_the_wait_limit_keeps_the_state(gpu, monkeypatch, precision, pure):
+    w = pillars()
+    choose(monkeypatch, chain=NEVER, pure=pure)
+    a = gpu.Lbm3.from_workload(w, precision=precision)
+    b = gpu.Lbm3.from_workload(w, precision=precision)
+    assert a.info()["step_kernels"] == 1
+    for n in (41, 60):
+        a.step(20)
+        a.set_copy_wait_limit(1 << 20)
+        assert a.info()["step_kernels"] == 2
+        a.step(n)
+        a.set_copy_wait_limit(-1)
+        assert a.info()["step_kernels"] == 1
+        a.step(30)
+        b.step(20 + n + 30)
+        same(a, b)
