@@ -837,7 +837,7 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
         if (e == cudaSuccess) e = cudaMemset(h->cw[b], 0, 3 * N * sizeof(double));
     if (e == cudaSuccess) e = cudaMemset(h->u, 0, 2 * N * sizeof(float));
     const char* one_env = std::getenv("LBM3_ONE_TILES");
-    const bool many = h->n_pure >= std::max(1, one_env ? std::atoi(one_env) : kOneTiles);
+    h->one = h->n_pure >= std::max(1, one_env ? std::atoi(one_env) : kOneTiles);
     // pure tiles through bulk tensor copies where the layout allows them (row pitch a multiple of
     // 16 bytes: nx % 4 == 0 for FP32 populations, nx % 8 == 0 for 16-bit offset planes);
     // LBM3_DISABLE_TMA=1 in the environment keeps the plain kernel
@@ -859,19 +859,6 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
                 ep = f32 ? step_tma_prepare() : step_tma16_prepare();
                 if (ep != cudaSuccess) cudaGetLastError();
             }
-            // SMs left free for the other kernels of a step while the persistent pure-tile kernel holds
-            // its own.  Where k_step_one takes most of the pure tiles, half of them beside the FP32 kernel
-            // and 2/5 beside the 16-bit one: us a step after 200 and 4500 steps with 30, 60, 76 and 105
-            // left, FP32 4096 x 2048 164 185 / 158 178 / 156 173 / 149 185, FP16 163 184 / 163 182 /
-            // 161 194 / -, BF16 2048 x 1024 61 83 / 61 83 / 61 88 / -.  Where it takes them all, the
-            // other tiles' share of the step's work, in units of a pure tile's SM time (such a tile 1.8,
-            // 0.038 per C_SB node).  LBM3_SPARE_SMS=<n> in the environment at lbm3_create sets the count
-            // instead.
-            const double wg = 1.8 * h->n_gen + 0.038 * h->nw;
-            int spare = many ? (f32 ? sms / 2 : sms * 2 / 5) : std::min(sms / 2, (int)std::lround(sms * wg / (wg + h->n_pure)));
-            if (const char* ov = std::getenv("LBM3_SPARE_SMS"))
-                spare = std::max(0, std::min(sms - 1, std::atoi(ov)));
-            h->tma_blocks = (f32 ? kTmaBlocksPerSm : kTma16BlocksPerSm) * (sms - spare);
             h->tma = e == cudaSuccess && ep == cudaSuccess && sms > 0;
             // FP32: the warp-specialised ring kernel, unless LBM3_PURE_KERNEL=tma asks for the
             // two-blocks-per-SM kernel (both give the same results)
@@ -879,23 +866,31 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
             if (h->tma && f32 && !(pk && std::strcmp(pk, "tma") == 0)) {
                 bool rm = true;
                 for (int b = 0; b < 2 && rm; b++) rm = make_box_map(P, h->pop[b].f, &h->tm_box[b]);
-                if (rm && step_ring_prepare() == cudaSuccess) {
-                    h->ring = true;
-                    h->ring_blocks = sms - spare;
-                } else {
-                    cudaGetLastError();
-                }
+                h->ring = rm && step_ring_prepare() == cudaSuccess;
+                if (!h->ring) cudaGetLastError();
             }
+            // the two-blocks-per-SM kernel takes every pure tile itself
+            if (h->tma && f32 && !h->ring) h->one = false;
+            // SMs left free for the other kernels of a step while the persistent pure-tile kernel holds
+            // its own.  Where k_step_one takes most of the pure tiles, half of them beside the FP32 kernel
+            // and 2/5 beside the 16-bit one: us a step after 200 and 4500 steps with 30, 60, 76 and 105
+            // left, FP32 4096 x 2048 164 185 / 158 178 / 156 173 / 149 185, FP16 163 184 / 163 182 /
+            // 161 194 / -, BF16 2048 x 1024 61 83 / 61 83 / 61 88 / -.  Where the persistent kernel takes
+            // them all, the other tiles' share of the step's work, in units of a pure tile's SM time (such a
+            // tile 1.8, 0.038 per C_SB node).  LBM3_SPARE_SMS=<n> in the environment at lbm3_create sets
+            // the count instead.
+            const double wg = 1.8 * h->n_gen + 0.038 * h->nw;
+            int spare = h->one ? (f32 ? sms / 2 : sms * 2 / 5)
+                               : std::min(sms / 2, (int)std::lround(sms * wg / (wg + h->n_pure)));
+            if (const char* ov = std::getenv("LBM3_SPARE_SMS"))
+                spare = std::max(0, std::min(sms - 1, std::atoi(ov)));
+            h->tma_blocks = (f32 ? kTmaBlocksPerSm : kTma16BlocksPerSm) * (sms - spare);
+            if (h->ring) h->ring_blocks = sms - spare;
         }
     }
     h->gen = TileSet{n_gen, (const int*)h->tile_mem[0], (const int4*)h->tile_mem[1], (const double2*)h->tile_mem[4], h->wang, h->gen.cache,
                      h->type, (const uint16_t*)h->tile_mem[2]};
     h->tiles_pure = (const int*)h->tile_mem[3];
-    {
-        // the two-blocks-per-SM kernel takes every pure tile itself
-        const bool tma_only = h->tma && g->precision == LBM3_FP32 && !h->ring;
-        h->one = !tma_only && many;
-    }
     if (e != cudaSuccess) {
         const int code = e == cudaErrorMemoryAllocation ? LBM3_ERR_OOM : LBM3_ERR_CUDA;
         release(h);

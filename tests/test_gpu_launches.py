@@ -2,6 +2,7 @@
 one-fluid launches, the tiles near solids beside them -- on grids small enough for the oracle, which by
 themselves would be done by one launch of every tile (LBM3_CHAIN_TILES=0 splits them); and what the
 tiles' words and cached lines say after a change from outside."""
+import numpy as np
 import pytest
 
 from paper_2102_04709_gb300 import workloads as W
@@ -56,3 +57,36 @@ def test_a_change_of_the_wait_limit_keeps_the_state(gpu, monkeypatch, precision,
         a.step(30)
         b.step(20 + n + 30)
         same(a, b)
+
+
+# ---- SMs of the two-blocks-per-SM kernel ----
+def test_the_kernel_that_takes_every_pure_tile_has_the_sms_for_it(gpu, monkeypatch):
+    """The half of the SMs that the one-fluid launch gets on large grids is not taken from the kernel
+    that leaves it no tile.  With 12 SMs left (the other tiles' share here) against half of 152, a step
+    bound by that kernel takes up to 140 / 76 = 1.8 times as long; the line is drawn half way."""
+    import torch
+    nx, ny = 2048, 1024
+    rho = np.zeros((3, ny, nx))
+    rho[2] = 1.0
+    w = W.Workload("box", nx, ny, 1, W.BC_PERIODIC, np.zeros((ny, nx), np.uint8), rho, np.full((ny, nx, 3), 90.0),
+                   (0.01,) * 3, (0.1,) * 3)
+    choose(monkeypatch, one="1200", chain="1200", pure="tma")
+    monkeypatch.delenv("LBM3_SPARE_SMS", raising=False)
+    a = gpu.Lbm3.from_workload(w)
+    monkeypatch.setenv("LBM3_SPARE_SMS", "12")
+    b = gpu.Lbm3.from_workload(w)
+    assert a.info()["pure_kernel"] == "bulk copies" and a.info()["step_kernels"] == 2
+
+    def time(s):
+        e = [torch.cuda.Event(enable_timing=True) for _ in range(2)]
+        torch.cuda.synchronize()
+        e[0].record()
+        s.step(65)
+        e[1].record()
+        torch.cuda.synchronize()
+        return e[0].elapsed_time(e[1])
+
+    for s in (a, b):
+        s.step(40)
+    ratio = sorted(time(a) / time(b) for _ in range(7))
+    assert ratio[3] < 1.4
