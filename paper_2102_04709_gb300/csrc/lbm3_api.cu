@@ -9,6 +9,9 @@
 #include <string>
 #include <vector>
 
+#include <sys/mman.h>
+#include <unistd.h>
+
 #include <cudaTypedefs.h>
 
 #include "../../include/lbm3.h"
@@ -405,13 +408,24 @@ int take_kernel_error(lbm3* h)
 }
 
 // First touch of the pages of an output array: while the device still works on the steps before, instead
-// of page by page in the middle of the copy with the device waiting.  (Values widened by the device and
-// copied straight to the caller's arrays, on the 4096 x 2048 grid behind 256 steps: 6.4 ms; as floats through
-// a vector, widened by the host: 27.  128 x 64 behind 8 steps: 58 and 157 us; through pinned memory 52
-// there, but five times longer from 512 x 512 on.)
+// of page by page in the middle of the copy with the device waiting.  The values stay: a call that fails
+// later has not written to the array.  (Values widened by the device and copied straight to the caller's
+// arrays, on the 4096 x 2048 grid behind 256 steps: 6.4 ms; as floats through a vector, widened by the
+// host: 27.  128 x 64 behind 8 steps: 58 and 157 us; through pinned memory 52 there, but five times longer
+// from 512 x 512 on.)
 void touch_pages(double* p, size_t n)
 {
-    for (size_t i = 0; i < n; i += 4096 / sizeof(double)) *const_cast<volatile double*>(p + i) = 0.0;
+    if (n == 0) return;
+    const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
+    const uintptr_t from = (uintptr_t)p / page * page, to = (uintptr_t)(p + n);
+#ifdef MADV_POPULATE_WRITE
+    if (madvise((void*)from, to - from, MADV_POPULATE_WRITE) == 0) return;
+#endif
+    // a kernel without it: one word of each page, written with what it holds
+    for (size_t i = 0; i < n; i += 4096 / sizeof(double)) {
+        volatile uint64_t* w = reinterpret_cast<volatile uint64_t*>(p + i);
+        *w = *w;
+    }
 }
 
 // the state was replaced from outside: every tile may hold every fluid

@@ -2,6 +2,8 @@
 one-fluid launches, the tiles near solids beside them -- on grids small enough for the oracle, which by
 themselves would be done by one launch of every tile (LBM3_CHAIN_TILES=0 splits them); and what the
 tiles' words and cached lines say after a change from outside."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -57,6 +59,30 @@ def test_a_change_of_the_wait_limit_keeps_the_state(gpu, monkeypatch, precision,
         a.step(30)
         b.step(20 + n + 30)
         same(a, b)
+
+
+# ---- what a failed read-back leaves ----
+def test_fields_that_fail_leave_the_arrays(gpu):
+    """lbm3_fields cannot be captured (it waits for the device): it says so and writes nothing."""
+    import torch
+    w = pillars()
+    stream = torch.cuda.Stream()
+    sim = gpu.Lbm3.from_workload(w, stream=stream.cuda_stream)
+    sim.step(3)
+    want = sim.fields()
+    rho, u = np.full(3 * w.n, 7.5), np.full(2 * w.n, -2.5)
+    rt = ctypes.CDLL("libcudart.so.13")
+    handle, graph = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p()
+    assert rt.cudaStreamBeginCapture(handle, 1) == 0  # this thread's calls only
+    code = gpu.load().lbm3_fields(sim._h, gpu._dp(rho), gpu._dp(u))
+    rt.cudaStreamEndCapture(handle, ctypes.byref(graph))
+    if graph.value:
+        rt.cudaGraphDestroy(graph)
+    rt.cudaGetLastError()
+    assert code == gpu.LBM3_ERR_CUDA
+    assert (rho == 7.5).all() and (u == -2.5).all()
+    for p, q in zip(sim.fields(), want):
+        assert np.array_equal(p, q)
 
 
 # ---- SMs of the two-blocks-per-SM kernel ----
