@@ -1124,9 +1124,10 @@ int lbm3_set_state(lbm3* h, const double* f_post, const double* wall_c)
     CUDA_TRY(h, pres_reset(h));
     CUDA_TRY(h, cudaMemsetAsync(h->err_flag, 0, sizeof(int), h->stream));
     launch_set_state(h->precision, h->P, dpost, h->type, h->pop[0], h->stream);
-    // both arrays: a step writes the C_SB nodes' values only
-    for (int b = 0; b < 2; b++)
-        CUDA_TRY(h, cudaMemcpyAsync(h->cw[b], wall_c, 3 * N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+    // both arrays: a step writes the C_SB nodes' values only (the second from the first: by way of the host
+    // it made the call 8 % longer)
+    CUDA_TRY(h, cudaMemcpyAsync(h->cw[0], wall_c, 3 * N * sizeof(double), cudaMemcpyHostToDevice, h->stream));
+    CUDA_TRY(h, cudaMemcpyAsync(h->cw[1], h->cw[0], 3 * N * sizeof(double), cudaMemcpyDeviceToDevice, h->stream));
     launch_wet_look(h->P, h->gen, h->n_went, h->cw[h->pp], h->stream);
     CUDA_TRY(h, cudaMemsetAsync(h->u, 0, 2 * N * sizeof(float), h->stream));
     CUDA_TRY(h, cudaFreeAsync(dpost, h->stream));
