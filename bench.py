@@ -224,6 +224,13 @@ def bytes_moved(w, sim, per_fluid):
     return int(per_tile[pure].sum()), int(per_tile.sum()) + w.n, int(nodes[pure & one].sum())
 
 
+def pure_gbs(moved, ms_pure, ms_other, steps):
+    """GB/s of the pure tiles' launches (moved: bytes_moved's), or, where a step is one launch of every
+    tile (no time of the pure ones), of that."""
+    b, ms = (moved[0], ms_pure) if ms_pure > 0 else (moved[1], ms_other)
+    return b / (ms / steps * 1e-3) / 1e9
+
+
 # ------------------------------------------------------------------------------------------
 # CPU oracle timing
 # ------------------------------------------------------------------------------------------
@@ -335,14 +342,13 @@ def run_ours(args):
     barrier()
     t0 = time.time()
     e0.record(stream)
-    ms_wet, ms_pure, ms_wall, ms_edge, ms_run = sim.step_timed_detail(args.steps)
-    ms_gen = ms_wall + ms_edge
+    _, ms_pure, ms_gen, _, ms_run = sim.step_timed_detail(args.steps)
     e1.record(stream)
     barrier()
     t1 = time.time()
     sampler.stop()
     # the device time of exactly the K steps, from the event before the first launch to the one
-    # after the last step (e0 -> e1 also holds the host's read-back of the 7 K per-launch events,
+    # after the last step (e0 -> e1 also holds the host's read-back of the 4 K per-launch events,
     # during which the device is idle)
     ms = max_over_ranks(ms_run, ws, "cuda")
     ms_call = max_over_ranks(e0.elapsed_time(e1), ws, "cuda")
@@ -382,7 +388,7 @@ def run_ours(args):
                 w.n, E2E_LONG, ws, max_over_ranks((tb - ta) * 1e3, ws, "cuda")), "unit": "MLUPS"}
 
     # the same steps through lbm3_step itself, which replays captured CUDA graphs of 8 steps and
-    # records no per-launch events (the timed region above records five events per step so that
+    # records no per-launch events (the timed region above records four events per step so that
     # the roofline can use each kernel's own duration)
     g0 = torch.cuda.Event(enable_timing=True)
     g1 = torch.cuda.Event(enable_timing=True)
@@ -406,13 +412,13 @@ def run_ours(args):
             sim.step(args.warmup)
             barrier()
             n_alt = max(args.steps // 2, 1)
-            _, msp, _, _, arun = sim.step_timed_detail(n_alt)
+            _, msp, msg, _, arun = sim.step_timed_detail(n_alt)
             barrier()
             ams = max_over_ranks(arun, ws, "cuda")
             alt[name] = {"value": job_mlups(w.n, n_alt, ws, ams), "unit": "MLUPS",
                          "ms_per_step": ams / n_alt, "steps": n_alt,
                          "bytes_per_fluid": 72 if p == 0 else 40,
-                         "pure_kernel_gbs": bytes_moved(w, sim, 72 if p == 0 else 40)[0] / (msp / n_alt * 1e-3) / 1e9}
+                         "pure_kernel_gbs": pure_gbs(bytes_moved(w, sim, 72 if p == 0 else 40), msp, msg, n_alt)}
 
     # adjoint: J = x-centroid of fluid 0 after 2000 steps of the 512 x 256 six-pillar case,
     # gradients for every wall-node angle and the inflow velocity; every state kept on the device
@@ -462,9 +468,9 @@ def run_ours(args):
         return
     value = job_mlups(w.n, args.steps, ws, ms)
     # dominant work: the fused step on the pure tiles (72 B per node where one fluid is around, which
-    # a launch of its own takes, 216 B elsewhere; no class bytes)
-    bytes_launch = bytes_pure
-    achieved = bytes_launch / (ms_pure / args.steps * 1e-3) / 1e9
+    # a launch of its own takes, 216 B elsewhere; no class bytes); on small grids, the one launch of all
+    bytes_launch = bytes_pure if ms_pure > 0 else bytes_step
+    achieved = pure_gbs((bytes_pure, bytes_step), ms_pure, ms_gen, args.steps)
     peak, peak_src = measured_peak()
     traffic = profiled_traffic(info["pure_nodes"])
     clocks = sampler.summary(t0, t1)
@@ -477,11 +483,9 @@ def run_ours(args):
                    "alt_storage": alt, "adjoint": adj, "lbm3_step_graphs": graphs,
                    "mflups": info["n_fluid"] * args.steps * ws / (ms * 1e-3) / 1e6,
                    "l2": "populations 2 x 0.91 GB > 129 MB L2: no flush between steps",
-                   "replicas": ws, "ms_wet_per_step": ms_wet / args.steps,
+                   "replicas": ws,
                    "ms_step_pure_tiles_per_step": ms_pure / args.steps,
                    "ms_step_other_tiles_per_step": ms_gen / args.steps,
-                   "ms_step_wall_tiles_per_step": ms_wall / args.steps,
-                   "ms_step_edge_tiles_per_step": ms_edge / args.steps,
                    "ms_call_per_step": ms_call / args.steps,
                    "timing": "ms_per_step: CUDA events on the main stream around exactly the "
                              "timed steps (before the first launch, after the last step's "
@@ -494,7 +498,8 @@ def run_ours(args):
                    "max_u": float(d[5])},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic, "peak_source": peak_src,
-                     "kernel": "k_step_one (pure tiles with one fluid around) beside " +
+                     "kernel": "k_tile (every tile, one launch a step)" if ms_pure == 0 else
+                               "k_step_one (pure tiles with one fluid around) beside " +
                                {"ring": "k_step_ring (the others, warp-specialised ring of bulk "
                                         "tensor copies)",
                                 "bulk copies": "k_step_tma16 (the others, bulk tensor copies)",

@@ -103,19 +103,20 @@ int lbm3_step(lbm3* h, int32_t nsteps);
 
 /* lbm3_step with per-launch timing: CUDA events are recorded around every launch on the stream
  * it runs on; after the last step the call synchronises and writes the summed times in ms:
- * ms_out[0] = wetting launch (none: about 0, the wetting is part of the tiles), ms_out[1] = pure tiles
+ * ms_out[0] = 0 (the wetting has no launch of its own, it is part of the tiles), ms_out[1] = pure tiles
  * (no solid within 3 nodes; main stream), ms_out[2] = the other tiles (side stream).  The pure-tile
- * launches overlap the other one.  On small grids, where one launch takes every tile, ms_out[2] is
- * its time and ms_out[1] about 0. */
+ * launches overlap the other one.  On small grids, where one launch takes every tile and begins under the
+ * end of the one before, no event stands between the steps: ms_out[2] is the whole run's time and
+ * ms_out[1] 0. */
 int lbm3_step_timed(lbm3* h, int32_t nsteps, double ms_out[3]);
 
-/* lbm3_step_timed with the device time of the run: ms_out[0] = wetting launch (none: about 0),
- * ms_out[1] = pure tiles, ms_out[2] = the other tiles (solids within 3 nodes, or halo crossing the
- * domain edge), ms_out[3] = edge tiles apart from those (none: about 0), summed over the
+/* lbm3_step_timed with the device time of the run: ms_out[0] = 0 (wetting), ms_out[1] = pure tiles,
+ * ms_out[2] = the other tiles (solids within 3 nodes, or halo crossing the domain edge), ms_out[3] = 0
+ * (edge tiles have no launch of their own), summed over the
  * steps in ms, and ms_out[4] = the device time of the whole run, from the event before the first
  * step's first launch to one recorded after the last step (the host's read-back of the events
- * after the run is outside it).  Synchronises.  lbm3_step_timed's ms_out[2] is the sum of
- * ms_out[2] and ms_out[3]. */
+ * after the run is outside it).  The steps run as lbm3_step runs them: replayed from a graph, with the
+ * event records of the split launches in it.  Synchronises. */
 int lbm3_step_timed_detail(lbm3* h, int32_t nsteps, double ms_out[5]);
 
 /* Copy the current post-streaming densities rho_k (host [3][ny][nx], 0 at solid nodes) and the

@@ -322,8 +322,8 @@ bool chained(const lbm3* h) { return h->chain && h->P.wait_polls == kCopyWaitPol
 // One timestep: fork the side streams off the main stream, run the pure tiles on the main stream
 // (those with several fluids around on a side stream of their own where launch_step_one takes the
 // others) and the other tiles, with the wetting of their solid boundary nodes, on the
-// higher-priority side stream; join.  With ev != NULL the launches are bracketed by the events ev[0..6]
-// (main: 0-1 pure tiles; side: 3-4 the other tiles; 2-3 and 5-6 enclose nothing).
+// higher-priority side stream; join.  With ev != NULL the launches of such a step are bracketed by events
+// (main stream: ev[0], ev[1], the pure tiles; side stream: ev[2], ev[3], the others).
 cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
 {
     cudaError_t e;
@@ -336,11 +336,9 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
     uint64_t* pout = h->pres[1 - h->pp];
     if (chained(h)) {
         // a small grid: every tile in one launch, one step behind the other on the main stream
-        for (int j = 0; ev && j < 4; j++) record_timing(h, ev[j], h->stream);
         TileSet all = h->gen;
         all.ntiles = h->n_gen + h->n_pure;
-        e = launch_tile(h->precision, h->P, all, fin, fo, cw_out, u, pin, pout, io, false, !ev, h->stream);
-        for (int j = 4; ev && j < 7; j++) record_timing(h, ev[j], h->stream);
+        e = launch_tile(h->precision, h->P, all, fin, fo, cw_out, u, pin, pout, io, false, true, h->stream);
         if (!io) h->cur = 1 - h->cur;
         h->pp = 1 - h->pp;
         return e;
@@ -348,7 +346,6 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
     if ((e = cudaEventRecord(h->ev_fork, h->stream)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(h->side, h->ev_fork, 0)) != cudaSuccess) return e;
     if (ev) record_timing(h, ev[2], h->side);
-    if (ev) record_timing(h, ev[3], h->side);
     // steps between the adjoint's slots write every plane and wall value: the tiles all of theirs
     const bool light = h->one && !io;
     e = launch_tile(h->precision, h->P, h->gen, fin, fo, cw_out, u, pin, pout, io, light, false, h->side);
@@ -356,7 +353,7 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
     // (behind the tiles that take long: in front of them, or of the pure tiles on either stream, it delays
     // what the step waits for, 5-10 % on the 2048 x 1024 pillars)
     if (light) launch_step_one(h->precision, h->P, h->gen, nullptr, 0, fin, fo, u, pin, pout, false, h->side);
-    if (ev) record_timing(h, ev[4], h->side);
+    if (ev) record_timing(h, ev[3], h->side);
     if (ev) record_timing(h, ev[0], h->stream);
     // pure tiles: those with several fluids around through the kernel of the storage and layout,
     // those with one (launch_step_one) beside it; the two-blocks-per-SM kernel takes them all
@@ -384,8 +381,6 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
         }
     }
     if (ev) record_timing(h, ev[1], h->stream);
-    if (ev) record_timing(h, ev[5], h->side);
-    if (ev) record_timing(h, ev[6], h->side);
     if ((e = cudaEventRecord(h->ev_join, h->side)) != cudaSuccess) return e;
     if ((e = cudaStreamWaitEvent(h->stream, h->ev_join, 0)) != cudaSuccess) return e;
     if (!io) h->cur = 1 - h->cur;
@@ -961,8 +956,13 @@ int lbm3_step_timed_detail(lbm3* h, int32_t nsteps, double ms_out[5])
     if (nsteps < 0) return fail(h, LBM3_ERR_INVALID, "nsteps < 0");
     if (!h->ready) return fail(h, LBM3_ERR_STATE, "lbm3_set_fields has not been called");
     for (int j = 0; j < 5; j++) ms_out[j] = 0.0;
-    std::vector<cudaEvent_t> ev(7 * (size_t)nsteps + 1);  // 7 per step, and the end of the run
+    // The run's begin and end, and four a step around its launches -- none where a step is one launch,
+    // which begins under the end of the one before as long as no event stands between them.
+    const bool whole = chained(h);
+    std::vector<cudaEvent_t> ev(2 + (whole ? 0 : 4 * (size_t)nsteps));
     for (auto& e : ev) CUDA_TRY(h, cudaEventCreate(&e));
+    const cudaEvent_t begin = ev[0], end = ev[1];
+    auto step_events = [&](int s) { return whole ? nullptr : &ev[2 + 4 * (size_t)s]; };
     // The steps are captured into one graph with the events as record nodes, so that they run
     // as lbm3_step runs them (replayed graphs) rather than launched one by one; launched one by
     // one if the capture fails.
@@ -976,9 +976,9 @@ int lbm3_step_timed_detail(lbm3* h, int32_t nsteps, double ms_out[5])
         cudaGraphExec_t x = nullptr;
         cudaError_t ec = cudaStreamBeginCapture(h->gcap, cudaStreamCaptureModeThreadLocal);
         if (ec == cudaSuccess) {
-            cudaError_t el = cudaSuccess;
-            for (int s = 0; s < nsteps && el == cudaSuccess; s++) el = enqueue_step(h, s == nsteps - 1, &ev[7 * (size_t)s]);
-            if (el == cudaSuccess) el = cudaEventRecordWithFlags(ev.back(), h->gcap, cudaEventRecordExternal);
+            cudaError_t el = cudaEventRecordWithFlags(begin, h->gcap, cudaEventRecordExternal);
+            for (int s = 0; s < nsteps && el == cudaSuccess; s++) el = enqueue_step(h, s == nsteps - 1, step_events(s));
+            if (el == cudaSuccess) el = cudaEventRecordWithFlags(end, h->gcap, cudaEventRecordExternal);
             ec = cudaStreamEndCapture(h->gcap, &g);
             if (el != cudaSuccess) ec = el;
         }
@@ -1000,23 +1000,23 @@ int lbm3_step_timed_detail(lbm3* h, int32_t nsteps, double ms_out[5])
         }
     }
     if (!ran) {
-        for (int s = 0; s < nsteps; s++) CUDA_TRY(h, enqueue_step(h, s == nsteps - 1, &ev[7 * (size_t)s]));
-        CUDA_TRY(h, cudaEventRecord(ev.back(), h->stream));  // after the last step's joins
+        CUDA_TRY(h, cudaEventRecord(begin, h->stream));
+        for (int s = 0; s < nsteps; s++) CUDA_TRY(h, enqueue_step(h, s == nsteps - 1, step_events(s)));
+        CUDA_TRY(h, cudaEventRecord(end, h->stream));  // after the last step's joins
         CUDA_TRY(h, cudaStreamSynchronize(h->stream));
     }
-    if (nsteps > 0) {
+    auto add = [&](int j, cudaEvent_t a, cudaEvent_t b) {
         float t = 0.f;
-        CUDA_TRY(h, cudaEventElapsedTime(&t, ev[0], ev.back()));
-        ms_out[4] = t;
-    }
-    for (int s = 0; s < nsteps; s++) {
-        const cudaEvent_t* E = &ev[7 * (size_t)s];
-        const int from[4] = {2, 0, 3, 5}, to[4] = {3, 1, 4, 6};
-        for (int j = 0; j < 4; j++) {
-            float t = 0.f;
-            CUDA_TRY(h, cudaEventElapsedTime(&t, E[from[j]], E[to[j]]));
-            ms_out[j] += t;
-        }
+        const cudaError_t e = cudaEventElapsedTime(&t, a, b);
+        ms_out[j] += t;
+        return e;
+    };
+    if (nsteps > 0) CUDA_TRY(h, add(4, begin, end));
+    if (whole) ms_out[2] = ms_out[4];
+    for (int s = 0; s < nsteps && !whole; s++) {
+        const cudaEvent_t* E = step_events(s);
+        CUDA_TRY(h, add(1, E[0], E[1]));
+        CUDA_TRY(h, add(2, E[2], E[3]));
     }
     for (auto& e : ev) cudaEventDestroy(e);
     return LBM3_OK;

@@ -182,7 +182,7 @@ class Lbm3:
 
     def step_timed(self, n):
         """Advance n steps; return CUDA-event times in ms summed over the steps:
-        (wetting launch -- none, about 0 --, pure tiles, the other tiles)."""
+        (0: the wetting has no launch of its own, pure tiles, the other tiles)."""
         out = np.zeros(3)
         _check(self._h, load().lbm3_step_timed(self._h, int(n), _dp(out)))
         return float(out[0]), float(out[1]), float(out[2])

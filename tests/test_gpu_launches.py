@@ -61,6 +61,20 @@ def test_a_change_of_the_wait_limit_keeps_the_state(gpu, monkeypatch, precision,
         same(a, b)
 
 
+# ---- times of launches that a step does not have ----
+def test_times_of_the_launches_there_are(gpu, monkeypatch):
+    """The wetting and the edge tiles have no launch of their own: exactly 0.  Where a step is one launch,
+    it is all of the run, which the timing must not slow down with events between the steps."""
+    choose(monkeypatch)
+    t = gpu.Lbm3.from_workload(pillars()).step_timed_detail(20)
+    assert t[0] == 0.0 and t[3] == 0.0 and 0.0 < t[1] <= t[4] and 0.0 < t[2] <= t[4]
+    choose(monkeypatch, chain=NEVER)
+    s = gpu.Lbm3.from_workload(pillars())
+    t = s.step_timed_detail(20)
+    assert t[:2] == (0.0, 0.0) and t[3] == 0.0 and t[2] == t[4] > 0.0
+    assert s.step_timed(3)[:2] == (0.0, 0.0)
+
+
 # ---- what a failed read-back leaves ----
 def test_fields_that_fail_leave_the_arrays(gpu):
     """lbm3_fields cannot be captured (it waits for the device): it says so and writes nothing."""
