@@ -61,6 +61,51 @@ def test_a_change_of_the_wait_limit_keeps_the_state(gpu, monkeypatch, precision,
         same(a, b)
 
 
+# ---- lines and words after new wall angles ----
+# A step reads lines that the step before looked for, and looks anew only where wall values change: new
+# angles have to replace them all at once.  Against a handle made with the new angles.
+def turned(w, theta):
+    new = w.angles.copy()
+    new[..., 0], new[..., 2] = theta, 180.0 - theta
+    return new
+
+
+@pytest.mark.parametrize("precision", [0, 1], ids=["fp32", "fp16"])
+@pytest.mark.parametrize("chain", [NEVER, "0"], ids=["one-launch", "split"])
+def test_wall_angles_replaced_between_steps(gpu, monkeypatch, precision, chain):
+    w = W.janus_cylinder(nx=256, ny=128, Rs=16.0, Rj=14.0)
+    choose(monkeypatch, one=ALWAYS, chain=chain)
+    a = gpu.Lbm3.from_workload(w, precision=precision)
+    a.step(20)
+    for theta in (70.0, 50.0):
+        f, c = a.get_state()
+        w.angles = turned(w, theta)
+        b = gpu.Lbm3.from_workload(w, precision=precision)
+        b.set_state(f, c)
+        a.set_state(f, c)  # the same encoding as b's, the lines still those of the old angles
+        a.set_wall_angles(w.angles.reshape(-1, 3)[a.wall_nodes()])
+        a.step(15)
+        b.step(15)
+        same(a, b)
+
+
+# Tiles near solids whose words say that nothing of the wetting changes, until the droplet's traces come.
+# (FP32: its populations survive get_state bit for bit, so a goes on without a set_state.)
+def test_wall_angles_replaced_in_settled_tiles(gpu, monkeypatch):
+    w = pillars(u_in=0.02)
+    choose(monkeypatch, one=ALWAYS)
+    a = gpu.Lbm3.from_workload(w)
+    a.step(20)
+    for theta in (70.0, 110.0):
+        w.angles = turned(w, theta)
+        b = gpu.Lbm3.from_workload(w)
+        b.set_state(*a.get_state())
+        a.set_wall_angles(w.angles.reshape(-1, 3)[a.wall_nodes()])
+        a.step(50)
+        b.step(50)
+        same(a, b)
+
+
 # ---- times of launches that a step does not have ----
 def test_times_of_the_launches_there_are(gpu, monkeypatch):
     """The wetting and the edge tiles have no launch of their own: exactly 0.  Where a step is one launch,
