@@ -159,6 +159,34 @@ def test_every_launch_gives_the_same_bits_across_the_seam(gpu, monkeypatch, prec
         same(*sims)
 
 
+# ---- the one-fluid and the trace way against the general one, in every storage ----
+# New wall angles (here the same ones) make every tile's word say "all fluids": the step after that takes
+# no short way anywhere.
+@pytest.mark.parametrize("precision", [0, 1, 2], ids=["fp32", "fp16", "bf16"])
+@pytest.mark.parametrize("name,nx,ny,chain", [("pillars", 320, 120, NEVER), ("pillars", 320, 120, "0"),
+                                              ("pillars", 319, 123, "0"), ("capillary", 320, 60, "0"),
+                                              ("capillary", 320, 60, NEVER)],
+                         ids=["one-launch", "bulk", "plain", "seam", "seam-one-launch"])
+def test_short_ways_match_the_general_one(gpu, monkeypatch, precision, name, nx, ny, chain):
+    if name == "pillars":
+        w = pillars(nx, ny, u_in=0.02)
+    else:
+        w = W.capillary(nx=nx, ny=ny, y_lo=6, y_hi=54, s0=60, Lg=60, nu=(0.1, 0.02, 0.1))
+    choose(monkeypatch, one=ALWAYS, chain=chain)
+    a = gpu.Lbm3.from_workload(w, precision=precision)
+    b = gpu.Lbm3.from_workload(w, precision=precision)
+    angles = w.angles.reshape(-1, 3)[a.wall_nodes()]
+    for n in (60, 120):
+        a.step(n)
+        for _ in range(n):
+            b.set_wall_angles(angles)
+            b.step(1)
+        same(a, b)
+    # there were traces to leave out, below the threshold of every storage, over many tiles
+    r = np.abs(a.fields()[0])
+    assert np.count_nonzero((r > 0) & (r < 1e-14)) > nx * ny // 16
+
+
 # ---- more boundary nodes in a tile's region than two passes of the wetting take ----
 # 2 x 2 posts at a spacing of 3: every 36 x 12 region holds 192 boundary nodes, three passes of 64.  (In the
 # oracle a disturbance of 1e-7 stays below 3e-7 over 80 steps of this set-up.)
