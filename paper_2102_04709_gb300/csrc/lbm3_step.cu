@@ -415,18 +415,21 @@ __device__ __forceinline__ void stress_at(const Params& P, const int (*t)[HX], c
 // ---- what the words of the tiles say (one byte per row of 32 nodes) ----
 // Bits 0-2: the fluids that the row's nodes hold; 0 only where it has no fluid node.  Bits 3-4: 0, or
 // d + 1 where the row is calm in fluid d: every node's total populations are at least kCalmMin, its
-// density at most kCalmRho, and the share C of the two other fluids at most kCalmShare, in what is
+// density at most kCalmRho, and the share C of the two other fluids at most calm_share(), in what is
 // stored.  (Bits 5-6 of byte 0: settled_steps.)
 //
 // Where everything that can reach a node within two links is calm in the same d, the other fluids stay
 // traces there: a pulled share is the mean of its sources' with the total populations as weights
-// (between 0 and kCalmShare; in the FP16 storage, where the traces' offsets round to 0 and the sources
-// keep w_a rho_k, at most 10 times that: 1.4 / (9 / 64)), so it is at most 2e-13 at every fluid node of
-// the phase-field region, and the wall values of the C_SB nodes there are compared with that.  A gradient
-// component of such a share is at most three times as large (the extrapolation beyond a C_SB node
-// doubles one value and subtracts another), those of C_d are rounding (1e-6) and come times a share in
-// G_kl, and |G_kl|^2 < 8e-25 for every pair: below kG2Eps, so the stress of Eq.(10) and the normals of
-// Eq.(13) are exact zeros.  What the recolouring splits is then C_k f alone, from the node's own
+// (between 0 and calm_share).  In the FP16 storage the traces' offsets round to 0 and the sources keep
+// w_a rho_k: at most 10 times that, 1.4 / (9 / 64).  In BF16 an offset C (f_a - w_a rho) is off by 2^-9 of
+// itself: summed over the eight that move, |f_a - w_a rho| is at most f_a + w_a 1.4, so 1 + 10 times the
+// pulled total; in the rest population, over a node's own eight, at most 2 x 1.4, 20 times it; 31 x 2^-9 =
+// 6 % more.  So a share is at most 2.02e-13 at every fluid node of the phase-field region, and the wall
+// values of the C_SB nodes there are compared with 2e-13.  (The pulled total is at least 9 / 64: positive
+// and finite.)  A gradient component of such a share is at most three times as large (the extrapolation
+// beyond a C_SB node doubles one value and subtracts another), those of C_d are rounding (1e-6) and come
+// times a share in G_kl, and |G_kl|^2 <= 18 x (2.02e-13)^2 < 8e-25 for every pair: below kG2Eps, so the
+// stress of Eq.(10) and the normals of Eq.(13) are exact zeros.  What the recolouring splits is then C_k f alone, from the node's own
 // populations: no halo, no phase fields, no barriers.  Traces spread by a node a step and soon are
 // in most tiles (of the 512 x 512 cylinder in 95 % after 1000 steps, of which 5 % hold shares above
 // 1e-12): us a step after 1000 steps without and with this, 512 x 512 23.6 / 19.7, the 800 x 375
@@ -434,12 +437,20 @@ __device__ __forceinline__ void stress_at(const Params& P, const int (*t)[HX], c
 constexpr float kCalmMin = 1.0f / 64.0f, kCalmRho = 1.4f, kCalmWall = 2e-13f;
 __host__ __device__ constexpr float calm_share(int store) { return store == kStoreF16 ? 1.9e-14f : 1.9e-13f; }
 
+// the smaller one, or NaN where one is NaN (fminf gives the other number)
+__device__ __forceinline__ float min_nan(float a, float b)
+{
+    float m;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+    return m;
+}
 // a node's part of the above: bits 3-5 the fluids with more than a trace, bit 6 not calm at all; f: the
 // total populations that are stored
 template <int STORE>
 __device__ __forceinline__ int calm_bits(const float f[kQ], float rho, float c0, float c1, float c2)
 {
-    const float m = fminf(fminf(fminf(fminf(f[0], f[1]), fminf(f[2], f[3])), fminf(fminf(f[4], f[5]), fminf(f[6], f[7]))), f[8]);
+    const float m = min_nan(min_nan(min_nan(min_nan(f[0], f[1]), min_nan(f[2], f[3])),
+                                    min_nan(min_nan(f[4], f[5]), min_nan(f[6], f[7]))), f[8]);
     constexpr float T = calm_share(STORE);
     return (fabsf(c0) > T ? 8 : 0) | (fabsf(c1) > T ? 16 : 0) | (fabsf(c2) > T ? 32 : 0) |
            (m >= kCalmMin && rho <= kCalmRho ? 0 : 64);
@@ -864,16 +875,26 @@ __device__ __forceinline__ void store_fluid(const Params& P, const Pop& out, int
 
 // One node that holds fluid k alone, from the 9 post-streaming populations f of that fluid: its
 // velocity and, in f, its post-collision populations; the same bits as collide_node and the
-// recolouring give with the other two fluids' zeros.  false where they would not be: a density
-// whose fraction does not come out as 1 (a zero, an infinity or a NaN), which spreads to the
-// populations of the absent fluids too.
-__device__ __forceinline__ bool collide_single(const Params& P, int k, float f[kQ], float r, float& ux, float& uy)
+// recolouring give with the other two fluids' zeros.  false where they would not be, as it spreads to
+// the populations of the absent fluids too: a density whose fraction does not come out as 1 (a zero, an
+// infinity or a NaN), or an infinity or a NaN among the post-collision populations (their sum is the
+// density, so not all of them can be positive then: it is looked for where they are not calm only).
+// still: whether they are (calm_bits).
+template <int STORE>
+__device__ __forceinline__ bool collide_single(const Params& P, int k, float f[kQ], float r, float& ux, float& uy,
+                                               bool& still)
 {
     const float c = fraction(r, r);
     const float D = r * (k == 0 ? P.inv_nu0 : (k == 1 ? P.inv_nu1 : P.inv_nu2));
     const float s1 = __fdividef(D, 0.5f * D + 3.0f);
     collide_mrt_free(f, r, s1, ux, uy);
-    return c == 1.0f;
+    bool plain = c == 1.0f;
+    still = calm_bits<STORE>(f, r, 0.0f, 0.0f, 0.0f) == 0;
+    if (!still) {
+#pragma unroll
+        for (int a = 0; a < kQ; a++) plain = plain && isfinite(f[a]);
+    }
+    return plain;
 }
 
 // One node at which |G_kl| vanishes for every pair (see calm_bits), from its 9 post-streaming totals f
@@ -1551,7 +1572,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
         // ---- one fluid: as in k_step_one ----
         if (!inside) return;
         const int k = __ffs(around | wp) - 1, i = own & kGeoIdx;
-        bool plain = true;
+        bool plain = true, still = true;
         float f[kQ], r = 1.0f, ux = 0.0f, uy = 0.0f;
         if (own_fluid) {
 #pragma unroll
@@ -1562,7 +1583,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
                 load_fluid<STORE>(P, fin, s & kGeoIdx, bb ? opp(a) : a, (s & kGeoPar) && k != 1 ? 2 - k : k, f[a]);
             }
             r = sum9(f);
-            plain = collide_single(P, k, f, r, ux, uy);
+            plain = collide_single<STORE>(P, k, f, r, ux, uy, still);
         }
         const bool all = __all_sync(0xffffffffu, plain);
         if (own_fluid) {
@@ -1579,7 +1600,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
             }
         }
         const unsigned some = __ballot_sync(0xffffffffu, own_fluid);
-        const bool still = __all_sync(0xffffffffu, !own_fluid || (calm_bits<STORE>(f, r, 0.0f, 0.0f, 0.0f) == 0));
+        still = __all_sync(0xffffffffu, still);
         if (lane == 0)
             *word = (uint8_t)((some ? (all ? 1 << k | (still ? (k + 1) << 3 : 0) : 7) : 0) | (tid == 0 ? quiet << 5 : 0));
         return;
@@ -1830,8 +1851,7 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
         bool plain = true, still = true;
         if (fluid) {
             r = sum9(f);
-            plain = collide_single(P, k, f, r, ux, uy);
-            still = calm_bits<STORE>(f, r, 0.0f, 0.0f, 0.0f) == 0;
+            plain = collide_single<STORE>(P, k, f, r, ux, uy, still);
             if (uout) {
                 uout[i] = ux;
                 uout[N + i] = uy;

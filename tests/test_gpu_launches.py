@@ -187,6 +187,35 @@ def test_short_ways_match_the_general_one(gpu, monkeypatch, precision, name, nx,
     assert np.count_nonzero((r > 0) & (r < 1e-14)) > nx * ny // 16
 
 
+# ---- a region of one fluid that diverges ----
+# Opposed streams just below the largest float: within some steps populations overflow, in the middle of
+# tiles whose words name that fluid alone.  What the collision makes of them -- infinities, NaN -- spreads
+# to the absent fluids and, through a density without a fraction, to the wall values as it does in the
+# general way (all words set to "all fluids" before every step).
+@pytest.mark.parametrize("precision", [0, 2], ids=["fp32", "bf16"])
+@pytest.mark.parametrize("chain,plain", [(NEVER, "0"), ("0", "0"), ("0", "1")], ids=["one-launch", "bulk", "plain"])
+@pytest.mark.parametrize("y,x", [(30, 60), (52, 128)], ids=["away", "at-the-wall"])
+def test_one_fluid_that_overflows(gpu, monkeypatch, precision, chain, plain, y, x):
+    w = W.janus_cylinder(nx=256, ny=128, Rs=10.0, Rj=9.0, nu=(0.01, 0.01, 0.01))
+    choose(monkeypatch, one=ALWAYS, chain=chain, plain=plain)
+    a = gpu.Lbm3.from_workload(w, precision=precision)
+    b = gpu.Lbm3.from_workload(w, precision=precision)
+    angles = w.angles.reshape(-1, 3)[a.wall_nodes()]
+    f, c = a.get_state()
+    f[1, 1, y, x - 3:x + 3] += 1e35
+    f[1, 3, y, x - 3:x + 3] -= 0.875e35
+    finite = []
+    for s in (a, b):
+        s.set_state(f, c)
+    for _ in range(12):
+        b.set_wall_angles(angles)
+        for s in (a, b):
+            s.step(1)
+        same(a, b)
+        finite.append(bool(np.isfinite(a.fields()[0]).all()))
+    assert finite[1] and not finite[-1]  # when it overflowed, words had come to name one fluid
+
+
 # ---- more boundary nodes in a tile's region than two passes of the wetting take ----
 # 2 x 2 posts at a spacing of 3: every 36 x 12 region holds 192 boundary nodes, three passes of 64.  (In the
 # oracle a disturbance of 1e-7 stays below 3e-7 over 80 steps of this set-up.)
