@@ -455,11 +455,28 @@ __device__ __forceinline__ int calm_bits(const float f[kQ], float rho, float c0,
     return (fabsf(c0) > T ? 8 : 0) | (fabsf(c1) > T ? 16 : 0) | (fabsf(c2) > T ? 32 : 0) |
            (m >= kCalmMin && rho <= kCalmRho ? 0 : 64);
 }
+// Whether all populations are numbers.  (A collision keeps their sum, the density: where one of them
+// overflows, another is far below 0 or no number.  So a calm node has none that is infinite or NaN.)
+__device__ __forceinline__ bool all_finite(const float f[kQ])
+{
+    bool finite = true;
+#pragma unroll
+    for (int a = 0; a < kQ; a++) finite = finite && isfinite(f[a]);
+    return finite;
+}
 __device__ __forceinline__ int present_bits(float r0, float r1, float r2)
 {
     return (r0 != 0.0f ? 1 : 0) | (r1 != 0.0f ? 2 : 0) | (r2 != 0.0f ? 4 : 0);
 }
-// the row's byte from the OR of its nodes' bits (a row without any density has NaNs in all planes)
+// The OR of the bits of a row's nodes, by the whole warp (bits 0: no fluid node), with all fluids where a
+// collision left infinities or NaN in f: C_k f is NaN there, also for a fluid with C_k = 0.
+__device__ __forceinline__ int row_bits(int bits, const float f[kQ])
+{
+    const int v = __reduce_or_sync(0xffffffffu, bits);
+    if (!(v & 64)) return v;
+    return __any_sync(0xffffffffu, (bits & 64) && !all_finite(f)) ? v | 7 : v;
+}
+// the row's byte from that (a row without any density has NaNs in all planes)
 __device__ __forceinline__ uint8_t row_byte(int v)
 {
     const int d = v >> 3 & 7;
@@ -877,24 +894,24 @@ __device__ __forceinline__ void store_fluid(const Params& P, const Pop& out, int
 // velocity and, in f, its post-collision populations; the same bits as collide_node and the
 // recolouring give with the other two fluids' zeros.  false where they would not be, as it spreads to
 // the populations of the absent fluids too: a density whose fraction does not come out as 1 (a zero, an
-// infinity or a NaN), or an infinity or a NaN among the post-collision populations (their sum is the
-// density, so not all of them can be positive then: it is looked for where they are not calm only).
-// still: whether they are (calm_bits).
-template <int STORE>
-__device__ __forceinline__ bool collide_single(const Params& P, int k, float f[kQ], float r, float& ux, float& uy,
-                                               bool& still)
+// infinity or a NaN).  So does what all_single looks for.
+__device__ __forceinline__ bool collide_single(const Params& P, int k, float f[kQ], float r, float& ux, float& uy)
 {
     const float c = fraction(r, r);
     const float D = r * (k == 0 ? P.inv_nu0 : (k == 1 ? P.inv_nu1 : P.inv_nu2));
     const float s1 = __fdividef(D, 0.5f * D + 3.0f);
     collide_mrt_free(f, r, s1, ux, uy);
-    bool plain = c == 1.0f;
-    still = calm_bits<STORE>(f, r, 0.0f, 0.0f, 0.0f) == 0;
-    if (!still) {
-#pragma unroll
-        for (int a = 0; a < kQ; a++) plain = plain && isfinite(f[a]);
-    }
-    return plain;
+    return c == 1.0f;
+}
+// Whether that holds at every node of a row, by the whole warp: plain (what collide_single says), and no
+// infinity or NaN among the populations f after the collision.  still: whether the node is calm, then whether
+// all are; only where they are not is f looked at.  Nodes that take no part: both true.
+__device__ __forceinline__ bool all_single(bool plain, bool& still, const float f[kQ])
+{
+    const bool mine = still;
+    still = __all_sync(0xffffffffu, still);
+    if (!still) plain = plain && (mine || all_finite(f));
+    return __all_sync(0xffffffffu, plain);
 }
 
 // One node at which |G_kl| vanishes for every pair (see calm_bits), from its 9 post-streaming totals f
@@ -1077,7 +1094,7 @@ __global__ void __launch_bounds__(TX* TY, 4) k_step_plain(const Params P, const 
     }
     store_recoloured<STORE>(P, fout, i, f, rc);
     // what this warp's nodes hold, for the tiles around this one in the next step
-    const int w = __reduce_or_sync(0xffffffffu, recoloured_bits<STORE>(f, r0, r1, r2, rc));
+    const int w = row_bits(recoloured_bits<STORE>(f, r0, r1, r2, rc), f);
     if (lx == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[ly] = row_byte(w);
 }
 
@@ -1583,9 +1600,10 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
                 load_fluid<STORE>(P, fin, s & kGeoIdx, bb ? opp(a) : a, (s & kGeoPar) && k != 1 ? 2 - k : k, f[a]);
             }
             r = sum9(f);
-            plain = collide_single<STORE>(P, k, f, r, ux, uy, still);
+            plain = collide_single(P, k, f, r, ux, uy);
+            still = calm_bits<STORE>(f, r, 0.0f, 0.0f, 0.0f) == 0;
         }
-        const bool all = __all_sync(0xffffffffu, plain);
+        const bool all = all_single(plain, still, f);
         if (own_fluid) {
             if (uout) {
                 uout[i] = ux;
@@ -1600,7 +1618,6 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
             }
         }
         const unsigned some = __ballot_sync(0xffffffffu, own_fluid);
-        still = __all_sync(0xffffffffu, still);
         if (lane == 0)
             *word = (uint8_t)((some ? (all ? 1 << k | (still ? (k + 1) << 3 : 0) : 7) : 0) | (tid == 0 ? quiet << 5 : 0));
         return;
@@ -1727,7 +1744,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
         bits = recoloured_bits<STORE>(f, r0, r1, r2, rc);
     }
     // what this row's fluid nodes hold, for the tiles around in the next step
-    const int v = __reduce_or_sync(0xffffffffu, bits);
+    const int v = row_bits(bits, f);
     if (lane == 0) *word = row_byte(v);
 }
 
@@ -1851,14 +1868,22 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
         bool plain = true, still = true;
         if (fluid) {
             r = sum9(f);
-            plain = collide_single<STORE>(P, k, f, r, ux, uy, still);
+            plain = collide_single(P, k, f, r, ux, uy);
+            still = calm_bits<STORE>(f, r, 0.0f, 0.0f, 0.0f) == 0;
+            // (what all_single does otherwise; so the 16-bit storages need 40 registers instead of 48)
+            if (PURE && !still) plain = plain && all_finite(f);
             if (uout) {
                 uout[i] = ux;
                 uout[N + i] = uy;
             }
         }
-        const bool all = __all_sync(0xffffffffu, plain);
-        still = __all_sync(0xffffffffu, still);
+        bool all;
+        if constexpr (PURE) {
+            all = __all_sync(0xffffffffu, plain);
+            still = __all_sync(0xffffffffu, still);
+        } else {
+            all = all_single(plain, still, f);
+        }
         const int rowold = (int)(old >> (8 * row)) & 7;
         // fluids to write: k, and those that this row of the buffer still holds, as zeros; all of
         // them where a density has no fraction
@@ -2133,7 +2158,7 @@ __global__ void __launch_bounds__(2 * TX * TY + 32, 1) k_step_ring(const Params 
                 o[P.off_plane[k * kQ + a]] =
                     rc.C[k] * f[a] + wq(a) * (rc.Vx[k] * (float)ex(a) + rc.Vy[k] * (float)ey(a));
         // what this warp's nodes hold, for the tiles around this one in the next step
-        const int w = __reduce_or_sync(0xffffffffu, recoloured_bits<kStoreF32>(f, r0, r1, r2, rc));
+        const int w = row_bits(recoloured_bits<kStoreF32>(f, r0, r1, r2, rc), f);
         if (lane == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = row_byte(w);
         // the next tile's phase fields overwrite ch / rh only after its own barriers; the stress
         // arrays after its phase-1 barrier, by which time every thread here has read them
@@ -2588,7 +2613,7 @@ __global__ void __launch_bounds__(TX* TY, kTma16BlocksPerSm) k_step_tma16(const 
                     v[9 * k + a] = rc.C[k] * f[a] + wq(a) * (rc.Vx[k] * (float)ex(a) + rc.Vy[k] * (float)ey(a));
             store_node<STORE>(fout, P.N, i, v);
             // what this warp's nodes hold, for the tiles around this one in the next step
-            const int w = __reduce_or_sync(0xffffffffu, recoloured_bits<STORE>(f, r0, r1, r2, rc));
+            const int w = row_bits(recoloured_bits<STORE>(f, r0, r1, r2, rc), f);
             if ((tid & 31) == 0) reinterpret_cast<uint8_t*>(pres_out + tile)[tid >> 5] = row_byte(w);
         }
     }

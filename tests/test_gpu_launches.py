@@ -216,6 +216,30 @@ def test_one_fluid_that_overflows(gpu, monkeypatch, precision, chain, plain, y, 
     assert finite[1] and not finite[-1]  # when it overflowed, words had come to name one fluid
 
 
+# What a collision makes of a density just below the largest float, in the general way: infinities in the
+# planes of one fluid, NaN in those of the absent ones, which the words of the next step must name.
+@pytest.mark.parametrize("precision", [0, 1, 2], ids=["fp32", "fp16", "bf16"])
+@pytest.mark.parametrize("chain", [NEVER, "0"], ids=["one-launch", "split"])
+def test_words_after_an_overflow_in_the_general_way(gpu, monkeypatch, precision, chain):
+    w = W.janus_cylinder(nx=256, ny=128, Rs=10.0, Rj=9.0, nu=(1.0, 1.0, 1.0))
+    choose(monkeypatch, one=ALWAYS, chain=chain)
+    a = gpu.Lbm3.from_workload(w, precision=precision)
+    b = gpu.Lbm3.from_workload(w, precision=precision)
+    angles = w.angles.reshape(-1, 3)[a.wall_nodes()]
+    f, c = a.get_state()
+    f[1, 1, 53, 127] = f[1, 3, 53, 129] = f[1, 2, 52, 128] = f[1, 2, 53, 128] = 1e38
+    for s in (a, b):
+        s.set_state(f, c)  # the words say "all fluids"
+        s.step(1)
+    assert not np.isfinite(a.fields()[0]).all()
+    for _ in range(4):
+        b.set_wall_angles(angles)
+        for s in (a, b):
+            s.step(1)
+        assert np.array_equal(a.get_state()[1], b.get_state()[1], equal_nan=True)
+        same(a, b)
+
+
 # ---- more boundary nodes in a tile's region than two passes of the wetting take ----
 # 2 x 2 posts at a spacing of 3: every 36 x 12 region holds 192 boundary nodes, three passes of 64.  (In the
 # oracle a disturbance of 1e-7 stays below 3e-7 over 80 steps of this set-up.)
