@@ -1298,8 +1298,9 @@ __device__ __forceinline__ void wet_look(const Params& P, const TileSet& T, int 
 // 4 k + 2 side + end -- pull one of the up to two nodes of a line each.  The values go to the region's
 // phase fields (rho := 1 there), to S.wv and, for the nodes that the tile owns, to cw_out.  A node
 // near several tiles is wetted by each of them, with the same result: 1.6 times the work of a pass
-// over the nodes, but no launch that the tiles have to wait for.  one: the fluids around; where that
-// is one, the nodes near the region hold it alone (C_k exactly 1 or 0) and need no pull.  Returns the
+// over the nodes, but no launch that the tiles have to wait for.  one: the fluids around where all that
+// can reach the region is calm, else 7; where that is one, the nodes near the region hold it alone and
+// with a positive density (C_k exactly 1 or 0), and need no pull.  Returns the
 // fluids with a nonzero wall value (bit k), in bit 3 whether some node's values are mixed, in bit 4
 // whether a line ends in a node that is not near, and in bit 5 whether some value of a fluid other than
 // calm - 1 is more than a trace.
@@ -1463,16 +1464,17 @@ __device__ __forceinline__ int fluids_reaching(const uint64_t* __restrict__ pres
 // Bits 5-6 of a tile's word (at most 2): for how many steps the wall values of every C_SB node that the
 // tile sees have been those of the one fluid around it alone, with lines that end in nodes near it.
 // After two both arrays of wall values hold them, and while the tiles around keep holding that fluid
-// alone nothing of the wetting changes.  (The tile itself is among those, and has a fluid node, so it
+// alone, and calm, nothing of the wetting changes.  (The tile itself is among those, and has a fluid node, so it
 // is the same fluid.)
 __device__ __forceinline__ int settled_steps(uint64_t word, int around)
 {
     return __popc((unsigned)around & 7u) == 1 ? (int)(word >> 5 & 3) : 0;
 }
-// a tile that needs no wetting and holds one fluid after the pull: k_step_one's
+// a tile that needs no wetting and holds one fluid after the pull: k_step_one's (calm around, bit 3: a
+// density that became zero or NaN there would reach the wall values in this step)
 __device__ __forceinline__ bool settled_single(int around, int cnt, uint64_t word)
 {
-    return __popc((unsigned)around & 7u) == 1 && (cnt == 0 || settled_steps(word, around) == 2);
+    return __popc((unsigned)around & 7u) == 1 && (cnt == 0 || ((around & 8) && settled_steps(word, around) == 2));
 }
 
 // One step of tile T.rec[blockIdx.x] (any kind): thread t < TX TY has the tile's node t, the next ones a
@@ -1569,7 +1571,7 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
     int wp = 0;
     if (cnt > 0) {
         const int b = __reduce_or_sync(
-            0xffffffffu, wet_entries<TX, TY, STORE>(P, T, e0, cnt, around, word_calm(mine), fin, cw_out, S));
+            0xffffffffu, wet_entries<TX, TY, STORE>(P, T, e0, cnt, calm ? around : 7, word_calm(mine), fin, cw_out, S));
         if (lane == 0 && b) atomicOr(&S.wall, b);
         __syncthreads();
         df = S.wall & 8;
@@ -1804,8 +1806,9 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
         tile = __shfl_sync(0xffffffffu, r, 0);
         const int cnt = __shfl_sync(0xffffffffu, r, 2);
         const uint64_t mine = pres_in[tile];
-        around = fluids_reaching(pres_in, lane >= kTileRecHead ? r : kNoTile, mine) & 7;
+        around = fluids_reaching(pres_in, lane >= kTileRecHead ? r : kNoTile, mine);
         if (!settled_single(around, cnt, mine)) return;
+        around &= 7;
         word = mine & 0x60;  // settled it stays
     }
     if (!PURE && row0 >= P.ny - (tile / ntx) * TY) {
