@@ -67,7 +67,10 @@ typedef struct lbm3_grid {
 /* Create a simulation.  Classifies nodes into C_FI, C_FB, C_SB, C_SI (Section II.B, any of the
  * 8 D2Q9 neighbours counts as contact), computes the outward solid normal at every C_SB node
  * with the eighth-order isotropic stencil of Eq.(19)-(20), builds the compact wall list and
- * allocates device memory (owned by the handle).  All host inputs are copied.
+ * allocates device memory (owned by the handle): 299 bytes per node with FP32 storage and 203 with
+ * 16-bit offsets, of which 48 are two arrays of FP64 wall values that take turns and 24 the scratch of
+ * lbm3_fields, and 16 per tile of 32 x 8 nodes; some hundred bytes more per C_SB node and per tile near
+ * solids.  All host inputs are copied.
  *   sigma  = (sigma_01, sigma_02, sigma_12), interfacial tensions of Eq.(10), > 0
  *   nu     = kinematic viscosity of each pure fluid, > 0 (mixture by Eq.(7))
  *   beta0  = reference segregation parameter of Eq.(14) (the paper uses 0.7)
@@ -91,8 +94,8 @@ int lbm3_set_fields(lbm3* h, const double* rho);
  * the SMs that the other tiles' share of the work leaves); the other tiles run beside them on an
  * internal higher-priority stream that is joined back before the call's work completes.  On grids
  * with many pure tiles those around which one fluid is stored are advanced by a launch of their own
- * that moves that fluid's populations only (the others' are zeros there).  The results do not depend
- * on which launch takes a tile.  The velocity of the last collision of the call is recorded for
+ * that moves that fluid's populations only (the others' are zeros there).  On small grids (up to 1200
+ * tiles) a step is one launch of all of them.  The results do not depend on which launch takes a tile.  The velocity of the last collision of the call is recorded for
  * lbm3_fields / lbm3_diag.  A bulk copy that does not complete within its wait limit is reported by
  * the next lbm3_diag.  While more
  * than 8 steps remain, blocks of 8 steps are launched as one CUDA graph, captured on an internal
@@ -188,9 +191,10 @@ int lbm3_adjoint_release(lbm3* h);
  * timestep, out[4] = wetting launches
  * per timestep (0: part of the fused step), out[5] = device bytes held by the handle, out[6] = algorithmic bytes of the
  * pure-tile launch, out[7] = nodes in pure tiles, out[8] = how the pure tiles move their
- * populations: 0 plain loads, 1 bulk tensor copies with two blocks per SM, 2 bulk tensor copies
- * through the warp-specialised ring (FP32 storage; LBM3_PURE_KERNEL=tma in the environment at
- * lbm3_create selects 1 instead).  Bulk copies need nx a multiple of 4 (FP32) or 8 (16-bit
+ * populations in a launch of their own: 0 plain loads, 1 bulk tensor copies with two blocks per SM, 2
+ * bulk tensor copies through the warp-specialised ring (FP32 storage; LBM3_PURE_KERNEL=tma in the
+ * environment at lbm3_create selects 1 instead); on small grids (out[3] = 1) that kernel runs only after
+ * lbm3_set_copy_wait_limit has lowered the limit, as one launch takes every tile.  Bulk copies need nx a multiple of 4 (FP32) or 8 (16-bit
  * offsets) and are disabled by LBM3_DISABLE_TMA=1. */
 int lbm3_info(const lbm3* h, int64_t out[9]);
 

@@ -356,10 +356,10 @@ cudaError_t step_tma16_prepare();
 void launch_step_tma(const Params& P, const int* tiles, int ntiles, int nblocks, const Pop& fout, float* u,
                      const CUtensorMap& tin_a, const CUtensorMap& tin_b, const CUtensorMap& tout, uint64_t* pres_out,
                      cudaStream_t s);
-// tiles around which pres_in holds one fluid, a warp each (any storage, any nx): the pure ones of the
-// list, and those of T in which nothing of the wetting changes (none of T if T.ntiles is 0); launch_tile
-// with `one`, and the launches below unless `all` is set, leave them out.  full_write: fout is not the
-// buffer that pres_out described before this step
+// tiles around which pres_in holds one fluid (any storage, any nx): the pure ones of the list, two warps
+// each, and those of T in which nothing of the wetting changes, a warp per row (none of T if T.ntiles is
+// 0); launch_tile with `one`, and the launches below unless `all` is set, leave them out.  full_write:
+// fout is not the buffer that pres_out described before this step
 void launch_step_one(int store, const Params& P, const TileSet& T, const int* tiles, int ntiles, const Pop& fin,
                      const Pop& fout, float* u, const uint64_t* pres_in, uint64_t* pres_out, bool full_write,
                      cudaStream_t s);

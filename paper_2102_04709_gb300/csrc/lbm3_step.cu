@@ -1911,12 +1911,9 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
         }
         const bool some = PURE || __ballot_sync(0xffffffffu, fluid);
         const int byte = some ? (all ? 1 << k | (still ? (k + 1) << 3 : 0) : 7) : 0;
-        if constexpr (RW == TY)
-            word |= (uint64_t)byte << (8 * row);
-        else if (lane == 0)
+        if (lane == 0)
             reinterpret_cast<uint8_t*>(pres_out + tile)[row] = (uint8_t)(byte | (row == 0 ? (int)word : 0));
     }
-    if (RW == TY && lane == 0) pres_out[tile] = word;
 }
 
 // Pure FP32 tiles through a ring of bulk tensor copies, warp-specialised: one producer warp and
