@@ -101,7 +101,10 @@ int lbm3_set_fields(lbm3* h, const double* rho);
  * than 8 steps remain, blocks of 8 steps are launched as one CUDA graph, captured on an internal
  * stream the first time it is needed (one graph per starting population buffer) and replayed on
  * the handle's stream: the same kernels in the same order, so the results do not depend on how
- * steps are split between calls.  If a capture fails the steps are launched one by one. */
+ * steps are split between calls.  If a capture fails the steps are launched one by one.  On grids with
+ * many pure tiles those with several fluids around are counted every 256 steps or more (a kernel and a
+ * copy of four bytes to pinned memory, for which nothing waits), and the count that has arrived says on
+ * how many SMs their launch goes from then on. */
 int lbm3_step(lbm3* h, int32_t nsteps);
 
 /* lbm3_step with per-launch timing: CUDA events are recorded around every launch on the stream

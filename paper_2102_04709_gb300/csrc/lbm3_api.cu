@@ -38,12 +38,17 @@ struct lbm3 {
     // population buffer, FP32 storage: the two parts of the source box and the destination tile;
     // 16-bit storage: the density box (tm_in_a) and the offset-plane box (tm_in_b)
     bool tma = false;
-    int tma_blocks = 0;  // persistent blocks of that kernel: kTmaBlocksPerSm per SM
+    // blocks of the persistent pure-tile kernel, and the index in use: [1] where so many pure tiles are
+    // its own that it needs the SMs that [0] leaves to launch_step_one (the same where that is not
+    // launched); see count_tiles
+    int pure_blocks[2] = {0, 0};
+    int many = 0;
+    unsigned *count_dev = nullptr, *count_host = nullptr;  // its tiles when last counted (host: pinned)
+    int count_limit = 0, count_age = 0;                    // [1] from this many on; steps since the count
     CUtensorMap tm_in_a[2], tm_in_b[2], tm_out[2];
     // FP32 pure tiles through the ring kernel (one producer warp, two consumer groups, one block
-    // per SM): tensor maps of each buffer with the whole pull box, and its block count
+    // per SM): tensor maps of each buffer with the whole pull box
     bool ring = false;
-    int ring_blocks = 0;
     CUtensorMap tm_box[2];
     int* widx = nullptr;
     double* wnrm = nullptr;
@@ -90,12 +95,12 @@ struct lbm3 {
     cudaStream_t side3 = nullptr;
     cudaEvent_t ev_join3 = nullptr;
     // CUDA graphs of kGraphSteps consecutive steps (an even count: a graph starts and ends on the
-    // same population buffer), one per starting buffer, captured on the internal stream gcap
+    // same population buffer), one per starting buffer (and launch size), captured on the internal stream gcap
     // when lbm3_step first needs them and replayed on the caller's stream; dropped when a
     // captured launch argument changes (lbm3_set_inflow).  graph_off: a capture failed, so steps
     // are launched one by one (the same kernels, the same results).
     cudaStream_t gcap = nullptr;
-    cudaGraphExec_t gexec[2] = {nullptr, nullptr};
+    cudaGraphExec_t gexec[2][2] = {};  // by `many` and starting buffer
     bool graph_off = false;
     size_t bytes = 0;
     int cur = 0;
@@ -193,13 +198,14 @@ void release(lbm3* h)
     adj_release(h);
     void* ptrs[] = {h->pop[0].f, h->pop[1].f, h->pop[0].rho, h->pop[1].rho, h->pop[0].off,
                     h->pop[1].off, h->type, h->cw[0], h->cw[1], h->u, h->scratch, h->partials, h->dout,
-                    h->widx, h->wnrm, h->wang, h->err_flag, h->gen.cache, h->pres[0], h->pres[1],
+                    h->widx, h->wnrm, h->wang, h->err_flag, h->gen.cache, h->pres[0], h->pres[1], h->count_dev,
                     h->tile_mem[0], h->tile_mem[1], h->tile_mem[2], h->tile_mem[3], h->tile_mem[4]};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     h->pop[0] = h->pop[1] = Pop{nullptr, nullptr, nullptr};
-    for (int c = 0; c < 2; c++)
-        if (h->gexec[c]) cudaGraphExecDestroy(h->gexec[c]);
+    if (h->count_host) cudaFreeHost(h->count_host);
+    for (int c = 0; c < 4; c++)
+        if (h->gexec[c / 2][c % 2]) cudaGraphExecDestroy(h->gexec[c / 2][c % 2]);
     if (h->gcap) cudaStreamDestroy(h->gcap);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->ev_join) cudaEventDestroy(h->ev_join);
@@ -358,18 +364,18 @@ cudaError_t enqueue_step(lbm3* h, bool last, cudaEvent_t* ev)
     // pure tiles: those with several fluids around through the kernel of the storage and layout,
     // those with one (launch_step_one) beside it; the two-blocks-per-SM kernel takes them all
     if (h->n_pure > 0 && h->tma && h->precision == LBM3_FP32 && !h->ring) {
-        launch_step_tma(h->P, h->tiles_pure, h->n_pure, h->tma_blocks, fo, u, h->tm_in_a[h->cur],
+        launch_step_tma(h->P, h->tiles_pure, h->n_pure, h->pure_blocks[h->many], fo, u, h->tm_in_a[h->cur],
                         h->tm_in_b[h->cur], h->tm_out[1 - h->cur], pout, h->stream);
     } else if (h->n_pure > 0) {
         const bool one = h->one;
         cudaStream_t ms = one ? h->side3 : h->stream;
         if (one && (e = cudaStreamWaitEvent(ms, h->ev_fork, 0)) != cudaSuccess) return e;
         if (h->ring)
-            launch_step_ring(h->P, h->tiles_pure, h->n_pure, h->ring_blocks, fo, u,
+            launch_step_ring(h->P, h->tiles_pure, h->n_pure, h->pure_blocks[h->many], fo, u,
                              io ? *h->io_box : h->tm_box[h->cur], pin, pout, !one, ms);
         else if (h->tma)
-            launch_step_tma16(h->precision, h->P, h->tiles_pure, h->n_pure, h->tma_blocks, fo, u, h->tm_in_a[h->cur],
-                              h->tm_in_b[h->cur], pin, pout, !one, ms);
+            launch_step_tma16(h->precision, h->P, h->tiles_pure, h->n_pure, h->pure_blocks[h->many], fo, u,
+                              h->tm_in_a[h->cur], h->tm_in_b[h->cur], pin, pout, !one, ms);
         else
             launch_step_plain(h->precision, h->P, h->tiles_pure, h->n_pure, fin, fo, u, pin, pout, !one, ms);
         if (one) {
@@ -434,9 +440,10 @@ cudaError_t pres_reset(lbm3* h)
 
 void drop_graphs(lbm3* h)
 {
-    for (int c = 0; c < 2; c++) {
-        if (h->gexec[c]) cudaGraphExecDestroy(h->gexec[c]);
-        h->gexec[c] = nullptr;
+    for (int c = 0; c < 4; c++) {
+        cudaGraphExec_t& g = h->gexec[c / 2][c % 2];
+        if (g) cudaGraphExecDestroy(g);
+        g = nullptr;
     }
     if (h->adj.gexec) cudaGraphExecDestroy(h->adj.gexec);
     h->adj.gexec = nullptr;
@@ -449,7 +456,8 @@ void drop_graphs(lbm3* h)
 cudaError_t graph_block(lbm3* h)
 {
     const int c = h->cur, pc = h->pp;
-    if (!h->gexec[c] && !h->graph_off) {
+    cudaGraphExec_t& x = h->gexec[h->many][c];
+    if (!x && !h->graph_off) {
         cudaStream_t user = h->stream;
         h->stream = h->gcap;
         cudaGraph_t g = nullptr;
@@ -463,22 +471,22 @@ cudaError_t graph_block(lbm3* h)
         h->stream = user;
         h->cur = c;
         h->pp = pc;
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&h->gexec[c], g, 0);
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&x, g, 0);
         if (g) cudaGraphDestroy(g);
         if (e != cudaSuccess) {
-            h->gexec[c] = nullptr;
+            x = nullptr;
             h->graph_off = true;
             cudaGetLastError();  // a failed capture leaves no sticky error; clear the last one
         }
     }
-    if (!h->gexec[c]) {
+    if (!x) {
         for (int s = 0; s < kGraphSteps; s++) {
             const cudaError_t e = enqueue_step(h, false, nullptr);
             if (e != cudaSuccess) return e;
         }
         return cudaSuccess;
     }
-    return cudaGraphLaunch(h->gexec[c], h->stream);  // ends on buffer c again
+    return cudaGraphLaunch(x, h->stream);  // ends on buffer c again
 }
 
 // Classes and flags of the nodes of a row but for its ends, with rows on either side: nine plain reads each
@@ -503,6 +511,57 @@ __attribute__((noinline)) long long classify_inside(const uint8_t* __restrict__ 
         n_fluid += !me;
     }
     return n_fluid;
+}
+
+// The persistent pure-tile kernel's blocks.  SMs left free for the other kernels of a step while it holds its
+// own: where it takes all pure tiles, the other tiles' share of the step's work, in units of a pure tile's SM
+// time (such a tile 1.8, 0.038 per C_SB node).  Where k_step_one takes most of them, half of the SMs (beside
+// the 16-bit kernel 2/5), and 1/5 once more than 3/10 (1/5) of the pure tiles hold or have several fluids
+// around.  us a step with 76 (60), 50 and 30 left, at the share that does:
+//   FP32 4096 x 2048  0.07 159 165 169, 0.23 188 196 202, 0.30 210 211 216, 0.39 248 236 241
+//   FP32 2048 x 1024  0.13 60 62 64, 0.26 69 70 72, 0.32 77 75 78, 0.50 103 97 98, 0.72 124 116 114
+//   FP16 4096 x 2048  0.07 162 162 165, 0.19 188 188 190, 0.23 203 197 198, 0.35 262 239 230
+//   FP16 2048 x 1024  0.13 63 64 64, 0.20 68 70 68, 0.27 77 78 75, 0.45 112 113 106
+// and all of them, after 100,000 steps of FP32 4096 x 2048, 486 430 404 (457 before there was a k_step_one).
+// LBM3_SPARE_SMS=<n> in the environment at lbm3_create sets the count instead.
+cudaError_t choose_blocks(lbm3* h, int sms)
+{
+    const bool f32 = h->precision == LBM3_FP32;
+    const double wg = 1.8 * h->n_gen + 0.038 * h->nw;
+    const int share = std::min(sms / 2, (int)std::lround(sms * wg / (wg + h->n_pure)));
+    int spare[2] = {h->one ? (f32 ? sms / 2 : sms * 2 / 5) : share, h->one ? sms / 5 : share};
+    if (const char* ov = std::getenv("LBM3_SPARE_SMS"))
+        spare[0] = spare[1] = std::max(0, std::min(sms - 1, std::atoi(ov)));
+    for (int b = 0; b < 2; b++)
+        h->pure_blocks[b] = (f32 ? (h->ring ? 1 : kTmaBlocksPerSm) : kTma16BlocksPerSm) * (sms - spare[b]);
+    if (spare[0] == spare[1]) return cudaSuccess;
+    h->count_limit = (int)((long long)h->n_pure * (f32 ? 3 : 2) / 10);
+    cudaError_t e = cudaMalloc((void**)&h->count_dev, sizeof(unsigned));
+    if (e == cudaSuccess) tally(h, sizeof(unsigned));
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&h->count_host, sizeof(unsigned));
+    if (e == cudaSuccess) *h->count_host = 0;
+    return e;
+}
+
+// How many blocks the persistent kernel gets from here on.  The tiles that are its own grow in number for
+// tens of thousands of steps, as the fluids' traces spread, and it needs more SMs then (pure_blocks); the
+// blocks of a launch that find no tile cost nearly what the others cost.  So every kCountSteps steps or
+// more its tiles are counted on the device, and the host takes the count that has arrived when it comes by:
+// it never waits, an old one makes the steps no less right, and the two launches give the same bits.
+constexpr int kCountSteps = 256;
+cudaError_t count_tiles(lbm3* h, int steps)
+{
+    if (!h->count_host || chained(h)) return cudaSuccess;
+    const unsigned n = *const_cast<volatile unsigned*>(h->count_host);
+    h->many = n > (unsigned)h->count_limit;
+    h->count_age += steps;
+    if (h->count_age < kCountSteps) return cudaSuccess;
+    h->count_age = 0;
+    cudaError_t e = cudaMemsetAsync(h->count_dev, 0, sizeof(unsigned), h->stream);
+    if (e != cudaSuccess) return e;
+    launch_count(h->P, h->tiles_pure, h->n_pure, h->pres[h->pp], h->count_dev, h->stream);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    return cudaMemcpyAsync(h->count_host, h->count_dev, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream);
 }
 
 }  // namespace
@@ -892,21 +951,7 @@ int lbm3_create(lbm3** out, const lbm3_grid* g, const uint8_t* solid, const doub
             }
             // the two-blocks-per-SM kernel takes every pure tile itself
             if (h->tma && f32 && !h->ring) h->one = false;
-            // SMs left free for the other kernels of a step while the persistent pure-tile kernel holds
-            // its own.  Where k_step_one takes most of the pure tiles, half of them beside the FP32 kernel
-            // and 2/5 beside the 16-bit one: us a step after 200 and 4500 steps with 30, 60, 76 and 105
-            // left, FP32 4096 x 2048 164 185 / 158 178 / 156 173 / 149 185, FP16 163 184 / 163 182 /
-            // 161 194 / -, BF16 2048 x 1024 61 83 / 61 83 / 61 88 / -.  Where the persistent kernel takes
-            // them all, the other tiles' share of the step's work, in units of a pure tile's SM time (such a
-            // tile 1.8, 0.038 per C_SB node).  LBM3_SPARE_SMS=<n> in the environment at lbm3_create sets
-            // the count instead.
-            const double wg = 1.8 * h->n_gen + 0.038 * h->nw;
-            int spare = h->one ? (f32 ? sms / 2 : sms * 2 / 5)
-                               : std::min(sms / 2, (int)std::lround(sms * wg / (wg + h->n_pure)));
-            if (const char* ov = std::getenv("LBM3_SPARE_SMS"))
-                spare = std::max(0, std::min(sms - 1, std::atoi(ov)));
-            h->tma_blocks = (f32 ? kTmaBlocksPerSm : kTma16BlocksPerSm) * (sms - spare);
-            if (h->ring) h->ring_blocks = sms - spare;
+            if (e == cudaSuccess) e = choose_blocks(h, sms);
         }
     }
     h->gen = TileSet{n_gen, (const int*)h->tile_mem[0], (const int4*)h->tile_mem[1], (const double2*)h->tile_mem[4], h->wang, h->gen.cache,
@@ -957,7 +1002,11 @@ int lbm3_step(lbm3* h, int32_t nsteps)
     // blocks of kGraphSteps steps through the graphs while at least one step remains after them;
     // the rest, and the last step (it writes the velocity), one by one
     int s = 0;
-    for (; s + kGraphSteps < nsteps; s += kGraphSteps) CUDA_TRY(h, graph_block(h));
+    for (; s + kGraphSteps < nsteps; s += kGraphSteps) {
+        CUDA_TRY(h, count_tiles(h, kGraphSteps));
+        CUDA_TRY(h, graph_block(h));
+    }
+    CUDA_TRY(h, count_tiles(h, nsteps - s));
     for (; s < nsteps; s++) CUDA_TRY(h, enqueue_step(h, s == nsteps - 1, nullptr));
     return LBM3_OK;
 }

@@ -363,6 +363,8 @@ void launch_step_tma(const Params& P, const int* tiles, int ntiles, int nblocks,
 void launch_step_one(int store, const Params& P, const TileSet& T, const int* tiles, int ntiles, const Pop& fin,
                      const Pop& fout, float* u, const uint64_t* pres_in, uint64_t* pres_out, bool full_write,
                      cudaStream_t s);
+// adds to *out how many of the tiles hold several fluids, or have them around (not launch_step_one's)
+void launch_count(const Params& P, const int* tiles, int ntiles, const uint64_t* pres, unsigned* out, cudaStream_t s);
 // pure FP32 tiles through a ring of three bulk-copy buffers, one producer warp and two consumer
 // groups per block, one block per SM (nblocks blocks): tensor map of fin with the whole pull box
 // (kTX + 8, kTY + 6, 27) over the [27][ny][nx] buffer

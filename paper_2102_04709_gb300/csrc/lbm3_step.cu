@@ -531,6 +531,14 @@ __device__ __forceinline__ int fluids_around_warp(const uint64_t* __restrict__ p
 }
 // one fluid: k_step_one's tiles
 __device__ __forceinline__ bool one_fluid(int around) { return __popc((unsigned)around & 7u) == 1; }
+__global__ void k_count(const Params P, const int* __restrict__ tiles, const int ntiles,
+                        const uint64_t* __restrict__ pres, unsigned* __restrict__ out)
+{
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool several = t < ntiles && !one_fluid(fluids_around(pres, tiles[t], (P.nx + kTX - 1) / kTX));
+    const unsigned n = __popc(__ballot_sync(0xffffffffu, several));
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(out, n);
+}
 // In the list of tiles of the kernels that move all 27 planes: the tile is calm, no gradients needed.
 constexpr int kCalmTile = 1 << 30;
 
@@ -2697,6 +2705,11 @@ void launch_step_tma16(int store, const Params& P, const int* tiles, int ntiles,
     else
         k_step_tma16<kTX, kTY, kStoreBF16><<<nb, dim3(kTX, kTY), step_tma16_smem_bytes(), s>>>(
             P, tiles, ntiles, fout, u, trho, toff, pres_in, pres_out, all);
+}
+
+void launch_count(const Params& P, const int* tiles, int ntiles, const uint64_t* pres, unsigned* out, cudaStream_t s)
+{
+    if (ntiles > 0) k_count<<<(ntiles + 255) / 256, 256, 0, s>>>(P, tiles, ntiles, pres, out);
 }
 
 void launch_step_one(int store, const Params& P, const TileSet& T, const int* tiles, int ntiles, const Pop& fin,
