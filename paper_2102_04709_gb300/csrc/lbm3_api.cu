@@ -214,22 +214,24 @@ void release(lbm3* h)
     if (h->side) cudaStreamDestroy(h->side);
 }
 
-// From this many pure tiles on, the tiles with one fluid around are launch_step_one's, and the pure
-// ones with several run beside them on a stream of their own.  On smaller grids the fluids soon reach
-// every tile, the step waits for the tiles near solids, and two more launches cost more than they hide:
-// after 1500 steps the 512 x 512 cylinder (805 pure tiles) took 25.5 us a step with them and 22.9
-// without, the 800 x 375 pillars (865) 28.6 and 28.9, the 1030 x 517 ones (1571) 36 and 42, a
-// 1024 x 1024 cylinder (3700) 60 and 67.  LBM3_ONE_TILES=<n> in the environment at lbm3_create sets
-// another line (same results).
+// From this many pure tiles on, the tiles with one fluid around are launch_step_one's, and the pure ones
+// with several run beside them on a stream of their own.  On smaller grids the fluids soon reach every
+// tile, the step waits for the tiles near solids, and two more launches cost more than they hide.  us a step
+// with them and without, after 300, 1500 and 6000 steps: the 512 x 512 cylinder (803 pure tiles) 22.9 22.9
+// 23.0 / 18.5 19.2 19.3, a 544 x 544 one (920) 23.0 25.4 25.5 / 20.5 21.9 22.0, the 800 x 375 pillars (865)
+// 20.1 21.6 27.0 / 22.7 24.0 26.1 (one launch of all tiles 20.2 21.4 23.7), the 1030 x 517 ones (1571) 26.5
+// 30.4 38.1 / 32.7 34.7 36.2, a 1024 x 1024 cylinder (3715) 36.8 40.0 58 / 55.7 57.7 60.7.
+// LBM3_ONE_TILES=<n> in the environment at lbm3_create sets another line (same results).
 constexpr int kOneTiles = 1200;
 
 // Tiles up to which a step is one launch of all of them (k_tile, two blocks per SM: four rounds of
 // blocks), one launch behind the other with no fork to the side streams and no join, and the start of a
 // step (its record, the geometry words) under the end of the one before (programmatic dependent launch).
 // Beyond, k_tile's time for a pure tile counts: us a step with the launches beside one another and with
-// one, after 300 and 1500 steps: 128 x 64 16.3 16.5 / 15.4 15.5, 450 x 31 18.1 18.2 / 16.7 17.0,
-// 2048 x 128 (1024 tiles) 17.3 19.2 / 16.8 17.3, the 512 x 512 cylinder (1024) 21.7 23.2 / 21.7 23.6, the
-// 800 x 375 pillars (1175) 23.4 29.3 / 21.5 25.0, the 1030 x 517 ones (2145) 27.4 36.1 / 36.8 44.9.
+// one, after 300, 1500 and 6000 steps: 128 x 64 16.9 17.0 16.9 / 15.5 15.2 15.2, 450 x 31 19.0 18.8 19.7 /
+// 17.6 17.3 17.8, 2048 x 128 (1024 tiles) 17.6 17.7 19.7 / 17.5 17.7 17.8, the 512 x 512 cylinder (1024) 18.5
+// 19.2 19.3 / 18.7 19.9 20.0, a 544 x 544 one (1156) 20.5 21.9 22.0 / 19.7 21.8 22.1, the 800 x 375 pillars
+// (1175) 22.7 24.0 26.1 / 20.2 21.4 23.7, the 1030 x 517 ones (2145) 32.7 34.7 36.2 / 35.0 39.6 46.7.
 // LBM3_CHAIN_TILES=<n> in the environment at lbm3_create sets another line (same results).
 constexpr int kChainTiles = 1200;
 

@@ -433,7 +433,7 @@ __device__ __forceinline__ void stress_at(const Params& P, const int (*t)[HX], c
 // populations: no halo, no phase fields, no barriers.  Traces spread by a node a step and soon are
 // in most tiles (of the 512 x 512 cylinder in 95 % after 1000 steps, of which 5 % hold shares above
 // 1e-12): us a step after 1000 steps without and with this, 512 x 512 23.6 / 19.7, the 800 x 375
-// pillars 22.8 / 21.2 and after 6000 28.1 / 24.2; bf16 2048 x 1024 after 4500 105 / 87.
+// pillars 22.8 / 21.2 and after 6000 28.1 / 24.2.
 constexpr float kCalmMin = 1.0f / 64.0f, kCalmRho = 1.4f, kCalmWall = 2e-13f;
 __host__ __device__ constexpr float calm_share(int store) { return store == kStoreF16 ? 1.9e-14f : 1.9e-13f; }
 
@@ -1501,7 +1501,7 @@ __device__ __forceinline__ bool settled_single(int around, int cnt, uint64_t wor
 // all that hangs on it in the next.  It takes the place of a wetting pass and two launches behind it:
 // a step of 128 x 64 took 17.5 us instead of 27.6, of 320 x 180 17.2 instead of 27.9, of the 800 x 375
 // pillars 28.6 instead of 35.5, and of the 4096 x 2048 ones 223 instead of 240 (with what came after --
-// one launch per step, calm tiles -- now 15.4, 16.4, 21 and 156).
+// one launch per step, calm tiles -- now 15.5, 16.7, 20 and 160 after some hundred steps).
 // (Measured and left out: many steps in one cooperative launch whose blocks wait for one another, 14 to
 // 80 us where this took 12 to 44; the region's populations copied to shared memory during the wetting,
 // no gain; 256 threads a tile, each with two nodes of the region in turn, 1.5 times slower.)
@@ -1774,14 +1774,15 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_tile(const Params P, const 
 //
 // A warp takes kOneRows rows of 32 nodes, two in flight: nothing is shared between threads, each
 // population is read once, and the loads of a warp are whole lines but for the shift by one node in x.
-// It is bound by HBM: alone on the 4096 x 2048 pillars 82 us for 547 MB, the rate of a copy, at 261
-// instructions a row (11 of them for the row's calm bits; 68 more with lane-wise plane addresses) and 64 %
-// issue, so what counts is warps in flight: no shared memory, no barriers.  (Two rows per thread in packed
-// single-precision instructions, with 62 registers instead of 40: 158 us a step instead of 156.)  On the 4096 x 2048 pillars, 97 % of whose
-// pure tiles are such, the pure tiles took 338 us a step (FP16: 410) in the kernels that move all 27
-// planes; the whole step, all kernels, takes 156 us with this one (FP16: 163).  (Inside the ring kernel,
-// with 9-plane boxes, the same tiles took 1200 cycles of a consumer group and 1500 of its one producer
-// each: 270 us.)
+// It is bound by HBM: alone on the 4096 x 2048 pillars 85 us for 547 MB, the rate of a copy, at some 310
+// instructions a row with the tile's look-up (12.2 M for the 39,000 rows of the 2048 x 1024 ones after 1500
+// steps; 68 more with lane-wise plane addresses) and 62 % issue, so what counts is warps in flight: no shared
+// memory, no barriers, 40 registers in every storage.  (Two rows per thread in packed single-precision
+// instructions, with 62 registers: 158 us a step instead of 156.)  On the 4096 x 2048 pillars, where 93 % of
+// the pure tiles are such after 200 steps, the pure tiles took 338 us a step (FP16: 410) in the kernels that
+// move all 27 planes; the whole step, all kernels, takes 160 us with this one (FP16: 162).  (Inside the ring
+// kernel, with 9-plane boxes, the same tiles took 1200 cycles of a consumer group and 1500 of its one
+// producer each: 270 us.)
 constexpr int kOneThreads = 128;
 // rows of a pure tile per warp (a tile near solids: 1, there are few of them and each row waits for its
 // flags first); 8, 4 and 2 rows: 180, 175 and 182 us a step of the 4096 x 2048 pillars
@@ -1881,7 +1882,7 @@ __global__ void __launch_bounds__(kOneThreads) k_step_one(const Params P, const 
             r = sum9(f);
             plain = collide_single(P, k, f, r, ux, uy);
             still = calm_bits<STORE>(f, r, 0.0f, 0.0f, 0.0f) == 0;
-            // (what all_single does otherwise; so the 16-bit storages need 40 registers instead of 48)
+            // (what all_single does otherwise; with this form the 16-bit storages need 40 registers, not 48)
             if (PURE && !still) plain = plain && all_finite(f);
             if (uout) {
                 uout[i] = ux;
