@@ -422,9 +422,10 @@ void touch_pages(double* p, size_t n)
     const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
     const uintptr_t from = (uintptr_t)p / page * page, to = (uintptr_t)(p + n);
 #ifdef MADV_POPULATE_WRITE
-    if (madvise((void*)from, to - from, MADV_POPULATE_WRITE) == 0) return;
+    // (small arrays mostly have their pages: 128 x 64 pays 2 us for the system calls)
+    if (n > (1u << 17) && madvise((void*)from, to - from, MADV_POPULATE_WRITE) == 0) return;
 #endif
-    // a kernel without it: one word of each page, written with what it holds
+    // else one word of each page, written with what it holds
     for (size_t i = 0; i < n; i += 4096 / sizeof(double)) {
         volatile uint64_t* w = reinterpret_cast<volatile uint64_t*>(p + i);
         *w = *w;
