@@ -213,7 +213,9 @@ int lbm3_set_stream(lbm3* h, void* stream);
  * tiles.  lbm3_fields, lbm3_diag and lbm3_adjoint_centroid then return LBM3_ERR_CUDA once (the
  * bit is cleared when reported, and by lbm3_set_fields / lbm3_set_state, which replace the state
  * whose tiles were skipped).  polls = 0 makes every wait give up at once, which is how the error
- * path is tested without faulting or hanging anything.  The paper has no counterpart. */
+ * path is tested without faulting or hanging anything.  A grid small enough for one launch of all tiles,
+ * which makes no bulk copies, takes the split launches for as long as the limit is not the default.  The
+ * paper has no counterpart. */
 int lbm3_set_copy_wait_limit(lbm3* h, int32_t polls);
 
 /* Block until all work enqueued by the handle is done. */
